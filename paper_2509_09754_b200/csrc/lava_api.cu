@@ -298,7 +298,8 @@ lava_status lava_score_layers(const lava_layer_desc* desc, int32_t n_layers, con
     else
       rc = launch_score_sm100(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
                               v_layer_stride, vbar_in, scores, vbar_out, entropy,
-                              (char*)workspace, lay.off_sm100, st);
+                              (char*)workspace, lay.off_sm100,
+                              reinterpret_cast<double2*>((char*)workspace + lay.off_ent), st);
   } else {
     rc = launch_score_generic(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
                               v_layer_stride, vbar_in, scores, vbar_out, entropy,
@@ -308,7 +309,9 @@ lava_status lava_score_layers(const lava_layer_desc* desc, int32_t n_layers, con
   // VATP: every position's own value-row norm, then the entropy of the final scores
   rc = launch_token_norm_scale(g, n_layers, v, v_layer_stride, scores, st);
   if (rc != LAVA_OK) return rc;
-  return launch_entropy_from_scores(g, n_layers, scores, entropy, st);
+  return launch_entropy_from_scores(g, n_layers, scores, entropy,
+                                    reinterpret_cast<double2*>((char*)workspace + lay.off_ent),
+                                    nullptr, nullptr, nullptr, st);
 }
 
 lava_status lava_score_layer(const lava_layer_desc* desc, const void* q_win, const void* k,

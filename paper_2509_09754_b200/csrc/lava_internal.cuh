@@ -110,7 +110,8 @@ Sm100Layout sm100_layout(const Geom& g, int n_layers);
 lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const void* k,
                                const void* v, long long q_ls, long long k_ls, long long v_ls,
                                const float* vbar_in, float* scores, float* vbar_out,
-                               double* entropy, char* ws_base, size_t ws_off, cudaStream_t stream);
+                               double* entropy, char* ws_base, size_t ws_off, double2* ent_scratch,
+                               cudaStream_t stream);
 // Tensor maps of the query window ([layer][batch*H_q*w rows][128]) and of K
 // ([layer][H_kv][tokens][128]) in boxes of 64 x 128 bf16 elements with the 128-byte swizzle.
 lava_status encode_score_maps(const Geom& g, int n_layers, const void* q, const void* k,
@@ -133,9 +134,12 @@ lava_status launch_score_tmem(const Geom& g, int n_layers, const void* q, const 
 lava_status launch_fill_ones(float* dst, long long count, cudaStream_t stream);
 lava_status launch_token_norm_scale(const Geom& g, int n_layers, const void* v, long long v_ls,
                                     float* scores, cudaStream_t stream);
-// entropy of every (layer, sequence) from the final score array (fixed summation order)
+// entropy of every (layer, sequence) from the final score array (fixed summation order); `scratch`
+// is the entropy area of the workspace.  Hands out the value norms too where vbar_out is given.
 lava_status launch_entropy_from_scores(const Geom& g, int n_layers, const float* scores,
-                                       double* entropy, cudaStream_t stream);
+                                       double* entropy, double2* scratch, const float* vbar_in,
+                                       const unsigned* vbar_bits, float* vbar_out,
+                                       cudaStream_t stream);
 lava_status launch_wo_norm(const void* w_o, int dtype, long long rows, long long cols,
                            float* out, cudaStream_t stream);
 lava_status launch_budgets(int n_layers, int batch, const double* entropy,

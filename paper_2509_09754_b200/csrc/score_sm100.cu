@@ -974,56 +974,75 @@ entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph2_max, int 
   }
 }
 
-// Split mode: the scores of a KV head are complete only after both halves of its query group
-// have been merged in memory, so the entropy of one (layer, sequence) is summed from the final
-// score array here (fixed order: thread-strided fp32 sums of at most a few hundred terms, then
-// fp64 across lanes and warps).  Also hands out the value norms.
+// Entropy of the final score arrays (split mode, where the scores of a KV head are complete only
+// after both halves of its query group have met in memory, and the per-token value term).  Bound by
+// the read of the scores and by latency, so a problem (a layer and sequence) of more than one slice
+// gets a block per slice and a second, small launch over the slices' sums: 16 + 3 us for 28 problems
+// of 524 160 scores (59 MB) and 25 + 3 us for 256 of 80 000 (82 MB); one block per problem, each a
+// serial chain of loads, took 253 and 122 us there, a cluster of eight CTAs with one launch 67 and
+// 72 us.  Up to kEntropySlice scores the one block is enough and saves the launch.  Sums in a fixed
+// order: thread-strided fp32 sums of 32 terms, then fp64.
+constexpr int kEntropySlice = 32768;
+
+// `part` NULL: one block per problem, which finishes it; else the sums of one slice each
 __global__ void __launch_bounds__(1024)
-entropy_from_scores_kernel(Geom g, const float* scores, double* entropy, const float* vbar_in,
-                           const unsigned* vbar_bits, float* vbar_out) {
-  __shared__ double rs[32], rt[32];
-  const int prob = blockIdx.x, layer = prob / g.batch, b = prob - layer * g.batch;
+entropy_from_scores_kernel(Geom g, const float* scores, double2* part, double* entropy,
+                           const float* vbar_in, const unsigned* vbar_bits, float* vbar_out) {
   if (batch_has_short_sequence(g)) return;
+  const int prob = blockIdx.y, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
-  if (vbar_out && (int)threadIdx.x < g.n_kv_heads) {
+  if (vbar_out && blockIdx.x == 0 && (int)threadIdx.x < g.n_kv_heads) {
     const size_t head = (size_t)prob * g.n_kv_heads + threadIdx.x;
     vbar_out[head] = vbar_in ? vbar_in[head] : __uint_as_float(vbar_bits[head]);
   }
-  const float* sc = scores + (size_t)layer * g.total_scores + s.score_off;
-  const long long count = (long long)g.n_kv_heads * s.prefix;
-  double sum_s = 0.0, sum_t = 0.0;
-  for (long long i0 = threadIdx.x; i0 < count; i0 += 1024 * 256) {
-    float es = 0.f, et = 0.f;  // at most 256 terms in fp32, then fp64
-    for (long long i = i0; i < count && i < i0 + 1024LL * 256; i += 1024) {
-      const float v = sc[i];
-      if (v > 0.f) {
-        es += v;
-        et += v * __logf(v);
-      }
-    }
-    sum_s += (double)es;
-    sum_t += (double)et;
+  const int count = g.n_kv_heads * s.prefix;  // fits: H_kv * total_tokens is below 2^31
+  const int i0 = (int)min((long long)count, (long long)blockIdx.x * kEntropySlice);
+  const int n = min(kEntropySlice, count - i0);
+  const float* sc = scores + (size_t)layer * g.total_scores + s.score_off + i0;
+  float es = 0.f, et = 0.f;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n; i += 1024) {
+    const float v = sc[i];
+    es += v;
+    et += v > 0.f ? v * __logf(v) : 0.f;
+  }
+  __shared__ double2 red[32];
+  double a = (double)es, c = (double)et;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    c += __shfl_down_sync(0xffffffffu, c, o);
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_double2(a, c);
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int i = 1; i < 32; ++i) {
+    a += red[i].x;
+    c += red[i].y;
+  }
+  if (part) part[(size_t)prob * gridDim.x + blockIdx.x] = make_double2(a, c);
+  else entropy[prob] = a > 0.0 ? (log(a) - c / a) / ((double)g.n_kv_heads * (double)s.n) : 0.0;
+}
+
+__global__ void __launch_bounds__(32)
+entropy_from_slices_kernel(Geom g, const double2* part, int slices, double* entropy) {
+  if (batch_has_short_sequence(g)) return;
+  const int prob = blockIdx.x, b = prob % g.batch;
+  const SeqInfo s = seq_info(g, b);
+  const int used = min(slices, ceil_div(g.n_kv_heads * s.prefix, kEntropySlice));
+  double a = 0.0, c = 0.0;
+  for (int i = threadIdx.x; i < used; i += 32) {
+    const double2 v = part[(size_t)prob * slices + i];
+    a += v.x;
+    c += v.y;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    sum_s += __shfl_down_sync(0xffffffffu, sum_s, o);
-    sum_t += __shfl_down_sync(0xffffffffu, sum_t, o);
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    c += __shfl_down_sync(0xffffffffu, c, o);
   }
-  if ((threadIdx.x & 31) == 0) {
-    rs[threadIdx.x >> 5] = sum_s;
-    rt[threadIdx.x >> 5] = sum_t;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, c = 0.0;
-    for (int i = 0; i < 32; ++i) {
-      a += rs[i];
-      c += rt[i];
-    }
-    double e = 0.0;
-    if (a > 0.0) e = (log(a) - c / a) / ((double)g.n_kv_heads * (double)s.n);
-    entropy[(size_t)layer * g.batch + b] = e;
-  }
+  if (threadIdx.x == 0)
+    entropy[prob] = a > 0.0 ? (log(a) - c / a) / ((double)g.n_kv_heads * (double)s.n) : 0.0;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1088,10 +1107,18 @@ int lead_extra_for(int chunk_tiles) {
 }  // namespace
 
 lava_status launch_entropy_from_scores(const Geom& g, int n_layers, const float* scores,
-                                       double* entropy, cudaStream_t stream) {
-  entropy_from_scores_kernel<<<n_layers * g.batch, 1024, 0, stream>>>(g, scores, entropy, nullptr,
-                                                                      nullptr, nullptr);
-  count_launches(1);
+                                       double* entropy, double2* scratch, const float* vbar_in,
+                                       const unsigned* vbar_bits, float* vbar_out,
+                                       cudaStream_t stream) {
+  // the scratch has room for H_kv * ceil(max_seqlen / 512) sums per problem
+  const long long most = (long long)g.n_kv_heads * (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
+  const int slices = most > kEntropySlice ? (int)((most + kEntropySlice - 1) / kEntropySlice) : 1;
+  const int problems = n_layers * g.batch;
+  entropy_from_scores_kernel<<<dim3(slices, problems), 1024, 0, stream>>>(
+      g, scores, slices > 1 ? scratch : nullptr, entropy, vbar_in, vbar_bits, vbar_out);
+  if (slices > 1)
+    entropy_from_slices_kernel<<<problems, 32, 0, stream>>>(g, scratch, slices, entropy);
+  count_launches(slices > 1 ? 2 : 1);
   return check_cuda(cudaGetLastError(), "entropy launch");
 }
 
@@ -1176,7 +1203,8 @@ lava_status encode_score_maps(const Geom& g, int n_layers, const void* q, const 
 lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const void* k,
                                const void* v, long long q_ls, long long k_ls, long long v_ls,
                                const float* vbar_in, float* scores, float* vbar_out,
-                               double* entropy, char* ws_base, size_t ws_off, cudaStream_t stream) {
+                               double* entropy, char* ws_base, size_t ws_off, double2* ent_scratch,
+                               cudaStream_t stream) {
   char* ws = ws_base + ws_off;
   const Sm100Layout lay = sm100_layout(g, n_layers);
 
@@ -1242,13 +1270,14 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
   rc = check_cuda(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kThreads), args,
                                               kSmemBytes, stream), "score (sm100) launch");
   if (rc != LAVA_OK) return rc;
-  if (p.split)
-    entropy_from_scores_kernel<<<n_layers * g.batch, 1024, 0, stream>>>(g, scores, entropy, vbar_in,
-                                                                        p.vbar_bits, vbar_out);
-  else
-    entropy_finalize_sm100_kernel<<<n_layers * g.batch, 256, 0, stream>>>(
-        g, p.ent_part, lay.chunks2, p.chunk_tiles * lay.out_keys, entropy, vbar_in, p.vbar_bits,
-        vbar_out);
+  if (p.split) {
+    count_launches(1);
+    return launch_entropy_from_scores(g, n_layers, scores, entropy, ent_scratch, vbar_in, p.vbar_bits,
+                                      vbar_out, stream);
+  }
+  entropy_finalize_sm100_kernel<<<n_layers * g.batch, 256, 0, stream>>>(
+      g, p.ent_part, lay.chunks2, p.chunk_tiles * lay.out_keys, entropy, vbar_in, p.vbar_bits,
+      vbar_out);
   count_launches(2);
   return check_cuda(cudaGetLastError(), "entropy finalize launch");
 }
