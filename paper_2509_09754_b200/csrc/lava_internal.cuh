@@ -99,9 +99,9 @@ lava_status launch_score_generic(const Geom& g, int n_layers, const void* q, con
                                  const float* vbar_in, float* scores, float* vbar_out,
                                  double* entropy, char* ws, const Workspace& lay,
                                  cudaStream_t stream);
-// Blackwell tensor-core score path (bf16, head_dim 128, G*w <= 128).
+// Blackwell tensor-core score path (bf16, w 16/32/64/128, G*w <= 256).
 struct Sm100Layout {
-  int heads_total, chunks1, chunks2, out_keys;  // chunks per head at max_seqlen, pass 1 / pass 2
+  int heads_total, chunks, out_keys;            // chunks: per head at max_seqlen
   int chunk_tiles;                              // tiles per chunk chosen for this launch
   size_t off_sync, sync_bytes, off_part, off_ent, total;
 };
@@ -112,7 +112,7 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
                                const float* vbar_in, float* scores, float* vbar_out,
                                double* entropy, char* ws_base, size_t ws_off, double2* ent_scratch,
                                cudaStream_t stream);
-// Tensor maps of the query window ([layer][batch*H_q*w rows][128]) and of K
+// Tensor maps of the single-pass kernel: the query window ([layer][batch*H_q*w rows][128]) and K
 // ([layer][H_kv][tokens][128]) in boxes of 64 x 128 bf16 elements with the 128-byte swizzle.
 lava_status encode_score_maps(const Geom& g, int n_layers, const void* q, const void* k,
                               long long q_ls, long long k_ls, CUtensorMap* map_q,

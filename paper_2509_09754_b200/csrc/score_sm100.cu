@@ -1,31 +1,41 @@
-// LAVa score, Blackwell path: bf16, head_dim 128, w in {16, 32, 64, 128}, up to 256 window-query
-// rows per KV head (a unit holds at most 128; larger query groups run as two units).
+// LAVa score, Blackwell path: bf16, head_dim 64 or 128, w in {16, 32, 64, 128}, up to 256
+// window-query rows per KV head (a unit holds at most 128; larger query groups run as two units).
 //
 // One persistent, warp-specialised kernel (one CTA per SM, cooperative launch so that every CTA
 // is resident) runs two pipelines over 128-key tiles of K, both fed by TMA into 128B-swizzled
 // shared memory and contracted with tcgen05.mma into TMEM:
 //
 //   pass 1 (statistics)  S = Q_g K^T  (rows = the unit's window queries, columns = keys)
-//       one thread per row reads its TMEM lane and keeps a running (max, sum of exp2) over the
-//       keys the query may see (Sec. 2: softmax over i <= j).  Work is dealt to CTAs in chunks
-//       of consecutive tiles of one head; a chunk's statistics leave the CTA once, through a
-//       publisher warp that also counts the head's published chunks.  Seven more warps stream
-//       the chunk's V rows for the value norm (Theorem 1: max_k ||V[k]||_1).
+//       one thread per row reads its TMEM lane and sums exp2 over the keys the query may see
+//       (Sec. 2: softmax over i <= j).  Work is dealt to CTAs in chunks of consecutive tiles of
+//       one head; a chunk's statistics leave the CTA once, through a publisher warp that also
+//       counts the head's published chunks.  Two more warps stream the chunk's V rows for the
+//       value norm (Theorem 1: max_k ||V[k]||_1).
 //   pass 2 (scores)      S^T = K Q_g^T (rows = keys, columns = window queries)
 //       one thread per key: a_h[i] = (1/w) sum_t exp2(z - lse_t) per query head in registers,
 //       pooled over the token axis through shared memory, scaled by Vbar * c_hat, reduced with
 //       the GQA group maximum, written once; entropy sums go to ordered per-chunk slots
 //       (Definition 1, Sec. 4.2, Sec. 4.3, Sec. 5.1 pooling).
 //
-// The exponentials bound the kernel, so the eight consumer warps are not split by pass: two
-// groups of four warps each own one TMEM buffer of BOTH pipelines and take their tiles in a
-// static order that alternates the passes, which keeps two exp-issuing warps on every scheduler.
+// Both passes use the same chunks.  Pass 1 of a CTA runs ahead of its own pass 2 by at most
+// `lead_slots` tiles (the pass-1 producer waits); pass 2 of a chunk waits for the head's statistics
+// from every CTA that holds a part of the head.  The lead is long enough for those waits to end and
+// short enough for pass 2 to find its K tiles in L2.
 //
-// Pass 2 trails pass 1 by a bounded number of tiles (K tiles are loaded with an evict-last hint
-// in pass 1 and evict-first in pass 2, V rows with evict-first), so part of its K tiles are
-// still in L2; how many depends on the chunk length (see chunk_tiles_for).  Every wait
-// (mbarrier, head counters) is bounded in time; on expiry the kernel sets
-// LAVA_DEV_WAIT_EXPIRED, drains its copies, frees TMEM and returns.
+// Sixteen consumer warps, four per scheduler, take the exponentials (two per logit): two groups of
+// four warps per pass, each with its own TMEM buffer, so that the loads, reductions, pooling and
+// hand-overs of one group run under the exponentials of the other three.
+//
+// Bound: 2 * G * w exponentials per key at 16 per clock and SM (0.53 ms for 32 layers x 32K tokens at
+// 32/8 heads, w 32) and K + V once from HBM plus K once from L2 (0.66 ms); measured 0.98 ms there
+// (1.17 ms with eight consumer warps that alternated the passes, the predecessor of this kernel).
+// What is left is mostly pass 2 waiting for a head's statistics.
+//
+// Every wait (mbarrier, head counters, chunk records, lead) is bounded in time; on expiry the
+// kernel sets LAVA_DEV_WAIT_EXPIRED, every role leaves at its next chunk, copies are drained, TMEM
+// is freed and the kernel returns.
+#include <type_traits>
+
 #include "sm100_ptx.cuh"
 
 namespace lava {
@@ -34,14 +44,15 @@ namespace {
 using namespace sm100;
 
 constexpr int kTile = 128;           // keys per tile
-constexpr int kThreads = 640;        // 20 warps: 5 service, 8 consumer, 7 value-norm
-constexpr int kVWarps = 7;
-constexpr int kVRows = kVWarps * 2;  // V rows per load step (16 threads per row)
-constexpr int kMma2Warp = 19;        // issues the pass-2 MMAs (warp 2 issues pass 1)
-constexpr int kStages = 2;           // K stages per pipeline
+constexpr int kVWarps = 2;
+constexpr int kFirstConsumer = 4;    // warps 4..11 pass 1, 12..19 pass 2
+constexpr int kPubWarp = 20, kFirstPrep = 21, kPrepWarps = 4, kFirstV = kFirstPrep + kPrepWarps;
+constexpr int kThreads = 32 * (kFirstV + kVWarps);
+constexpr int kVRows = 32;           // V rows per stage
+constexpr int kRing = 16;            // chunk records a CTA keeps
+constexpr int kMaxLeadChunks = 12;   // pass 1 is never further ahead than this (see Chunk)
 constexpr int kMaxBatch = 512;       // sequences the in-kernel chunk schedule can index
-constexpr uint32_t kTileBytes = 128 * 128 * 2;  // one [128 x 128] bf16 tile = 2 swizzled blocks
-constexpr uint32_t kHalfBytes = kTileBytes / 2;
+constexpr uint32_t kBlockBytes = 128 * 64 * 2;  // one 128-row, 64-column swizzled block
 
 // shared memory map (bytes from a 1024-aligned base)
 // Two small operands in the un-swizzled K-major layout (8 x 16-byte core matrices, 128 B apart
@@ -52,126 +63,211 @@ constexpr uint32_t kHalfBytes = kTileBytes / 2;
 constexpr uint32_t kOffOnes = 0;
 constexpr uint32_t kOffBias = 4096;          // two slots of 4 KB
 constexpr uint32_t kSmallTileBytes = 4096;
-constexpr uint32_t kOffQ1 = 16384;
-constexpr uint32_t kOffQ2 = kOffQ1 + kTileBytes;
-constexpr uint32_t kOffK1 = kOffQ2 + kTileBytes;
-constexpr uint32_t kOffK2 = kOffK1 + kStages * kTileBytes;
-constexpr uint32_t kOffMisc = kOffK2 + kStages * kTileBytes;  // 16 KB + 192 KB
-constexpr uint32_t kMiscBytes = 15360;
-constexpr uint32_t kSmemBytes = kOffMisc + kMiscBytes + 1024;  // + alignment slack
-
-struct Prep {                 // what the score warps need to know about a head
-  float scale;                // Vbar * c_hat
-  float pad[3];
+constexpr uint32_t kOffQ1 = 12288;
+constexpr uint32_t kMiscBytes = 19456;
+// K is loaded in blocks of 64 columns (16 KB), each a stage of its own: a block is free again after
+// its own four MMAs, and the shared memory that the query tiles leave divides more evenly between
+// the passes.  V has kV pieces of 32 rows per warp.
+template <int D>
+struct Smem {
+  static constexpr int kBlocks = D / 64;                          // blocks per tile
+  static constexpr int kK1 = D == 128 ? 3 : 4, kK2 = D == 128 ? 3 : 4, kV = D == 128 ? 2 : 4;
+  static constexpr uint32_t kTileBytes = kBlockBytes * kBlocks;   // [128 x D] bf16
+  static constexpr uint32_t kVBytes = kVRows * 128 * kBlocks;     // [32 x D] bf16
+  static constexpr uint32_t kOffQ2 = kOffQ1 + kTileBytes;
+  static constexpr uint32_t kOffK1 = kOffQ2 + kTileBytes;
+  static constexpr uint32_t kOffK2 = kOffK1 + kK1 * kBlockBytes;
+  static constexpr uint32_t kOffV = kOffK2 + kK2 * kBlockBytes;
+  static constexpr uint32_t kOffMisc = kOffV + kVWarps * kV * kVBytes;
+  static constexpr uint32_t kBytes = kOffMisc + kMiscBytes + 1024;  // + alignment slack
 };
 
+// What the roles need to know about a chunk.  The pass-1 producer, which is the first to need it,
+// decodes a chunk once and leaves the record in a ring in shared memory; with the index arithmetic
+// in every role, the integer divisions and the instruction fetches they cost outweighed the
+// exponentials.  A record is overwritten kRing chunks later: the producer is at most kMaxLeadChunks
+// + 1 chunks ahead of pass 2, pass 2 of a chunk waits for the chunk's value norm and statistics, and
+// the pass-1 roles are ahead of both.
+struct Chunk {
+  int ord;     // the CTA's ordinal of the chunk
+  int rhead;   // linear KV head index = (layer * batch + b) * H_kv + kvh (value norms)
+  int head;    // linear index of the scored unit (a KV head, or one half of its query group in
+               // split mode): counters, chunk partials and entropy slots are per unit
+  int layer, kvh;
+  int half;    // which half of the query group (0 unless split)
+  int q_row0;  // first row of the unit in the query-window matrix of a layer
+  int group;   // query heads of the unit
+  int slot;    // head * cph_max + chunk number inside the head: index of the chunk's scratch
+  int cph;     // chunks of this head
+  int tile1, n1, tile2, n2;  // first tile and number of tiles, pass 1 and pass 2
+  int n, prefix, tok0;       // the sequence
+  long long score_base;      // first score of the KV head
+};
+
+constexpr int kMaxStages = 4;
 struct Misc {
-  unsigned long long k1_full[kStages], k1_empty[kStages], k2_full[kStages], k2_empty[kStages];
+  unsigned long long k1_full[kMaxStages], k1_empty[kMaxStages], k2_full[kMaxStages],
+      k2_empty[kMaxStages], v_full[kVWarps][kMaxStages];
   unsigned long long q1_full, q1_empty, q2_full, q2_empty;
   unsigned long long s1_full[2], s1_empty[2], s2_full[2], s2_empty[2];
-  unsigned long long pub_full[2], pub_empty[2], prep_full[2], prep_empty[2];
-  unsigned long long gsync[2];        // rendezvous of the four warps of a consumer group
+  unsigned long long pub_full[2], pub_empty[2], prep_full[2], prep_empty[2], fold_full[2];
   unsigned long long drain, drain2;
   uint32_t tmem_base;
   volatile int abort_flag;
   long long wait_cycles;              // limit of the waits that an abort may end (launch parameter)
-  int sched_total1, sched_total2;     // chunks per layer of pass 1 / pass 2
-  int lead_tiles;                     // tile slots pass 1 runs ahead of pass 2 in a CTA's order
+  int sched_total;                    // chunks per layer
+  int lead_slots;                     // tile slots pass 1 may be ahead of pass 2 in a CTA
+  volatile int p2_slot;               // first pass-2 tile slot that has not been issued yet
+  volatile int go[2][2];              // [parity][group]: pass-2 group takes the next chunk
+  int ck_count;                       // chunk records written so far
+  float scale[2];                     // Vbar * c_hat of a prepared chunk's head
   alignas(16) float pub[2][2][128];   // [slot][group][query]: log2-sum-exp of a finished chunk
-  Prep prep[2];
+  float fold[2][kPrepWarps][128];     // [slot][prep warp][query]: log2-sum-exp of its chunks
   alignas(16) float a[2][2][4][kTile];  // [group][tile parity][query head][key]: window means
-  int pref1[kMaxBatch + 1], pref2[kMaxBatch + 1];  // exclusive scans of chunks per sequence
+  alignas(16) Chunk ring[kRing];
+  int pref[kMaxBatch + 1];            // exclusive scan of chunks per sequence
 };
 static_assert(sizeof(Misc) <= kMiscBytes, "misc region too small");
 
 struct Sm100Params {
   Geom g;
   int n_layers;
-  int chunk_tiles;          // tiles per chunk
+  int chunk_tiles;          // pass-1 tiles per chunk
+  int chunk_slots;          // tile slots per chunk: no chunk of either pass has more tiles
   int out_keys;             // keys a pass-2 tile owns: 128 - 2 * pool_radius
-  int cph1_max, cph2_max;   // chunks per head at max_seqlen (strides of the scratch arrays)
-  int lead_extra;           // tiles pass 1 leads pass 2 by, beyond what head completion needs
+  int cph_max;              // chunks per head at max_seqlen (stride of the scratch arrays)
+  int lead_extra;           // slots added to the lead that head completion needs
   int split;                // 1: every KV head is scored as two halves of its query group
   int g0;                   // query heads in the first half (split mode)
   long long wait_cycles;    // SM cycles after which a wait on another role or CTA gives up
   const float* vbar_in;
   float* scores;
   float* vbar_out;
-  const char* v;
-  long long v_ls;
   // scratch
-  float* part;              // [heads_total][cph1_max][128] log2-sum-exp per chunk and query
+  float* part;              // [heads_total][cph_max][128] log2-sum-exp per chunk and query
   int* counters;            // [heads_total] published pass-1 chunks
   int* vcount;              // [heads_total] finished value-norm warps
   unsigned* vbar_bits;      // [heads_total]
-  float2* ent_part;         // [heads_total][cph2_max][8 consumer warps] (sum s, sum s ln s)
+  float2* ent_part;         // [heads_total][cph_max][8 consumer warps] (sum s, sum s ln s)
   unsigned* status;
 };
 
 // ------------------------------------------------------------------------------------------
-// chunk schedule (identical in every role and every CTA, so no descriptors travel)
+// chunk schedule (identical in every CTA)
 // ------------------------------------------------------------------------------------------
-struct Chunk {
-  int head;    // linear index of the scored unit (a KV head, or one half of its query group in
-               // split mode): counters, chunk partials and entropy slots are per unit
-  int rhead;   // linear KV head index = (layer * batch + b) * H_kv + kvh (value norms)
-  int layer, b, kvh;
-  int half;    // which half of the query group (0 unless split)
-  int q0;      // first query head of the unit inside the sequence's H_q heads
-  int group;   // query heads of the unit
-  int index;   // chunk number inside the head
-  int cph;     // chunks of this head
-  int tile0, ntiles;
-  SeqInfo s;
-};
-
-__device__ inline int tiles_of(const Sm100Params& p, const SeqInfo& s, int pass) {
-  return pass == 1 ? ceil_div(s.n, kTile) : ceil_div(s.prefix, p.out_keys);
+__device__ inline void st_release_cta(int* p, int v) {
+  asm volatile("st.release.cta.shared::cta.s32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v) : "memory");
+}
+__device__ inline int ld_acquire_cta(const int* p) {
+  int v;
+  asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+  return v;
 }
 
-__device__ inline Chunk decode_chunk(const Sm100Params& p, const Misc* m, int c, int pass) {
-  const int* pref = pass == 1 ? m->pref1 : m->pref2;
-  const int per_layer = pass == 1 ? m->sched_total1 : m->sched_total2;
-  Chunk ck;
-  ck.layer = c / per_layer;
-  const int r = c - ck.layer * per_layer;
-  const int hkv = p.g.n_kv_heads << p.split;  // scored units per sequence
-  int lo = 0, hi = p.g.batch;  // largest b with hkv * pref[b] <= r
+// Writes the record of the CTA's chunk number `ord` (one thread).
+__device__ __noinline__ void decode_chunk(const Sm100Params& p, Misc* m, int ord) {
+  const int c = blockIdx.x + ord * gridDim.x;
+  const Geom& g = p.g;
+  const int layer = c / m->sched_total;
+  const int r = c - layer * m->sched_total;
+  const int units = g.n_kv_heads << p.split;  // scored units per sequence
+  int lo = 0, hi = g.batch;  // largest b with units * pref[b] <= r
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
-    if (hkv * pref[mid] <= r) lo = mid; else hi = mid;
+    if (units * m->pref[mid] <= r) lo = mid; else hi = mid;
   }
-  ck.b = lo;
-  ck.cph = pref[lo + 1] - pref[lo];
-  const int r2 = r - hkv * pref[lo];
-  const int unit = r2 / ck.cph;
-  ck.index = r2 - unit * ck.cph;
-  ck.head = (ck.layer * p.g.batch + ck.b) * hkv + unit;
-  ck.half = p.split ? (unit & 1) : 0;
-  ck.kvh = unit >> p.split;
-  ck.rhead = (ck.layer * p.g.batch + ck.b) * p.g.n_kv_heads + ck.kvh;
-  ck.group = p.split ? (ck.half ? p.g.group - p.g0 : p.g0) : p.g.group;
-  ck.q0 = ck.kvh * p.g.group + ck.half * p.g0;
-  ck.s = seq_info(p.g, ck.b);
-  // the head's tiles are spread evenly over its chunks (none longer than chunk_tiles): a short
-  // last chunk would leave the CTAs with unequal loads
-  const long long tiles = tiles_of(p, ck.s, pass);
-  ck.tile0 = (int)(ck.index * tiles / ck.cph);
-  ck.ntiles = (int)((ck.index + 1) * tiles / ck.cph) - ck.tile0;
-  return ck;
+  const int b = lo, cph = m->pref[lo + 1] - m->pref[lo];
+  const int r2 = r - units * m->pref[lo];
+  const int unit = r2 / cph, index = r2 - unit * cph;
+  const SeqInfo s = seq_info(g, b);
+  const int half = p.split ? (unit & 1) : 0, kvh = unit >> p.split;
+  Chunk& ck = m->ring[ord % kRing];
+  ck.ord = ord;
+  ck.layer = layer;
+  ck.cph = cph;
+  ck.head = (layer * g.batch + b) * units + unit;
+  ck.half = half;
+  ck.kvh = kvh;
+  ck.rhead = (layer * g.batch + b) * g.n_kv_heads + kvh;
+  ck.group = p.split ? (half ? g.group - p.g0 : p.g0) : g.group;
+  ck.q_row0 = (b * g.n_q_heads + kvh * g.group + half * p.g0) * g.window;
+  ck.slot = ((layer * g.batch + b) * units + unit) * p.cph_max + index;
+  ck.n = s.n;
+  ck.prefix = s.prefix;
+  ck.tok0 = (int)s.tok0;
+  ck.score_base = (long long)layer * g.total_scores + s.score_off + (long long)kvh * s.prefix;
+  // the head's tiles are spread evenly over its chunks, in both passes: a short last chunk would
+  // leave the CTAs with unequal loads
+  const int tiles1 = ceil_div(s.n, kTile), base1 = tiles1 / cph, more1 = tiles1 - base1 * cph;
+  ck.tile1 = index * base1 + min(index, more1);
+  ck.n1 = base1 + (index < more1 ? 1 : 0);
+  const int tiles2 = ceil_div(s.prefix, p.out_keys), base2 = tiles2 / cph, more2 = tiles2 - base2 * cph;
+  ck.tile2 = index * base2 + min(index, more2);
+  ck.n2 = base2 + (index < more2 ? 1 : 0);
+  st_release_cta(&m->ck_count, ord + 1);
+}
+
+// Waits for the record of chunk number `ord`; false once the CTA is aborting without it.
+__device__ __noinline__ bool chunk_wait(Misc* m, int ord, unsigned* status) {
+  const long long t0 = clock64();
+  while (ld_acquire_cta(&m->ck_count) <= ord) {
+    if (m->abort_flag) return false;
+    __nanosleep(32);
+    if (clock64() - t0 > m->wait_cycles) give_up(m, status);
+  }
+  return true;
+}
+__device__ inline bool chunk_ready(Misc* m, int ord, unsigned* status) {
+  if (ld_acquire_cta(&m->ck_count) > ord) return true;
+  return chunk_wait(m, ord, status);
+}
+
+// Bounded wait, out of line behind a first try (see wait_bar).
+__device__ __noinline__ bool wait_long(uint32_t bar, uint32_t parity, Misc* m, unsigned* status,
+                                       bool heed_abort) {
+  return wait_bar(bar, parity, m, status, heed_abort);
+}
+__device__ inline bool wait_for(uint32_t bar, uint32_t parity, Misc* m, unsigned* status,
+                                bool heed_abort = true) {
+  if (mbar_try(bar, parity, 1000)) return true;
+  return wait_long(bar, parity, m, status, heed_abort);
+}
+
+// ------------------------------------------------------------------------------------------
+// exponential sums
+// ------------------------------------------------------------------------------------------
+// sum of exp2(c * scale + shift) over 16 values
+template <bool SHIFT>
+__device__ inline float exp_sum16(const float* c, float scale, float shift) {
+  float2 s0 = make_float2(0.f, 0.f), s1 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float2 x = make_float2(c[2 * i], c[2 * i + 1]);
+    x = SHIFT ? __ffma2_rn(x, make_float2(scale, scale), make_float2(shift, shift))
+              : __fmul2_rn(x, make_float2(scale, scale));
+    x.x = fast_exp2(x.x);
+    x.y = fast_exp2(x.y);
+    if (i & 1) s1 = __fadd2_rn(s1, x);
+    else s0 = __fadd2_rn(s0, x);
+  }
+  s0 = __fadd2_rn(s0, s1);
+  return s0.x + s0.y;
 }
 
 // ------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------
-template <int W>
+template <int W, int D>
 __global__ void __launch_bounds__(kThreads, 1)
 lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
-                        const __grid_constant__ CUtensorMap map_k, const Sm100Params p) {
+                        const __grid_constant__ CUtensorMap map_k,
+                        const __grid_constant__ CUtensorMap map_v,
+                        const __grid_constant__ Sm100Params p) {
+  using S = Smem<D>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* gen = smem_raw + (base - smem_u32(smem_raw));
-  Misc* m = reinterpret_cast<Misc*>(gen + kOffMisc);
+  Misc* m = reinterpret_cast<Misc*>(gen + S::kOffMisc);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const Geom& g = p.g;
   const int units = g.n_kv_heads << p.split;  // scored units per sequence
@@ -180,70 +276,48 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
     return;
   }
 
-  // ---- chunk schedule: exclusive scans of chunks per sequence, both passes -------------------
+  // ---- chunk schedule: exclusive scan of chunks per sequence ---------------------------------
   {
-    __shared__ int wsum[2][kThreads / 32];
-    int c1 = 0, c2 = 0;
-    if ((int)threadIdx.x < g.batch) {
-      const SeqInfo s = seq_info(g, threadIdx.x);
-      if (s.n < g.window && blockIdx.x == 0) atomicOr(p.status, LAVA_DEV_SHORT_SEQUENCE);
-      c1 = ceil_div(ceil_div(s.n, kTile), p.chunk_tiles);
-      c2 = ceil_div(ceil_div(s.prefix, p.out_keys), p.chunk_tiles);
-    }
-    int i1 = c1, i2 = c2;
+    __shared__ int wsum[kThreads / 32];
+    int c1 = 0;
+    if ((int)threadIdx.x < g.batch)
+      c1 = ceil_div(ceil_div(seq_info(g, threadIdx.x).n, kTile), p.chunk_tiles);
+    int i1 = c1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y1 = __shfl_up_sync(0xffffffffu, i1, o), y2 = __shfl_up_sync(0xffffffffu, i2, o);
-      if (lane >= o) {
-        i1 += y1;
-        i2 += y2;
-      }
+      const int y1 = __shfl_up_sync(0xffffffffu, i1, o);
+      if (lane >= o) i1 += y1;
     }
-    if (lane == 31) {
-      wsum[0][warp] = i1;
-      wsum[1][warp] = i2;
-    }
+    if (lane == 31) wsum[warp] = i1;
     __syncthreads();
-    int b1 = 0, b2 = 0;
-    for (int wdx = 0; wdx < warp; ++wdx) {
-      b1 += wsum[0][wdx];
-      b2 += wsum[1][wdx];
-    }
-    if ((int)threadIdx.x < g.batch) {
-      m->pref1[threadIdx.x + 1] = b1 + i1;
-      m->pref2[threadIdx.x + 1] = b2 + i2;
-    }
-    if (threadIdx.x == 0) {
-      m->pref1[0] = 0;
-      m->pref2[0] = 0;
-    }
+    int b1 = 0;
+    for (int wdx = 0; wdx < warp; ++wdx) b1 += wsum[wdx];
+    if ((int)threadIdx.x < g.batch) m->pref[threadIdx.x + 1] = b1 + i1;
+    if (threadIdx.x == 0) m->pref[0] = 0;
     __syncthreads();
     if (threadIdx.x == 0) {
-      m->sched_total1 = units * m->pref1[g.batch];
-      m->sched_total2 = units * m->pref2[g.batch];
-      // How far pass 1 must lead pass 2 in a CTA's own order (see the consumer warps).  With
-      // rho = pass-2 chunks per pass-1 chunk: rho * (1 + (longest head + drift) / grid) chunks,
-      // where drift is how far the two passes' chunk numbering can diverge inside a layer.
-      const double t1 = (double)m->sched_total1, t2 = (double)m->sched_total2;
-      const double rho = t1 > 0.0 ? t2 / t1 : 1.0;
-      double drift = 0.0, longest = 0.0;
-      for (int b = 0; b < g.batch; ++b) {
-        const double c1 = m->pref1[b + 1] - m->pref1[b], c2 = m->pref2[b + 1] - m->pref2[b];
-        const double at = fabs(units * (m->pref1[b] * rho - m->pref2[b]));
-        drift = fmax(drift, at + units * fabs(c1 * rho - c2));
-        longest = fmax(longest, c1);
-      }
-      const double lead = p.chunk_tiles * rho * (1.0 + (longest + drift) / (double)gridDim.x);
-      m->lead_tiles = (int)ceil(lead) + p.lead_extra;
+      m->sched_total = units * m->pref[g.batch];
+      // Chunk number c belongs to CTA c mod grid.  Let c be the lowest chunk whose pass 2 has not
+      // finished in any CTA.  It needs pass 1 (and the value norms) of its head's chunks c' < c +
+      // cph, in split mode of both halves' (c + 2 cph); each of them belongs to a CTA whose own
+      // next pass-2 chunk is c'' >= c, so c' lies at most (cph - 1) / grid ordinals beyond it.
+      // With a lead of that many chunks plus one chunk's tiles every such wait ends.  The extra
+      // slots cover the skew between CTAs and the time the statistics take to travel.
+      int longest = 1;
+      for (int b = 0; b < g.batch; ++b) longest = max(longest, m->pref[b + 1] - m->pref[b]);
+      longest <<= p.split;
+      const int need = p.chunk_slots * ((longest - 1) / (int)gridDim.x) + p.chunk_tiles;
+      m->lead_slots = min(need + p.lead_extra, kMaxLeadChunks * p.chunk_slots);
     }
   }
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(smem_u32(&m->k1_full[s]), 1);
       mbar_init(smem_u32(&m->k1_empty[s]), 1);
       mbar_init(smem_u32(&m->k2_full[s]), 1);
       mbar_init(smem_u32(&m->k2_empty[s]), 1);
+      for (int w = 0; w < kVWarps; ++w) mbar_init(smem_u32(&m->v_full[w][s]), 1);
     }
     mbar_init(smem_u32(&m->q1_full), 1);
     mbar_init(smem_u32(&m->q1_empty), 1);
@@ -254,15 +328,17 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
       mbar_init(smem_u32(&m->s1_empty[s]), 4);   // one arrival per warp of the group
       mbar_init(smem_u32(&m->s2_full[s]), 1);
       mbar_init(smem_u32(&m->s2_empty[s]), 4);
-      mbar_init(smem_u32(&m->pub_full[s]), 8);   // the eight consumer warps
+      mbar_init(smem_u32(&m->pub_full[s]), 8);   // the eight pass-1 warps
       mbar_init(smem_u32(&m->pub_empty[s]), 1);
-      mbar_init(smem_u32(&m->prep_full[s]), 1);
-      mbar_init(smem_u32(&m->prep_empty[s]), 8);
-      mbar_init(smem_u32(&m->gsync[s]), 4);
+      mbar_init(smem_u32(&m->prep_full[s]), kPrepWarps);
+      mbar_init(smem_u32(&m->fold_full[s]), kPrepWarps);
+      mbar_init(smem_u32(&m->prep_empty[s]), 8);  // the eight pass-2 warps
     }
     mbar_init(smem_u32(&m->drain), 1);
     mbar_init(smem_u32(&m->drain2), 1);
     m->abort_flag = 0;
+    m->p2_slot = 0;
+    m->ck_count = 0;
     m->wait_cycles = p.wait_cycles;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -279,237 +355,176 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = m->tmem_base;
-  const long long total1 = (long long)p.n_layers * m->sched_total1;
-  const long long total2 = (long long)p.n_layers * m->sched_total2;
+  const int total = p.n_layers * m->sched_total;  // chunks (fits: checked on the host)
+  const int nchunks = total > (int)blockIdx.x ? (total - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-  if (warp == 0) {
-    // ================= pass-1 producer: Q of the head, K tiles =============================
-    if (lane == 0) {
-      const uint64_t keep = policy_evict_last();
-      int q_loads = 0;
-      long long n = 0;  // K loads issued
-      for (long long c = blockIdx.x; c < total1 && !m->abort_flag; c += gridDim.x) {
-        const Chunk ck = decode_chunk(p, m, c, 1);
-        if (!wait_bar(smem_u32(&m->q1_empty), (q_loads & 1) ^ 1, m, p.status)) break;
-        {
-          const uint32_t bar = smem_u32(&m->q1_full);
-          mbar_expect_tx(bar, kTileBytes);
-          const int row0 = (ck.b * g.n_q_heads + ck.q0) * W;
-          tma_load_3d(base + kOffQ1, &map_q, 0, row0, ck.layer, bar);
-          tma_load_3d(base + kOffQ1 + kHalfBytes, &map_q, 64, row0, ck.layer, bar);
-          ++q_loads;
-        }
-        bool ok = true;
-        for (int t = 0; t < ck.ntiles && ok; ++t) {
-          const int st = (int)(n % kStages);
-          ok = wait_bar(smem_u32(&m->k1_empty[st]), (uint32_t)((n / kStages) & 1) ^ 1, m, p.status);
-          if (!ok) break;
-          const uint32_t bar = smem_u32(&m->k1_full[st]);
-          mbar_expect_tx(bar, kTileBytes);
-          const int tok = (int)ck.s.tok0 + (ck.tile0 + t) * kTile;
-          tma_load_4d(base + kOffK1 + st * kTileBytes, &map_k, 0, tok, ck.kvh, ck.layer, bar, keep);
-          tma_load_4d(base + kOffK1 + st * kTileBytes + kHalfBytes, &map_k, 64, tok, ck.kvh,
-                      ck.layer, bar, keep);
-          ++n;
-        }
-        if (!ok) break;
-      }
-      // copies still in flight land before this CTA gives up its shared memory
-      for (long long j = (n > kStages ? n - kStages : 0); j < n; ++j)
-        wait_bar(smem_u32(&m->k1_full[j % kStages]), (uint32_t)((j / kStages) & 1), m, p.status,
-                 false);
-      if (q_loads > 0)
-        wait_bar(smem_u32(&m->q1_full), (uint32_t)((q_loads - 1) & 1), m, p.status, false);
-    }
-  } else if (warp == 1) {
-    // ================= pass-2 producer: head data for the score warps, Q, K tiles ============
-    const uint64_t drop = policy_evict_first();
-    int q_loads = 0;
-    long long n = 0, j = 0;  // K loads issued, chunks prepared
-    for (long long c = blockIdx.x; c < total2; c += gridDim.x, ++j) {
-      const Chunk ck = decode_chunk(p, m, c, 2);
-      const int slot = (int)(j & 1);
-      // wait until every pass-1 chunk of the head has been published and its value norm is final
-      bool ok = true;
-      const int cph1 = ceil_div(ceil_div(ck.s.n, kTile), p.chunk_tiles);
-      if (lane == 0) {
-        const int want_v = p.vbar_in ? 0 : kVWarps * cph1;
-        const long long t0 = clock64();
-        while (ld_acquire(&p.counters[ck.head]) < cph1 ||
-               (want_v && ld_acquire(&p.vcount[ck.rhead]) < want_v)) {
-          if (m->abort_flag) break;
-          __nanosleep(100);
-          if (clock64() - t0 > m->wait_cycles) give_up(m, p.status);
-        }
-        ok = !m->abort_flag &&
-             wait_bar(smem_u32(&m->prep_empty[slot]), (uint32_t)((j >> 1) & 1) ^ 1, m, p.status);
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+  // MMA issuer of one pass.  The whole warp walks the loop and one elected lane issues: descriptors
+  // and addresses stay warp-uniform.  (With one lane walking the loop and building descriptors for
+  // every instruction, issuing a tile took up to 4000 cycles beside busy consumer warps.)
+  auto issue_mmas = [&](auto first_pass) {
+    constexpr bool kFirst = decltype(first_pass)::value;
+    constexpr int kStages = kFirst ? S::kK1 : S::kK2;
+    unsigned long long* k_full = kFirst ? m->k1_full : m->k2_full;
+    unsigned long long* k_empty = kFirst ? m->k1_empty : m->k2_empty;
+    unsigned long long* s_full = kFirst ? m->s1_full : m->s2_full;
+    unsigned long long* s_empty = kFirst ? m->s1_empty : m->s2_empty;
+    const uint32_t q_full = smem_u32(kFirst ? &m->q1_full : &m->q2_full);
+    const uint32_t q_empty = smem_u32(kFirst ? &m->q1_empty : &m->q2_empty);
+    const uint64_t q_desc = make_desc(base + (kFirst ? kOffQ1 : S::kOffQ2));
+    const uint64_t k_desc0 = make_desc(base + (kFirst ? S::kOffK1 : S::kOffK2));
+    const uint64_t ones_desc = make_desc_plain(base + kOffOnes);
+    const uint64_t bias_desc0 = make_desc_plain(base + kOffBias);
+    const uint32_t d_base = tmem + (kFirst ? 0u : 256u);
+    int q_uses = 0;                      // query tiles used
+    uint32_t buf_uses = 0;               // bit b: parity of the uses of accumulator b
+    int st = 0;                          // K stage of the next block
+    uint32_t st_phase = 0;
+    bool ok = true;
+    for (int j = 0; j < nchunks && ok; ++j) {
+      if (!kFirst) m->p2_slot = j * p.chunk_slots;
+      ok = __all_sync(0xffffffffu, chunk_ready(m, j, p.status));
       if (!ok) break;
-      // Fold the head's chunk partials, in chunk order, into one log2-sum-exp per window query
-      // (lane l: queries 4l .. 4l+3).  Every CTA that scores a chunk of the head does this for
-      // itself, with the same operations in the same order, so all of them get the same bits
-      // and no CTA waits for another one's fold.
-      {
-        const float4* pp =
-            reinterpret_cast<const float4*>(p.part + (size_t)ck.head * p.cph1_max * 128) + lane;
-        float big[4], sum[4];
+      const int nt = kFirst ? m->ring[j % kRing].n1 : m->ring[j % kRing].n2;
+      const int tile0 = kFirst ? m->ring[j % kRing].tile1 : m->ring[j % kRing].tile2;
+      const uint64_t bias_desc = bias_desc0 + (uint64_t)((j & 1) * (kSmallTileBytes >> 4));
+      if (!kFirst)
+        ok = __all_sync(0xffffffffu, wait_for(smem_u32(&m->prep_full[j & 1]), (uint32_t)((j >> 1) & 1), m,
+                                              p.status));
+      if (nt == 0) continue;  // (pass 2 of a head without candidates)
+      ok = ok && wait_for(q_full, (uint32_t)(q_uses & 1), m, p.status);
+      ok = __all_sync(0xffffffffu, ok);
+      ++q_uses;
+      for (int t = 0; t < nt && ok; ++t) {
+        const int buf = (tile0 + t) & 1;
+        ok = wait_for(smem_u32(&s_empty[buf]), ((buf_uses >> buf) & 1) ^ 1, m, p.status);
+        buf_uses ^= 1u << buf;
+        const uint32_t d = d_base + (uint32_t)buf * 128u;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          big[q] = -INFINITY;
-          sum[q] = 0.f;
-        }
-#pragma unroll 1
-        for (int i0 = 0; i0 < cph1; i0 += 16) {
-          float4 pr[16];
-#pragma unroll
-          for (int u = 0; u < 16; ++u)
-            pr[u] = (i0 + u < cph1) ? __ldcg(pp + (size_t)(i0 + u) * 32)
-                                    : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            float l[16];
-#pragma unroll
-            for (int u = 0; u < 16; ++u)
-              l[u] = q == 0 ? pr[u].x : q == 1 ? pr[u].y : q == 2 ? pr[u].z : pr[u].w;
-            float bm = l[0];
-#pragma unroll
-            for (int u = 1; u < 16; ++u) bm = fmaxf(bm, l[u]);
-            const float nb = fmaxf(big[q], bm);
-            const float ref = nb == -INFINITY ? 0.f : nb;  // keeps -inf - -inf out of the exponent
-            float acc = sum[q] * fast_exp2(big[q] - ref);
-#pragma unroll
-            for (int u = 0; u < 16; ++u) acc += fast_exp2(l[u] - ref);
-            sum[q] = acc;
-            big[q] = nb;
-          }
-        }
-        // per window query: minus the log2-sum-exp in logit units, as three bf16 terms
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = 4 * lane + q;
-          uint32_t w0 = 0xf149u, w1 = 0;  // about -1e30 for a query without any key
-          if (sum[q] > 0.f) {
-            const float b = -(big[q] + fast_log2(sum[q])) / g.scale_log2;
-            const __nv_bfloat16 b0 = __float2bfloat16_rn(b);
-            const float r1 = b - __bfloat162float(b0);
-            const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 b2 = __float2bfloat16_rn(r1 - __bfloat162float(b1));
-            w0 = (uint32_t)__bfloat16_as_ushort(b0) | ((uint32_t)__bfloat16_as_ushort(b1) << 16);
-            w1 = (uint32_t)__bfloat16_as_ushort(b2);
-          }
-          *reinterpret_cast<uint4*>(gen + kOffBias + slot * kSmallTileBytes + r * 16) =
-              make_uint4(w0, w1, 0, 0);
-        }
-      }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      if (lane == 0) {
-        const float vb = p.vbar_in ? p.vbar_in[ck.rhead]
-                                   : __uint_as_float(__ldcg(p.vbar_bits + ck.rhead));
-        m->prep[slot].scale = vb * g.c_hat;
-      }
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(smem_u32(&m->prep_full[slot]));
-        ok = wait_bar(smem_u32(&m->q2_empty), (q_loads & 1) ^ 1, m, p.status);
-        if (ok) {
-          const uint32_t bar = smem_u32(&m->q2_full);
-          mbar_expect_tx(bar, kTileBytes);
-          const int row0 = (ck.b * g.n_q_heads + ck.q0) * W;
-          tma_load_3d(base + kOffQ2, &map_q, 0, row0, ck.layer, bar);
-          tma_load_3d(base + kOffQ2 + kHalfBytes, &map_q, 64, row0, ck.layer, bar);
-          ++q_loads;
-        }
-        for (int t = 0; t < ck.ntiles && ok; ++t) {
-          const int st = (int)(n % kStages);
-          ok = wait_bar(smem_u32(&m->k2_empty[st]), (uint32_t)((n / kStages) & 1) ^ 1, m, p.status);
-          if (!ok) break;
-          const uint32_t bar = smem_u32(&m->k2_full[st]);
-          mbar_expect_tx(bar, kTileBytes);
-          // the tile starts pool_radius keys before the first key it owns (halo for pooling)
-          const int tok = (int)ck.s.tok0 + (ck.tile0 + t) * p.out_keys - g.pool_radius;
-          tma_load_4d(base + kOffK2 + st * kTileBytes, &map_k, 0, tok, ck.kvh, ck.layer, bar, drop);
-          tma_load_4d(base + kOffK2 + st * kTileBytes + kHalfBytes, &map_k, 64, tok, ck.kvh,
-                      ck.layer, bar, drop);
-          ++n;
-        }
-      }
-      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-      if (!ok) break;
-    }
-    if (lane == 0) {
-      for (long long i = (n > kStages ? n - kStages : 0); i < n; ++i)
-        wait_bar(smem_u32(&m->k2_full[i % kStages]), (uint32_t)((i / kStages) & 1), m, p.status,
-                 false);
-      if (q_loads > 0)
-        wait_bar(smem_u32(&m->q2_full), (uint32_t)((q_loads - 1) & 1), m, p.status, false);
-    }
-  } else if (warp == 2 || warp == kMma2Warp) {
-    // ================= MMA issuers: warp 2 serves pass 1, the last warp pass 2 ================
-    if (lane == 0) {
-      const bool first = warp == 2;
-      const int pass = first ? 1 : 2;
-      const long long total = first ? total1 : total2;
-      unsigned long long* k_full = first ? m->k1_full : m->k2_full;
-      unsigned long long* k_empty = first ? m->k1_empty : m->k2_empty;
-      unsigned long long* s_full = first ? m->s1_full : m->s2_full;
-      unsigned long long* s_empty = first ? m->s1_empty : m->s2_empty;
-      const uint32_t q_full = smem_u32(first ? &m->q1_full : &m->q2_full);
-      const uint32_t q_empty = smem_u32(first ? &m->q1_empty : &m->q2_empty);
-      const uint32_t q_addr = base + (first ? kOffQ1 : kOffQ2);
-      const uint32_t k_addr = base + (first ? kOffK1 : kOffK2);
-      const uint32_t d_base = tmem + (first ? 0u : 256u);
-      long long n = 0;
-      int q_uses = 0;
-      bool ok = true;
-      for (long long c = blockIdx.x; c < total && ok; c += gridDim.x) {
-        const int nt = decode_chunk(p, m, c, pass).ntiles;
-        const int slot = q_uses & 1;  // chunk ordinal parity = slot of the head's bias tile
-        ok = wait_bar(q_full, (uint32_t)(q_uses & 1), m, p.status);
-        if (ok && !first)
-          ok = wait_bar(smem_u32(&m->prep_full[slot]), (uint32_t)((q_uses >> 1) & 1), m, p.status);
-        ++q_uses;
-        for (int t = 0; t < nt && ok; ++t, ++n) {
-          const int st = (int)(n % kStages), buf = (int)(n & 1);
-          ok = wait_bar(smem_u32(&k_full[st]), (uint32_t)((n / kStages) & 1), m, p.status) &&
-               wait_bar(smem_u32(&s_empty[buf]), (uint32_t)((n >> 1) & 1) ^ 1, m, p.status);
+        for (int x = 0; x < S::kBlocks; ++x) {
+          ok = ok && wait_for(smem_u32(&k_full[st]), st_phase, m, p.status);
+          ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t d = d_base + (uint32_t)buf * 128u;
-          const uint32_t kt = k_addr + st * kTileBytes;
+          const uint64_t k_desc = k_desc0 + (uint64_t)(st * (kBlockBytes >> 4));
+          if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint32_t off = (uint32_t)(kk >> 2) * kHalfBytes + (uint32_t)(kk & 3) * 32u;
-            // pass 1: D[query, key] = Q K^T; pass 2: D[key, query] = K Q^T
-            if (first) umma_bf16(d, make_desc(q_addr + off), make_desc(kt + off), kIdesc, kk > 0);
-            else umma_bf16(d, make_desc(kt + off), make_desc(q_addr + off), kIdesc, kk > 0);
+            for (int kk = 0; kk < 4; ++kk) {
+              const uint64_t ko = kk * 2, qo = x * (kBlockBytes >> 4) + kk * 2;
+              // pass 1: D[query, key] = Q K^T; pass 2: D[key, query] = K Q^T
+              umma_bf16(d, kFirst ? q_desc + qo : k_desc + ko, kFirst ? k_desc + ko : q_desc + qo,
+                        kIdesc, x + kk > 0);
+            }
+            umma_commit(smem_u32(&k_empty[st]));
+            if (x == S::kBlocks - 1) {
+              // pass 2: one more k-step adds minus the log2-sum-exp of every window query
+              if (!kFirst) umma_bf16(d, ones_desc, bias_desc, kIdesc, 1);
+              umma_commit(smem_u32(&s_full[buf]));
+              // the query tile may be replaced once the MMAs of its last user have completed
+              if (t == nt - 1) umma_commit(q_empty);
+              if (!kFirst) m->p2_slot = j * p.chunk_slots + t + 1;
+            }
           }
-          // pass 2: one more k-step adds minus the log2-sum-exp of every window query
-          if (!first)
-            umma_bf16(d, make_desc_plain(base + kOffOnes),
-                      make_desc_plain(base + kOffBias + slot * kSmallTileBytes), kIdesc, 1);
-          umma_commit(smem_u32(&k_empty[st]));
-          umma_commit(smem_u32(&s_full[buf]));
+          __syncwarp();
+          if (++st == kStages) {
+            st = 0;
+            st_phase ^= 1;
+          }
         }
-        // the query tile may be replaced once the MMAs of its last user have completed
-        if (ok) umma_commit(q_empty);
       }
-      // every MMA this thread issued has completed before TMEM is released
-      unsigned long long* drain = first ? &m->drain : &m->drain2;
-      umma_commit(smem_u32(drain));
-      wait_bar(smem_u32(drain), 0, m, p.status, false);
     }
+    if (!kFirst) m->p2_slot = 0x3fffffff;
+    // every MMA this warp issued has completed before TMEM is released
+    const uint32_t drain = smem_u32(kFirst ? &m->drain : &m->drain2);
+    if (elect_one()) umma_commit(drain);
+    __syncwarp();
+    wait_for(drain, 0, m, p.status, false);
+  };
+
+  // TMA producer of one pass (one lane): the chunk records (pass 1), the head's query tile, K blocks.
+  auto produce = [&](auto first_pass) {
+    constexpr bool kFirst = decltype(first_pass)::value;
+    constexpr int kStages = kFirst ? S::kK1 : S::kK2;
+    unsigned long long* k_full = kFirst ? m->k1_full : m->k2_full;
+    unsigned long long* k_empty = kFirst ? m->k1_empty : m->k2_empty;
+    const uint32_t q_full = smem_u32(kFirst ? &m->q1_full : &m->q2_full);
+    const uint32_t q_empty = smem_u32(kFirst ? &m->q1_empty : &m->q2_empty);
+    const uint32_t dst0 = base + (kFirst ? S::kOffK1 : S::kOffK2);
+    // pass 2 reads the K rows a second time, from L2
+    const uint64_t policy = kFirst ? policy_evict_last() : policy_evict_first();
+    const int step = kFirst ? kTile : p.out_keys;
+    int q_loads = 0, n = 0;  // n: K blocks issued
+    int st = 0;
+    uint32_t st_phase = 0;
+    bool ok = true;
+    if (kFirst && nchunks > 0) decode_chunk(p, m, 0);
+    for (int j = 0; j < nchunks && ok; ++j) {
+      if (!kFirst && !chunk_ready(m, j, p.status)) break;
+      const Chunk& ck = m->ring[j % kRing];
+      const int nt = kFirst ? ck.n1 : ck.n2, kvh = ck.kvh, layer = ck.layer;
+      // a pass-2 tile starts pool_radius keys before the first key it owns (halo for pooling)
+      int tok = ck.tok0 + (kFirst ? ck.tile1 * kTile : ck.tile2 * p.out_keys - g.pool_radius);
+      for (int t = 0; t < nt && ok; ++t, tok += step) {
+        if (kFirst) {
+          const int slot = j * p.chunk_slots + t;
+          if (slot > m->p2_slot + m->lead_slots) {
+            const long long t0 = clock64();
+            while (slot > m->p2_slot + m->lead_slots && !m->abort_flag) {
+              __nanosleep(32);
+              if (clock64() - t0 > m->wait_cycles) give_up(m, p.status);
+            }
+          }
+          ok = !m->abort_flag;
+        }
+#pragma unroll 1
+        for (int x = 0; x < S::kBlocks && ok; ++x) {
+          ok = wait_for(smem_u32(&k_empty[st]), st_phase ^ 1, m, p.status);
+          if (!ok) break;
+          const uint32_t bar = smem_u32(&k_full[st]);
+          mbar_expect_tx(bar, kBlockBytes);
+          tma_load_5d(dst0 + st * kBlockBytes, &map_k, 0, tok, x, kvh, layer, bar, policy);
+          ++n;
+          if (++st == kStages) {
+            st = 0;
+            st_phase ^= 1;
+          }
+        }
+        if (ok && t == 0) {  // after the first K tile: the last MMAs still hold the query tile
+          if (kFirst && j + 1 < nchunks) decode_chunk(p, m, j + 1);
+          ok = wait_for(q_empty, (q_loads & 1) ^ 1, m, p.status);
+          if (ok) {
+            mbar_expect_tx(q_full, S::kTileBytes);
+            tma_load_4d_plain(base + (kFirst ? kOffQ1 : S::kOffQ2), &map_q, 0, ck.q_row0, 0, layer,
+                              q_full);
+            ++q_loads;
+          }
+        }
+      }
+    }
+    // copies still in flight land before this CTA gives up its shared memory
+    for (int i = max(0, n - kStages); i < n; ++i)
+      wait_for(smem_u32(&k_full[i % kStages]), (uint32_t)((i / kStages) & 1), m, p.status, false);
+    if (q_loads > 0) wait_for(q_full, (uint32_t)((q_loads - 1) & 1), m, p.status, false);
+  };
+
+  if (warp == 0) {
+    if (lane == 0) produce(std::true_type{});
+  } else if (warp == 1) {
+    if (lane == 0) produce(std::false_type{});
+  } else if (warp == 2) {
+    issue_mmas(std::true_type{});
   } else if (warp == 3) {
+    issue_mmas(std::false_type{});
+  } else if (warp == kPubWarp) {
     // ================= publisher: chunk statistics leave the CTA ============================
-    long long j = 0;
-    for (long long c = blockIdx.x; c < total1; c += gridDim.x, ++j) {
-      const Chunk ck = decode_chunk(p, m, c, 1);
-      const int slot = (int)(j & 1);
+    for (int j = 0; j < nchunks; ++j) {
+      const int slot = j & 1;
       bool ok = true;
       if (lane == 0)
-        ok = wait_bar(smem_u32(&m->pub_full[slot]), (uint32_t)((j >> 1) & 1), m, p.status);
+        ok = chunk_ready(m, j, p.status) &&
+             wait_for(smem_u32(&m->pub_full[slot]), (uint32_t)((j >> 1) & 1), m, p.status);
       ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
       if (!ok) break;
+      const Chunk& ck = m->ring[j % kRing];
       // lane l carries rows 4l .. 4l+3; the two consumer groups' partials are merged first
       {
         const float4 a4 = reinterpret_cast<const float4*>(m->pub[slot][0])[lane];
@@ -519,7 +534,7 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
         o4.y = lse2(a4.y, b4.y);
         o4.z = lse2(a4.z, b4.z);
         o4.w = lse2(a4.w, b4.w);
-        float* dst = p.part + ((size_t)ck.head * p.cph1_max + ck.index) * 128;
+        float* dst = p.part + (size_t)ck.slot * 128;
         reinterpret_cast<float4*>(dst)[lane] = o4;
       }
       __syncwarp();
@@ -529,278 +544,272 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
         red_add_release(&p.counters[ck.head], 1);
       }
     }
-  } else if (warp >= 4 && warp < 12) {
-    // ================= consumers: two groups of four warps, each serving BOTH passes ==========
-    // Group 0 owns TMEM buffer 0 of either pipeline (the even tiles a CTA sees), group 1 buffer
-    // 1, so the exponential unit of every scheduler has two warps to draw from.
-    //   pass 1: thread = (query head, window query) row, running (max, sum of exp2) per chunk
-    //   pass 2: thread = key, window-mean attention per query head, pooling, score, entropy
-    // The order in which the tiles are taken is static and alternates tile by tile: counting a
-    // CTA's tiles in slots (chunk ordinal * chunk_tiles + tile), the pass-1 tile comes first
-    // while its slot, scaled to pass-2 slots, is at most lead_tiles beyond the next pass-2
-    // slot.  The lead is long enough that every pass-1 chunk of a head precedes, in every CTA,
-    // every pass-2 tile of that head or a later one, so the wait for a head's statistics
-    // always ends; it is short enough to keep the K tiles between the two passes in L2, and the
-    // fine alternation keeps both TMA/MMA pipelines busy all the time.
-    constexpr int NH = 128 / W;  // query heads that fit the 128 columns
-    const int grp = (warp - 4) >> 2, quad = warp & 3, row = quad * 32 + lane;
-    const int t_in_win = row % W;
+  } else if (warp >= kFirstPrep && warp < kFirstPrep + kPrepWarps) {
+    // ================= head data for pass 2: normalisers and value norm =======================
+    // Four warps: the fold is part of the chain from pass 1 of a head to its pass 2, and one warp
+    // took four dependent rounds of loads (4.3 us per chunk) for a head of 32 chunks.
+    const int pw = warp - kFirstPrep;
+    for (int j = 0; j < nchunks; ++j) {
+      if (!__all_sync(0xffffffffu, chunk_ready(m, j, p.status))) break;
+      const Chunk& ck = m->ring[j % kRing];
+      const int slot = j & 1;
+      const uint32_t phase = (uint32_t)((j >> 1) & 1);
+      const int cph = ck.cph, nt = ck.n2;
+      // wait until every pass-1 chunk of the head has been published and its value norm is final
+      bool ok = true;
+      if (lane == 0) {
+        const int want_v = p.vbar_in ? 0 : (kVWarps * cph) << p.split;
+        const long long t0 = clock64();
+        while (ld_acquire(&p.counters[ck.head]) < cph ||
+               (pw == 0 && want_v && ld_acquire(&p.vcount[ck.rhead]) < want_v)) {
+          if (m->abort_flag) break;
+          __nanosleep(32);
+          if (clock64() - t0 > m->wait_cycles) give_up(m, p.status);
+        }
+        ok = !m->abort_flag && wait_for(smem_u32(&m->prep_empty[slot]), phase ^ 1, m, p.status);
+      }
+      ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+      if (!ok) break;
+      // Fold the head's chunk partials into one log2-sum-exp per window query: warp w takes chunks
+      // w, w + 4, ... (lane l: queries 4l .. 4l+3), then query 32 w + l from the four warps' sums.
+      // Every CTA that scores a chunk of the head does this for itself, with the same operations in
+      // the same order, so all of them get the same bits and no CTA waits for another one's fold.
+      if (nt > 0) {
+        const float4* pp =
+            reinterpret_cast<const float4*>(p.part + (size_t)ck.head * p.cph_max * 128) + lane;
+        float big[4], sum[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          big[q] = -INFINITY;
+          sum[q] = 0.f;
+        }
+#pragma unroll 1
+        for (int i0 = pw; i0 < cph; i0 += 8 * kPrepWarps) {
+          float4 pr[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int i = i0 + u * kPrepWarps;
+            pr[u] = i < cph ? __ldcg(pp + (size_t)i * 32)
+                            : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            float l[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              l[u] = q == 0 ? pr[u].x : q == 1 ? pr[u].y : q == 2 ? pr[u].z : pr[u].w;
+            float bm = l[0];
+#pragma unroll
+            for (int u = 1; u < 8; ++u) bm = fmaxf(bm, l[u]);
+            const float nb = fmaxf(big[q], bm);
+            const float ref = nb == -INFINITY ? 0.f : nb;  // keeps -inf - -inf out of the exponent
+            float acc = sum[q] * fast_exp2(big[q] - ref);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += fast_exp2(l[u] - ref);
+            sum[q] = acc;
+            big[q] = nb;
+          }
+        }
+        float4 mine;
+        mine.x = sum[0] > 0.f ? big[0] + fast_log2(sum[0]) : -INFINITY;
+        mine.y = sum[1] > 0.f ? big[1] + fast_log2(sum[1]) : -INFINITY;
+        mine.z = sum[2] > 0.f ? big[2] + fast_log2(sum[2]) : -INFINITY;
+        mine.w = sum[3] > 0.f ? big[3] + fast_log2(sum[3]) : -INFINITY;
+        reinterpret_cast<float4*>(m->fold[slot][pw])[lane] = mine;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&m->fold_full[slot]));
+        if (!__all_sync(0xffffffffu, wait_for(smem_u32(&m->fold_full[slot]), phase, m, p.status))) break;
+        // this lane's query: minus the log2-sum-exp in logit units, as three bf16 terms
+        const int r = 32 * pw + lane;
+        const float lse = lse2(lse2(m->fold[slot][0][r], m->fold[slot][1][r]),
+                               lse2(m->fold[slot][2][r], m->fold[slot][3][r]));
+        uint32_t w0 = 0xf149u, w1 = 0;  // about -1e30 for a query without any key
+        if (lse > -INFINITY) {
+          const float b = -lse / g.scale_log2;
+          const __nv_bfloat16 b0 = __float2bfloat16_rn(b);
+          const float r1 = b - __bfloat162float(b0);
+          const __nv_bfloat16 b1 = __float2bfloat16_rn(r1);
+          const __nv_bfloat16 b2 = __float2bfloat16_rn(r1 - __bfloat162float(b1));
+          w0 = (uint32_t)__bfloat16_as_ushort(b0) | ((uint32_t)__bfloat16_as_ushort(b1) << 16);
+          w1 = (uint32_t)__bfloat16_as_ushort(b2);
+        }
+        *reinterpret_cast<uint4*>(gen + kOffBias + slot * kSmallTileBytes + r * 16) =
+            make_uint4(w0, w1, 0, 0);
+        if (pw == 0 && lane == 0) {
+          const float vb = p.vbar_in ? p.vbar_in[ck.rhead]
+                                     : __uint_as_float(__ldcg(p.vbar_bits + ck.rhead));
+          m->scale[slot] = vb * g.c_hat;
+        }
+      } else {
+        if (lane == 0) mbar_arrive(smem_u32(&m->fold_full[slot]));  // keeps the phases in step
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&m->prep_full[slot]));
+    }
+  } else if (warp >= kFirstConsumer && warp < kFirstConsumer + 8) {
+    // ================= pass-1 consumers: softmax statistics ==================================
+    // Group 0 takes the even tiles of a head, group 1 the odd ones (not every other tile of the CTA:
+    // the partial sums, and with them the last bits of the scores, depend on the head alone then).  A
+    // thread's row is summed
+    // relative to a reference exponent taken from the first block of its chunk, not to a running
+    // maximum: fp32 sums keep their relative precision at any scale, the reference is moved by
+    // whole powers of two (exactly) when the sum grows, and a tile that would overflow, or that
+    // holds keys some row may not see, is done with a running maximum.  This takes the maximum, and
+    // the chain it forms in front of the exponentials, out of the loop.
+    const int grp = (warp - kFirstConsumer) >> 2, quad = warp & 3, row = quad * 32 + lane;
+    const float sc2 = g.scale_log2;
+    const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)grp * 128u;
+    uint32_t uses = 0;  // tiles this group has taken
+    for (int j = 0; j < nchunks; ++j) {
+      if (!__all_sync(0xffffffffu, chunk_ready(m, j, p.status))) break;
+      const Chunk& ck = m->ring[j % kRing];
+      const int rows = ck.group * W, nt = ck.n1, key0 = ck.tile1 * kTile;
+      // keys this query may see: i < n and i <= P + t (rows beyond the unit see all; their sums
+      // are not published)
+      const int last = row < rows ? min(ck.n, ck.prefix + row % W + 1) : 0x3fffffff;
+      const bool active = quad * 32 < rows;
+      float z = 0.f, ref = -INFINITY;
+      bool seeded = false;
+      for (int t = (grp ^ ck.tile1) & 1; t < nt; t += 2, ++uses) {
+        wait_for(smem_u32(&m->s1_full[grp]), uses & 1, m, p.status);
+        __syncwarp();
+        if (active) {
+          tc_fence_after();
+          const int limit = last - (key0 + t * kTile);
+          bool careful = !__all_sync(0xffffffffu, limit >= kTile);
+          const float z0 = z, r0 = ref;
+#pragma unroll 1
+          for (;;) {
+#pragma unroll 1
+            for (int blk = 0; blk < 4; ++blk) {
+              float cur[32];
+              tmem_ld32_issue(taddr + blk * 32, cur);
+              tmem_ld_wait(cur);
+              if (careful || !seeded) {
+                // hide the keys this query may not see, then bring the reference up to the block's
+                // maximum
+                const int cnt = limit - blk * 32;
+                float top = -INFINITY;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) {
+                  cur[i] = i < cnt ? cur[i] : -INFINITY;
+                  top = fmaxf(top, cur[i]);
+                }
+                top *= sc2;
+                if (top > ref) {
+                  z *= fast_exp2(ref - top);
+                  ref = top;
+                }
+                seeded = true;
+              }
+              const float shift = ref == -INFINITY ? 0.f : -ref;  // (no visible key so far)
+              z += exp_sum16<true>(cur, sc2, shift) + exp_sum16<true>(cur + 16, sc2, shift);
+            }
+            if (careful || !__any_sync(0xffffffffu, !(z < 1e30f))) break;
+            z = z0;
+            ref = r0;
+            careful = true;
+          }
+          if (z > 65536.f) {
+            const int e = (__float_as_int(z) >> 23) - 127;
+            z = __int_as_float(__float_as_int(z) - (e << 23));
+            ref += (float)e;
+          }
+          tc_fence_before();
+        }
+        __syncwarp();  // every lane has finished reading the accumulator
+        if (lane == 0) mbar_arrive(smem_u32(&m->s1_empty[grp]));
+      }
+      // hand the chunk's statistics (as one log2-sum-exp) to the publisher warp
+      const int slot = j & 1;
+      wait_for(smem_u32(&m->pub_empty[slot]), (uint32_t)((j >> 1) & 1) ^ 1, m, p.status);
+      m->pub[slot][grp][row] = row < rows && z > 0.f ? ref + fast_log2(z) : -INFINITY;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&m->pub_full[slot]));
+    }
+  } else if (warp >= kFirstConsumer + 8 && warp < kFirstConsumer + 16) {
+    // ================= pass-2 consumers: scores of 128 - 2 * pool_radius keys per tile =========
+    const int grp = (warp - kFirstConsumer - 8) >> 2, quad = warp & 3, row = quad * 32 + lane;
     const int rad = g.pool_radius;
     const float inv_w = 1.0f / (float)W;
     const float sc2 = g.scale_log2;
     const bool avg = g.pool_kind == LAVA_POOL_AVG;
-    const uint32_t gbar = smem_u32(&m->gsync[grp]);
-    uint32_t gphase = 0;
-    bool alive = true;
-    // rendezvous of the group's four warps (bounded, and it ends when the CTA aborts)
-    auto group_sync = [&]() {
-      __syncwarp();  // the lanes' shared-memory writes are ordered before lane 0's arrival
-      if (lane == 0) mbar_arrive(gbar);
-      if (!__all_sync(0xffffffffu, wait_bar(gbar, gphase & 1, m, p.status))) alive = false;
-      ++gphase;
-    };
-
-    // ---- cursors over the CTA's chunks of both passes ---------------------------------------
-    // the order rule compares (pass-1 slot) * S2 with (pass-2 slot + lead) * S1; both sides are
-    // kept as running sums so that a step costs an addition
-    const long long sched1 = m->sched_total1, sched2 = m->sched_total2;
-    long long ord1 = 0, ord2 = (long long)m->lead_tiles * sched1;
-    // Tile n of a pass (counted over the CTA) belongs to group n & 1, so a group's own tiles are
-    // two apart: t is the index of its next own tile inside the open chunk (it may point past the
-    // chunk's end, into a later chunk), n the tile's number in the CTA.
-    int c1 = blockIdx.x, t1 = grp, n1 = grp, j1 = 0, last1 = 0;
-    ord1 += grp * sched2;
-    bool has1 = c1 < total1;
-    Chunk k1;
-    float mx = -INFINITY, z = 0.f;
-    auto open1 = [&]() {
-      k1 = decode_chunk(p, m, c1, 1);
-      // keys this query may see: i < n and i <= P + t
-      last1 = row < k1.group * W ? min(k1.s.n, k1.s.prefix + t_in_win + 1) : 0;
-    };
-    if (has1) open1();
-    int c2 = blockIdx.x, t2 = grp, n2 = grp, j2 = 0;
-    ord2 += grp * sched1;
-    bool has2 = c2 < total2, prepped = false;
-    Chunk k2;
-    float es = 0.f, et = 0.f;  // entropy sums of this thread's keys over the chunk
-    float* dst_head = nullptr;   // score row of the open chunk's KV head
-    float chunk_scale = 0.f;     // Vbar * c_hat of that head
-    auto open2 = [&]() {
-      k2 = decode_chunk(p, m, c2, 2);
-      dst_head = p.scores + (size_t)k2.layer * g.total_scores + k2.s.score_off +
-                 (long long)k2.kvh * k2.s.prefix;
-    };
-    if (has2) open2();
-
-    while (alive) {
-      // ---- close the pass-1 chunks that lie before this group's next tile ---------------------
-      while (has1 && t1 >= k1.ntiles) {
-        // hand the chunk's statistics (as one log2-sum-exp) to the publisher warp
-        const int slot = j1 & 1;
-        if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&m->pub_empty[slot]),
-                                              (uint32_t)((j1 >> 1) & 1) ^ 1, m, p.status))) {
-          alive = false;
-          break;
-        }
-        m->pub[slot][grp][row] = z > 0.f ? mx + fast_log2(z) : -INFINITY;
+    const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + 256u + (uint32_t)grp * 128u;
+    constexpr int kBph = W >= 32 ? W / 32 : 1;  // 32-column blocks per query head
+    uint32_t uses = 0;  // tiles this group has taken
+    for (int j = 0; j < nchunks; ++j) {
+      // the group's four warps decide together whether they take the chunk (an abort may come
+      // between one warp's look and another's, and they meet at a hardware barrier per tile)
+      if (quad == 0) {
+        const bool ok = __all_sync(0xffffffffu, chunk_ready(m, j, p.status));
+        if (lane == 0) m->go[j & 1][grp] = ok;
+      }
+      named_bar_sync(1 + grp, 128);
+      if (!m->go[j & 1][grp]) break;
+      const Chunk& ck = m->ring[j % kRing];
+      const int nt = ck.n2, prefix = ck.prefix, group = ck.group, tile2 = ck.tile2, ck_slot = ck.slot;
+      float* dst_head = p.scores + ck.score_base;
+      float es = 0.f, et = 0.f;  // entropy sums of this thread's keys over the chunk
+      wait_for(smem_u32(&m->prep_full[j & 1]), (uint32_t)((j >> 1) & 1), m, p.status);
+      const float chunk_scale = m->scale[j & 1];
+      for (int t = (grp ^ tile2) & 1; t < nt; t += 2, ++uses) {
+        const int tile = tile2 + t, par = uses & 1;
+        wait_for(smem_u32(&m->s2_full[grp]), (uint32_t)par, m, p.status);
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&m->pub_full[slot]));
-        mx = -INFINITY;
-        z = 0.f;
-        ++j1;
-        c1 += gridDim.x;
-        ord1 += (long long)(p.chunk_tiles - k1.ntiles) * sched2;  // the next chunk starts a new run of slots
-        t1 -= k1.ntiles;
-        has1 = c1 < total1;
-        if (has1) open1();
-      }
-      // ---- the same for pass 2 ----------------------------------------------------------------
-      while (alive && has2 && t2 >= k2.ntiles) {
-        // entropy sums of the chunk in a fixed order: keys of a thread, lanes of a warp; the
-        // eight warp sums of a chunk are added up, in order, by the finishing kernel
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          es += __shfl_down_sync(0xffffffffu, es, o);
-          et += __shfl_down_sync(0xffffffffu, et, o);
-        }
-        if (lane == 0) {
-          p.ent_part[((size_t)k2.head * p.cph2_max + k2.index) * 8 + grp * 4 + quad] =
-              make_float2(es, et);
-          mbar_arrive(smem_u32(&m->prep_empty[j2 & 1]));
-        }
-        es = 0.f;
-        et = 0.f;
-        prepped = false;
-        ++j2;
-        c2 += gridDim.x;
-        ord2 += (long long)(p.chunk_tiles - k2.ntiles) * sched1;
-        t2 -= k2.ntiles;
-        has2 = c2 < total2;
-        if (has2) open2();
-      }
-      if (!alive || (!has1 && !has2)) break;
-
-      bool take1 = has1;
-      if (has1 && has2) take1 = ord1 <= ord2;
-
-      if (take1) {
-        // ---- a pass-1 tile: running softmax statistics of 128 keys ------------------------------
-        if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&m->s1_full[grp]),
-                                              (uint32_t)((n1 >> 1) & 1), m, p.status)))
-          break;
         tc_fence_after();
-        const int limit = max(0, min(kTile, last1 - (k1.tile0 + t1) * kTile));
-        const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)grp * 128u;
-#pragma unroll 1
-        for (int blk = 0; blk < 4; ++blk) {
-          const int cnt = limit - blk * 32;
-          float cur[32];
-          tmem_ld32_issue(taddr + blk * 32, cur);
-          tmem_ld_wait(cur);
-          if (cnt >= 32) {
-            // stage by stage (maxima, scaled differences, exponentials, a fixed summation tree)
-            // four running maxima (few live registers; the chains are independent)
-            float t[4] = {cur[0], cur[1], cur[2], cur[3]};
-#pragma unroll
-            for (int i = 4; i < 32; i += 4) {
-              t[0] = fmaxf(t[0], cur[i]);
-              t[1] = fmaxf(t[1], cur[i + 1]);
-              t[2] = fmaxf(t[2], cur[i + 2]);
-              t[3] = fmaxf(t[3], cur[i + 3]);
-            }
-            const float nm = fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])) * sc2;
-            if (nm > mx) {
-              z *= fast_exp2(mx - nm);
-              mx = nm;
-            }
-            const float neg = -mx;
-#pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-              const float2 r = __ffma2_rn(make_float2(cur[i], cur[i + 1]), make_float2(sc2, sc2),
-                                          make_float2(neg, neg));
-              cur[i] = r.x;
-              cur[i + 1] = r.y;
-            }
-#pragma unroll
-            for (int i = 0; i < 32; ++i) cur[i] = fast_exp2(cur[i]);
-            z += tree_sum32(cur);
-          } else if (cnt > 0) {
-            float bm = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (i < cnt) bm = fmaxf(bm, cur[i]);
-            const float nm = bm * sc2;
-            if (nm > mx) {
-              z *= fast_exp2(mx - nm);
-              mx = nm;
-            }
-            float zz = 0.f;
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (i < cnt) zz += fast_exp2(fmaf(cur[i], sc2, -mx));
-            z += zz;
-          }
-        }
-        tc_fence_before();
-        __syncwarp();  // every lane has finished reading the accumulator
-        if (lane == 0) mbar_arrive(smem_u32(&m->s1_empty[grp]));
-        t1 += 2;
-        n1 += 2;
-        ord1 += 2 * sched2;
-      } else {
-        // ---- a pass-2 tile: scores of 128 - 2 * pool_radius keys --------------------------------
-        if (!prepped) {
-          if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&m->prep_full[j2 & 1]),
-                                                (uint32_t)((j2 >> 1) & 1), m, p.status)))
-            break;
-          prepped = true;
-          chunk_scale = m->prep[j2 & 1].scale;
-        }
-        if (!__all_sync(0xffffffffu, wait_bar(smem_u32(&m->s2_full[grp]),
-                                              (uint32_t)((n2 >> 1) & 1), m, p.status)))
-          break;
-        const int tile = k2.tile0 + t2;
-        tc_fence_after();
-        float acc[NH];
-#pragma unroll
-        for (int h = 0; h < NH; ++h) acc[h] = 0.f;
-        const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + 256u + (uint32_t)grp * 128u;
-        // window queries come in blocks of 32 columns; a block lies inside one query head when
-        // W >= 32, and holds two heads when W == 16
-        const int nblk = (k2.group * W + 31) >> 5;  // 32-column blocks of window queries in use
+        // lane <-> key: the tile starts pool_radius keys before the first key it owns; keys
+        // outside the prefix hold the neutral element of both pools (values are >= 0)
+        const int i = tile * p.out_keys - rad + row;
+        const bool inside = i >= 0 && i < prefix;
+        float(*abuf)[kTile] = m->a[grp][par];
+        // window queries come in blocks of 32 columns; a head spans W / 32 blocks, or half a one.
+        // The MMA has already subtracted the log-sum-exp: p = exp2(scale * logit).  Max-pooling
+        // commutes with the group maximum, so only average pooling keeps the heads apart.
+        float top = 0.f, sum = 0.f;
+        const int nblk = (group * W + 31) >> 5;
 #pragma unroll 1
         for (int blk = 0; blk < nblk; ++blk) {
           float cur[32];
           tmem_ld32_issue(taddr + blk * 32, cur);
           tmem_ld_wait(cur);
-          // the MMA has already subtracted the log-sum-exp: p = exp2(scale * logit)
-#pragma unroll
-          for (int i = 0; i < 32; i += 2) {
-            const float2 r = __fmul2_rn(make_float2(cur[i], cur[i + 1]), make_float2(sc2, sc2));
-            cur[i] = fast_exp2(r.x);
-            cur[i + 1] = fast_exp2(r.y);
-          }
+          const float lo = exp_sum16<false>(cur, sc2, 0.f);
+          const float hi = exp_sum16<false>(cur + 16, sc2, 0.f);
           if (W >= 32) {
-            const float sum = tree_sum32(cur);
-            const int h = (blk * 32) / W;
-#pragma unroll
-            for (int hh = 0; hh < NH; ++hh)
-              if (hh == h) acc[hh] += sum;
+            sum += lo + hi;
+            if ((blk + 1) % kBph == 0) {
+              if (avg) abuf[blk / kBph][row] = inside ? sum * inv_w : 0.f;
+              top = fmaxf(top, sum);
+              sum = 0.f;
+            }
           } else {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              cur[i] += cur[i + 8];
-              cur[16 + i] += cur[24 + i];
+            if (avg) {  // at most four heads (checked on the host)
+              abuf[2 * blk][row] = inside ? lo * inv_w : 0.f;
+              abuf[2 * blk + 1][row] = inside ? hi * inv_w : 0.f;
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              cur[i] += cur[i + 4];
-              cur[16 + i] += cur[20 + i];
-            }
-            const float s0 = (cur[0] + cur[1]) + (cur[2] + cur[3]);
-            const float s1 = (cur[16] + cur[17]) + (cur[18] + cur[19]);
-#pragma unroll
-            for (int hh = 0; hh < NH; hh += 2)
-              if (hh == 2 * blk) {
-                acc[hh] += s0;
-                if (hh + 1 < NH) acc[hh + 1] += s1;
-              }
+            top = fmaxf(top, lo);
+            if (2 * blk + 1 < group) top = fmaxf(top, hi);
           }
         }
+        if (!avg) abuf[0][row] = inside ? top * inv_w : 0.f;
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&m->s2_empty[grp]));
-        // lane <-> key: the tile starts pool_radius keys before the first key it owns; keys
-        // outside the prefix hold the neutral element of both pools (values are >= 0)
-        const int ab = (int)((n2 >> 1) & 1);
-        const int i = tile * p.out_keys - rad + row;
-        const bool inside = i >= 0 && i < k2.s.prefix;
-        float(*abuf)[kTile] = m->a[grp][ab];
-        if (avg) {
-#pragma unroll
-          for (int h = 0; h < NH; ++h)
-            if (h < 4 && h < k2.group) abuf[h][row] = inside ? acc[h] * inv_w : 0.f;
-        } else {
-          // max-pooling commutes with the group maximum: reduce over the query heads first
-          float top = 0.f;
-#pragma unroll
-          for (int h = 0; h < NH; ++h)
-            if (h < k2.group) top = fmaxf(top, acc[h] * inv_w);
-          abuf[0][row] = inside ? top : 0.f;
-        }
-        group_sync();
-        if (!alive) break;
-        const int own_lo = tile * p.out_keys, own_hi = min(k2.s.prefix, own_lo + p.out_keys);
+        // One rendezvous per tile: the buffers alternate, so whoever writes this one again has
+        // passed the rendezvous of the tile in between, which every reader of this tile precedes.
+        // All four warps make the same tiles whatever their waits returned.
+        named_bar_sync(1 + grp, 128);
+        const int own_lo = tile * p.out_keys, own_hi = min(prefix, own_lo + p.out_keys);
         if (i >= own_lo && i < own_hi) {
           float best = 0.f;
           if (avg) {
-            for (int h = 0; h < k2.group; ++h) {
+            for (int h = 0; h < group; ++h) {
               const float* a = &abuf[h][row];
               float pv = 0.f;
               for (int q = -rad; q <= rad; ++q) pv += a[q];
-              best = fmaxf(best, pv / (float)g.pool_kernel);
+              best = fmaxf(best, pv);
             }
+            best = best / (float)g.pool_kernel;  // monotone: the maximum may be taken first
           } else {
             const float* a = &abuf[0][row];
             if (rad == 3) {
@@ -822,99 +831,116 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
             et += sc * __logf(sc);
           }
         }
-        t2 += 2;
-        n2 += 2;
-        ord2 += 2 * sched1;
+      }
+      // entropy sums of the chunk in a fixed order: keys of a thread, lanes of a warp; the
+      // eight warp sums of a chunk are added up, in order, by the finishing kernel
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        es += __shfl_down_sync(0xffffffffu, es, o);
+        et += __shfl_down_sync(0xffffffffu, et, o);
+      }
+      if (lane == 0) {
+        p.ent_part[(size_t)ck_slot * 8 + grp * 4 + quad] = make_float2(es, et);
+        mbar_arrive(smem_u32(&m->prep_empty[j & 1]));
       }
     }
-  } else if (warp >= 12 && warp < 12 + kVWarps) {
+  } else if (warp >= kFirstV) {
     // ================= value-norm warps: the V rows of the CTA's pass-1 chunks ===============
-    // Row L1 norms through the register-operand tensor path: a warp takes 16 rows at a time,
-    // clears the sign bits of the packed bf16 values and multiplies the 16 x 128 slab by a matrix
-    // of ones (mma.sync m16n8k16, fp32 accumulate, exact products), which leaves the row sums in
-    // the accumulator.  Which of a row's values lands in which k slot does not matter for a
-    // sum, so every thread simply loads 16-byte pieces: thread (g, t) of a warp, g = lane / 4,
-    // t = lane % 4, owns pieces t, t+4, t+8, t+12 of rows g and g+8.  Seven warps cover 112 rows
-    // per step; one step is in flight while the previous one is reduced.
+    // Row L1 norms through the register-operand tensor path: the sign bits of the packed bf16
+    // values are cleared and the rows multiplied by a matrix of ones (mma.sync m16n8k16, fp32
+    // accumulate, exact products).  Which of a row's values lands in which k slot does not matter
+    // for a sum, so the swizzled piece is read straight through, 16 bytes per lane: lanes 8r..8r+7
+    // hold 64 values of row r, which are rows 2r and 2r + 1 of the operand; four rows go in as the
+    // operand's rows 0..7 and four more as its rows 8..15.  Each warp loads its own pieces of 32
+    // rows, kV of them ahead; in split mode the two halves of a query group share the head's rows.
     if (!p.vbar_in) {
-      const int vw = warp - 12;                   // 0..6
-      const int gq = lane >> 2, tq = lane & 3;
-      struct Group {
-        const char* base;  // this thread's first 16 bytes of row 0 of the sequence
-        int row0, row_hi, head;
-        bool last;         // last group of its chunk
-      };
-      int c = blockIdx.x;
-      Chunk ck;
-      int grp = 0, ngrp = 0;
-      auto next_group = [&](Group& gr) -> bool {
-        while (grp == ngrp) {
-          if (c >= total1 || m->abort_flag) return false;
-          ck = decode_chunk(p, m, c, 1);
-          c += gridDim.x;
-          grp = 0;
-          ngrp = ceil_div(min(ck.s.n, (ck.tile0 + ck.ntiles) * kTile) - ck.tile0 * kTile, 8 * kVRows);
-          if (ck.half) ngrp = 0;  // the head's V rows belong to the first half's chunks
-        }
-        gr.base = p.v + ((size_t)ck.layer * p.v_ls + (long long)ck.kvh * g.v_sh +
-                         ck.s.tok0 * g.v_st) * 2 + tq * 16;
-        gr.row0 = ck.tile0 * kTile + grp * 8 * kVRows + vw * 16 + gq;
-        gr.row_hi = min(ck.s.n, (ck.tile0 + ck.ntiles) * kTile);
-        gr.head = ck.rhead;
-        gr.last = ++grp == ngrp;
-        return true;
-      };
-      // buf[0..3]: pieces of row g, buf[4..7]: pieces of row g + 8 (zeros beyond the chunk)
-      auto issue = [&](uint4 (&buf)[8], const Group& gr) {
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          const int row = gr.row0 + half * 8;
-          const char* src = gr.base + (long long)row * g.v_st * 2;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            buf[half * 4 + q] = make_uint4(0, 0, 0, 0);
-            if (row < gr.row_hi) buf[half * 4 + q] = ld_stream16(src + q * 64);
-          }
-        }
-      };
-      float best = 0.f;
+      const int vw = warp - kFirstV, parts = kVWarps << p.split;
       const uint32_t ones = 0x3f803f80u;  // bf16 (1, 1)
-      auto reduce = [&](const uint4 (&buf)[8], const Group& gr) {
-        float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;  // d0: row g, d2: row g + 8
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const uint4 lo = buf[q], hi = buf[4 + q];
-          // two k = 16 steps per pair of pieces: (x, y) and (z, w)
-          mma_bf16_16816(d0, d1, d2, d3, lo.x & 0x7fff7fffu, hi.x & 0x7fff7fffu,
-                         lo.y & 0x7fff7fffu, hi.y & 0x7fff7fffu, ones, ones);
-          mma_bf16_16816(d0, d1, d2, d3, lo.z & 0x7fff7fffu, hi.z & 0x7fff7fffu,
-                         lo.w & 0x7fff7fffu, hi.w & 0x7fff7fffu, ones, ones);
-        }
-        best = fmaxf(best, fmaxf(d0, d2));
-        if (gr.last) {  // warp-uniform
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-          if (lane == 0) {
-            atomicMax(&p.vbar_bits[gr.head], __float_as_uint(best));
-            __threadfence();
-            atomicAdd(&p.vcount[gr.head], 1);
-          }
-          best = 0.f;
-        }
+      const uint64_t drop = policy_evict_first();
+      const uint32_t stage0 = S::kOffV + vw * S::kV * S::kVBytes;
+      struct Cursor {
+        int j, row, end;  // chunk ordinal, next row of this warp, end of the chunk's rows
       };
-      uint4 bufa[8], bufb[8];
-      Group ga, gb;
-      bool have_a = next_group(ga), have_b = false;
-      if (have_a) issue(bufa, ga);
-      while (have_a) {
-        have_b = next_group(gb);
-        if (have_b) issue(bufb, gb);
-        reduce(bufa, ga);
-        if (!have_b) break;
-        have_a = next_group(ga);
-        if (have_a) issue(bufa, ga);
-        reduce(bufb, gb);
+      auto open = [&](Cursor& cur) {
+        const Chunk& ck = m->ring[cur.j % kRing];
+        if (ck.ord != cur.j) give_up(m, p.status);  // (cannot happen, see Chunk)
+        cur.row = ck.tile1 * kTile + (vw + kVWarps * ck.half) * kVRows;
+        cur.end = min(ck.n, (ck.tile1 + ck.n1) * kTile);
+      };
+      Cursor ld = {-1, 0, 0}, us = {-1, 0, 0};  // loads issued, pieces used
+      int nl = 0, nu = 0;
+      float best = 0.f;
+      while (!__any_sync(0xffffffffu, m->abort_flag)) {
+        // ---- issue loads as far as stages and chunk records allow ------------------------------
+        while (nl - nu < S::kV) {
+          if (ld.row >= ld.end) {
+            const bool more = ld.j + 1 < nchunks && ld_acquire_cta(&m->ck_count) > ld.j + 1;
+            if (!__all_sync(0xffffffffu, more)) break;
+            ++ld.j;
+            open(ld);
+            continue;
+          }
+          const int st = nl % S::kV;
+          if (lane == 0) {
+            const Chunk& ck = m->ring[ld.j % kRing];
+            const uint32_t bar = smem_u32(&m->v_full[vw][st]);
+            mbar_expect_tx(bar, S::kVBytes);
+            tma_load_5d(base + stage0 + st * S::kVBytes, &map_v, 0, ck.tok0 + ld.row, 0, ck.kvh,
+                        ck.layer, bar, drop);
+          }
+          ld.row += parts * kVRows;
+          ++nl;
+        }
+        // ---- close the chunks whose pieces have all been used ----------------------------------
+        while (us.row >= us.end) {
+          if (us.j >= 0) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+            if (lane == 0) {
+              const int head = m->ring[us.j % kRing].rhead;
+              atomicMax(&p.vbar_bits[head], __float_as_uint(best));
+              red_add_release(&p.vcount[head], 1);
+            }
+            best = 0.f;
+          }
+          if (us.j + 1 >= nchunks || !__all_sync(0xffffffffu, chunk_ready(m, us.j + 1, p.status))) {
+            us.j = nchunks;
+            break;
+          }
+          ++us.j;
+          open(us);
+        }
+        if (us.j >= nchunks) break;
+        if (nl == nu) continue;  // (the record has only just arrived)
+        const int st = nu % S::kV;
+        wait_for(smem_u32(&m->v_full[vw][st]), (uint32_t)((nu / S::kV) & 1), m, p.status);
+        const uint8_t* piece = gen + stage0 + st * S::kVBytes + lane * 16;
+#pragma unroll 2
+        for (int r8 = 0; r8 < kVRows / 8; ++r8) {
+          float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+#pragma unroll
+          for (int x = 0; x < S::kBlocks; ++x) {
+            const uint8_t* src = piece + x * (kVRows * 128) + r8 * 1024;
+            const uint4 lo = *reinterpret_cast<const uint4*>(src);
+            const uint4 hi = *reinterpret_cast<const uint4*>(src + 512);
+            mma_bf16_16816(d0, d1, d2, d3, lo.x & 0x7fff7fffu, hi.x & 0x7fff7fffu,
+                           lo.y & 0x7fff7fffu, hi.y & 0x7fff7fffu, ones, ones);
+            mma_bf16_16816(d0, d1, d2, d3, lo.z & 0x7fff7fffu, hi.z & 0x7fff7fffu,
+                           lo.w & 0x7fff7fffu, hi.w & 0x7fff7fffu, ones, ones);
+          }
+          d0 += __shfl_xor_sync(0xffffffffu, d0, 4);
+          d2 += __shfl_xor_sync(0xffffffffu, d2, 4);
+          const int row = us.row + r8 * 8 + (lane >> 3);
+          if (row < us.end) best = fmaxf(best, d0);
+          if (row + 4 < us.end) best = fmaxf(best, d2);
+        }
+        __syncwarp();  // every lane has read the stage before it is loaded again
+        us.row += parts * kVRows;
+        ++nu;
       }
+      // copies still in flight land before this CTA gives up its shared memory
+      for (; nu < nl; ++nu)
+        wait_for(smem_u32(&m->v_full[vw][nu % S::kV]), (uint32_t)((nu / S::kV) & 1), m, p.status, false);
     }
   }
 
@@ -927,13 +953,13 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
 
 // entropy of one (layer, sequence) from the per-chunk sums, folded in a fixed order
 __global__ void __launch_bounds__(256)
-entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph2_max, int chunk_keys,
+entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph_max, int chunk_tiles,
                               double* entropy, const float* vbar_in, const unsigned* vbar_bits,
                               float* vbar_out) {
   __shared__ double rs[8], rt[8];
   const int prob = blockIdx.x, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
-  const int used = ceil_div(s.prefix, chunk_keys);
+  const int used = ceil_div(ceil_div(s.n, kTile), chunk_tiles);
   const int total = g.n_kv_heads * used;
   if (vbar_out && (int)threadIdx.x < g.n_kv_heads) {
     const size_t head = (size_t)prob * g.n_kv_heads + threadIdx.x;
@@ -942,7 +968,7 @@ entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph2_max, int 
   double sum_s = 0.0, sum_t = 0.0;
   for (int i = threadIdx.x; i < total; i += 256) {
     const int kvh = i / used, t = i - kvh * used;
-    const float2* e = ent_part + (((size_t)prob * g.n_kv_heads + kvh) * cph2_max + t) * 8;
+    const float2* e = ent_part + (((size_t)prob * g.n_kv_heads + kvh) * cph_max + t) * 8;
     double cs = 0.0, ct = 0.0;  // the eight consumer warps of the chunk, in order
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -1068,13 +1094,7 @@ EncodeTiledFn encode_fn() {
 
 size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Tiles per chunk.  A chunk boundary costs a reload of the head's query tile and a hand-over
-// of statistics, so chunks should be long; but the launch needs many more chunks than CTAs to
-// balance (chunks are dealt round-robin), and a head finishes pass 1 sooner when more CTAs
-// share it.  Default: about twelve chunks per CTA, between 4 and 32 tiles.  LAVA_SM100_CHUNK_TILES
-// overrides it (option "score_chunk_tiles").
-constexpr int kMinChunkTiles = 4, kMaxChunkTiles = 64;
-constexpr int kSmallLaunchChunkTiles = 8;  // floor of the chosen length: shorter chunks cost more in boundaries than they balance
+constexpr int kMinChunkTiles = 4;
 
 // Query groups of more than 128 window-query rows are scored as two halves (each a unit of its
 // own with at most 128 rows); returns the number of query heads in the first half, 0 if the
@@ -1082,26 +1102,28 @@ constexpr int kSmallLaunchChunkTiles = 8;  // floor of the chosen length: shorte
 int sm100_first_half(const Geom& g) {
   return g.group * g.window > 128 ? (g.group + 1) / 2 : 0;
 }
+
+// Tiles per chunk.  A boundary costs a reload of the query tile, a publication and a fold, but pass 2
+// can only start once a whole head is through pass 1, and what lies between the passes has to stay in
+// L2 (chunk + lead tiles of 32 KB in 148 CTAs).  Score call in us for 4 / 8 / 16 tiles: 32 layers x
+// 32K tokens 1079 / 981 / 1151, 32 x 8K 292 / 269 / 286, 28 layers x 128K (7 query heads per KV head)
+// 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With fewer than sixteen tiles per CTA in
+// all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
+// 8K (fourteen tiles per CTA) 64 / 66.
 int chunk_tiles_for(const Geom& g, int n_layers) {
   if (options().score_chunk_tiles > 0) return options().score_chunk_tiles;
   const long long tiles = (long long)n_layers * (g.n_kv_heads << (sm100_first_half(g) ? 1 : 0)) *
                           ceil_div((int)g.total_tokens, kTile);
   const int sms = sm_count() > 0 ? sm_count() : 148;  // without a device: the part this is tuned for
-  // at least four chunks per CTA, and at least three chunks in a sequence of average length (a
-  // batch of short sequences would otherwise be dealt in a few unequal pieces)
-  long long r = tiles / ((long long)sms * 4);
-  const long long mean_tiles = ceil_div((int)(g.total_tokens / g.batch), kTile);
-  if (r > mean_tiles / 3) r = mean_tiles / 3;
-  if (r < kSmallLaunchChunkTiles) r = mean_tiles < kSmallLaunchChunkTiles ? mean_tiles : kSmallLaunchChunkTiles;
-  return (int)(r < kMinChunkTiles ? kMinChunkTiles : r > kMaxChunkTiles ? kMaxChunkTiles : r);
+  return tiles >= 16LL * sms ? 8 : kMinChunkTiles;
 }
 
-// Tiles pass 1 leads pass 2 by beyond what head completion needs (covers the time a head's
-// statistics take to be published and folded, and the skew between CTAs): half a chunk.
-// LAVA_SM100_LEAD_TILES overrides it.
-int lead_extra_for(int chunk_tiles) {
+// Slots pass 1 leads pass 2 by beyond what head completion needs.  4 / 8 / 12 / 16 slots with chunks of
+// eight tiles: 1300 / 1002 / 981 / 1134 us at 32 layers x 32K; shorter leads let pass 2 wait for the
+// statistics, longer ones lose its K tiles from L2 (0 % more DRAM reads than K and V at 8, 15 % at 16).
+int lead_extra_for() {
   const int forced = options().score_lead_tiles;
-  return forced >= 0 ? forced : (chunk_tiles + 1) / 2;
+  return forced >= 0 ? forced : 12;
 }
 
 }  // namespace
@@ -1123,7 +1145,7 @@ lava_status launch_entropy_from_scores(const Geom& g, int n_layers, const float*
 }
 
 bool sm100_supported(const Geom& g) {
-  if (g.dtype != LAVA_BF16 || g.head_dim != 128) return false;
+  if (g.dtype != LAVA_BF16 || (g.head_dim != 64 && g.head_dim != 128)) return false;
   if (g.window != 16 && g.window != 32 && g.window != 64 && g.window != 128) return false;
   // heads of one scored unit: the whole query group, or its larger half when the group has more
   // than 128 window-query rows
@@ -1142,28 +1164,66 @@ Sm100Layout sm100_layout(const Geom& g, int n_layers) {
   l.heads_total = n_layers * g.batch * (g.n_kv_heads << (sm100_first_half(g) ? 1 : 0));  // units
   l.out_keys = kTile - 2 * g.pool_radius;
   const int tiles1 = ceil_div(g.max_seqlen, kTile);
-  const int tiles2 = ceil_div(max(1, g.max_seqlen - g.window), l.out_keys);
-  l.chunks1 = ceil_div(tiles1, r);  // chunks per head, pass 1
-  l.chunks2 = ceil_div(tiles2, r);  // chunks per head, pass 2
+  l.chunks = ceil_div(tiles1, r);  // chunks per head
   size_t off = 0;
   l.off_sync = off;   // chunk counters, value-norm counters and bits: zeroed every launch
   off = up256(off + sizeof(int) * 3 * (size_t)l.heads_total);
   l.sync_bytes = off;
   l.off_part = off;
-  off = up256(off + sizeof(float) * 128 * (size_t)l.heads_total * l.chunks1);
+  off = up256(off + sizeof(float) * 128 * (size_t)l.heads_total * l.chunks);
   l.off_ent = off;
-  off = up256(off + sizeof(float2) * 8 * (size_t)l.heads_total * l.chunks2);
+  off = up256(off + sizeof(float2) * 8 * (size_t)l.heads_total * l.chunks);
   // The size asked of the caller does not depend on the chunk length chosen for this launch
   // (a workspace sized for a whole model also serves calls on fewer layers): it is the size
   // at the shortest chunk.
   const int rmin = r < kMinChunkTiles ? r : kMinChunkTiles;
   size_t cap = up256(sizeof(int) * 3 * (size_t)l.heads_total);
   cap = up256(cap + sizeof(float) * 128 * (size_t)l.heads_total * ceil_div(tiles1, rmin));
-  cap = up256(cap + sizeof(float2) * 8 * (size_t)l.heads_total * ceil_div(tiles2, rmin));
+  cap = up256(cap + sizeof(float2) * 8 * (size_t)l.heads_total * ceil_div(tiles1, rmin));
   l.total = cap > off ? cap : off;
   return l;
 }
 
+// Tensor map of K or V ([layer][H_kv][tokens][d]) in boxes of `box_rows` tokens and `box_blocks`
+// column blocks: the d columns are split into blocks of 64 (one swizzled row of 128 bytes) as a
+// dimension of its own.
+static lava_status encode_rows_map(const Geom& g, int n_layers, const void* x, long long sh,
+                                   long long st, long long ls, int box_rows, int box_blocks,
+                                   CUtensorMap* map) {
+  EncodeTiledFn encode = encode_fn();
+  if (!encode) return fail(LAVA_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
+  const cuuint64_t blocks = (cuuint64_t)g.head_dim / 64;
+  const cuuint64_t dims[5] = {64, (cuuint64_t)g.total_tokens, blocks, (cuuint64_t)g.n_kv_heads,
+                              (cuuint64_t)n_layers};
+  const cuuint64_t hs = (cuuint64_t)sh * 2;
+  const cuuint64_t lb = n_layers > 1 ? (cuuint64_t)ls * 2 : hs * (cuuint64_t)g.n_kv_heads;
+  const cuuint64_t strides[4] = {(cuuint64_t)st * 2, 128, hs > 0 ? hs : 256, lb > 0 ? lb : 256};
+  const cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_blocks, 1, 1};
+  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return fail(LAVA_ERR_CUDA, "tensor map for K or V could not be encoded");
+  return LAVA_OK;
+}
+
+// The same for the window queries, [layer][batch*H_q*w rows][d], a whole tile per copy.
+static lava_status encode_query_map(const Geom& g, int n_layers, const void* q, long long ls,
+                                    CUtensorMap* map) {
+  EncodeTiledFn encode = encode_fn();
+  if (!encode) return fail(LAVA_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
+  const cuuint64_t rows = (cuuint64_t)g.batch * g.n_q_heads * g.window, d = (cuuint64_t)g.head_dim;
+  const cuuint64_t dims[4] = {64, rows, d / 64, (cuuint64_t)n_layers};
+  const cuuint64_t strides[3] = {d * 2, 128, n_layers > 1 ? (cuuint64_t)ls * 2 : rows * d * 2};
+  const cuuint32_t box[4] = {64, kTile, (cuuint32_t)(d / 64), 1}, es[4] = {1, 1, 1, 1};
+  if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(q), dims, strides, box, es,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return fail(LAVA_ERR_CUDA, "tensor map for the query window could not be encoded");
+  return LAVA_OK;
+}
+
+// The maps of the single-pass kernel (head_dim 128): boxes of one block of 64 columns.
 lava_status encode_score_maps(const Geom& g, int n_layers, const void* q, const void* k,
                               long long q_ls, long long k_ls, CUtensorMap* map_q_out,
                               CUtensorMap* map_k_out) {
@@ -1208,10 +1268,14 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
   char* ws = ws_base + ws_off;
   const Sm100Layout lay = sm100_layout(g, n_layers);
 
-  CUtensorMap map_q, map_k;
+  CUtensorMap map_q, map_k, map_v;
   {
-    const lava_status mrc = encode_score_maps(g, n_layers, q, k, q_ls, k_ls, &map_q, &map_k);
+    lava_status mrc = encode_query_map(g, n_layers, q, q_ls, &map_q);
+    if (mrc == LAVA_OK) mrc = encode_rows_map(g, n_layers, k, g.k_sh, g.k_st, k_ls, kTile, 1, &map_k);
+    if (mrc == LAVA_OK && !vbar_in)
+      mrc = encode_rows_map(g, n_layers, v, g.v_sh, g.v_st, v_ls, kVRows, g.head_dim / 64, &map_v);
     if (mrc != LAVA_OK) return mrc;
+    if (vbar_in) map_v = map_k;  // V is not read
   }
 
   const int sms = sm_count();
@@ -1223,17 +1287,17 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
   p.n_layers = n_layers;
   p.chunk_tiles = lay.chunk_tiles;
   p.out_keys = lay.out_keys;
-  p.cph1_max = lay.chunks1;
-  p.cph2_max = lay.chunks2;
-  p.lead_extra = lead_extra_for(lay.chunk_tiles);
+  p.cph_max = lay.chunks;
+  // a head of cph chunks has at most 128 R cph keys, hence at most 128 R cph / out_keys + 1 tiles
+  // in pass 2, spread evenly over the chunks
+  p.chunk_slots = ceil_div(lay.chunk_tiles * kTile, lay.out_keys) + 2;
+  p.lead_extra = lead_extra_for();
   p.g0 = sm100_first_half(g);
   p.split = p.g0 ? 1 : 0;
   p.wait_cycles = options().wait_limit_cycles;
   p.vbar_in = vbar_in;
   p.scores = scores;
   p.vbar_out = vbar_out;
-  p.v = (const char*)v;
-  p.v_ls = v_ls;
   p.counters = reinterpret_cast<int*>(ws + lay.off_sync);
   p.vcount = p.counters + lay.heads_total;
   p.vbar_bits = reinterpret_cast<unsigned*>(p.vcount + lay.heads_total);
@@ -1250,25 +1314,27 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
     if (rc != LAVA_OK) return rc;
   }
 
-  void (*kern)(const CUtensorMap, const CUtensorMap, const Sm100Params) = nullptr;
+  void (*kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const Sm100Params) = nullptr;
+  const bool wide = g.head_dim == 128;
   switch (g.window) {
-    case 16: kern = lava_score_sm100_kernel<16>; break;
-    case 32: kern = lava_score_sm100_kernel<32>; break;
-    case 64: kern = lava_score_sm100_kernel<64>; break;
-    default: kern = lava_score_sm100_kernel<128>; break;
+    case 16: kern = wide ? lava_score_sm100_kernel<16, 128> : lava_score_sm100_kernel<16, 64>; break;
+    case 32: kern = wide ? lava_score_sm100_kernel<32, 128> : lava_score_sm100_kernel<32, 64>; break;
+    case 64: kern = wide ? lava_score_sm100_kernel<64, 128> : lava_score_sm100_kernel<64, 64>; break;
+    default: kern = wide ? lava_score_sm100_kernel<128, 128> : lava_score_sm100_kernel<128, 64>; break;
   }
-  rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kSmemBytes), "cudaFuncSetAttribute(sm100 score)");
+  const int smem = wide ? (int)Smem<128>::kBytes : (int)Smem<64>::kBytes;
+  rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                  "cudaFuncSetAttribute(sm100 score)");
   if (rc != LAVA_OK) return rc;
-  // an upper bound on the pass-1 chunks; CTAs beyond the real count find no work and exit
-  const long long chunks = (long long)lay.heads_total * lay.chunks1;
-  if ((long long)lay.heads_total * (lay.chunks2 > lay.chunks1 ? lay.chunks2 : lay.chunks1) > 0x3fffffffLL)
-    return fail(LAVA_ERR_UNSUPPORTED, "too many chunks for the 32-bit chunk index");
+  // an upper bound on the chunks; CTAs beyond the real count find no work and exit
+  const long long chunks = (long long)lay.heads_total * lay.chunks;
+  if (chunks * p.chunk_slots > 0x3fffffffLL)
+    return fail(LAVA_ERR_UNSUPPORTED, "too many tiles for the 32-bit tile index");
   const int grid = (int)(chunks < sms ? chunks : sms);
   // Cooperative launch: the CTAs wait on one another's flags, so all must be resident at once.
-  void* args[3] = {&map_q, &map_k, &p};
+  void* args[4] = {&map_q, &map_k, &map_v, &p};
   rc = check_cuda(cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kThreads), args,
-                                              kSmemBytes, stream), "score (sm100) launch");
+                                              smem, stream), "score (sm100) launch");
   if (rc != LAVA_OK) return rc;
   if (p.split) {
     count_launches(1);
@@ -1276,8 +1342,7 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
                                       vbar_out, stream);
   }
   entropy_finalize_sm100_kernel<<<n_layers * g.batch, 256, 0, stream>>>(
-      g, p.ent_part, lay.chunks2, p.chunk_tiles * lay.out_keys, entropy, vbar_in, p.vbar_bits,
-      vbar_out);
+      g, p.ent_part, lay.chunks, p.chunk_tiles, entropy, vbar_in, p.vbar_bits, vbar_out);
   count_launches(2);
   return check_cuda(cudaGetLastError(), "entropy finalize launch");
 }

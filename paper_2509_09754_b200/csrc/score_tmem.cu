@@ -1053,6 +1053,7 @@ int first_unit_heads(const Geom& g) { return g.group * g.window > 128 ? (g.group
 // a pooling radius of at most 4, and a head short enough for a part with up to 160 SMs.  Whether
 // a launch really fits is decided against the actual grid in tmem_fits.
 bool tmem_supported(const Geom& g) {
+  if (g.head_dim != 128) return false;
   if (!sm100_supported(g)) return false;
   if (g.pool_radius > kMaxRadius) return false;
   const int nunit = first_unit_heads(g) ? 2 : 1;

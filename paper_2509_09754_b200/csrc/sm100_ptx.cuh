@@ -32,6 +32,16 @@ __device__ inline void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ inline void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// true in one lane of a fully active warp
+__device__ inline bool elect_one() {
+  uint32_t pred;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(pred));
+  return pred != 0;
+}
+// hardware barrier `id` for `count` threads of the CTA
+__device__ inline void named_bar_sync(int id, int count) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
 // Blocking form: the thread is suspended until the phase completes or a time limit (at most
 // about `ns` nanoseconds) passes, so a waiting warp does not occupy issue slots.
 __device__ inline bool mbar_try(uint32_t bar, uint32_t parity, uint32_t ns) {
@@ -68,6 +78,14 @@ __device__ inline void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0,
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       ".L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
       ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "l"(policy)
+      : "memory");
+}
+__device__ inline void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2,
+                                   int c3, int c4, uint32_t bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      ".L2::cache_hint [%0], [%1, {%3, %4, %5, %6, %7}], [%2], %8;"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "l"(policy)
       : "memory");
 }
 __device__ inline void tma_load_4d_plain(uint32_t dst, const CUtensorMap* map, int c0, int c1,
