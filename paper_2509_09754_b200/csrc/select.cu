@@ -6,9 +6,9 @@
 // after head and in ascending position, every entry above tau plus the first ties in flat
 // index order.  Equal scores therefore resolve to the lower flat index, deterministically.
 //
-// One thread-block cluster of 8 CTAs works on one (layer, sequence); each CTA owns a
-// contiguous eighth of the flat array.  Histograms and counts are exchanged through
-// distributed shared memory with hardware cluster barriers (no spin waits, no global atomics).
+// One thread-block cluster works on one (layer, sequence); each CTA owns a contiguous part of the
+// flat array.  Histograms are exchanged through distributed shared memory with hardware cluster
+// barriers (no spin waits, no global atomics).
 #include <cooperative_groups.h>
 
 #include "lava_internal.cuh"
@@ -18,229 +18,92 @@ namespace cg = cooperative_groups;
 namespace lava {
 namespace {
 
-constexpr int kCluster = 8;
 constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 2048;
+constexpr int kCoarse = kBins / 32;
+constexpr int kCopies = 4;           // interleaved copies of the histogram: one 16-byte cell per bin
+constexpr int kCacheVec = 3584;      // vectors of four keys kept in shared memory: two CTAs fit an SM
+constexpr int kMaskVec = kBins * kCopies * 4;  // mask bytes that fit where the copies were
+constexpr int kMaxCluster = 16;
+constexpr int kSoloKeys = 8192;      // keys that one CTA takes before another is worth its barriers
+constexpr int kFullKeys = 65536;     // keys per CTA up to which CTAs are saved to fit one wave
+constexpr int kMaxPerHead = 524288;  // positions per head, per-head selection
+constexpr int kMaxHeld = 524288;     // entries per list, as the interface promises
+constexpr int kDynSmem = kBins * kCopies * 4 + kCacheVec * 16;
 
 struct SelectShared {
-  unsigned hist[kBins];     // this CTA's digit histogram; peers read it through DSMEM
-  unsigned total[kBins];    // cluster-wide histogram (every CTA builds the same copy)
-  unsigned warp_sum[kWarps + 1];
-  unsigned counts[2];       // entries above tau / equal to tau inside this CTA's chunk
-  unsigned found_digit, found_before;
-  int head_before[1];       // placeholder to keep the struct trivially sized
+  // By parity of the pass: a CTA may fill the next pass's while peers still read this one's.
+  unsigned hist[2][kBins];
+  alignas(8) unsigned coarse[2][kCoarse];  // sums of 32 bins
+  // Peers' sums of the bins in question, [rank][lane]: fetched by one warp per peer, read by all.
+  uint2 peer_coarse[kMaxCluster][32];
+  unsigned peer_fine[kMaxCluster][32];
+  uint2 warp_cnt[kWarps];       // (above tau, equal to tau) per warp
 };
 
-// Inclusive block scan of one unsigned per thread (thread order); returns (exclusive, total).
-__device__ inline unsigned block_exclusive_scan(unsigned x, unsigned* warp_sum, unsigned* total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned incl = x;
+// The two halves of a cluster barrier: what a CTA does between them overlaps the wait for its peers.
+__device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// Address of the same shared-memory location in CTA `rank` of the cluster, and loads through it.
+__device__ inline uint32_t peer_addr(const unsigned* p, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return a;
+}
+__device__ inline unsigned peer_load(const unsigned* p, int rank) {
+  unsigned x;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(peer_addr(p, rank)) : "memory");
+  return x;
+}
+__device__ inline uint2 peer_load2(const unsigned* p, int rank) {
+  uint2 x;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];"
+               : "=r"(x.x), "=r"(x.y) : "r"(peer_addr(p, rank)) : "memory");
+  return x;
+}
+
+// Inclusive sum over the lanes before and including this one.
+__device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
+    const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
   }
-  __syncthreads();  // protects warp_sum against readers of the previous call
-  if (lane == 31) warp_sum[warp] = incl;
-  __syncthreads();
-  unsigned before = 0, all = 0;
-#pragma unroll
-  for (int wdx = 0; wdx < kWarps; ++wdx) {
-    const unsigned v = warp_sum[wdx];
-    if (wdx < warp) before += v;
-    all += v;
-  }
-  *total = all;
-  return before + incl - x;
+  return x;
 }
-
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kThreads)
-select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
-                   int* head_offsets) {
-  if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
-  __shared__ SelectShared sh;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int prob = blockIdx.y, layer = prob / g.batch, b = prob - layer * g.batch;
-  const SeqInfo s = seq_info(g, b);
-  const long long m_total = (long long)g.n_kv_heads * s.prefix;  // candidates
-  const unsigned* keys =
-      reinterpret_cast<const unsigned*>(scores + (size_t)layer * g.total_scores + s.score_off);
-  int* out = keep_idx + (size_t)layer * g.total_scores + s.score_off;
-  int* hoff = head_offsets + (size_t)prob * (g.n_kv_heads + 1);
-
-  const long long window_rows = (long long)g.n_kv_heads * min(g.window, s.n);
-  long long k_sel = layer_budget[prob] - window_rows;
-  if (k_sel < 0) k_sel = 0;
-  if (k_sel > m_total) k_sel = m_total;
-
-  // contiguous chunk of this CTA
-  const long long per = (m_total + kCluster - 1) / kCluster;
-  const long long c0 = min(m_total, per * rank), c1 = min(m_total, c0 + per);
-
-  // ---- radix passes: find tau and the number of ties to take -------------------------------
-  unsigned prefix_val = 0, prefix_mask = 0;
-  long long k_rem = k_sel;
-  if (k_sel > 0) {
-    const int shifts[3] = {21, 10, 0};
-    const int widths[3] = {11, 11, 10};
-#pragma unroll 1
-    for (int pass = 0; pass < 3; ++pass) {
-      const int shift = shifts[pass];
-      const unsigned dmask = (1u << widths[pass]) - 1u;
-      for (int i = threadIdx.x; i < kBins; i += kThreads) sh.hist[i] = 0;
-      __syncthreads();
-      for (long long i0 = c0; i0 < c1; i0 += kThreads) {  // warp-uniform trip count
-        const long long i = i0 + threadIdx.x;
-        const unsigned key = i < c1 ? keys[i] : 0u;
-        const bool mine = i < c1 && (key & prefix_mask) == prefix_val;
-        const unsigned digit = (key >> shift) & dmask;
-        // Scores of one layer crowd into a few exponent buckets, so most lanes of a row share
-        // the digit of the first active lane: those are counted by one atomic, the rest add
-        // their own (spread digits rarely collide).
-        const unsigned active = __ballot_sync(0xffffffffu, mine);
-        if (active) {
-          const int leader = __ffs(active) - 1;
-          const unsigned d0 = __shfl_sync(0xffffffffu, digit, leader);
-          const unsigned same = __ballot_sync(0xffffffffu, mine && digit == d0);
-          if ((int)(threadIdx.x & 31) == leader) atomicAdd(&sh.hist[d0], (unsigned)__popc(same));
-          else if (mine && digit != d0) atomicAdd(&sh.hist[digit], 1u);
-        }
-      }
-      cluster.sync();  // every CTA's histogram is complete
-      for (int i = threadIdx.x; i < kBins; i += kThreads) {
-        unsigned sum = 0;
-#pragma unroll
-        for (int r = 0; r < kCluster; ++r) sum += cluster.map_shared_rank(sh.hist, r)[i];
-        sh.total[i] = sum;
-      }
-      cluster.sync();  // peers have finished reading this CTA's histogram
-      // Walk the digits from the top: thread t owns digits [kBins-1-4t-3, kBins-1-4t].
-      unsigned mine4[4], local = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        mine4[j] = sh.total[kBins - 1 - (threadIdx.x * 4 + j)];
-        local += mine4[j];
-      }
-      unsigned all;
-      unsigned before = block_exclusive_scan(local, sh.warp_sum, &all);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // `before` entries have a larger digit than this one
-        if ((long long)before < k_rem && k_rem <= (long long)before + mine4[j]) {
-          sh.found_digit = kBins - 1 - (threadIdx.x * 4 + j);
-          sh.found_before = before;
-        }
-        before += mine4[j];
-      }
-      __syncthreads();
-      prefix_val |= sh.found_digit << shift;
-      prefix_mask |= dmask << shift;
-      k_rem -= sh.found_before;
-      __syncthreads();
-    }
-  }
-  const unsigned tau = k_sel > 0 ? prefix_val : 0xffffffffu;
-  const unsigned ties_wanted = k_sel > 0 ? (unsigned)k_rem : 0u;  // >= 1 when k_sel > 0
-
-  // ---- count (above, equal) per CTA chunk ---------------------------------------------------
-  unsigned n_gt = 0, n_eq = 0;
-  for (long long i = c0 + threadIdx.x; i < c1; i += kThreads) {
-    const unsigned key = keys[i];
-    n_gt += key > tau;
-    n_eq += key == tau;
-  }
-  unsigned tot_gt, tot_eq;
-  block_exclusive_scan(n_gt, sh.warp_sum, &tot_gt);
-  block_exclusive_scan(n_eq, sh.warp_sum, &tot_eq);
-  if (threadIdx.x == 0) {
-    sh.counts[0] = tot_gt;
-    sh.counts[1] = tot_eq;
-  }
-  cluster.sync();
-  unsigned kept_base = 0, tie_base = 0;  // kept entries / ties in lower-ranked chunks
-  for (int r = 0; r < rank; ++r) {
-    const unsigned* c = cluster.map_shared_rank(sh.counts, r);
-    const unsigned gt = c[0], eq = c[1];
-    const unsigned room = ties_wanted > tie_base ? ties_wanted - tie_base : 0u;
-    kept_base += gt + min(eq, room);
-    tie_base += eq;
-  }
-  cluster.sync();  // counts stay valid until every CTA has read them
-
-  // ---- ordered compaction of this CTA's chunk ---------------------------------------------
-  unsigned kept_run = kept_base, tie_run = tie_base;
-  for (long long i0 = c0; i0 < c1; i0 += kThreads) {
-    const long long i = i0 + threadIdx.x;
-    const bool valid = i < c1;
-    const unsigned key = valid ? keys[i] : 0u;
-    const bool gt = valid && key > tau, eq = valid && key == tau;
-    unsigned tile_eq, tile_keep;
-    const unsigned eq_before = block_exclusive_scan(eq ? 1u : 0u, sh.warp_sum, &tile_eq);
-    const bool keep = gt || (eq && tie_run + eq_before < ties_wanted);
-    const unsigned keep_before = block_exclusive_scan(keep ? 1u : 0u, sh.warp_sum, &tile_keep);
-    if (valid) {
-      const int head = (int)(i / s.prefix);
-      const int pos = (int)(i - (long long)head * s.prefix);
-      if (keep) out[kept_run + keep_before] = pos;
-      // the first entry of a head records how many kept entries precede the head
-      if (pos == 0) hoff[head] = (int)(kept_run + keep_before) + head * g.window;
-    }
-    kept_run += tile_keep;
-    tie_run += tile_eq;
-  }
-  if (rank == 0 && threadIdx.x == 0) {
-    hoff[g.n_kv_heads] = (int)(k_sel + window_rows);
-    if (s.prefix == 0)  // no candidates: every head holds only its (possibly short) window
-      for (int h = 0; h < g.n_kv_heads; ++h) hoff[h] = h * min(g.window, s.n);
-  }
-}
-
-
-// ------------------------------------------------------------------------------------------
-// Register-resident variant: every thread keeps E consecutive keys in registers for all passes,
-// so element order is thread order and nothing in the passes or the emit needs a warp vote.
-// Keys reach the registers through a padded shared-memory staging area (coalesced global reads,
-// conflict-free 16-byte shared reads).  The digit histogram is kept in kRep interleaved copies
-// (copy = lane mod kRep): layer scores crowd into a few exponent buckets, and a single copy
-// would serialise the shared-memory atomics of a warp on those few addresses.  Kept positions
-// are packed in shared memory and leave with coalesced stores.  Serves problems of up to 32768
-// keys per CTA (cluster of 8 or 16 CTAs); larger ones take the streaming kernel above.
-// ------------------------------------------------------------------------------------------
-constexpr int kRegMaxPerCta = 32768;
-
-struct RegShared {
-  unsigned hist[kBins];    // this CTA's folded histogram; peers read it through DSMEM
-  unsigned total[kBins];   // cluster-wide histogram (peers write their share of the bins)
-  unsigned warp_sum[kWarps + 1];
-  unsigned found_digit, found_before;
-  uint2 cta_cnt;           // (above tau, equal to tau) inside this CTA; peers read it
-};
-
-template <int E>
-struct RegCfg {
-  static constexpr int kRep = E >= 64 ? 16 : E >= 32 ? 8 : 4;  // histogram copies
-  static constexpr int kMinCtas = E >= 64 ? 1 : 2;  // CTAs per SM the kernel is compiled for
-  static constexpr int kPad = E + 4;             // staging words per thread (bank spread)
-  static constexpr int kStageWords = kThreads * kPad;
-  static constexpr int kHistWords = kBins * kRep;
-  static constexpr int kBigWords = kStageWords > kHistWords ? kStageWords : kHistWords;
-};
 
 // LIST selects among the entries a layer still holds (Algorithm 2: a lower layer is evicted
 // again with its stored scores): the keys of problem p are the `held` scores of its list, in
 // list order, which is ascending flat index, so ties still go to the lower flat index.  The
 // kept entries' scores and positions are copied to the new list and `src_pos` records where in
 // the old list each came from.
-template <int E, bool LIST>
-__global__ void __launch_bounds__(kThreads, RegCfg<E>::kMinCtas)
-select_topk_reg_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
-                       int* head_offsets, HeldLists io) {
-  using Cfg = RegCfg<E>;
+//
+// Bound by latency (barriers, remote shared memory) at prompt lengths up to 8K and by shared-memory
+// atomics and reads beyond; the keys are 4 bytes a position.  So: a cluster no larger than the keys
+// ask for, and no barrier at all for one CTA; one barrier per pass, after which one warp of each CTA
+// narrows the digit down in two steps (64 sums, then the 32 bins below one of them) instead of adding
+// up all 2048 bins; the counts of lower-ranked CTAs fall out of the same reads.  Keys are read as
+// 16-byte vectors, the first 14336 of a CTA stay in shared memory and the rest are read again from L2,
+// so two CTAs share an SM whatever the length.  Kept entries are found once per vector as a mask and
+// a warp emits its contiguous part of the keys with votes.  Against two kernels (keys in registers; all
+// passes from memory) with a fixed cluster of 8 or 16, all 2048 bins added up and two barriers per pass:
+// 32 layers of 1K / 8K / 32K: 20.5 / 27 / 99 us before, 11.4 / 19.4 / 39 now; 28 layers of 128K with 4
+// heads: 164 -> 49; 128 ragged problems of up to 32K with 8 heads: 259 -> 87.
+template <bool LIST>
+__global__ void __launch_bounds__(kThreads, 2)
+select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
+                   int* head_offsets, HeldLists io) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  uint4* cells = reinterpret_cast<uint4*>(dyn);  // histogram copies of one bin; later the masks
+  unsigned* copies = reinterpret_cast<unsigned*>(dyn);
+  unsigned char* masks = dyn;
+  uint4* cache = reinterpret_cast<uint4*>(dyn + kBins * kCopies * 4);
+  __shared__ SelectShared sh;
+  for (int i = threadIdx.x; i < kBins; i += kThreads) cells[i] = make_uint4(0u, 0u, 0u, 0u);
   if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
-  extern __shared__ __align__(16) unsigned big[];  // staging / histogram copies / packed output
-  __shared__ RegShared sh;
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   // one cluster per (layer, sequence); with per-head selection (the "- head dynamic" ablation of
@@ -249,220 +112,333 @@ select_topk_reg_kernel(Geom g, const float* scores, const long long* layer_budge
   const int cl = blockIdx.x / csize;
   const int prob = per_head ? cl / g.n_kv_heads : cl, layer = prob / g.batch, b = prob - layer * g.batch;
   const int head0 = per_head ? cl - prob * g.n_kv_heads : 0;  // first head of this problem
-  const int lane = threadIdx.x & 31;
+  const int n_heads = per_head ? 1 : g.n_kv_heads;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const SeqInfo s = seq_info(g, b);
   const int win = min(g.window, s.n);
   const int* hoff_old = LIST ? io.hoff_old + (size_t)prob * (g.n_kv_heads + 1) : nullptr;
-  // candidates (fits 31 bits): the whole prefix of every head, or what the list still holds
-  const int m_total = LIST ? max(0, hoff_old[g.n_kv_heads] - g.n_kv_heads * win)
-                           : (per_head ? 1 : g.n_kv_heads) * s.prefix;
+  // candidates: the whole prefix of every head, or what the list still holds
+  const long long m_total = LIST ? max(0, hoff_old[g.n_kv_heads] - g.n_kv_heads * win)
+                                 : (long long)n_heads * s.prefix;
+  const int active = (int)min((long long)csize, max(1ll, (m_total + kSoloKeys - 1) / kSoloKeys));
   const long long window_rows = (long long)g.n_kv_heads * win;
-  long long k_sel = layer_budget[prob] - window_rows;
-  if (k_sel < 0) k_sel = 0;
+  long long k_want = layer_budget[prob] - window_rows;
+  if (k_want < 0) k_want = 0;
   int out_base = 0;  // kept entries of the heads before this problem's first head
   if (per_head) {
     // even shares of the selectable entries, the first (k mod H_kv) heads one more; a head
     // never keeps more than it has
-    const long long share = k_sel / g.n_kv_heads, extra = k_sel % g.n_kv_heads;
+    const long long share = k_want / g.n_kv_heads, extra = k_want % g.n_kv_heads;
     out_base = share >= s.prefix ? head0 * s.prefix
                                  : (int)(head0 * share + min((long long)head0, extra));
-    k_sel = share + (head0 < extra ? 1 : 0);
+    k_want = share + (head0 < extra ? 1 : 0);
   }
-  if (k_sel > m_total) k_sel = m_total;
+  const unsigned k_sel = (unsigned)min(k_want, m_total);
+  if (rank >= active) {  // no keys: take part in the barriers of those that have some
+    if (active > 1)
+      for (int i = 0; i < (k_sel > 0 ? 4 : 1); ++i) cluster.sync();
+    return;
+  }
   const long long old0 = LIST ? io.row_off_old[prob] : 0, new0 = LIST ? io.row_off_new[prob] : 0;
-  const unsigned* keys = reinterpret_cast<const unsigned*>(
-      LIST ? io.score_old + old0
-           : scores + (size_t)layer * g.total_scores + s.score_off + (long long)head0 * s.prefix);
-  int* out = LIST ? io.pos_new + new0
-                  : keep_idx + (size_t)layer * g.total_scores + s.score_off + out_base;
   int* hoff = head_offsets + (size_t)prob * (g.n_kv_heads + 1);
 
-  // this CTA's range; thread t owns its elements [t E, t E + E)
-  const int per = (m_total + csize - 1) / csize;
-  const int c0 = min(m_total, per * rank), c1 = min(m_total, c0 + per);
-  const int n_cta = c1 - c0;
-  const int n_mine = max(0, min(E, n_cta - (int)threadIdx.x * E));  // valid keys of this thread
-#pragma unroll 8
-  for (int i = threadIdx.x; i < n_cta; i += kThreads)
-    big[(i / E) * Cfg::kPad + (i % E)] = keys[c0 + i];
-  __syncthreads();
-  unsigned key[E];
-#pragma unroll
-  for (int j = 0; j < E; j += 4) {
-    const uint4 q = *reinterpret_cast<const uint4*>(&big[threadIdx.x * Cfg::kPad + j]);
-    key[j] = q.x;
-    key[j + 1] = q.y;
-    key[j + 2] = q.z;
-    key[j + 3] = q.w;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < Cfg::kHistWords / 4; i += kThreads)
-    reinterpret_cast<uint4*>(big)[i] = make_uint4(0u, 0u, 0u, 0u);
-  __syncthreads();
+  // this CTA's range [c0, c0 + n) and the aligned vectors that hold it; key e is element e + mis
+  const long long per = (m_total + active - 1) / active;
+  const long long c0 = min(m_total, per * rank);
+  const int n = (int)(min(m_total, c0 + per) - c0);
+  const unsigned* keys = reinterpret_cast<const unsigned*>(
+      LIST ? io.score_old + old0
+           : scores + (size_t)layer * g.total_scores + s.score_off + (long long)head0 * s.prefix) + c0;
+  const int mis = (int)((reinterpret_cast<uintptr_t>(keys) >> 2) & 3);
+  const uint4* vecs = reinterpret_cast<const uint4*>(keys - mis);
+  const int n_vec = n > 0 ? (mis + n + 3) / 4 : 0;
+  auto inside = [&](int e) { return (unsigned)e < (unsigned)n; };
+  auto fetch = [&](int v) {  // only the vectors at the two ends hold anything but this CTA's keys
+    const int e = 4 * v - mis;
+    if (e >= 0 && e + 4 <= n) return vecs[v];
+    uint4 q;
+    q.x = inside(e) ? keys[e] : 0u;
+    q.y = inside(e + 1) ? keys[e + 1] : 0u;
+    q.z = inside(e + 2) ? keys[e + 2] : 0u;
+    q.w = inside(e + 3) ? keys[e + 3] : 0u;
+    return q;
+  };
+  auto again = [&](int v) { return v < kCacheVec ? cache[v] : fetch(v); };
+  // vectors va..vb (and those between) hold nothing but this CTA's keys
+  auto whole = [&](int va, int vb) { return 4 * va - mis >= 0 && 4 * vb + 4 - mis <= n; };
 
   // ---- radix passes: find tau and the number of ties to take -------------------------------
-  unsigned prefix_val = 0, prefix_mask = 0;
-  long long k_rem = k_sel;
+  unsigned digits = 0, mask = 0;  // key bits found so far, and which these are
+  unsigned k_rem = k_sel;         // entries with those bits that are wanted
+  unsigned gt_lower = 0, eq_lower = 0;  // entries above / equal to tau in the CTAs before this one
   if (k_sel > 0) {
-    const int shifts[3] = {21, 10, 0};
-    const int widths[3] = {11, 11, 10};
-    unsigned* my_copy = big + (lane & (Cfg::kRep - 1));
-#pragma unroll 1
+    unsigned* my_copy = copies + (lane & (kCopies - 1));
+#pragma unroll
     for (int pass = 0; pass < 3; ++pass) {
-      const int shift = shifts[pass];
-      const unsigned dmask = (1u << widths[pass]) - 1u;
+      const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+      const unsigned dmask = pass == 2 ? 1023u : 2047u;
+      auto tally = [&](unsigned key) {
+        if (pass == 0 || ((key ^ digits) & mask) == 0u)
+          atomicAdd(&my_copy[((key >> shift) & dmask) * kCopies], 1u);
+      };
+      for (int v0 = threadIdx.x; v0 < n_vec; v0 += 4 * kThreads) {
+        uint4 q[4];
+        if (whole(v0, v0 + 3 * kThreads)) {
 #pragma unroll
-      for (int j = 0; j < E; ++j) {
-        const unsigned digit = (key[j] >> shift) & dmask;
-        if (j < n_mine && (key[j] & prefix_mask) == prefix_val)
-          atomicAdd(&my_copy[digit * Cfg::kRep], 1u);
-      }
-      __syncthreads();
-      // Fold the copies and clear them: consecutive lanes take consecutive 16-byte pieces
-      // (conflict-free); kRep / 4 neighbouring lanes hold the pieces of one bin.
-      for (int i = threadIdx.x; i < Cfg::kHistWords / 4; i += kThreads) {
-        uint4* cell = reinterpret_cast<uint4*>(big) + i;
-        const uint4 q = *cell;
-        *cell = make_uint4(0u, 0u, 0u, 0u);
-        unsigned sum = q.x + q.y + q.z + q.w;
-#pragma unroll
-        for (int o = 1; o < Cfg::kRep / 4; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if ((i & (Cfg::kRep / 4 - 1)) == 0) sh.hist[i / (Cfg::kRep / 4)] = sum;
-      }
-      cluster.sync();  // every CTA's histogram is complete
-      // CTA r sums bins [r * kBins / csize, ...) over the cluster and hands the sums to every
-      // CTA: each thread issues independent remote loads, then csize remote stores.
-      {
-        const int share = kBins / csize;  // 256 or 128
-        if ((int)threadIdx.x < share) {
-          const int bin = rank * share + threadIdx.x;
-          unsigned sum = 0;
-          for (int r0 = 0; r0 < csize; r0 += 8) {  // cluster sizes are 8 and 16
-            unsigned part[8];
-#pragma unroll
-            for (int r = 0; r < 8; ++r) part[r] = cluster.map_shared_rank(sh.hist, r0 + r)[bin];
-#pragma unroll
-            for (int r = 0; r < 8; ++r) sum += part[r];
+          for (int u = 0; u < 4; ++u) {
+            const int v = v0 + u * kThreads;
+            q[u] = pass > 0 && v < kCacheVec ? cache[v] : vecs[v];
           }
-          for (int r = 0; r < csize; ++r) cluster.map_shared_rank(sh.total, r)[bin] = sum;
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (pass == 0 && v0 + u * kThreads < kCacheVec) cache[v0 + u * kThreads] = q[u];
+            tally(q[u].x);
+            tally(q[u].y);
+            tally(q[u].z);
+            tally(q[u].w);
+          }
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int v = v0 + u * kThreads;
+            if (v < n_vec) q[u] = pass == 0 ? fetch(v) : again(v);
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int v = v0 + u * kThreads, e = 4 * v - mis;
+            if (pass == 0 && v < min(n_vec, kCacheVec)) cache[v] = q[u];
+            if (inside(e)) tally(q[u].x);
+            if (inside(e + 1)) tally(q[u].y);
+            if (inside(e + 2)) tally(q[u].z);
+            if (inside(e + 3)) tally(q[u].w);
+          }
         }
       }
-      cluster.sync();  // all sums have arrived; peers have finished reading this CTA's histogram
-      // Walk the digits from the top: thread t owns digits [kBins-1-4t-3, kBins-1-4t].
-      unsigned mine4[4], local = 0;
+      __syncthreads();
+      unsigned* hist = sh.hist[pass & 1];
+      unsigned* coarse = sh.coarse[pass & 1];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        mine4[j] = sh.total[kBins - 1 - (threadIdx.x * 4 + j)];
-        local += mine4[j];
+      for (int i = 0; i < kBins / kThreads; ++i) {  // add the copies up and clear them
+        const int bin = i * kThreads + threadIdx.x;
+        const uint4 q = cells[bin];
+        cells[bin] = make_uint4(0u, 0u, 0u, 0u);
+        const unsigned sum = q.x + q.y + q.z + q.w;
+        hist[bin] = sum;
+        const unsigned all = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0) coarse[bin >> 5] = all;
       }
-      unsigned all;
-      unsigned before = block_exclusive_scan(local, sh.warp_sum, &all);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if ((long long)before < k_rem && k_rem <= (long long)before + mine4[j]) {
-          sh.found_digit = kBins - 1 - (threadIdx.x * 4 + j);
-          sh.found_before = before;
+      // every CTA's histogram is complete; then warp r fetches from CTA r and all warps find the same
+      if (active > 1) {
+        cluster.sync();
+        if (warp < active) sh.peer_coarse[warp][lane] = peer_load2(coarse + 2 * (31 - lane), warp);
+      }
+      __syncthreads();
+      // lane l has the coarse bins 63 - 2l (y) and 62 - 2l (x): the highest digits first
+      uint2 c = make_uint2(0u, 0u), c_lower = c;
+      if (active > 1) {
+        for (int r = 0; r < active; ++r) {
+          const uint2 x = sh.peer_coarse[r][lane];
+          c.x += x.x;
+          c.y += x.y;
+          if (r < rank) {
+            c_lower.x += x.x;
+            c_lower.y += x.y;
+          }
         }
-        before += mine4[j];
+      } else {
+        c = *reinterpret_cast<const uint2*>(coarse + 2 * (31 - lane));
       }
-      __syncthreads();
-      prefix_val |= sh.found_digit << shift;
-      prefix_mask |= dmask << shift;
-      k_rem -= sh.found_before;
-      __syncthreads();
+      unsigned before = warp_inclusive(c.x + c.y, lane) - c.x - c.y;
+      unsigned hit = __ballot_sync(0xffffffffu, before < k_rem && k_rem <= before + c.x + c.y);
+      int src = __ffs(hit) - 1;
+      const bool second = k_rem > before + c.y;  // meaningful in lane src
+      unsigned lower = lane < src ? c_lower.x + c_lower.y : (lane == src && second ? c_lower.y : 0u);
+      const int group = __shfl_sync(0xffffffffu, kCoarse - 1 - 2 * lane - (second ? 1 : 0), src);
+      k_rem -= __shfl_sync(0xffffffffu, before + (second ? c.y : 0u), src);
+      // then the 32 bins of that one
+      unsigned f = 0, f_lower = 0;
+      const unsigned* bins = hist + group * 32 + 31 - lane;
+      if (active > 1) {
+        if (warp < active) sh.peer_fine[warp][lane] = peer_load(bins, warp);
+        __syncthreads();
+        for (int r = 0; r < active; ++r) {
+          const unsigned x = sh.peer_fine[r][lane];
+          f += x;
+          if (r < rank) f_lower += x;
+        }
+      } else {
+        f = *bins;
+      }
+      before = warp_inclusive(f, lane) - f;
+      hit = __ballot_sync(0xffffffffu, before < k_rem && k_rem <= before + f);
+      src = __ffs(hit) - 1;
+      k_rem -= __shfl_sync(0xffffffffu, before, src);
+      if (active > 1) {
+        if (lane < src) lower += f_lower;
+        gt_lower += __reduce_add_sync(0xffffffffu, lower);
+        eq_lower = __shfl_sync(0xffffffffu, f_lower, src);
+      }
+      digits |= (unsigned)(group * 32 + 31 - src) << shift;
+      mask |= dmask << shift;
     }
   }
-  const unsigned tau = k_sel > 0 ? prefix_val : 0xffffffffu;
-  const unsigned ties_wanted = k_sel > 0 ? (unsigned)k_rem : 0u;  // >= 1 when k_sel > 0
+  if (active > 1) cluster_arrive();  // this CTA reads no peer's shared memory any more
+  const unsigned tau = k_sel > 0 ? digits : 0xffffffffu;
+  const unsigned ties_wanted = k_sel > 0 ? k_rem : 0u;  // >= 1 when k_sel > 0
 
-  // ---- counts: per thread, then block scan (both counts packed, each at most 32768) ----------
+  // ---- what is kept: every warp takes consecutive vectors; a mask byte per vector (above tau in
+  // the low half, equal to it in the high half), and counts that place the warp's first entry ----
+  const int per_warp = (n_vec + kThreads - 1) / kThreads * 32;
+  const int v_first = min(n_vec, warp * per_warp), v_last = min(n_vec, v_first + per_warp);
+  auto compare = [&](const uint4& q) {
+    if (max(max(q.x, q.y), max(q.z, q.w)) < tau) return 0u;
+    const unsigned gt = (q.x > tau ? 1u : 0u) | (q.y > tau ? 2u : 0u) | (q.z > tau ? 4u : 0u) |
+                        (q.w > tau ? 8u : 0u);
+    const unsigned eq = (q.x == tau ? 16u : 0u) | (q.y == tau ? 32u : 0u) | (q.z == tau ? 64u : 0u) |
+                        (q.w == tau ? 128u : 0u);
+    return gt | eq;
+  };
+  auto ends = [&](int v) {  // mask bits of the keys of this CTA
+    const int e = 4 * v - mis;
+    return (inside(e) ? 17u : 0u) | (inside(e + 1) ? 34u : 0u) | (inside(e + 2) ? 68u : 0u) |
+           (inside(e + 3) ? 136u : 0u);
+  };
+  // without a pass nothing has been put into shared memory (and nothing is kept)
+  const int n_cached = k_sel > 0 ? kCacheVec : 0;
+  auto key_of = [&](int v) { return v < n_cached ? cache[v] : fetch(v); };
   unsigned n_gt = 0, n_eq = 0;
+  for (int v0 = v_first + lane; v0 < v_last; v0 += 128) {
+    uint4 q[4];
+    unsigned m[4];
+    if (v0 + 96 < v_last && whole(v0, v0 + 96)) {
 #pragma unroll
-  for (int j = 0; j < E; ++j) {
-    n_gt += (j < n_mine && key[j] > tau) ? 1u : 0u;
-    n_eq += (j < n_mine && key[j] == tau) ? 1u : 0u;
-  }
-  unsigned cta_packed;
-  const unsigned before_packed = block_exclusive_scan(n_gt | (n_eq << 16), sh.warp_sum, &cta_packed);
-  const unsigned gt_before = before_packed & 0xffffu, eq_before = before_packed >> 16;
-  const unsigned cta_gt = cta_packed & 0xffffu, cta_eq = cta_packed >> 16;
-  if (threadIdx.x == 0) sh.cta_cnt = make_uint2(cta_gt, cta_eq);
-  cluster.sync();
-  unsigned gt_cta_before = 0, eq_cta_before = 0;  // counts in the CTAs before this one
+      for (int u = 0; u < 4; ++u) q[u] = v0 + 32 * u < n_cached ? cache[v0 + 32 * u] : vecs[v0 + 32 * u];
 #pragma unroll
-  for (int r = 0; r < 16; ++r)
-    if (r < rank) {
-      const uint2 c = *cluster.map_shared_rank(&sh.cta_cnt, r);
-      gt_cta_before += c.x;
-      eq_cta_before += c.y;
-    }
-  // ties are taken in element order: the earliest ties_wanted of them
-  const unsigned ties_before_cta = min(eq_cta_before, ties_wanted);
-  const unsigned kept_cta_before = gt_cta_before + ties_before_cta;
-  const unsigned cta_kept = cta_gt + (min(eq_cta_before + cta_eq, ties_wanted) - ties_before_cta);
-
-  // ---- ordered emit: pack the kept positions in shared memory, then store them coalesced -----
-  {
-    const unsigned tie0 = eq_cta_before + eq_before;  // index of this thread's first tie
-    const unsigned slot0 = gt_before + (min(tie0, ties_wanted) - ties_before_cta);  // in the CTA
-    // bit j of keep_mask: key j is retained (above tau, or one of the first ties_wanted ties)
-    unsigned long long keep_mask = 0ull;
-    {
-      unsigned ties_seen = 0;
-#pragma unroll
-      for (int j = 0; j < E; ++j) {
-        const bool eq = j < n_mine && key[j] == tau;
-        const bool keep = (j < n_mine && key[j] > tau) || (eq && tie0 + ties_seen < ties_wanted);
-        keep_mask |= (unsigned long long)keep << j;
-        ties_seen += eq ? 1u : 0u;
-      }
-    }
-    int* packed = reinterpret_cast<int*>(big);
-    if (LIST) {
-      if (n_mine > 0) {
-        const int first = c0 + (int)threadIdx.x * E;
-        // heads whose list segment starts inside this thread's keys
-        for (int h = 0; h < g.n_kv_heads; ++h) {
-          const int j = hoff_old[h] - h * win - first;
-          if (j >= 0 && j < n_mine)
-            hoff[h] = (int)(kept_cta_before + slot0) + __popcll(keep_mask & ((1ull << j) - 1ull)) +
-                      h * win;
-        }
-#pragma unroll
-        for (int j = 0; j < E; ++j)
-          if ((keep_mask >> j) & 1ull)
-            packed[slot0 + __popcll(keep_mask & ((1ull << j) - 1ull))] = first + j;
-      }
-      __syncthreads();
-      for (unsigned i = threadIdx.x; i < cta_kept; i += kThreads) {
-        const int p = packed[i];
-        const long long o = new0 + kept_cta_before + i;
-        io.pos_new[o] = io.pos_old[old0 + p];
-        io.score_new[o] = io.score_old[old0 + p];
-        io.src_pos[o] = p;
-      }
+      for (int u = 0; u < 4; ++u) m[u] = compare(q[u]);
     } else {
-    if (n_mine > 0) {
-      const int first = c0 + (int)threadIdx.x * E;
-      int head = first / s.prefix;
-      const int pos0 = first - head * s.prefix;
-      // heads that start inside this thread's keys record how many kept entries precede them
-      for (int j = pos0 == 0 ? 0 : s.prefix - pos0; j < n_mine; j += s.prefix) {
-        const int h = head0 + (first + j) / s.prefix;
-        hoff[h] = out_base + (int)(kept_cta_before + slot0) +
-                  __popcll(keep_mask & ((1ull << j) - 1ull)) + h * g.window;
-      }
 #pragma unroll
-      for (int j = 0; j < E; ++j) {
-        int pos = pos0 + j;
-        while (pos >= s.prefix) pos -= s.prefix;  // at most once unless heads are shorter than E
-        if ((keep_mask >> j) & 1ull)
-          packed[slot0 + __popcll(keep_mask & ((1ull << j) - 1ull))] = pos;
+      for (int u = 0; u < 4; ++u) {
+        const int v = v0 + 32 * u;
+        m[u] = v < v_last ? compare(key_of(v)) & ends(v) : 0u;
       }
     }
-    __syncthreads();
-    for (unsigned i = threadIdx.x; i < cta_kept; i += kThreads) out[kept_cta_before + i] = packed[i];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (v0 + 32 * u < min(v_last, kMaskVec)) masks[v0 + 32 * u] = (unsigned char)m[u];
+      n_gt += __popc(m[u] & 15u);
+      n_eq += __popc(m[u] >> 4);
     }
+  }
+  n_gt = __reduce_add_sync(0xffffffffu, n_gt);
+  n_eq = __reduce_add_sync(0xffffffffu, n_eq);
+  if (lane == 0) sh.warp_cnt[warp] = make_uint2(n_gt, n_eq);
+  __syncthreads();
+  const uint2 wc = lane < warp ? sh.warp_cnt[lane & (kWarps - 1)] : make_uint2(0u, 0u);
+  gt_lower += __reduce_add_sync(0xffffffffu, wc.x);
+  unsigned tie_run = eq_lower + __reduce_add_sync(0xffffffffu, wc.y);
+  unsigned kept_run = gt_lower + min(tie_run, ties_wanted);  // kept entries before this row
+
+  // ---- ordered emit: 32 vectors at a time ----------------------------------------------------
+  int* out = LIST ? io.pos_new + new0
+                  : keep_idx + (size_t)layer * g.total_scores + s.score_off + out_base;
+  // first key of head h, counted from this CTA's first (held inside what the arithmetic can take)
+  auto head_start = [&](int h) {
+    const long long at = (LIST ? (long long)(hoff_old[h] - h * win) : (long long)h * s.prefix) - c0;
+    return (int)min((long long)n, at);
+  };
+  int next_head = n_heads;  // first head that starts at or after this warp's first key
+  int next_start = n;
+  int head_begin = 0;       // first key of the head that the row's first key belongs to
+  if (v_first < v_last) {
+    const int first = max(0, 4 * v_first - mis);
+    if (LIST) {
+      next_head = 0;
+      for (int h0 = 0; h0 < n_heads; h0 += 32)
+        next_head += __popc(__ballot_sync(0xffffffffu, h0 + lane < n_heads && head_start(h0 + lane) < first));
+    } else {
+      next_head = (int)((c0 + first + s.prefix - 1) / s.prefix);
+      head_begin = (int)((long long)(next_head - 1) * s.prefix - c0);
+    }
+    if (next_head < n_heads) next_start = head_start(next_head);
+  }
+  for (int v0 = v_first; v0 < v_last; v0 += 32) {
+    const int v = v0 + lane, e = 4 * v - mis;
+    unsigned m = 0;
+    if (v < v_last) m = v < kMaskVec ? masks[v] : compare(key_of(v)) & ends(v);
+    const int row0 = 4 * v0 - mis, row1 = min(n, row0 + 128);
+    const bool starts = next_start < row1;  // a head starts in this row
+    if (!__any_sync(0xffffffffu, m != 0u) && !starts) continue;
+    unsigned keep = m & 15u;
+    const unsigned eq = m >> 4;
+    if (__any_sync(0xffffffffu, eq != 0u)) {  // ties are taken in order: the first ties_wanted
+      const unsigned c = __popc(eq);
+      const unsigned upto = warp_inclusive(c, lane);
+      unsigned tie = tie_run + upto - c;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((eq >> j) & 1u) {
+          if (tie < ties_wanted) keep |= 1u << j;
+          ++tie;
+        }
+      tie_run += __shfl_sync(0xffffffffu, upto, 31);
+    }
+    unsigned vote[4], row_kept = 0, slot = kept_run;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      vote[j] = __ballot_sync(0xffffffffu, (keep >> j) & 1u);
+      row_kept += __popc(vote[j]);
+      slot += __popc(vote[j] & ((1u << lane) - 1u));
+    }
+    if (keep) {
+      if (LIST) {
+        const uint4 q = key_of(v);
+        const unsigned key[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((keep >> j) & 1u) {
+            out[slot] = io.pos_old[old0 + c0 + e + j];
+            io.score_new[new0 + slot] = __uint_as_float(key[j]);
+            io.src_pos[new0 + slot] = (int)c0 + e + j;
+            ++slot;
+          }
+      } else {
+        int pos = e - head_begin;
+        if (starts) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if ((keep >> j) & 1u) {
+              int at = pos + j;
+              while (at >= s.prefix) at -= s.prefix;
+              out[slot] = at;
+              ++slot;
+            }
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            if ((keep >> j) & 1u) {
+              out[slot] = pos + j;
+              ++slot;
+            }
+        }
+      }
+    }
+    // heads that start in this row record how many kept entries precede them
+    while (next_start < row1) {
+      const int at = next_start - row0, l = at >> 2;
+      unsigned before = kept_run;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        before += __popc(vote[j] & ((1u << l) - 1u));
+        if (j < (at & 3)) before += (vote[j] >> l) & 1u;
+      }
+      const int h = head0 + next_head;
+      if (lane == 0) hoff[h] = out_base + (int)before + h * win;
+      head_begin = next_start;
+      ++next_head;
+      next_start = next_head < n_heads ? head_start(next_head) : n;
+    }
+    kept_run += row_kept;
   }
   if (rank == 0 && threadIdx.x == 0) {
     if (LIST) {
@@ -479,27 +455,37 @@ select_topk_reg_kernel(Geom g, const float* scores, const long long* layer_budge
       if (head0 == g.n_kv_heads - 1) hoff[g.n_kv_heads] = out_base + (int)k_sel + (int)window_rows;
     }
   }
-  cluster.sync();  // peers may still be reading this CTA's counts
+  if (active > 1) cluster_wait();  // peers may still be reading this CTA's histograms
 }
 
-template <int E, bool LIST = false>
-cudaError_t launch_reg(const Geom& g, int problems, int csize, const float* scores,
-                       const long long* layer_budget, int* keep_idx, int* head_offsets,
-                       cudaStream_t stream, HeldLists io = HeldLists()) {
-  auto kern = select_topk_reg_kernel<E, LIST>;
-  const int big_bytes = RegCfg<E>::kBigWords * (int)sizeof(unsigned);
-  {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, big_bytes);
-    if (e != cudaSuccess) return e;
-  }
-  if (csize > 8) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
+// CTAs per problem.  A CTA takes 8192 keys before another pays for the barriers (32 problems of 7936
+// keys: 11.4 us with one CTA each, 12.9 with two; one of 65K: 15 with eight CTAs, 20 with four).  Once all
+// problems together have more CTAs than the device holds at two per SM, fewer and fuller ones do, up to
+// 65536 keys each (32 x 262K keys: 39 us in one wave of 8 CTAs per problem, 70 in two of 16; 28 x 524K:
+// 49 with 8, 66 with 16; 128 problems of up to 262K: 87, 108, 165 with 64K, 32K and 16K keys per CTA).
+int cluster_size(long long m_max, int problems) {
+  if (options().select_cluster) return options().select_cluster;
+  int c = 1;
+  while (c < kMaxCluster && m_max > (long long)c * kSoloKeys) c *= 2;
+  const int slots = 2 * (sm_count() > 0 ? sm_count() : 1);
+  while (c > 1 && (long long)c * problems > slots && m_max <= (long long)(c / 2) * kFullKeys) c /= 2;
+  return c;
+}
+
+template <bool LIST>
+lava_status launch(const Geom& g, int problems, long long m_max, const float* scores,
+                   const long long* layer_budget, int* keep_idx, int* head_offsets,
+                   cudaStream_t stream, const HeldLists& io, const char* what) {
+  const int csize = cluster_size(m_max, problems);
+  auto kern = select_topk_kernel<LIST>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
+  if (e == cudaSuccess && csize > 8)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return check_cuda(e, what);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(csize * problems);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = big_bytes;
+  cfg.dynamicSmemBytes = kDynSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeClusterDimension;
@@ -508,7 +494,9 @@ cudaError_t launch_reg(const Geom& g, int problems, int csize, const float* scor
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, g, scores, layer_budget, keep_idx, head_offsets, io);
+  e = cudaLaunchKernelEx(&cfg, kern, g, scores, layer_budget, keep_idx, head_offsets, io);
+  count_launches(1);
+  return check_cuda(e, what);
 }
 
 }  // namespace
@@ -518,52 +506,24 @@ lava_status launch_select(const Geom& g, int n_layers, const float* scores,
                           unsigned* status, cudaStream_t stream) {
   (void)status;
   const bool per_head = (g.flags & LAVA_FLAG_PER_HEAD_TOPK) != 0;
-  // candidates of the largest problem; the register-resident kernel takes up to 32768 per CTA
+  // candidates of the largest problem
   const long long m_max = (long long)(per_head ? 1 : g.n_kv_heads) *
                           (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
   const int problems = n_layers * g.batch * (per_head ? g.n_kv_heads : 1);
-  // 16 CTAs once a cluster of 8 would need 64 keys per thread: at 32 keys per thread two CTAs
-  // share an SM
-  int csize = m_max <= 8LL * (kRegMaxPerCta / 2) ? 8 : 16;
-  if (options().select_cluster == 8 && m_max <= 8LL * kRegMaxPerCta) csize = 8;
-  if (options().select_cluster == 16) csize = 16;
-  if (m_max <= (long long)csize * kRegMaxPerCta) {
-    const long long per = (m_max + csize - 1) / csize;
-    const int e = (int)((per + kThreads - 1) / kThreads);  // keys per thread
-    cudaError_t err;
-    if (e <= 8) err = launch_reg<8>(g, problems, csize, scores, layer_budget, keep_idx, head_offsets, stream);
-    else if (e <= 16) err = launch_reg<16>(g, problems, csize, scores, layer_budget, keep_idx, head_offsets, stream);
-    else if (e <= 32) err = launch_reg<32>(g, problems, csize, scores, layer_budget, keep_idx, head_offsets, stream);
-    else err = launch_reg<64>(g, problems, csize, scores, layer_budget, keep_idx, head_offsets, stream);
-    count_launches(1);
-    return check_cuda(err, "select_topk launch");
-  }
-  if (per_head)
-    return fail(LAVA_ERR_UNSUPPORTED, "per-head selection covers up to 524288 positions per head");
-  dim3 grid(kCluster, n_layers * g.batch);
-  select_topk_kernel<<<grid, kThreads, 0, stream>>>(g, scores, layer_budget, keep_idx,
-                                                    head_offsets);
-  count_launches(1);
-  return check_cuda(cudaGetLastError(), "select_topk launch");
+  if (per_head && m_max > kMaxPerHead)
+    return fail(LAVA_ERR_UNSUPPORTED, "per-head selection covers up to %d positions per head", kMaxPerHead);
+  return launch<false>(g, problems, m_max, scores, layer_budget, keep_idx, head_offsets, stream,
+                       HeldLists(), "select_topk launch");
 }
 
 lava_status launch_reselect(const Geom& g, int problems, long long max_held,
                             const long long* layer_budget, int* head_offsets_new,
                             const HeldLists& io, cudaStream_t stream) {
   if (problems < 1) return LAVA_OK;
-  int csize = max_held <= 8LL * (kRegMaxPerCta / 2) ? 8 : 16;
-  if (max_held > (long long)csize * kRegMaxPerCta)
-    return fail(LAVA_ERR_UNSUPPORTED, "a layer may hold at most %d entries per sequence here",
-                16 * kRegMaxPerCta);
-  const long long per = (max_held + csize - 1) / csize;
-  const int e = (int)((per + kThreads - 1) / kThreads);
-  cudaError_t err;
-  if (e <= 8) err = launch_reg<8, true>(g, problems, csize, nullptr, layer_budget, nullptr, head_offsets_new, stream, io);
-  else if (e <= 16) err = launch_reg<16, true>(g, problems, csize, nullptr, layer_budget, nullptr, head_offsets_new, stream, io);
-  else if (e <= 32) err = launch_reg<32, true>(g, problems, csize, nullptr, layer_budget, nullptr, head_offsets_new, stream, io);
-  else err = launch_reg<64, true>(g, problems, csize, nullptr, layer_budget, nullptr, head_offsets_new, stream, io);
-  count_launches(1);
-  return check_cuda(err, "reselect launch");
+  if (max_held > kMaxHeld)
+    return fail(LAVA_ERR_UNSUPPORTED, "a layer may hold at most %d entries per sequence here", kMaxHeld);
+  return launch<true>(g, problems, max_held, nullptr, layer_budget, nullptr, head_offsets_new, stream,
+                      io, "reselect launch");
 }
 
 }  // namespace lava
