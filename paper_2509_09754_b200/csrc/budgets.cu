@@ -64,6 +64,7 @@ budgets_kernel(int n_layers, int batch, const double* entropy, const long long* 
                long long* row_off, unsigned* status) {
   __shared__ double sh_e[kSeqs<J>][J * 32];
   __shared__ long long sh_frac[kSeqs<J>][J * 32];  // bits of the fractional part (>= 0); -1: not active
+  in_stream_order();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int b = blockIdx.x * (blockDim.x >> 5) + warp;
   if (b < batch) {
@@ -185,6 +186,7 @@ budgets_kernel(int n_layers, int batch, const double* entropy, const long long* 
 
 __global__ void __launch_bounds__(1024)
 row_offsets_kernel(int count, const long long* budget, long long* row_off) {
+  in_stream_order();
   prefix_rows(count, budget, row_off);
 }
 
@@ -194,10 +196,10 @@ int launch(int n_layers, int batch, const double* entropy, const long long* tota
            cudaStream_t stream) {
   const int seqs = batch < kSeqs<J> ? batch : kSeqs<J>;
   const int blocks = (batch + seqs - 1) / seqs;
-  budgets_kernel<J><<<blocks, 32 * seqs, 0, stream>>>(n_layers, batch, entropy, total, lo, hi, mode, budget,
-                                                      row_off, status);
+  launch_in_order(budgets_kernel<J>, blocks, 32 * seqs, 0, stream, n_layers, batch, entropy, total, lo, hi,
+                  mode, budget, row_off, status);
   if (blocks == 1) return 1;
-  row_offsets_kernel<<<1, 1024, 0, stream>>>(n_layers * batch, budget, row_off);
+  launch_in_order(row_offsets_kernel, 1, 1024, 0, stream, n_layers * batch, budget, row_off);
   return 2;
 }
 

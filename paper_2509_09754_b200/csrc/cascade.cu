@@ -61,6 +61,7 @@ CascadeLayout cascade_layout(const Geom& g, int n_layers, long long rows) {
 __global__ void cascade_init_kernel(Geom g, int n_layers, long long rows, const long long* total_in,
                                     long long* total_now, long long* floor_out, long long* cap_out,
                                     unsigned* status) {
+  in_stream_order();
   if (blockIdx.x != 0 || threadIdx.x != 0) return;
   long long need = 0;
   bool bad = false;
@@ -92,6 +93,7 @@ __global__ void cascade_init_kernel(Geom g, int n_layers, long long rows, const 
 __global__ void __launch_bounds__(256)
 cascade_adopt_kernel(Geom g, const float* scores_full, const int* keep_full, const int* head_offsets,
                      const long long* row_off, float* score_list, int* pos_list) {
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
   const int b = blockIdx.y;
   const SeqInfo s = seq_info(g, b);
@@ -114,6 +116,7 @@ __global__ void __launch_bounds__(256)
 cascade_move_kernel(Geom g, const int* src_pos, const int* hoff_old_all, const int* hoff_new_all,
                     const long long* roff_old, const long long* roff_new, const char* k_old,
                     const char* v_old, char* k_new, char* v_new, int blocks_per_head) {
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
   const int prob = blockIdx.z, b = prob % g.batch, kvh = blockIdx.y;
   const SeqInfo s = seq_info(g, b);
@@ -205,10 +208,9 @@ lava_status lava_cascade_begin(lava_cascade* h, const int64_t* total_budget, voi
                                void* stream) {
   if (!h || !total_budget || !workspace) return fail(LAVA_ERR_INVALID_ARG, "NULL argument");
   const CascadeLayout& c = h->lay;
-  cascade_init_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(
-      h->g, h->n_layers, h->rows, (const long long*)total_budget,
-      (long long*)(h->state + c.off_total), (long long*)(h->state + c.off_floor),
-      (long long*)(h->state + c.off_cap), (unsigned*)workspace);
+  launch_in_order(cascade_init_kernel, 1, 32, 0, (cudaStream_t)stream, h->g, h->n_layers, h->rows, (const
+                  long long*)total_budget, (long long*)(h->state + c.off_total), (long long*)(h->state +
+                  c.off_floor), (long long*)(h->state + c.off_cap), (unsigned*)workspace);
   count_launches(1);
   lava_status rc = check_cuda(cudaGetLastError(), "cascade init launch");
   h->begun = rc == LAVA_OK;
@@ -257,10 +259,9 @@ lava_status lava_cascade_step(lava_cascade* h, const void* q_win, const void* k,
   if (rc != LAVA_OK) return rc;
   if (g.total_scores > 0) {
     dim3 grid(std::max(1, std::min(64, sm_count() * 4 / std::max(1, g.batch))), g.batch);
-    cascade_adopt_kernel<<<grid, 256, 0, st>>>(g, scores_full, keep_full,
-                                               hoff_new + lb_t * (g.n_kv_heads + 1),
-                                               roff_new + lb_t, (float*)(base + c.off_score[to]),
-                                               (int*)(base + c.off_pos[to]));
+    launch_in_order(cascade_adopt_kernel, grid, 256, 0, st, g, scores_full, keep_full, hoff_new + lb_t *
+                    (g.n_kv_heads + 1), roff_new + lb_t, (float*)(base + c.off_score[to]), (int*)(base +
+                    c.off_pos[to]));
     count_launches(1);
     rc = check_cuda(cudaGetLastError(), "cascade adopt launch");
     if (rc != LAVA_OK) return rc;
@@ -285,9 +286,9 @@ lava_status lava_cascade_step(lava_cascade* h, const void* q_win, const void* k,
     int bph = std::max(1, (sms * 8 + heads_total - 1) / heads_total);
     bph = std::min(bph, std::max(1, (g.max_seqlen + 15) / 16));
     dim3 grid(bph, g.n_kv_heads, t * g.batch);
-    cascade_move_kernel<<<grid, 256, 0, st>>>(g, io.src_pos, io.hoff_old, hoff_new, io.row_off_old,
-                                              roff_new, base + c.off_k[from], base + c.off_v[from],
-                                              base + c.off_k[to], base + c.off_v[to], bph);
+    launch_in_order(cascade_move_kernel, grid, 256, 0, st, g, io.src_pos, io.hoff_old, hoff_new,
+                    io.row_off_old, roff_new, base + c.off_k[from], base + c.off_v[from], base +
+                    c.off_k[to], base + c.off_v[to], bph);
     count_launches(1);
     rc = check_cuda(cudaGetLastError(), "cascade move launch");
     if (rc != LAVA_OK) return rc;

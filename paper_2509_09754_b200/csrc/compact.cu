@@ -13,6 +13,7 @@ __global__ void __launch_bounds__(256)
 compact_kernel(Geom g, const char* k, const char* v, long long k_ls, long long v_ls,
                const int* keep_idx, const int* head_offsets, const long long* row_off,
                char* k_out, char* v_out, int blocks_per_head) {
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
   const int prob = blockIdx.z, layer = prob / g.batch, b = prob - layer * g.batch;
   const int kvh = blockIdx.y;
@@ -59,11 +60,11 @@ lava_status launch_compact(const Geom& g, int n_layers, const void* k, const voi
   const int max_useful = (g.max_seqlen + 15) / 16;
   if (blocks_per_head > max_useful) blocks_per_head = max_useful;
   dim3 grid(blocks_per_head, g.n_kv_heads, n_layers * g.batch);
-  compact_kernel<<<grid, 256, 0, stream>>>(g, (const char*)k, (const char*)v, k_ls, v_ls, keep_idx,
-                                           head_offsets, row_off, (char*)k_out, (char*)v_out,
-                                           blocks_per_head);
+  const cudaError_t e = launch_in_order(compact_kernel, grid, 256, 0, stream, g, (const char*)k,
+                                        (const char*)v, k_ls, v_ls, keep_idx, head_offsets, row_off,
+                                        (char*)k_out, (char*)v_out, blocks_per_head);
   count_launches(1);
-  return check_cuda(cudaGetLastError(), "compact_kv launch");
+  return check_cuda(e, "compact_kv launch");
 }
 
 }  // namespace lava

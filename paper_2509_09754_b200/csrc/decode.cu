@@ -320,6 +320,7 @@ __device__ inline void fold_chunks(const float* src, size_t stride, int n, float
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32)
 decode_kernel(const DecodeParams p) {
+  in_stream_order();
   using S = Stage<D>;
   extern __shared__ __align__(128) unsigned char stage_mem[];
   __shared__ int2 wsum[kWarps];
@@ -494,6 +495,7 @@ decode_kernel(const DecodeParams p) {
 // for nothing.
 __global__ void __launch_bounds__(1024)
 list_chunks_kernel(const DecodeParams p) {
+  in_stream_order();
   __shared__ int wsum[32];
   __shared__ int base;
   const Geom& g = p.g;
@@ -531,6 +533,7 @@ list_chunks_kernel(const DecodeParams p) {
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32)
 decode_listed_kernel(const DecodeParams p) {
+  in_stream_order();
   extern __shared__ __align__(128) unsigned char stage_mem[];
   const Geom& g = p.g;
   const int n_items = *p.n_items;
@@ -550,6 +553,7 @@ decode_listed_kernel(const DecodeParams p) {
 template <int D>
 __global__ void __launch_bounds__(kWarps * 32)
 decode_combine_kernel(const DecodeParams p) {
+  in_stream_order();
   const Geom& g = p.g;
   const int u = blockIdx.x * kWarps + (threadIdx.x >> 5), head = u / g.group, q = u - head * g.group;
   if (head >= p.heads) return;
@@ -570,6 +574,7 @@ __device__ inline float elem(const void* ptr, int dtype, long long i) {
 
 __global__ void __launch_bounds__(128)
 decode_generic_kernel(const DecodeParams p) {
+  in_stream_order();
   __shared__ float q[128], pr[128], red[4];
   const Geom& g = p.g;
   const int h = blockIdx.x, prob = blockIdx.y, kvh = h / g.group, d = g.head_dim;
@@ -658,11 +663,12 @@ lava_status launch_decode(const DecodeParams& p, int n_layers, cudaStream_t stre
   const long long most = (long long)part_slots(p.g, n_layers);
   const int grid = (int)std::max<long long>(1, std::min<long long>(slots, (most + kWarps - 1) / kWarps));
   if (list) {
-    list_chunks_kernel<<<1, 1024, 0, stream>>>(p);
-    decode_listed_kernel<D><<<grid, kWarps * 32, Stage<D>::kSmem, stream>>>(p);
-    decode_combine_kernel<D><<<(p.heads * p.g.group + kWarps - 1) / kWarps, kWarps * 32, 0, stream>>>(p);
+    launch_in_order(list_chunks_kernel, 1, 1024, 0, stream, p);
+    launch_in_order(decode_listed_kernel<D>, grid, kWarps * 32, Stage<D>::kSmem, stream, p);
+    launch_in_order(decode_combine_kernel<D>, (p.heads * p.g.group + kWarps - 1) / kWarps, kWarps * 32,
+                    0, stream, p);
   } else {
-    decode_kernel<D><<<grid, kWarps * 32, Stage<D>::kSmem, stream>>>(p);
+    launch_in_order(decode_kernel<D>, grid, kWarps * 32, Stage<D>::kSmem, stream, p);
   }
   count_launches(list ? 3 : 1);
   return check_cuda(cudaGetLastError(), "decode attention launch");
@@ -714,7 +720,7 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
   cudaStream_t st = (cudaStream_t)stream;
   const bool tensor_path = g.dtype == LAVA_BF16 && g.group <= 8;
   if (!tensor_path) {
-    decode_generic_kernel<<<dim3(g.n_q_heads, n_layers * g.batch), 128, 0, st>>>(p);
+    launch_in_order(decode_generic_kernel, dim3(g.n_q_heads, n_layers * g.batch), 128, 0, st, p);
     count_launches(1);
     return check_cuda(cudaGetLastError(), "decode attention launch");
   }

@@ -116,6 +116,7 @@ __device__ inline void for_each_logit(const Tiles& t, const Geom& g, F&& f) {
 // ------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 value_norm_partial_kernel(Geom g, const char* v, long long v_ls, float* vpart, int n_vslices) {
+  in_stream_order();
   const int prob = blockIdx.z, layer = prob / g.batch, b = prob - layer * g.batch;
   const int kvh = blockIdx.y, slice = blockIdx.x;
   const SeqInfo s = seq_info(g, b);
@@ -167,6 +168,7 @@ value_norm_partial_kernel(Geom g, const char* v, long long v_ls, float* vpart, i
 __global__ void __launch_bounds__(kThreads)
 stats_partial_kernel(Geom g, const char* q, const char* k, long long q_ls, long long k_ls,
                      float2* stats, int n_slices) {
+  in_stream_order();
   extern __shared__ float smem[];
   const Tiles t = carve(smem, g);
   __shared__ float run_m[128], run_z[128];
@@ -225,6 +227,7 @@ stats_partial_kernel(Geom g, const char* q, const char* k, long long q_ls, long 
 __global__ void combine_kernel(Geom g, const float2* stats, int n_slices, const float* vpart,
                                int n_vslices, const float* vbar_in, float* neg_lse, float* vbar,
                                float* vbar_out, unsigned* status) {
+  in_stream_order();
   const int prob = blockIdx.y, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
   const int used = ceil_div(s.n, kSlice);
@@ -265,6 +268,7 @@ __global__ void __launch_bounds__(kThreads)
 score_kernel(Geom g, const char* q, const char* k, long long q_ls, long long k_ls,
              const float* neg_lse, const float* vbar, float* scores, double2* ent_part,
              int n_slices) {
+  in_stream_order();
   extern __shared__ float smem[];
   const Tiles t = carve(smem, g);
   // a[h_local][i - a_lo], window-mean attention of every head of the group on the slice + halo
@@ -364,6 +368,7 @@ score_kernel(Geom g, const char* q, const char* k, long long q_ls, long long k_l
 // ------------------------------------------------------------------------------------------
 __global__ void entropy_finalize_kernel(Geom g, const double2* ent_part, int n_slices,
                                         double* entropy) {
+  in_stream_order();
   const int prob = blockIdx.x, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
   const int used = ceil_div(s.prefix, kSlice);
@@ -404,8 +409,8 @@ lava_status launch_score_generic(const Geom& g, int n_layers, const void* q, con
 
   if (!vbar_in) {
     dim3 grid(lay.n_vslices, g.n_kv_heads, problems);
-    value_norm_partial_kernel<<<grid, 256, 0, stream>>>(g, (const char*)v, v_ls, vpart,
-                                                        lay.n_vslices);
+    launch_in_order(value_norm_partial_kernel, grid, 256, 0, stream, g, (const char*)v, v_ls, vpart,
+                    lay.n_vslices);
   }
   const size_t tile_bytes = tiles_bytes(g);
   const size_t score_bytes =
@@ -424,21 +429,20 @@ lava_status launch_score_generic(const Geom& g, int n_layers, const void* q, con
     return fail(LAVA_ERR_UNSUPPORTED, "window/group too large for the generic score kernel");
   {
     dim3 grid(lay.n_slices, g.n_q_heads, problems);
-    stats_partial_kernel<<<grid, kThreads, tile_bytes, stream>>>(
-        g, (const char*)q, (const char*)k, q_ls, k_ls, stats, lay.n_slices);
+    launch_in_order(stats_partial_kernel, grid, kThreads, tile_bytes, stream, g, (const char*)q, (const
+                    char*)k, q_ls, k_ls, stats, lay.n_slices);
   }
   {
     dim3 grid(g.n_q_heads + 1, problems);
-    combine_kernel<<<grid, 128, 0, stream>>>(g, stats, lay.n_slices, vpart, lay.n_vslices, vbar_in,
-                                            neg_lse, vbar, vbar_out, status);
+    launch_in_order(combine_kernel, grid, 128, 0, stream, g, stats, lay.n_slices, vpart, lay.n_vslices,
+                    vbar_in, neg_lse, vbar, vbar_out, status);
   }
   {
     dim3 grid(lay.n_slices, g.n_kv_heads, problems);
-    score_kernel<<<grid, kThreads, score_bytes, stream>>>(g, (const char*)q, (const char*)k, q_ls,
-                                                         k_ls, neg_lse, vbar, scores, ent_part,
-                                                         lay.n_slices);
+    launch_in_order(score_kernel, grid, kThreads, score_bytes, stream, g, (const char*)q, (const char*)k,
+                    q_ls, k_ls, neg_lse, vbar, scores, ent_part, lay.n_slices);
   }
-  entropy_finalize_kernel<<<problems, 32, 0, stream>>>(g, ent_part, lay.n_slices, entropy);
+  launch_in_order(entropy_finalize_kernel, problems, 32, 0, stream, g, ent_part, lay.n_slices, entropy);
   count_launches(vbar_in ? 4 : 5);
   return check_cuda(cudaGetLastError(), "score (generic) launch");
 }

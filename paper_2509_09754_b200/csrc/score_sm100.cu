@@ -956,6 +956,7 @@ __global__ void __launch_bounds__(256)
 entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph_max, int chunk_tiles,
                               double* entropy, const float* vbar_in, const unsigned* vbar_bits,
                               float* vbar_out) {
+  in_stream_order();
   __shared__ double rs[8], rt[8];
   const int prob = blockIdx.x, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
@@ -1014,6 +1015,7 @@ constexpr int kEntropySlice = 32768;
 __global__ void __launch_bounds__(1024)
 entropy_from_scores_kernel(Geom g, const float* scores, double2* part, double* entropy,
                            const float* vbar_in, const unsigned* vbar_bits, float* vbar_out) {
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;
   const int prob = blockIdx.y, layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
@@ -1052,6 +1054,7 @@ entropy_from_scores_kernel(Geom g, const float* scores, double2* part, double* e
 
 __global__ void __launch_bounds__(32)
 entropy_from_slices_kernel(Geom g, const double2* part, int slices, double* entropy) {
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;
   const int prob = blockIdx.x, b = prob % g.batch;
   const SeqInfo s = seq_info(g, b);
@@ -1136,10 +1139,10 @@ lava_status launch_entropy_from_scores(const Geom& g, int n_layers, const float*
   const long long most = (long long)g.n_kv_heads * (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
   const int slices = most > kEntropySlice ? (int)((most + kEntropySlice - 1) / kEntropySlice) : 1;
   const int problems = n_layers * g.batch;
-  entropy_from_scores_kernel<<<dim3(slices, problems), 1024, 0, stream>>>(
-      g, scores, slices > 1 ? scratch : nullptr, entropy, vbar_in, vbar_bits, vbar_out);
+  launch_in_order(entropy_from_scores_kernel, dim3(slices, problems), 1024, 0, stream, g, scores, slices
+                  > 1 ? scratch : nullptr, entropy, vbar_in, vbar_bits, vbar_out);
   if (slices > 1)
-    entropy_from_slices_kernel<<<problems, 32, 0, stream>>>(g, scratch, slices, entropy);
+    launch_in_order(entropy_from_slices_kernel, problems, 32, 0, stream, g, scratch, slices, entropy);
   count_launches(slices > 1 ? 2 : 1);
   return check_cuda(cudaGetLastError(), "entropy launch");
 }
@@ -1341,8 +1344,8 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
     return launch_entropy_from_scores(g, n_layers, scores, entropy, ent_scratch, vbar_in, p.vbar_bits,
                                       vbar_out, stream);
   }
-  entropy_finalize_sm100_kernel<<<n_layers * g.batch, 256, 0, stream>>>(
-      g, p.ent_part, lay.chunks, p.chunk_tiles, entropy, vbar_in, p.vbar_bits, vbar_out);
+  launch_in_order(entropy_finalize_sm100_kernel, n_layers * g.batch, 256, 0, stream, g, p.ent_part,
+                  lay.chunks, p.chunk_tiles, entropy, vbar_in, p.vbar_bits, vbar_out);
   count_launches(2);
   return check_cuda(cudaGetLastError(), "entropy finalize launch");
 }

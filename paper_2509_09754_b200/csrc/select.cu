@@ -103,6 +103,7 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
   uint4* cache = reinterpret_cast<uint4*>(dyn + kBins * kCopies * 4);
   __shared__ SelectShared sh;
   for (int i = threadIdx.x; i < kBins; i += kThreads) cells[i] = make_uint4(0u, 0u, 0u, 0u);
+  in_stream_order();
   if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
@@ -487,13 +488,15 @@ lava_status launch(const Geom& g, int problems, long long m_max, const float* sc
   cfg.blockDim = dim3(kThreads);
   cfg.dynamicSmemBytes = kDynSmem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = csize;
-  attr.val.clusterDim.y = 1;
-  attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = csize;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   e = cudaLaunchKernelEx(&cfg, kern, g, scores, layer_budget, keep_idx, head_offsets, io);
   count_launches(1);
   return check_cuda(e, what);
