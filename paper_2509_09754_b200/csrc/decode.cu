@@ -566,56 +566,103 @@ decode_combine_kernel(const DecodeParams p) {
                    (size_t)g.group * (D + 4), n, dst);
 }
 
-// Any geometry: one block per (query head, layer*sequence), tiles of 128 rows.
-__device__ inline float elem(const void* ptr, int dtype, long long i) {
-  return dtype == LAVA_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(ptr)[i])
-                            : reinterpret_cast<const float*>(ptr)[i];
-}
+// Any geometry: one block per (query head, layer*sequence), tiles of 1024 rows in the base-2 domain.
+// Bound by latency: a warp takes every eighth group of rows with 16-byte loads, d / 4 or d / 8 lanes per
+// row, so that all rows of a small head are in flight at once (128 threads with a row each and scalar
+// loads took 12 us for one fp32 layer of 8 heads, this takes 4).  Sums are taken in a fixed order.
+constexpr int kGenThreads = 256;
+constexpr int kGenTile = 1024;
 
-__global__ void __launch_bounds__(128)
+template <int D, bool BF16>
+__global__ void __launch_bounds__(kGenThreads)
 decode_generic_kernel(const DecodeParams p) {
   in_stream_order();
-  __shared__ float q[128], pr[128], red[4];
+  constexpr int kPer = BF16 ? 8 : 4;     // elements per 16-byte load
+  constexpr int kLanes = D / kPer;       // lanes per row: 8, 16 or 32
+  constexpr int kGroups = kGenThreads / kLanes;
+  __shared__ float pr[kGenTile], red[8];
+  __shared__ float sums[kGroups][D];
   const Geom& g = p.g;
-  const int h = blockIdx.x, prob = blockIdx.y, kvh = h / g.group, d = g.head_dim;
+  const int h = blockIdx.x, prob = blockIdx.y, kvh = h / g.group;
   const int* hoff = p.head_offsets + (size_t)prob * (g.n_kv_heads + 1);
   const int len = hoff[kvh + 1] - hoff[kvh];
-  const long long row0 = p.row_off[prob] + hoff[kvh];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < d) q[tid] = elem(p.q, g.dtype, ((long long)prob * g.n_q_heads + h) * d + tid);
-  __syncthreads();
-  float m = -INFINITY, l = 0.f, acc = 0.f;
-  for (int i0 = 0; i0 < len; i0 += 128) {
-    const int i = i0 + tid;
-    float x = -INFINITY;
-    if (i < len) {
-      float z = 0.f;
-      for (int c = 0; c < d; ++c) z = fmaf(q[c], elem(p.k_rows, g.dtype, (row0 + i) * d + c), z);
-      x = z * g.scale_log2;
+  const char* k = p.k_rows + (p.row_off[prob] + hoff[kvh]) * (D / kPer * 16);
+  const char* v = p.v_rows + (p.row_off[prob] + hoff[kvh]) * (D / kPer * 16);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, group = tid / kLanes, c = tid % kLanes;
+  auto unpack = [](const uint4& raw, float (&x)[kPer]) {
+    if constexpr (BF16) {
+      const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        x[2 * j] = bf16_lo(w[j]);
+        x[2 * j + 1] = bf16_hi(w[j]);
+      }
+    } else {
+      x[0] = __uint_as_float(raw.x);
+      x[1] = __uint_as_float(raw.y);
+      x[2] = __uint_as_float(raw.z);
+      x[3] = __uint_as_float(raw.w);
     }
-    float bm = x;
-    for (int o = 16; o > 0; o >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-    if (lane == 0) red[warp] = bm;
+  };
+  auto block_reduce = [&](float x, auto op) {  // the same order in every thread
+    for (int o = 16; o > 0; o >>= 1) x = op(x, __shfl_xor_sync(0xffffffffu, x, o));
     __syncthreads();
-    const float m_new = fmaxf(m, fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3])));
-    const float e = exp2f(x - m_new);
-    pr[tid] = e;
-    float bs = e;
-    for (int o = 16; o > 0; o >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, o);
+    if (lane == 0) red[warp] = x;
     __syncthreads();
-    if (lane == 0) red[warp] = bs;
-    __syncthreads();
+    x = red[0];
+    for (int w = 1; w < kGenThreads / 32; ++w) x = op(x, red[w]);
+    return x;
+  };
+  float q[kPer];
+  unpack(reinterpret_cast<const uint4*>(p.q)[((long long)prob * g.n_q_heads + h) * kLanes + c], q);
+  float m = -INFINITY, l = 0.f, acc[kPer] = {};
+  for (int i0 = 0; i0 < len; i0 += kGenTile) {
+    const int cnt = min(kGenTile, len - i0);
+    float best = -INFINITY;
+#pragma unroll 4
+    for (int r0 = 0; r0 < cnt; r0 += kGroups) {
+      const int r = r0 + group;
+      float x[kPer], z = 0.f;
+      unpack(r < cnt ? reinterpret_cast<const uint4*>(k)[(long long)(i0 + r) * kLanes + c] : uint4{}, x);
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) z = fmaf(q[j], x[j], z);
+      for (int o = kLanes / 2; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      z *= g.scale_log2;
+      if (r < cnt) {
+        best = fmaxf(best, z);
+        if (c == 0) pr[r] = z;
+      }
+    }
+    const float m_new = fmaxf(m, block_reduce(best, [](float a, float b) { return fmaxf(a, b); }));
+    float sum = 0.f;
+    for (int r = tid; r < cnt; r += kGenThreads) {
+      const float e = exp2f(pr[r] - m_new);
+      pr[r] = e;
+      sum += e;
+    }
+    sum = block_reduce(sum, [](float a, float b) { return a + b; });  // also: all of pr is written
     const float corr = exp2f(m - m_new);
-    l = l * corr + ((red[0] + red[1]) + (red[2] + red[3]));
-    acc *= corr;
+    l = l * corr + sum;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) acc[j] *= corr;
     m = m_new;
-    if (tid < d) {
-      const int cnt = min(128, len - i0);
-      for (int r = 0; r < cnt; ++r) acc = fmaf(pr[r], elem(p.v_rows, g.dtype, (row0 + i0 + r) * d + tid), acc);
+#pragma unroll 4
+    for (int r = group; r < cnt; r += kGroups) {
+      float x[kPer];
+      unpack(reinterpret_cast<const uint4*>(v)[(long long)(i0 + r) * kLanes + c], x);
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) acc[j] = fmaf(pr[r], x[j], acc[j]);
     }
-    __syncthreads();
+    __syncthreads();  // pr is written again
   }
-  if (tid < d) p.out[((size_t)prob * g.n_q_heads + h) * d + tid] = len > 0 ? acc / l : 0.f;
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) sums[group][c * kPer + j] = acc[j];
+  __syncthreads();
+  if (tid < D) {
+    float x = 0.f;
+    for (int i = 0; i < kGroups; ++i) x += sums[i][tid];
+    p.out[((size_t)prob * g.n_q_heads + h) * D + tid] = len > 0 ? x / l : 0.f;
+  }
 }
 
 inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -720,7 +767,11 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
   cudaStream_t st = (cudaStream_t)stream;
   const bool tensor_path = g.dtype == LAVA_BF16 && g.group <= 8;
   if (!tensor_path) {
-    launch_in_order(decode_generic_kernel, dim3(g.n_q_heads, n_layers * g.batch), 128, 0, st, p);
+    auto kern = g.dtype == LAVA_BF16 ? (g.head_dim == 64 ? decode_generic_kernel<64, true>
+                                                         : decode_generic_kernel<128, true>)
+                                     : (g.head_dim == 64 ? decode_generic_kernel<64, false>
+                                                         : decode_generic_kernel<128, false>);
+    launch_in_order(kern, dim3(g.n_q_heads, n_layers * g.batch), kGenThreads, 0, st, p);
     count_launches(1);
     return check_cuda(cudaGetLastError(), "decode attention launch");
   }

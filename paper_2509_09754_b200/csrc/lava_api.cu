@@ -139,21 +139,28 @@ Workspace workspace_layout(const lava_layer_desc* d, int n_layers) {
   Workspace w;
   const int max_seqlen = d->max_seqlen > 0 ? d->max_seqlen : (int)d->total_tokens;
   const size_t problems = (size_t)n_layers * d->batch;
-  w.n_slices = ceil_div(max_seqlen, Workspace::kSlice);
-  w.n_vslices = ceil_div(max_seqlen, Workspace::kVSlice);
+  // 64 keys per block up to 2048 tokens, 128 up to 4096, 256 up to 8192, then 512.  Score call in us with
+  // 64 / 128 / 512: one fp32 layer of 1000 tokens with 8 heads 32 / 41 / 122, of 4000 44 / 44 / 123, of 2000
+  // with 32 heads of 128 84 / 66 / 203; 32 layers x 32 heads of 4000 2046 / 1597 / 1397; 16 layers of 8000
+  // - / 2769 / 2722.  The rule looks at the length alone, so a layer gives the same bits alone and among
+  // others.
+  w.slice_keys = 64;
+  while (w.slice_keys < 512 && max_seqlen > 32 * w.slice_keys) w.slice_keys *= 2;
+  w.n_slices = ceil_div(max_seqlen, w.slice_keys);
+  // scores are pooled over up to 8 neighbours on either side: with them a slice is whole tiles of 64 keys
+  w.score_keys = d->pool_kind != LAVA_POOL_NONE && d->pool_kernel / 2 > 8 ? w.slice_keys : w.slice_keys - 16;
+  w.n_score_slices = ceil_div(max_seqlen, w.score_keys);
   size_t off = Workspace::kStatusBytes;
   w.off_vpart = off;
-  off = round_up(off + problems * d->n_kv_heads * w.n_vslices * sizeof(float), 256);
+  off = round_up(off + problems * d->n_kv_heads * w.n_slices * sizeof(float), 256);
   w.off_stats = off;
   off = round_up(off + problems * d->n_q_heads * w.n_slices * d->window * sizeof(float2), 256);
   w.off_lse = off;
   off = round_up(off + problems * d->n_q_heads * d->window * sizeof(float), 256);
-  w.off_vbar = off;
-  off = round_up(off + problems * d->n_kv_heads * sizeof(float), 256);
   w.off_ones = off;
   off = round_up(off + problems * d->n_kv_heads * sizeof(float), 256);
   w.off_ent = off;
-  off = round_up(off + problems * d->n_kv_heads * w.n_slices * sizeof(double2), 256);
+  off = round_up(off + problems * d->n_kv_heads * w.n_score_slices * sizeof(double2), 256);
   w.off_sm100 = off;
   Geom g;
   const bool tensor_path = make_geom(d, &g) == LAVA_OK && sm100_supported(g);

@@ -64,10 +64,9 @@ __device__ inline bool batch_has_short_sequence(const Geom& g) {
 // Workspace layout (byte offsets from the workspace base), identical for every caller.
 struct Workspace {
   static constexpr size_t kStatusBytes = 256;
-  static constexpr int kSlice = 512;    // keys per block in the generic score kernels
-  static constexpr int kVSlice = 1024;  // V rows per block in the value-norm kernel
-  size_t off_vpart, off_stats, off_lse, off_vbar, off_ones, off_ent, off_sm100, off_tmem, total;
-  int n_slices, n_vslices;
+  // generic score path: keys per block of the statistics (and rows of V), and of the scores
+  int slice_keys, n_slices, score_keys, n_score_slices;
+  size_t off_vpart, off_stats, off_lse, off_ones, off_ent, off_sm100, off_tmem, total;
 };
 Workspace workspace_layout(const lava_layer_desc* d, int n_layers);
 
