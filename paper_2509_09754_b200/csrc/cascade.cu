@@ -88,60 +88,6 @@ __global__ void cascade_init_kernel(Geom g, int n_layers, long long rows, const 
   }
 }
 
-// Scores and positions of the entries the new layer keeps, taken from its full arrays into its
-// list (the list of sequence b starts at row_off[b]).
-__global__ void __launch_bounds__(256)
-cascade_adopt_kernel(Geom g, const float* scores_full, const int* keep_full, const int* head_offsets,
-                     const long long* row_off, float* score_list, int* pos_list) {
-  in_stream_order();
-  if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
-  const int b = blockIdx.y;
-  const SeqInfo s = seq_info(g, b);
-  const int win = min(g.window, s.n);
-  const int* hoff = head_offsets + (size_t)b * (g.n_kv_heads + 1);
-  const int kept = hoff[g.n_kv_heads] - g.n_kv_heads * win;
-  const long long base = row_off[b];
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < kept; j += gridDim.x * blockDim.x) {
-    int head = 0;
-    while (head + 1 < g.n_kv_heads && hoff[head + 1] - (head + 1) * win <= j) ++head;
-    const int pos = keep_full[s.score_off + j];
-    pos_list[base + j] = pos;
-    score_list[base + j] = scores_full[s.score_off + (long long)head * s.prefix + pos];
-  }
-}
-
-// Rows of the lower layers move from the old arena to their place in the new one: for
-// (layer, sequence, head) the kept rows named by the source map, then the w window rows.
-__global__ void __launch_bounds__(256)
-cascade_move_kernel(Geom g, const int* src_pos, const int* hoff_old_all, const int* hoff_new_all,
-                    const long long* roff_old, const long long* roff_new, const char* k_old,
-                    const char* v_old, char* k_new, char* v_new, int blocks_per_head) {
-  in_stream_order();
-  if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
-  const int prob = blockIdx.z, b = prob % g.batch, kvh = blockIdx.y;
-  const SeqInfo s = seq_info(g, b);
-  const int win = min(g.window, s.n);
-  const int row_bytes = g.head_dim * (g.dtype == LAVA_BF16 ? 2 : 4);
-  const int lanes = row_bytes / 16;
-  const int* ho = hoff_old_all + (size_t)prob * (g.n_kv_heads + 1);
-  const int* hn = hoff_new_all + (size_t)prob * (g.n_kv_heads + 1);
-  const int h0 = hn[kvh], rows = hn[kvh + 1] - h0, kept = rows - win;
-  const long long new0 = roff_new[prob], old0 = roff_old[prob];
-  const int* src = src_pos + new0 + (h0 - kvh * win);  // this head's entries of the new list
-  const long long old_window0 = old0 + ho[kvh + 1] - win;
-  const int rows_per_iter = blockDim.x / lanes;
-  const int sub = threadIdx.x / lanes, c = threadIdx.x - sub * lanes;
-  for (int r = blockIdx.x * rows_per_iter + sub; r < rows; r += blocks_per_head * rows_per_iter) {
-    // entry p of the old list sits in old row p + kvh*win of the sequence's segment
-    const long long from = r < kept ? old0 + src[r] + (long long)kvh * win : old_window0 + (r - kept);
-    const uint4 kk = *reinterpret_cast<const uint4*>(k_old + from * row_bytes + c * 16);
-    const uint4 vv = *reinterpret_cast<const uint4*>(v_old + from * row_bytes + c * 16);
-    const long long dst = (new0 + h0 + r) * row_bytes + c * 16;
-    *reinterpret_cast<uint4*>(k_new + dst) = kk;
-    *reinterpret_cast<uint4*>(v_new + dst) = vv;
-  }
-}
-
 }  // namespace
 }  // namespace lava
 
@@ -250,49 +196,24 @@ lava_status lava_cascade_step(lava_cascade* h, const void* q_win, const void* k,
                       (const long long*)(base + c.off_floor), (const long long*)(base + c.off_cap),
                       h->mode, budget_new, roff_new, (unsigned*)workspace, st);
   if (rc != LAVA_OK) return rc;
-  // Evict(B_t, s_t, K_t, V_t): layer-wide top-k of the full layer, rows and list entries
-  rc = launch_select(g, 1, scores_full, budget_new + lb_t, keep_full,
-                     hoff_new + lb_t * (g.n_kv_heads + 1), (unsigned*)workspace, st);
+  // Evict(B_t, s_t, K_t, V_t): layer-wide top-k of the full layer; Evict(B_l, s_l, K_l, V_l) for every
+  // lower layer, from what it still holds; then the rows of both
+  HeldLists io;
+  io.score_old = (const float*)(base + c.off_score[from]);
+  io.pos_old = (const int*)(base + c.off_pos[from]);
+  io.row_off_old = (const long long*)(base + c.off_roff[from]);
+  io.hoff_old = (const int*)(base + c.off_hoff[from]);
+  io.score_new = (float*)(base + c.off_score[to]);
+  io.pos_new = (int*)(base + c.off_pos[to]);
+  io.src_pos = (int*)(base + c.off_src);
+  io.row_off_new = roff_new;
+  const long long prefix_max = g.max_seqlen > g.window ? g.max_seqlen - g.window : 0;
+  const long long max_held = std::min<long long>((long long)g.n_kv_heads * prefix_max, h->rows);
+  rc = launch_select_cascade(g, t * g.batch, max_held, scores_full, budget_new, keep_full, hoff_new, io, st);
   if (rc != LAVA_OK) return rc;
-  rc = launch_compact(g, 1, k, v, 0, 0, keep_full, hoff_new + lb_t * (g.n_kv_heads + 1),
-                      roff_new + lb_t, base + c.off_k[to], base + c.off_v[to], st);
+  rc = launch_cascade_rows(g, t * g.batch, io, hoff_new, base + c.off_k[from], base + c.off_v[from], k, v,
+                           keep_full, base + c.off_k[to], base + c.off_v[to], st);
   if (rc != LAVA_OK) return rc;
-  if (g.total_scores > 0) {
-    dim3 grid(std::max(1, std::min(64, sm_count() * 4 / std::max(1, g.batch))), g.batch);
-    launch_in_order(cascade_adopt_kernel, grid, 256, 0, st, g, scores_full, keep_full, hoff_new + lb_t *
-                    (g.n_kv_heads + 1), roff_new + lb_t, (float*)(base + c.off_score[to]), (int*)(base +
-                    c.off_pos[to]));
-    count_launches(1);
-    rc = check_cuda(cudaGetLastError(), "cascade adopt launch");
-    if (rc != LAVA_OK) return rc;
-  }
-  // Evict(B_l, s_l, K_l, V_l) for every lower layer, from what it still holds
-  if (t > 0) {
-    HeldLists io;
-    io.score_old = (const float*)(base + c.off_score[from]);
-    io.pos_old = (const int*)(base + c.off_pos[from]);
-    io.row_off_old = (const long long*)(base + c.off_roff[from]);
-    io.hoff_old = (const int*)(base + c.off_hoff[from]);
-    io.score_new = (float*)(base + c.off_score[to]);
-    io.pos_new = (int*)(base + c.off_pos[to]);
-    io.src_pos = (int*)(base + c.off_src);
-    io.row_off_new = roff_new;
-    const long long prefix_max = g.max_seqlen > g.window ? g.max_seqlen - g.window : 0;
-    const long long max_held = std::min<long long>((long long)g.n_kv_heads * prefix_max, h->rows);
-    rc = launch_reselect(g, t * g.batch, max_held, budget_new, hoff_new, io, st);
-    if (rc != LAVA_OK) return rc;
-    const int heads_total = t * g.batch * g.n_kv_heads;
-    const int sms = sm_count() > 0 ? sm_count() : 1;
-    int bph = std::max(1, (sms * 8 + heads_total - 1) / heads_total);
-    bph = std::min(bph, std::max(1, (g.max_seqlen + 15) / 16));
-    dim3 grid(bph, g.n_kv_heads, t * g.batch);
-    launch_in_order(cascade_move_kernel, grid, 256, 0, st, g, io.src_pos, io.hoff_old, hoff_new,
-                    io.row_off_old, roff_new, base + c.off_k[from], base + c.off_v[from], base +
-                    c.off_k[to], base + c.off_v[to], bph);
-    count_launches(1);
-    rc = check_cuda(cudaGetLastError(), "cascade move launch");
-    if (rc != LAVA_OK) return rc;
-  }
   h->layers_done = t + 1;
   h->begun = true;
   return LAVA_OK;

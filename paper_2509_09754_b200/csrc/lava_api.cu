@@ -360,9 +360,10 @@ lava_status lava_select_topk_layers(const lava_layer_desc* desc, int32_t n_layer
     return fail(LAVA_ERR_INVALID_ARG, "NULL argument");
   if ((long long)n_layers * g.batch > 65535)
     return fail(LAVA_ERR_UNSUPPORTED, "n_layers*batch must be <= 65535");
+  (void)workspace;
   (void)workspace_bytes;
   return launch_select(g, n_layers, scores, (const long long*)layer_budget, keep_idx, head_offsets,
-                       (unsigned*)workspace, (cudaStream_t)stream);
+                       (cudaStream_t)stream);
 }
 
 lava_status lava_select_topk(const lava_layer_desc* desc, const float* scores,

@@ -171,7 +171,7 @@ lava_status launch_budgets(int n_layers, int batch, const double* entropy,
                            cudaStream_t stream);
 lava_status launch_select(const Geom& g, int n_layers, const float* scores,
                           const long long* layer_budget, int* keep_idx, int* head_offsets,
-                          unsigned* status, cudaStream_t stream);
+                          cudaStream_t stream);
 // Lists of what every (layer, sequence) still holds during Algorithm 2's cascade: score and
 // position of each held prefix entry, heads in order and positions ascending inside a head; the
 // list of problem p starts at entry row_off[p] and its heads are delimited like the packed rows
@@ -186,10 +186,17 @@ struct HeldLists {
   int* src_pos = nullptr;           // for every new entry: its index in the old list
   const long long* row_off_new = nullptr;
 };
-// Re-selection of `problems` (layer, sequence) lists, each down to layer_budget[p] rows.
-lava_status launch_reselect(const Geom& g, int problems, long long max_held,
-                            const long long* layer_budget, int* head_offsets_new,
-                            const HeldLists& io, cudaStream_t stream);
+// One step of the cascade: `n_lists` (layer, sequence) lists, each down to layer_budget[p] rows, and after
+// them, in every array by problem, the sequences of the new layer from its full scores.  The new layer's
+// kept entries become its lists, score_new and pos_new from row_off_new[problem] on.
+lava_status launch_select_cascade(const Geom& g, int n_lists, long long max_held, const float* scores,
+                                  const long long* layer_budget, int* keep_idx, int* head_offsets,
+                                  const HeldLists& io, cudaStream_t stream);
+// The rows of such a step: those of the lists from the old copy of the cache to the new, and the new
+// layer's from its K and V.
+lava_status launch_cascade_rows(const Geom& g, int n_lists, const HeldLists& io, const int* hoff_new,
+                                const char* k_old, const char* v_old, const void* k, const void* v,
+                                const int* keep_idx, char* k_new, char* v_new, cudaStream_t stream);
 lava_status launch_compact(const Geom& g, int n_layers, const void* k, const void* v,
                            long long k_ls, long long v_ls, const int* keep_idx,
                            const int* head_offsets, const long long* row_off, void* k_out,

@@ -79,7 +79,8 @@ __device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 // again with its stored scores): the keys of problem p are the `held` scores of its list, in
 // list order, which is ascending flat index, so ties still go to the lower flat index.  The
 // kept entries' scores and positions are copied to the new list and `src_pos` records where in
-// the old list each came from.
+// the old list each came from.  ADOPT also starts such a list: the kept entries' scores and positions of a
+// layer that is evicted for the first time (17 us at 8K; 15 and 3 with a kernel of its own for the list).
 //
 // Bound by latency (barriers, remote shared memory) at prompt lengths up to 8K and by shared-memory
 // atomics and reads beyond; the keys are 4 bytes a position.  So: a cluster no larger than the keys
@@ -92,25 +93,19 @@ __device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 // passes from memory) with a fixed cluster of 8 or 16, all 2048 bins added up and two barriers per pass:
 // 32 layers of 1K / 8K / 32K: 20.5 / 27 / 99 us before, 11.4 / 19.4 / 39 now; 28 layers of 128K with 4
 // heads: 164 -> 49; 128 ragged problems of up to 32K with 8 heads: 259 -> 87.
-template <bool LIST>
-__global__ void __launch_bounds__(kThreads, 2)
-select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
-                   int* head_offsets, HeldLists io) {
-  extern __shared__ __align__(16) unsigned char dyn[];
+template <bool LIST, bool ADOPT>
+__device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* dyn, const Geom& g, int cl,
+                                               const float* scores, const long long* layer_budget,
+                                               int* keep_idx, int* head_offsets, const HeldLists& io) {
   uint4* cells = reinterpret_cast<uint4*>(dyn);  // histogram copies of one bin; later the masks
   unsigned* copies = reinterpret_cast<unsigned*>(dyn);
   unsigned char* masks = dyn;
   uint4* cache = reinterpret_cast<uint4*>(dyn + kBins * kCopies * 4);
-  __shared__ SelectShared sh;
-  for (int i = threadIdx.x; i < kBins; i += kThreads) cells[i] = make_uint4(0u, 0u, 0u, 0u);
-  in_stream_order();
-  if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
   cg::cluster_group cluster = cg::this_cluster();
   const int csize = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   // one cluster per (layer, sequence); with per-head selection (the "- head dynamic" ablation of
   // Sec. 5.4) one per (layer, sequence, KV head), each on its head's segment alone
   const bool per_head = !LIST && (g.flags & LAVA_FLAG_PER_HEAD_TOPK) != 0;
-  const int cl = blockIdx.x / csize;
   const int prob = per_head ? cl / g.n_kv_heads : cl, layer = prob / g.batch, b = prob - layer * g.batch;
   const int head0 = per_head ? cl - prob * g.n_kv_heads : 0;  // first head of this problem
   const int n_heads = per_head ? 1 : g.n_kv_heads;
@@ -140,7 +135,7 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
       for (int i = 0; i < (k_sel > 0 ? 4 : 1); ++i) cluster.sync();
     return;
   }
-  const long long old0 = LIST ? io.row_off_old[prob] : 0, new0 = LIST ? io.row_off_new[prob] : 0;
+  const long long old0 = LIST ? io.row_off_old[prob] : 0, new0 = LIST || ADOPT ? io.row_off_new[prob] : 0;
   int* hoff = head_offsets + (size_t)prob * (g.n_kv_heads + 1);
 
   // this CTA's range [c0, c0 + n) and the aligned vectors that hold it; key e is element e + mis
@@ -403,24 +398,24 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
             ++slot;
           }
       } else {
-        int pos = e - head_begin;
-        if (starts) {
+        const int pos = e - head_begin;
+        unsigned to = slot;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if ((keep >> j) & 1u) {
-              int at = pos + j;
+        for (int j = 0; j < 4; ++j)
+          if ((keep >> j) & 1u) {
+            int at = pos + j;
+            if (starts)
               while (at >= s.prefix) at -= s.prefix;
-              out[slot] = at;
-              ++slot;
-            }
+            out[to] = at;
+            if (ADOPT) io.pos_new[new0 + to] = at;
+            ++to;
           }
-        } else {
+        if (ADOPT) {  // the list of what the layer holds from now on
+          const uint4 q = key_of(v);
+          const unsigned key[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
           for (int j = 0; j < 4; ++j)
-            if ((keep >> j) & 1u) {
-              out[slot] = pos + j;
-              ++slot;
-            }
+            if ((keep >> j) & 1u) io.score_new[new0 + slot++] = __uint_as_float(key[j]);
         }
       }
     }
@@ -459,6 +454,20 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
   if (active > 1) cluster_wait();  // peers may still be reading this CTA's histograms
 }
 
+template <bool LIST, bool ADOPT>
+__global__ void __launch_bounds__(kThreads, 2)
+select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
+                   int* head_offsets, HeldLists io) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ SelectShared sh;
+  for (int i = threadIdx.x; i < kBins; i += kThreads)
+    reinterpret_cast<uint4*>(dyn)[i] = make_uint4(0u, 0u, 0u, 0u);
+  in_stream_order();
+  if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
+  select_problem<LIST, ADOPT>(sh, dyn, g, blockIdx.x / cg::this_cluster().num_blocks(), scores, layer_budget,
+                              keep_idx, head_offsets, io);
+}
+
 // CTAs per problem.  A CTA takes 8192 keys before another pays for the barriers (32 problems of 7936
 // keys: 11.4 us with one CTA each, 12.9 with two; one of 65K: 15 with eight CTAs, 20 with four).  Once all
 // problems together have more CTAs than the device holds at two per SM, fewer and fuller ones do, up to
@@ -473,12 +482,10 @@ int cluster_size(long long m_max, int problems) {
   return c;
 }
 
-template <bool LIST>
-lava_status launch(const Geom& g, int problems, long long m_max, const float* scores,
-                   const long long* layer_budget, int* keep_idx, int* head_offsets,
-                   cudaStream_t stream, const HeldLists& io, const char* what) {
+template <typename... P, typename... A>
+lava_status launch(void (*kern)(P...), int problems, long long m_max, const char* what, cudaStream_t stream,
+                   A... args) {
   const int csize = cluster_size(m_max, problems);
-  auto kern = select_topk_kernel<LIST>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmem);
   if (e == cudaSuccess && csize > 8)
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -497,7 +504,7 @@ lava_status launch(const Geom& g, int problems, long long m_max, const float* sc
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  e = cudaLaunchKernelEx(&cfg, kern, g, scores, layer_budget, keep_idx, head_offsets, io);
+  e = cudaLaunchKernelEx(&cfg, kern, P(args)...);
   count_launches(1);
   return check_cuda(e, what);
 }
@@ -506,8 +513,7 @@ lava_status launch(const Geom& g, int problems, long long m_max, const float* sc
 
 lava_status launch_select(const Geom& g, int n_layers, const float* scores,
                           const long long* layer_budget, int* keep_idx, int* head_offsets,
-                          unsigned* status, cudaStream_t stream) {
-  (void)status;
+                          cudaStream_t stream) {
   const bool per_head = (g.flags & LAVA_FLAG_PER_HEAD_TOPK) != 0;
   // candidates of the largest problem
   const long long m_max = (long long)(per_head ? 1 : g.n_kv_heads) *
@@ -515,18 +521,25 @@ lava_status launch_select(const Geom& g, int n_layers, const float* scores,
   const int problems = n_layers * g.batch * (per_head ? g.n_kv_heads : 1);
   if (per_head && m_max > kMaxPerHead)
     return fail(LAVA_ERR_UNSUPPORTED, "per-head selection covers up to %d positions per head", kMaxPerHead);
-  return launch<false>(g, problems, m_max, scores, layer_budget, keep_idx, head_offsets, stream,
-                       HeldLists(), "select_topk launch");
+  return launch(select_topk_kernel<false, false>, problems, m_max, "select_topk launch", stream, g, scores,
+                layer_budget, keep_idx, head_offsets, HeldLists());
 }
 
-lava_status launch_reselect(const Geom& g, int problems, long long max_held,
-                            const long long* layer_budget, int* head_offsets_new,
-                            const HeldLists& io, cudaStream_t stream) {
-  if (problems < 1) return LAVA_OK;
-  if (max_held > kMaxHeld)
+lava_status launch_select_cascade(const Geom& g, int n_lists, long long max_held, const float* scores,
+                                  const long long* layer_budget, int* keep_idx, int* head_offsets,
+                                  const HeldLists& io, cudaStream_t stream) {
+  if (n_lists > 0 && max_held > kMaxHeld)
     return fail(LAVA_ERR_UNSUPPORTED, "a layer may hold at most %d entries per sequence here", kMaxHeld);
-  return launch<true>(g, problems, max_held, nullptr, layer_budget, nullptr, head_offsets_new, stream,
-                      io, "reselect launch");
+  if (n_lists > 0) {
+    const lava_status rc = launch(select_topk_kernel<true, false>, n_lists, max_held, "reselect launch", stream,
+                                  g, nullptr, layer_budget, nullptr, head_offsets, io);
+    if (rc != LAVA_OK) return rc;
+  }
+  const long long m_max = (long long)g.n_kv_heads * (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
+  HeldLists adopt = io;
+  adopt.row_off_new += n_lists;
+  return launch(select_topk_kernel<false, true>, g.batch, m_max, "cascade selection launch", stream, g, scores,
+                layer_budget + n_lists, keep_idx, head_offsets + (size_t)n_lists * (g.n_kv_heads + 1), adopt);
 }
 
 }  // namespace lava
