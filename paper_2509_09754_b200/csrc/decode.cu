@@ -402,18 +402,21 @@ decode_kernel(const DecodeParams p) {
       const long long row0 = p.row_off[prob] + h0 + row_lo;
       attend_rows<D, false>(p, stage_mem, head, p.k_rows + row0 * S::kRowBytes, p.v_rows + row0 * S::kRowBytes,
                      nkeys, cb, n == 1, (size_t)chunk);
+      if (n > 1) {
+        __threadfence();
+        __syncwarp();
+        for (int c = chunk + lane; c < chunk + run; c += 32)
+          *reinterpret_cast<volatile unsigned long long*>(p.stamps + c) = p.stamp;
+      }
       chunk += run;
     }
-    __threadfence();
-    __syncwarp();
-    for (int c = c0 + lane; c < c1; c += 32)
-      *reinterpret_cast<volatile unsigned long long*>(p.stamps + c) = p.stamp;
   }
 
   // ---- heads of several chunks: a block that finds all partial results there folds them ----------
   // Every warp leaves its stamps before its block looks, so the last one to leave one sees them all;
-  // two blocks that both do fold the same values in the same order.  The stamps are cleared after the
-  // fold, so that a replayed launch (a captured graph carries its stamp) starts without them.
+  // two blocks that both do fold the same values in the same order.  Only chunks of such heads are stamped,
+  // and the stamps are cleared after the fold, so that a replayed launch (a captured graph carries its
+  // stamp) starts without any, whatever the row counts were that the launch before it found.
   const int b0 = start_at[0].z, b1 = start_at[kWarps].z;  // this block's chunks
   if (b1 <= b0) return;
   __syncthreads();
