@@ -6,22 +6,26 @@
 // One new token's query heads attend to the rows of their KV head:
 //     out[h] = softmax_i( sm_scale * q[h] . K^[g(h)][i] ) V^[g(h)]
 //
-// bf16, one kernel: a head's rows are cut into chunks whose length depends on the head alone (so that
-// a layer gives the same bits whatever else is in the call); every warp of a fixed grid takes
-// consecutive chunks, as many as start in its even share of all blocks of 16 rows, and keeps a running
-// (max, sum, output) per chunk in the base-2 domain.  A head of one chunk is finished there; of a
-// longer head the partial results go to memory and the block that comes last folds them, in chunk
-// order.  Row counts live on the device, so each block derives the split itself from head_offsets.
+// bf16: a head's rows are cut into chunks of 512, a chunk into parts of 128.  The running maximum, which
+// the probabilities are rounded to bf16 against, starts anew with a chunk and runs through its parts in
+// order; a part sums from zero and the parts, then the chunks, are folded in order.  A layer therefore
+// gives the same bits whatever else is in the call and whichever of the two paths serves it.
+//
+// Calls of few rows, one kernel: the blocks of a fixed grid take consecutive chunks, as many as start in
+// their even share of all parts, and a warp takes a part.  Its maximum needs those of the parts before it,
+// so the warp keeps the logits of its rows in registers until the block's warps have met, then multiplies
+// V; the parts are folded through shared memory.  A head of one chunk is finished there; of a longer head
+// the partial results go to memory and the block that comes last folds them.  Row counts live on the
+// device, so each block derives the split itself from head_offsets.
 // K and V blocks of 16 rows are staged per warp in shared memory with cp.async (XOR-swizzled 16-byte
-// pieces, loads in flight across the chunks of a head) and read with ldmatrix for mma.sync m16n8k16:
-// S = Q K^T with the queries padded to the 16 rows of the A operand, then O += P V with V read
-// transposed.  Other geometries take a plain CUDA-core kernel.
+// pieces) and read with ldmatrix for mma.sync m16n8k16: S = Q K^T with the queries padded to the 16 rows
+// of the A operand, then O += P V with V read transposed.  Other geometries take a plain CUDA-core kernel.
 //
 // Bound by latency: a layer's few rows.  Calls that may hold many (see listed()) are bound by the read of
-// the packed rows and take three kernels: a list of chunks of 512 rows, a warp per chunk, a fold.
-// Three kernels for every call, with a block per query head in the fold, took 27-32 us for one layer of
-// 1K to 64K prompts; the one kernel takes 19-21.  32 layers x 64 heads of 128 rows (67 MB): 61 -> 59.
-// Head dimension 64 was a CUDA-core kernel: a call behind the eviction of a 32K prompt went from 145 to 20.
+// the packed rows and take three kernels: a list of the chunks, a warp per chunk, a fold.  One layer of a
+// batch of 8 ragged prompts (64 heads of 128 rows on average): 23 us with three kernels for every call, 15
+// with one kernel whose chunks had 128 rows and were rounded on their own, 12 with this one; 256 heads of
+// 2048 rows (268 MB): 54 (5.0 TB/s).
 #include <algorithm>
 #include <atomic>
 #include <random>
@@ -34,12 +38,12 @@ namespace {
 
 using namespace sm100;
 
-constexpr int kBlk = 16;        // rows per step
+constexpr int kBlk = 16;         // rows per step
 constexpr int kWarps = 4;
-constexpr int kMinChunk = 8;    // blocks per chunk of a short head: 128 rows
-constexpr int kMaxChunks = 64;  // chunks per head: two per lane in the fold
-constexpr int kListChunk = 32;  // blocks per chunk of the listed path: 512 rows
-constexpr int kFoldWords = 32 * kMaxChunks / 32;  // bits for the stamps of 32 heads
+constexpr int kPartBlocks = 8;   // blocks per part of a chunk
+constexpr int kPartRows = kPartBlocks * kBlk;
+constexpr int kChunkRows = kWarps * kPartRows;
+constexpr int kMaxChunks = 256;  // chunks per head that the fold of the one kernel can look at
 
 struct DecodeParams {
   Geom g;
@@ -48,14 +52,15 @@ struct DecodeParams {
   const char* v_rows;
   const int* head_offsets;  // [layers, batch, H_kv + 1]
   const long long* row_off; // [layers * batch (+1)]
-  float* part;              // [chunks][group][d + 4]: outputs, running max, running sum, padding
+  float* part;              // [chunks][group][d]: partial results of the heads of several chunks,
+  float2* part_ml;          // [chunks][group]: and the running max and sum they are relative to
   unsigned long long* stamps;  // [chunks]: the launch's stamp once the partial result is there
   unsigned long long stamp;
   float* out;               // [layers, batch, H_q, d]
   int heads;                // layers * batch * H_kv
   int2* items;              // listed path: (head, chunk) of every chunk that has rows
   int* n_items;
-  int chunks_max;           // listed path: partial results per head
+  int chunks_max;           // chunks per head at max_seqlen
 };
 
 __device__ inline void cp_async16(uint32_t saddr, const void* src, bool valid) {
@@ -87,14 +92,19 @@ __device__ inline void ldmatrix_x4(uint32_t& r0, uint32_t& r1, uint32_t& r2, uin
                : "memory");
 }
 
+// One tile = 16 rows of K or of V, 16-byte pieces XOR-swizzled by the row.
 template <int D>
-struct Stage {
+struct Tile {
   static constexpr int kRowBytes = 2 * D, kPieces = kRowBytes / 16;
-  static constexpr int kTileBytes = kBlk * kRowBytes;  // 16 rows of K or of V
-  static constexpr int kBytes = 2 * kTileBytes;        // K tile, then V tile
-  static constexpr int kStages = D == 128 ? 3 : 6;
-  static constexpr int kSmem = kWarps * kStages * kBytes;
+  static constexpr int kBytes = kBlk * kRowBytes;
+  // Tiles per warp, a warp per chunk (pairs of a K and a V tile) and a warp per part: what covers the
+  // latency of a load with two blocks per SM.  (d = 64, a warp per part, 128 x 2048 and 512 x 700 rows:
+  // 26.7 and 33.9 us with 12 tiles, 25.6 and 32.3 with 8.)
+  static constexpr int kRing = D == 128 ? 6 : 12, kPartRing = D == 128 ? 6 : 8;
+  static constexpr int kFoldStride = D + 8;        // floats per query of a part's result (bank spread)
 };
+static_assert(8 * Tile<64>::kFoldStride * 4 <= Tile<64>::kPartRing * Tile<64>::kBytes &&
+              8 * Tile<128>::kFoldStride * 4 <= Tile<128>::kPartRing * Tile<128>::kBytes, "a part's result fits its ring");
 
 __device__ inline unsigned long long ld_relaxed64(const unsigned long long* p) {
   unsigned long long v;
@@ -102,182 +112,196 @@ __device__ inline unsigned long long ld_relaxed64(const unsigned long long* p) {
   return v;
 }
 
+// Rows of a head; no more than the partial results have room for.
 __device__ inline int head_len(const DecodeParams& p, int h) {
   const int prob = h / p.g.n_kv_heads, kvh = h - prob * p.g.n_kv_heads;
   const int* hoff = p.head_offsets + (size_t)prob * (p.g.n_kv_heads + 1) + kvh;
-  return max(0, hoff[1] - hoff[0]);
+  return (int)min((long long)max(0, hoff[1] - hoff[0]), (long long)p.chunks_max * kChunkRows);
 }
-// Blocks per chunk and chunks of a head of `len` rows: chunks of 128 rows, longer ones when there
-// would be more than 64.
-__device__ inline int chunk_blocks(int len) {
-  const int blocks = (len + kBlk - 1) / kBlk;
-  return blocks > kMinChunk * kMaxChunks ? (blocks + kMaxChunks - 1) / kMaxChunks : kMinChunk;
-}
-__device__ inline int head_chunks(int len) {
-  const int blocks = (len + kBlk - 1) / kBlk, cb = chunk_blocks(len);
-  return (blocks + cb - 1) / cb;
-}
+__device__ inline int head_parts(int len) { return (len + kPartRows - 1) / kPartRows; }
+__device__ inline int head_chunks(int len) { return (len + kChunkRows - 1) / kChunkRows; }
 
-// Attention of one warp over `nkeys` consecutive rows of one head, in chunks of `cb` blocks: the result
-// itself where the rows are the whole head, else a partial result per chunk from slot `slot` on.
-template <int D, bool kOneChunk>
-__device__ __forceinline__ void attend_rows(const DecodeParams& p, unsigned char* stage_mem, int head,
-                                            const char* krow, const char* vrow, int nkeys, int cb,
-                                            bool whole, size_t slot) {
-  using S = Stage<D>;
-  constexpr int kStages = S::kStages, kSteps = D / 16, kOut = D / 8;
-  const Geom& g = p.g;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int qrow = lane >> 2, t = lane & 3;  // row and column pair of the MMA fragments
-  const uint32_t sbase = smem_u32(stage_mem) + warp * (kStages * S::kBytes);
-  const float sc2 = g.scale_log2;
-  const int mi = lane >> 3, r8 = lane & 7;
-  // query fragments (A operand, 16 x 16 per k-step): rows 0..G-1 hold the head's queries
-  uint32_t qa[kSteps][2];
+// Query fragments of a KV head (A operand, 16 x 16 per k-step): rows 0..G-1 hold the head's queries.
+template <int D>
+__device__ __forceinline__ void load_queries(const DecodeParams& p, int head, uint32_t (&qa)[D / 16][2]) {
+  const int lane = threadIdx.x & 31, qrow = lane >> 2, t = lane & 3;
 #pragma unroll
-  for (int s = 0; s < kSteps; ++s) qa[s][0] = qa[s][1] = 0u;
-  if (qrow < g.group) {
-    const char* qh = (const char*)p.q + ((size_t)head * g.group + qrow) * S::kRowBytes;
+  for (int s = 0; s < D / 16; ++s) qa[s][0] = qa[s][1] = 0u;
+  if (qrow < p.g.group) {
+    const char* qh = (const char*)p.q + ((size_t)head * p.g.group + qrow) * Tile<D>::kRowBytes;
 #pragma unroll
-    for (int s = 0; s < kSteps; ++s) {
+    for (int s = 0; s < D / 16; ++s) {
       qa[s][0] = *reinterpret_cast<const uint32_t*>(qh + (16 * s + 2 * t) * 2);
       qa[s][1] = *reinterpret_cast<const uint32_t*>(qh + (16 * s + 8 + 2 * t) * 2);
     }
   }
-  const int nblk = (nkeys + kBlk - 1) / kBlk;
-  // one stage = 16 K rows and 16 V rows, 16-byte pieces XOR-swizzled by the row; rows past the
-  // end are filled with zeros
-  auto fill = [&](int blk, int stage) {
-    const uint32_t st = sbase + stage * S::kBytes;
+}
+
+// Loads block `blk` of `nkeys` rows into the tile at `dst`; rows past the end are filled with zeros.
+template <int D>
+__device__ __forceinline__ void fill_tile(uint32_t dst, const char* rows, int blk, int nkeys) {
+  using T = Tile<D>;
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < kBlk * S::kPieces / 32; ++i) {
-      const int idx = lane + 32 * i, r = idx / S::kPieces, pc = idx % S::kPieces;
-      const int key = blk * kBlk + r;
-      const bool ok = key < nkeys;
-      const long long off = (long long)(ok ? key : 0) * S::kRowBytes + pc * 16;
-      const uint32_t dst = st + r * S::kRowBytes + ((pc ^ (r & 7)) << 4);
-      cp_async16(dst, krow + off, ok);
-      cp_async16(dst + S::kTileBytes, vrow + off, ok);
+  for (int i = 0; i < kBlk * T::kPieces / 32; ++i) {
+    const int idx = lane + 32 * i, r = idx / T::kPieces, pc = idx % T::kPieces;
+    const int key = blk * kBlk + r;
+    const bool ok = key < nkeys;
+    cp_async16(dst + r * T::kRowBytes + ((pc ^ (r & 7)) << 4),
+               rows + (long long)(ok ? key : 0) * T::kRowBytes + pc * 16, ok);
+  }
+}
+
+// Base-2 logits of the block's 16 rows for query row lane / 4 at keys 2t, 2t+1 (+8), -inf past the end;
+// returns their maximum over the query's four lanes.
+template <int D>
+__device__ __forceinline__ float block_logits(uint32_t k_tile, const uint32_t (&qa)[D / 16][2], float sc2,
+                                              int blk, int nkeys, float (&x)[4]) {
+  using T = Tile<D>;
+  const int lane = threadIdx.x & 31, t = lane & 3, mi = lane >> 3, r8 = lane & 7;
+  float s[2][4];
+  s[0][0] = s[0][1] = s[0][2] = s[0][3] = 0.f;
+  s[1][0] = s[1][1] = s[1][2] = s[1][3] = 0.f;
+  // matrices of one k-step: (keys 0-7, piece 2s), (keys 0-7, piece 2s+1), (keys 8-15, ...)
+  const int key_l = (mi >> 1) * 8 + r8;
+#pragma unroll
+  for (int ks = 0; ks < D / 16; ++ks) {
+    uint32_t b0, b1, b2, b3;
+    const int pc = 2 * ks + (mi & 1);
+    ldmatrix_x4(b0, b1, b2, b3, k_tile + key_l * T::kRowBytes + ((pc ^ (key_l & 7)) << 4));
+    mma_bf16_16816(s[0][0], s[0][1], s[0][2], s[0][3], qa[ks][0], 0u, qa[ks][1], 0u, b0, b1);
+    mma_bf16_16816(s[1][0], s[1][1], s[1][2], s[1][3], qa[ks][0], 0u, qa[ks][1], 0u, b2, b3);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int key = blk * kBlk + (u >> 1) * 8 + 2 * t + (u & 1);
+    x[u] = key < nkeys ? __fmul_rn(s[u >> 1][u & 1], sc2) : -INFINITY;
+  }
+  float bm = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
+  bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
+  return fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
+}
+
+// The block's probabilities against the running maximum m_new (finite: every block has at least one valid
+// key), added to the sums; `corr` takes what is there to the new maximum.
+template <int D>
+__device__ __forceinline__ void block_values(uint32_t v_tile, const float (&x)[4], float m_new, float corr,
+                                             float& l_run, float (&o)[D / 8][4]) {
+  using T = Tile<D>;
+  const int lane = threadIdx.x & 31, mi = lane >> 3, r8 = lane & 7;
+  float pr[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) pr[u] = fast_exp2(__fsub_rn(x[u], m_new));
+  l_run = fmaf(l_run, corr, __fadd_rn(__fadd_rn(pr[0], pr[1]), __fadd_rn(pr[2], pr[3])));
+  if (__any_sync(0xffffffffu, corr != 1.f)) {
+#pragma unroll
+    for (int nd = 0; nd < D / 8; ++nd) {
+      o[nd][0] *= corr;
+      o[nd][1] *= corr;
     }
+  }
+  const uint32_t pa0 = pack_bf16(pr[0], pr[1]), pa2 = pack_bf16(pr[2], pr[3]);
+  // d = 64: the probabilities enter as two bf16 terms (error 2^-17), as precise as fp32 products
+  // were on the CUDA-core path that used to serve it
+  uint32_t pb0 = 0u, pb2 = 0u;
+  if (D == 64) {
+    pb0 = pack_bf16(pr[0] - bf16_lo(pa0), pr[1] - bf16_hi(pa0));
+    pb2 = pack_bf16(pr[2] - bf16_lo(pa2), pr[3] - bf16_hi(pa2));
+  }
+  const int key_l = (mi & 1) * 8 + r8;
+#pragma unroll
+  for (int nd = 0; nd < D / 8; nd += 2) {
+    uint32_t b0, b1, b2, b3;
+    const int pc = nd + (mi >> 1);
+    ldmatrix_x4_trans(b0, b1, b2, b3, v_tile + key_l * T::kRowBytes + ((pc ^ (key_l & 7)) << 4));
+    mma_bf16_16816(o[nd][0], o[nd][1], o[nd][2], o[nd][3], pa0, 0u, pa2, 0u, b0, b1);
+    mma_bf16_16816(o[nd + 1][0], o[nd + 1][1], o[nd + 1][2], o[nd + 1][3], pa0, 0u, pa2, 0u, b2, b3);
+    if (D == 64) {
+      mma_bf16_16816(o[nd][0], o[nd][1], o[nd][2], o[nd][3], pb0, 0u, pb2, 0u, b0, b1);
+      mma_bf16_16816(o[nd + 1][0], o[nd + 1][1], o[nd + 1][2], o[nd + 1][3], pb0, 0u, pb2, 0u, b2, b3);
+    }
+  }
+}
+
+// Sum over the four lanes of a query.
+__device__ __forceinline__ float query_sum(float x) {
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x + __shfl_xor_sync(0xffffffffu, x, 2);
+}
+
+// One warp, one chunk: its parts one after the other.
+template <int D>
+__device__ __forceinline__ void attend_chunk(const DecodeParams& p, unsigned char* stage_mem, int head,
+                                             const char* krow, const char* vrow, int nkeys, bool whole,
+                                             size_t slot) {
+  using T = Tile<D>;
+  constexpr int kStages = T::kRing / 2, kOut = D / 8;  // a stage: a K tile and a V tile
+  const Geom& g = p.g;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, qrow = lane >> 2, t = lane & 3;
+  const uint32_t ring = smem_u32(stage_mem) + warp * (T::kRing * T::kBytes);
+  const int nblk = (nkeys + kBlk - 1) / kBlk;
+  uint32_t qa[D / 16][2];
+  load_queries<D>(p, head, qa);
+  auto fill = [&](int blk) {
+    if (blk < nblk) {
+      const uint32_t st = ring + (blk % kStages) * (2 * T::kBytes);
+      fill_tile<D>(st, krow, blk, nkeys);
+      fill_tile<D>(st + T::kBytes, vrow, blk, nkeys);
+    }
+    cp_async_commit();
   };
 #pragma unroll
-  for (int s = 0; s < kStages - 1; ++s) {
-    if (s < nblk) fill(s, s);
-    cp_async_commit();
-  }
-  float o[kOut][4];
+  for (int s = 0; s < kStages - 1; ++s) fill(s);
+  float o[kOut][4], acc[kOut][2];
 #pragma unroll
-  for (int nd = 0; nd < kOut; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
-  float m_run = -INFINITY, l_run = 0.f;
-  int chunk_end = cb - 1;  // last block of the current chunk
-
+  for (int nd = 0; nd < kOut; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = acc[nd][0] = acc[nd][1] = 0.f;
+  float m_run = -INFINITY, m_part = -INFINITY, l_run = 0.f, l = 0.f;
   for (int blk = 0; blk < nblk; ++blk) {
-    if (blk + kStages - 1 < nblk) fill(blk + kStages - 1, (blk + kStages - 1) % kStages);
-    cp_async_commit();
+    fill(blk + kStages - 1);
     cp_async_wait<kStages - 1>();
     __syncwarp();
-    const uint32_t st = sbase + (blk % kStages) * S::kBytes;
-    // ---- S = Q K^T for 16 rows: two 8-key tiles, D / 16 k-steps -----------------------------
-    float s[2][4];
-    s[0][0] = s[0][1] = s[0][2] = s[0][3] = 0.f;
-    s[1][0] = s[1][1] = s[1][2] = s[1][3] = 0.f;
-    {
-      // matrices of one k-step: (keys 0-7, piece 2s), (keys 0-7, piece 2s+1), (keys 8-15, ...)
-      const int key_l = (mi >> 1) * 8 + r8;
-#pragma unroll
-      for (int ks = 0; ks < kSteps; ++ks) {
-        uint32_t b0, b1, b2, b3;
-        const int pc = 2 * ks + (mi & 1);
-        ldmatrix_x4(b0, b1, b2, b3, st + key_l * S::kRowBytes + ((pc ^ (key_l & 7)) << 4));
-        mma_bf16_16816(s[0][0], s[0][1], s[0][2], s[0][3], qa[ks][0], 0u, qa[ks][1], 0u, b0, b1);
-        mma_bf16_16816(s[1][0], s[1][1], s[1][2], s[1][3], qa[ks][0], 0u, qa[ks][1], 0u, b2, b3);
-      }
-    }
-    // ---- running softmax of query row qrow over its keys 2t, 2t+1 (+8) ------------------------
+    const uint32_t st = ring + (blk % kStages) * (2 * T::kBytes);
     float x[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int key = blk * kBlk + (u >> 1) * 8 + 2 * t + (u & 1);
-      x[u] = key < nkeys ? s[u >> 1][u & 1] * sc2 : -INFINITY;
-    }
-    float bm = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));
-    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 1));
-    bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 2));
-    const float m_new = fmaxf(m_run, bm);  // finite: every block has at least one valid key
-    const float corr = fast_exp2(m_run - m_new);
-    float pr[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) pr[u] = fast_exp2(x[u] - m_new);
-    l_run = l_run * corr + ((pr[0] + pr[1]) + (pr[2] + pr[3]));
+    const float m_new = fmaxf(m_run, block_logits<D>(st, qa, g.scale_log2, blk, nkeys, x));
+    block_values<D>(st + T::kBytes, x, m_new, fast_exp2(__fsub_rn(m_run, m_new)), l_run, o);
     m_run = m_new;
-    if (__any_sync(0xffffffffu, corr != 1.f)) {
+    __syncwarp();  // the stage may be refilled by the next iteration
+    if (blk + 1 == nblk || blk % kPartBlocks == kPartBlocks - 1) {  // end of a part
+      const float c = fast_exp2(__fsub_rn(m_part, m_run));
+      l = fmaf(l, c, query_sum(l_run));
+      l_run = 0.f;
+      m_part = m_run;
 #pragma unroll
       for (int nd = 0; nd < kOut; ++nd) {
-        o[nd][0] *= corr;
-        o[nd][1] *= corr;
-      }
-    }
-    const uint32_t pa0 = pack_bf16(pr[0], pr[1]), pa2 = pack_bf16(pr[2], pr[3]);
-    // d = 64: the probabilities enter as two bf16 terms (error 2^-17), as precise as fp32 products
-    // were on the CUDA-core path that used to serve it
-    uint32_t pb0 = 0u, pb2 = 0u;
-    if (D == 64) {
-      pb0 = pack_bf16(pr[0] - bf16_lo(pa0), pr[1] - bf16_hi(pa0));
-      pb2 = pack_bf16(pr[2] - bf16_lo(pa2), pr[3] - bf16_hi(pa2));
-    }
-    // ---- O += P V --------------------------------------------------------------------------
-    {
-      const int key_l = (mi & 1) * 8 + r8;
-#pragma unroll
-      for (int nd = 0; nd < kOut; nd += 2) {
-        uint32_t b0, b1, b2, b3;
-        const int pc = nd + (mi >> 1);
-        ldmatrix_x4_trans(b0, b1, b2, b3,
-                          st + S::kTileBytes + key_l * S::kRowBytes + ((pc ^ (key_l & 7)) << 4));
-        mma_bf16_16816(o[nd][0], o[nd][1], o[nd][2], o[nd][3], pa0, 0u, pa2, 0u, b0, b1);
-        mma_bf16_16816(o[nd + 1][0], o[nd + 1][1], o[nd + 1][2], o[nd + 1][3], pa0, 0u, pa2, 0u, b2, b3);
-        if (D == 64) {
-          mma_bf16_16816(o[nd][0], o[nd][1], o[nd][2], o[nd][3], pb0, 0u, pb2, 0u, b0, b1);
-          mma_bf16_16816(o[nd + 1][0], o[nd + 1][1], o[nd + 1][2], o[nd + 1][3], pb0, 0u, pb2, 0u, b2, b3);
-        }
-      }
-    }
-    __syncwarp();  // the stage may be refilled by the next iteration
-    // ---- end of the chunk ------------------------------------------------------------------
-    if (blk + 1 == nblk || (!kOneChunk && blk == chunk_end)) {
-      l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
-      l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
-      if (qrow < g.group) {
-        const float scale = whole ? 1.0f / l_run : 1.0f;
-        float* dst = whole ? p.out + ((size_t)head * g.group + qrow) * D
-                            : p.part + (slot * g.group + qrow) * (D + 4);
-#pragma unroll
-        for (int nd = 0; nd < kOut; ++nd)
-          *reinterpret_cast<float2*>(dst + nd * 8 + 2 * t) = make_float2(o[nd][0] * scale, o[nd][1] * scale);
-        if (!whole && t == 0) *reinterpret_cast<float2*>(dst + D) = make_float2(m_run, l_run);
-      }
-      if (!kOneChunk) {
-#pragma unroll
-        for (int nd = 0; nd < kOut; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
-        m_run = -INFINITY;
-        l_run = 0.f;
-        chunk_end += cb;
-        ++slot;
+        acc[nd][0] = fmaf(acc[nd][0], c, o[nd][0]);
+        acc[nd][1] = fmaf(acc[nd][1], c, o[nd][1]);
+        o[nd][0] = o[nd][1] = 0.f;
       }
     }
   }
   cp_async_wait<0>();
   __syncwarp();  // the stages may be filled again
+  if (qrow < g.group) {
+    const float div = whole ? l : 1.0f;
+    float* dst = whole ? p.out + ((size_t)head * g.group + qrow) * D : p.part + (slot * g.group + qrow) * D;
+#pragma unroll
+    for (int nd = 0; nd < kOut; ++nd)
+      *reinterpret_cast<float2*>(dst + nd * 8 + 2 * t) = make_float2(acc[nd][0] / div, acc[nd][1] / div);
+    if (!whole && t == 0) p.part_ml[slot * g.group + qrow] = make_float2(m_run, l);
+  }
 }
 
-// One warp: the partial results of `n` chunks, `stride` floats apart, folded in chunk order.
+// One warp: the partial results of the `n` chunks of query q of a head, from slot `slot` on, folded in
+// chunk order.
 template <int D>
-__device__ inline void fold_chunks(const float* src, size_t stride, int n, float* dst) {
+__device__ inline void fold_chunks(const DecodeParams& p, size_t slot, int q, int n, float* dst) {
   constexpr int kCols = D / 32;  // columns per lane
   using Cols = typename std::conditional<D == 128, float4, float2>::type;
   const int lane = threadIdx.x & 31;
+  const float* src = p.part + (slot * p.g.group + q) * D;
+  const size_t stride = (size_t)p.g.group * D;
   auto stats = [&](int i) {  // max and sum of chunk i
-    return i < n ? __ldcg(reinterpret_cast<const float2*>(src + i * stride + D)) : make_float2(-INFINITY, 0.f);
+    return i < n ? __ldcg(p.part_ml + (slot + i) * p.g.group + q) : make_float2(-INFINITY, 0.f);
   };
   float2 ml0 = stats(lane), ml1 = stats(lane + 32);
   float m = fmaxf(ml0.x, ml1.x);
@@ -321,107 +345,208 @@ template <int D>
 __global__ void __launch_bounds__(kWarps * 32)
 decode_kernel(const DecodeParams p) {
   in_stream_order();
-  using S = Stage<D>;
+  using T = Tile<D>;
+  constexpr int kOut = D / 8;
   extern __shared__ __align__(128) unsigned char stage_mem[];
   __shared__ int2 wsum[kWarps];
-  __shared__ int3 start_at[kWarps + 1];  // head, chunk inside it, chunk among all
+  __shared__ int3 start_at[2];  // this block's first chunk and the next block's: head, chunk in it, chunk of all
+  __shared__ float part_max[kWarps][8];   // [warp][query]: largest logit of the warp's part
+  __shared__ float2 part_ml[kWarps][8];   // running max and sum at its end
   __shared__ int fold_head[32], fold_first[32], fold_n[32], fold_count, fold_next, fold_lo, fold_hi;
-  __shared__ unsigned fold_there[kFoldWords];
+  __shared__ unsigned fold_there[kMaxChunks];  // bits for the stamps of 32 heads
   const Geom& g = p.g;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int warps = gridDim.x * kWarps;
 
-  // ---- the split: blocks and chunks of all heads, and where this block's warps start --------------
+  // ---- the split: parts and chunks of all heads, and where this block starts ----------------------
   {
     const int hpt = (p.heads + kWarps * 32 - 1) / (kWarps * 32);
     const int h0 = min(p.heads, tid * hpt), h1 = min(p.heads, h0 + hpt);
-    int blocks = 0, chunks = 0;
+    int parts = 0, chunks = 0;
 #pragma unroll 4
     for (int h = h0; h < h1; ++h) {
       const int len = head_len(p, h);
-      blocks += (len + kBlk - 1) / kBlk;
+      parts += head_parts(len);
       chunks += head_chunks(len);
       if (len == 0 && h % (int)gridDim.x == (int)blockIdx.x)  // no rows: the outputs are zeros
         for (int c = 0; c < g.group * D; ++c) p.out[(size_t)h * g.group * D + c] = 0.f;
     }
-    int bi = blocks, ci = chunks;
+    int pi = parts, ci = chunks;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, bi, o), z = __shfl_up_sync(0xffffffffu, ci, o);
+      const int y = __shfl_up_sync(0xffffffffu, pi, o), z = __shfl_up_sync(0xffffffffu, ci, o);
       if (lane >= o) {
-        bi += y;
+        pi += y;
         ci += z;
       }
     }
-    if (lane == 31) wsum[warp] = make_int2(bi, ci);
+    if (lane == 31) wsum[warp] = make_int2(pi, ci);
     __syncthreads();
-    int b_before = bi - blocks, c_before = ci - chunks, b_total = 0, c_total = 0;
+    int p_before = pi - parts, c_before = ci - chunks, p_total = 0, c_total = 0;
     for (int w = 0; w < kWarps; ++w) {
       if (w < warp) {
-        b_before += wsum[w].x;
+        p_before += wsum[w].x;
         c_before += wsum[w].y;
       }
-      b_total += wsum[w].x;
+      p_total += wsum[w].x;
       c_total += wsum[w].y;
     }
-    for (int w = 0; w <= kWarps; ++w) {
-      // the first chunk that starts at or after the warp's share
-      const int s = (int)((long long)b_total * (blockIdx.x * kWarps + w) / warps);
-      if (s >= b_total) {
+    for (int w = 0; w < 2; ++w) {
+      // the first chunk that starts at or after the block's share
+      const int s = (int)((long long)p_total * (blockIdx.x + w) / gridDim.x);
+      if (s >= p_total) {
         if (tid == 0) start_at[w] = make_int3(p.heads, 0, c_total);
-      } else if (s >= b_before && s < b_before + blocks) {
-        int at = b_before, c = c_before, h = h0, len = head_len(p, h);
-        while (at + (len + kBlk - 1) / kBlk <= s) {
-          at += (len + kBlk - 1) / kBlk;
+      } else if (s >= p_before && s < p_before + parts) {
+        int at = p_before, c = c_before, h = h0, len = head_len(p, h);
+        while (at + head_parts(len) <= s) {
+          at += head_parts(len);
           c += head_chunks(len);
           len = head_len(p, ++h);
         }
-        const int cb = chunk_blocks(len), in_head = (s - at + cb - 1) / cb;
+        const int in_head = (s - at + kWarps - 1) / kWarps;
         const bool next = in_head == head_chunks(len);  // inside the head's last chunk
         start_at[w] = make_int3(next ? h + 1 : h, next ? 0 : in_head, c + in_head);
       }
     }
     __syncthreads();
   }
-  const int c0 = start_at[warp].z, c1 = start_at[warp + 1].z;
-  const int first_head = start_at[0].x;
+  const int c0 = start_at[0].z, c1 = start_at[1].z, first_head = start_at[0].x;  // this block's chunks
+  if (c1 <= c0) return;
   // chunks of the block's first 32 heads, wanted at the end (loaded here, under the rows' latency)
   int n_mine = warp == 0 && first_head + lane < p.heads ? head_chunks(head_len(p, first_head + lane)) : 0;
 
-  if (c1 > c0) {
-    int head = start_at[warp].x, in_head = start_at[warp].y;
-    for (int chunk = c0; chunk < c1; ++head, in_head = 0) {
-      // ---- a run: this warp's consecutive chunks of one head -------------------------------------
-      const int prob = head / g.n_kv_heads, kvh = head - prob * g.n_kv_heads;
-      const int* hoff = p.head_offsets + (size_t)prob * (g.n_kv_heads + 1) + kvh;
-      const int h0 = hoff[0], len = hoff[1] - h0;
-      if (len <= 0) continue;
-      const int cb = chunk_blocks(len), n = head_chunks(len);
-      const int run = min(n - in_head, c1 - chunk);
-      const int row_lo = in_head * cb * kBlk, nkeys = min(len, (in_head + run) * cb * kBlk) - row_lo;
-      const long long row0 = p.row_off[prob] + h0 + row_lo;
-      attend_rows<D, false>(p, stage_mem, head, p.k_rows + row0 * S::kRowBytes, p.v_rows + row0 * S::kRowBytes,
-                     nkeys, cb, n == 1, (size_t)chunk);
-      if (n > 1) {
-        __threadfence();
-        __syncwarp();
-        for (int c = chunk + lane; c < chunk + run; c += 32)
-          *reinterpret_cast<volatile unsigned long long*>(p.stamps + c) = p.stamp;
+  const int qrow = lane >> 2, t = lane & 3;  // row and column pair of the MMA fragments
+  unsigned char* const ring_mem = stage_mem + warp * (T::kPartRing * T::kBytes);
+  const uint32_t ring = smem_u32(ring_mem);
+  int head = first_head, in_head = start_at[0].y;
+  bool several = false;  // a chunk here belongs to a head of several
+  for (int chunk = c0; chunk < c1;) {
+    // ---- a round: as many of the next chunks as the four warps take a part each of ----------------
+    int used = 0, my_head = 0, my_chunk = 0, first = 0, parts = 0, nkeys = 0;
+    bool whole = false;
+    const char *krow = nullptr, *vrow = nullptr;
+    while (chunk < c1) {
+      const int len = head_len(p, head);
+      const int lo = in_head * kChunkRows, n = head_parts(min(kChunkRows, len - lo));
+      if (used + n > kWarps) break;
+      if (len > 0) {
+        if (warp >= used && warp < used + n) {
+          const int prob = head / g.n_kv_heads, kvh = head - prob * g.n_kv_heads;
+          const int part_lo = lo + (warp - used) * kPartRows;
+          const long long row0 = p.row_off[prob] + p.head_offsets[(size_t)prob * (g.n_kv_heads + 1) + kvh] + part_lo;
+          krow = p.k_rows + row0 * T::kRowBytes;
+          vrow = p.v_rows + row0 * T::kRowBytes;
+          nkeys = min(kPartRows, len - part_lo);
+          my_head = head;
+          my_chunk = chunk;
+          first = used;
+          parts = n;
+          whole = len <= kChunkRows;
+        }
+        several |= len > kChunkRows;
+        used += n;
+        ++chunk;
       }
-      chunk += run;
+      if (++in_head * kChunkRows >= len) {
+        ++head;
+        in_head = 0;
+      }
+    }
+    // ---- logits of the part, K tiles first and V tiles behind them --------------------------------
+    const int nblk = (nkeys + kBlk - 1) / kBlk;
+    uint32_t qa[D / 16][2];
+    float x[kPartBlocks][4], bm[kPartBlocks], top = -INFINITY;
+    auto fill = [&](int i) {
+      if (i < 2 * nblk)
+        fill_tile<D>(ring + (i % T::kPartRing) * T::kBytes, i < nblk ? krow : vrow, i < nblk ? i : i - nblk, nkeys);
+      cp_async_commit();
+    };
+    if (nblk > 0) {
+      load_queries<D>(p, my_head, qa);
+#pragma unroll
+      for (int s = 0; s < T::kPartRing - 1; ++s) fill(s);
+#pragma unroll
+      for (int b = 0; b < kPartBlocks; ++b)
+        if (b < nblk) {
+          fill(b + T::kPartRing - 1);
+          cp_async_wait<T::kPartRing - 1>();
+          __syncwarp();
+          bm[b] = block_logits<D>(ring + (b % T::kPartRing) * T::kBytes, qa, g.scale_log2, b, nkeys, x[b]);
+          top = fmaxf(top, bm[b]);
+          __syncwarp();  // the tile may be refilled by the next iteration
+        }
+    }
+    if (t == 0) part_max[warp][qrow] = top;
+    __syncthreads();
+    // ---- probabilities against the chunk's running maximum, times V -------------------------------
+    if (nblk > 0) {
+      float m_run = -INFINITY, l_run = 0.f, o[kOut][4];
+      for (int w = first; w < warp; ++w) m_run = fmaxf(m_run, part_max[w][qrow]);
+#pragma unroll
+      for (int nd = 0; nd < kOut; ++nd) o[nd][0] = o[nd][1] = o[nd][2] = o[nd][3] = 0.f;
+#pragma unroll
+      for (int b = 0; b < kPartBlocks; ++b)
+        if (b < nblk) {
+          const int i = nblk + b;
+          fill(i + T::kPartRing - 1);
+          cp_async_wait<T::kPartRing - 1>();
+          __syncwarp();
+          const float m_new = fmaxf(m_run, bm[b]);
+          block_values<D>(ring + (i % T::kPartRing) * T::kBytes, x[b], m_new, fast_exp2(__fsub_rn(m_run, m_new)),
+                          l_run, o);
+          m_run = m_new;
+          __syncwarp();
+        }
+      cp_async_wait<0>();
+      l_run = query_sum(l_run);
+      if (t == 0) part_ml[warp][qrow] = make_float2(m_run, l_run);
+      if (qrow < g.group) {
+        float* dst = reinterpret_cast<float*>(ring_mem) + qrow * T::kFoldStride;  // all tiles have been read
+#pragma unroll
+        for (int nd = 0; nd < kOut; ++nd)
+          *reinterpret_cast<float2*>(dst + nd * 8 + 2 * t) = make_float2(o[nd][0], o[nd][1]);
+      }
+    }
+    __syncthreads();
+    // ---- the chunk: its parts in order, by the warps that made them --------------------------------
+    if (nblk > 0) {
+      for (int e = (warp - first) * 32 + lane; e < g.group * (D / 4); e += parts * 32) {
+        const int q = e / (D / 4), col = e % (D / 4) * 4;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        float m = -INFINITY, l = 0.f;
+        for (int w = first; w < first + parts; ++w) {
+          const float2 ml = part_ml[w][q];
+          const float4 f = *reinterpret_cast<const float4*>(
+              reinterpret_cast<const float*>(stage_mem + w * (T::kPartRing * T::kBytes)) + q * T::kFoldStride + col);
+          const float c = fast_exp2(__fsub_rn(m, ml.x));
+          l = fmaf(l, c, ml.y);
+          a.x = fmaf(a.x, c, f.x);
+          a.y = fmaf(a.y, c, f.y);
+          a.z = fmaf(a.z, c, f.z);
+          a.w = fmaf(a.w, c, f.w);
+          m = ml.x;
+        }
+        const size_t at = (size_t)(whole ? my_head : my_chunk) * g.group + q;
+        if (whole) a = make_float4(a.x / l, a.y / l, a.z / l, a.w / l);
+        else if (col == 0) p.part_ml[at] = make_float2(m, l);
+        *reinterpret_cast<float4*>((whole ? p.out : p.part) + at * D + col) = a;
+      }
+    }
+    __syncthreads();  // the rings and the parts' figures may be written again
+    if (nblk > 0 && !whole && warp == first && lane == 0) {
+      __threadfence();  // (what the chunk's warps have written, before the stamp)
+      *reinterpret_cast<volatile unsigned long long*>(p.stamps + my_chunk) = p.stamp;
     }
   }
 
   // ---- heads of several chunks: a block that finds all partial results there folds them ----------
-  // Every warp leaves its stamps before its block looks, so the last one to leave one sees them all;
+  // Every block leaves its stamps before it looks, so the last one to leave one sees them all;
   // two blocks that both do fold the same values in the same order.  Only chunks of such heads are stamped,
   // and the stamps are cleared after the fold, so that a replayed launch (a captured graph carries its
   // stamp) starts without any, whatever the row counts were that the launch before it found.
-  const int b0 = start_at[0].z, b1 = start_at[kWarps].z;  // this block's chunks
-  if (b1 <= b0) return;
+  if (!several) return;
   __syncthreads();
   __threadfence();
-  int head0 = first_head, base = b0 - start_at[0].y;  // 32 heads at a time, the first one's first chunk
+  int head0 = first_head, base = c0 - start_at[0].y;  // 32 heads at a time, the first one's first chunk
   int at = 0, n = 0;                                   // warp 0: this lane's head
   while (true) {
     if (warp == 0) {
@@ -433,14 +558,14 @@ decode_kernel(const DecodeParams p) {
         if (lane >= o) incl += y;
       }
       at = base + incl - n;
-      const unsigned mine = __ballot_sync(0xffffffffu, n > 0 && at < b1);  // heads with a chunk here
+      const unsigned mine = __ballot_sync(0xffffffffu, n > 0 && at < c1);  // heads with a chunk here
       const int last = mine ? 31 - __clz(mine) : 0;
       const int hi = __shfl_sync(0xffffffffu, at + n, last);
       const int end = __shfl_sync(0xffffffffu, base + incl, 31);
       if (lane == 0) {
         fold_lo = base;
         fold_hi = mine ? hi : base;
-        fold_next = end < b1 && head0 + 32 < p.heads ? 1 : 0;
+        fold_next = end < c1 && head0 + 32 < p.heads ? 1 : 0;
       }
       base = end;
     }
@@ -455,7 +580,7 @@ decode_kernel(const DecodeParams p) {
     __threadfence();
     __syncthreads();
     if (warp == 0) {
-      bool fold = n > 1 && at < b1;
+      bool fold = n > 1 && at < c1;
       for (int i = at - lo; fold && i < at - lo + n;) {  // whole words where they lie inside the head
         const int left = min(32 - (i & 31), at - lo + n - i);
         const unsigned want = (left == 32 ? 0xffffffffu : (1u << left) - 1u) << (i & 31);
@@ -477,9 +602,7 @@ decode_kernel(const DecodeParams p) {
     const bool more = fold_next != 0;
     for (int u = warp; u < count * g.group; u += kWarps) {
       const int e = u / g.group, q = u - e * g.group, n = fold_n[e];  // (n: of this head)
-      const float* src = p.part + ((size_t)fold_first[e] * g.group + q) * (D + 4);
-      const size_t stride = (size_t)g.group * (D + 4);
-      fold_chunks<D>(src, stride, n, p.out + ((size_t)fold_head[e] * g.group + q) * D);
+      fold_chunks<D>(p, fold_first[e], q, n, p.out + ((size_t)fold_head[e] * g.group + q) * D);
     }
     __syncthreads();  // (the list is written again, and the stamps go)
     for (int e = warp; e < count; e += kWarps)
@@ -491,7 +614,7 @@ decode_kernel(const DecodeParams p) {
   }
 }
 
-// Many long heads: chunks of 512 rows in a list, one per warp, and a kernel of its own for the fold.
+// Many long heads: the chunks in a list, one per warp, and a kernel of its own for the fold.
 // Row counts live on the device, so the list of (head, chunk) pairs that have rows is built
 // there: one block walks the heads in order (exclusive scan of their chunk counts) and writes
 // the pairs; the attention kernel then runs a fixed grid over that list and no CTA is launched
@@ -501,19 +624,13 @@ list_chunks_kernel(const DecodeParams p) {
   in_stream_order();
   __shared__ int wsum[32];
   __shared__ int base;
-  const Geom& g = p.g;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
   for (int h0 = 0; h0 < p.heads; h0 += 1024) {
     const int h = h0 + threadIdx.x;
     int cnt = 0;
-    if (h < p.heads) {
-      const int prob = h / g.n_kv_heads, kvh = h - prob * g.n_kv_heads;
-      const int* hoff = p.head_offsets + (size_t)prob * (g.n_kv_heads + 1);
-      const int len = hoff[kvh + 1] - hoff[kvh];
-      cnt = len > 0 ? min((len + kListChunk * kBlk - 1) / (kListChunk * kBlk), p.chunks_max) : 0;
-    }
+    if (h < p.heads) cnt = head_chunks(head_len(p, h));
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -543,12 +660,11 @@ decode_listed_kernel(const DecodeParams p) {
   for (int item = blockIdx.x * kWarps + (threadIdx.x >> 5); item < n_items; item += gridDim.x * kWarps) {
     const int2 it = p.items[item];
     const int prob = it.x / g.n_kv_heads, kvh = it.x - prob * g.n_kv_heads;
-    const int* hoff = p.head_offsets + (size_t)prob * (g.n_kv_heads + 1) + kvh;
-    const int h0 = hoff[0], len = hoff[1] - h0, lo = it.y * kListChunk * kBlk;
-    const long long row0 = p.row_off[prob] + h0 + lo;
-    attend_rows<D, true>(p, stage_mem, it.x, p.k_rows + row0 * Stage<D>::kRowBytes,
-                   p.v_rows + row0 * Stage<D>::kRowBytes, min(kListChunk * kBlk, len - lo), kListChunk,
-                   len <= kListChunk * kBlk, (size_t)it.x * p.chunks_max + it.y);
+    const int len = head_len(p, it.x), lo = it.y * kChunkRows;
+    const long long row0 = p.row_off[prob] + p.head_offsets[(size_t)prob * (g.n_kv_heads + 1) + kvh] + lo;
+    attend_chunk<D>(p, stage_mem, it.x, p.k_rows + row0 * Tile<D>::kRowBytes,
+                    p.v_rows + row0 * Tile<D>::kRowBytes, min(kChunkRows, len - lo), len <= kChunkRows,
+                    (size_t)it.x * p.chunks_max + it.y);
   }
 }
 
@@ -560,13 +676,11 @@ decode_combine_kernel(const DecodeParams p) {
   const Geom& g = p.g;
   const int u = blockIdx.x * kWarps + (threadIdx.x >> 5), head = u / g.group, q = u - head * g.group;
   if (head >= p.heads) return;
-  const int n = (head_len(p, head) + kListChunk * kBlk - 1) / (kListChunk * kBlk);
+  const int n = head_chunks(head_len(p, head));
   float* dst = p.out + ((size_t)head * g.group + q) * D;
   if (n == 0)
     for (int c = threadIdx.x & 31; c < D; c += 32) dst[c] = 0.f;
-  if (n > 1)
-    fold_chunks<D>(p.part + ((size_t)head * p.chunks_max * g.group + q) * (D + 4),
-                   (size_t)g.group * (D + 4), n, dst);
+  if (n > 1) fold_chunks<D>(p, (size_t)head * p.chunks_max, q, n, dst);
 }
 
 // Any geometry: one block per (query head, layer*sequence), tiles of 1024 rows in the base-2 domain.
@@ -669,23 +783,25 @@ decode_generic_kernel(const DecodeParams p) {
 }
 
 inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
-// Which path: the single kernel saves two launches and has more, shorter chunks; the listed one streams
-// with less imbalance and folds all heads at once.  Only the longest length is known here, so the line
-// lies at the most rows that the call may hold.  Single / listed, us (rows that there are, most rows):
-// 8 heads x 2048 rows, 0.26 M: 19 / 28; 256 x 128, 0.26 M: 20 / 27; 64 x 128, 1.0 M: 21 / 32; 256 x 512,
-// 2.1 M: 31 / 31; 112 x 1024, 3.7 M: 35 / 31; 256 x 2048, 8.4 M: 66 / 60; 2048 x 128, 34 M: 55 / 56.
+// Which path (the results are the same): the one kernel saves two launches and spreads a chunk over four
+// warps; the listed one streams with less imbalance and folds all heads at once.  Only the longest length
+// is known here, so the line lies at the most rows that the call may hold, and at more heads than a block
+// takes in three rounds.  One / listed, us (heads x average rows, longest): 128 x 128, 1K: 10 / 15;
+// 512 x 128, 2K: 12 / 17; 256 x 512, 8K: 22 / 26; 112 x 1024, 32K: 22 / 26; 300 x 1000, 6K: 44 / 37;
+// 512 x 700, 6K: 47 / 41; 256 x 2048, 32K: 65 / 54; 1024 x 128, 2K: 21 / 19; 1024 x 500, 3K: 69 / 66;
+// 2000 x 31, 300: 20 / 17; 2048 x 128, 16K: 43 / 38.
+int chunks_per_head(const Geom& g) { return (g.max_seqlen + kChunkRows - 1) / kChunkRows; }
 bool listed(const Geom& g, int n_layers) {
-  return (long long)n_layers * g.batch * g.n_kv_heads * g.max_seqlen >= (3ll << 20);
+  const long long heads = (long long)n_layers * g.batch * g.n_kv_heads;
+  return heads * g.max_seqlen >= (3ll << 20) || heads > 6ll * (sm_count() > 0 ? sm_count() : 148) ||
+         chunks_per_head(g) > kMaxChunks;
 }
 // partial results of all heads at most
 size_t part_slots(const Geom& g, int n_layers) {
-  const int step = (listed(g, n_layers) ? kListChunk : kMinChunk) * kBlk;
-  int longest = (g.max_seqlen + step - 1) / step;
-  if (!listed(g, n_layers)) longest = std::min(kMaxChunks, longest);
-  return (size_t)n_layers * g.batch * g.n_kv_heads * longest;
+  return (size_t)n_layers * g.batch * g.n_kv_heads * chunks_per_head(g);
 }
 size_t part_bytes(const Geom& g, int n_layers) {
-  return up256(part_slots(g, n_layers) * g.group * (g.head_dim + 4) * sizeof(float));
+  return up256(part_slots(g, n_layers) * g.group * (g.head_dim + 2) * sizeof(float));
 }
 // a stamp, or an entry of the list, per partial result; the length of the list
 size_t slot_bytes(const Geom& g, int n_layers) { return up256(part_slots(g, n_layers) * 8) + 256; }
@@ -705,8 +821,9 @@ template <int D>
 lava_status launch_decode(const DecodeParams& p, int n_layers, cudaStream_t stream) {
   const bool list = listed(p.g, n_layers);
   const void* kern = list ? (const void*)decode_listed_kernel<D> : (const void*)decode_kernel<D>;
-  const lava_status rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                         Stage<D>::kSmem), "decode attention attribute");
+  const int smem = kWarps * (list ? Tile<D>::kRing : Tile<D>::kPartRing) * Tile<D>::kBytes;
+  const lava_status rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
+                                    "decode attention attribute");
   if (rc != LAVA_OK) return rc;
   // two blocks fit an SM (shared memory); fewer when there cannot be a chunk for every warp
   const long long slots = (long long)(sm_count() > 0 ? sm_count() : 1) * 2;
@@ -714,11 +831,11 @@ lava_status launch_decode(const DecodeParams& p, int n_layers, cudaStream_t stre
   const int grid = (int)std::max<long long>(1, std::min<long long>(slots, (most + kWarps - 1) / kWarps));
   if (list) {
     launch_in_order(list_chunks_kernel, 1, 1024, 0, stream, p);
-    launch_in_order(decode_listed_kernel<D>, grid, kWarps * 32, Stage<D>::kSmem, stream, p);
+    launch_in_order(decode_listed_kernel<D>, grid, kWarps * 32, smem, stream, p);
     launch_in_order(decode_combine_kernel<D>, (p.heads * p.g.group + kWarps - 1) / kWarps, kWarps * 32,
                     0, stream, p);
   } else {
-    launch_in_order(decode_kernel<D>, grid, kWarps * 32, Stage<D>::kSmem, stream, p);
+    launch_in_order(decode_kernel<D>, grid, kWarps * 32, smem, stream, p);
   }
   count_launches(list ? 3 : 1);
   return check_cuda(cudaGetLastError(), "decode attention launch");
@@ -761,6 +878,7 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
   p.row_off = (const long long*)layer_row_offset;
   p.out = out;
   p.part = nullptr;
+  p.part_ml = nullptr;
   p.stamps = nullptr;
   p.stamp = 0;
   p.items = nullptr;
@@ -783,12 +901,13 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
     return fail(LAVA_ERR_WORKSPACE, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
   if (!aligned16(workspace)) return fail(LAVA_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
   p.part = (float*)workspace;
+  p.part_ml = (float2*)(p.part + part_slots(g, n_layers) * g.group * g.head_dim);
   char* per_slot = (char*)workspace + part_bytes(g, n_layers);
   p.stamps = (unsigned long long*)per_slot;
   p.stamp = next_stamp();
   p.items = (int2*)per_slot;
   p.n_items = (int*)(per_slot + slot_bytes(g, n_layers) - 256);
-  p.chunks_max = (g.max_seqlen + kListChunk * kBlk - 1) / (kListChunk * kBlk);
+  p.chunks_max = chunks_per_head(g);
   return g.head_dim == 128 ? launch_decode<128>(p, n_layers, st) : launch_decode<64>(p, n_layers, st);
 }
 

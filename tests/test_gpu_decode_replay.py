@@ -15,7 +15,7 @@ def test_a_replay_sees_the_row_counts_of_its_own_time(d):
     short, long = [90] * heads, [0] * heads
     for h in range(0, heads, kv):
         long[h] = 4096
-    # the last chunk of 129 and of 513 rows holds one row, so its block is the first to look for the others
+    # a last chunk of one row: its block is the first to look for the others
     pairs = [[n, 0] * (heads // 2) for n in (129, 513)]
     layouts = [short, pairs[0], short, pairs[1], short, long, [500] * heads, [32768] + [0] * (heads - 1), short]
     g = torch.Generator(device="cuda").manual_seed(5)
