@@ -886,7 +886,10 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
   p.chunks_max = 0;
   p.heads = n_layers * g.batch * g.n_kv_heads;
   cudaStream_t st = (cudaStream_t)stream;
-  const bool tensor_path = g.dtype == LAVA_BF16 && g.group <= 8;
+  const size_t need = part_bytes(g, n_layers) + slot_bytes(g, n_layers);
+  const bool room = workspace && workspace_bytes >= need && aligned16(workspace);
+  // the interface asks for a workspace at d = 128 only: d = 64 without one takes the plain kernel
+  const bool tensor_path = g.dtype == LAVA_BF16 && g.group <= 8 && (g.head_dim == 128 || room);
   if (!tensor_path) {
     auto kern = g.dtype == LAVA_BF16 ? (g.head_dim == 64 ? decode_generic_kernel<64, true>
                                                          : decode_generic_kernel<128, true>)
@@ -896,7 +899,6 @@ lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_
     count_launches(1);
     return check_cuda(cudaGetLastError(), "decode attention launch");
   }
-  const size_t need = part_bytes(g, n_layers) + slot_bytes(g, n_layers);
   if (!workspace || workspace_bytes < need)
     return fail(LAVA_ERR_WORKSPACE, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
   if (!aligned16(workspace)) return fail(LAVA_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
