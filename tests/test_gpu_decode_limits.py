@@ -1,4 +1,5 @@
-"""Decode attention at the limits of its arguments: head dimension 64 without a workspace."""
+"""Decode attention at the limits of its arguments: head dimension 64 without a workspace, and heads that
+hold more rows than max_seqlen says."""
 import ctypes
 
 import pytest
@@ -42,3 +43,20 @@ def test_head_dimension_64_needs_no_workspace(n_bytes):
                                    n_bytes or 0, torch.cuda.current_stream().cuda_stream)
     assert rc == 0
     _close(out, q, k, v, rows, group, 2.0 ** -15)
+
+
+@pytest.mark.parametrize("d", [128, 64])
+def test_heads_longer_than_max_seqlen_stay_inside_the_workspace(d):
+    # a workspace of one chunk of 512 rows per head: up to there all rows count, and nothing is written past it
+    rows, group = [500, 40000, 512, 513], 4
+    desc, q, k, v, hoff, roff, out = _setup(d, rows, group, 300)
+    n = lava.lava_decode_workspace_bytes(desc, 1)
+    buf = torch.full((n + 65536,), 85, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        lava.lava_decode_attention(desc, q, k, v, hoff, roff, out, buf[:n])
+    assert bool((buf[n:] == 85).all())
+    tol = 2.0 ** -8 if d == 128 else 2.0 ** -15
+    _close(out[:group], q[:group], k[:500], v[:500], [500], group, tol)
+    at = 500 + 40000
+    _close(out[2 * group:3 * group], q[2 * group:3 * group], k[at:at + 512], v[at:at + 512], [512], group, tol)
+    assert bool(torch.isfinite(out).all())
