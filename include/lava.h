@@ -344,8 +344,8 @@ LAVA_API lava_status lava_cascade_get(const lava_cascade* h, lava_cascade_view* 
  *                     runs on the tensor path with it and on the plain kernel without it; unused
  *                     otherwise
  * bf16 with group <= 8 runs on the tensor path; with d = 128 the probabilities are rounded to bf16
- * before they multiply V (error <= 2^-8 * sum_i p_i |V[i][c]| per output), with d = 64 they enter as
- * two bf16 terms (2^-17).  Other geometries run a plain fp32 kernel.  A head holds at most max_seqlen
+ * before they multiply V (error <= 2^-8 * sum_i p_i |V[i][c]| per output), with d = 64 they keep
+ * all 24 bits.  Other geometries run a plain fp32 kernel.  A head holds at most max_seqlen
  * rows.  lava_decode_attention is the one-layer form (pointers of that layer). */
 LAVA_API size_t lava_decode_workspace_bytes(const lava_layer_desc* desc, int32_t n_layers);
 LAVA_API lava_status lava_decode_attention_layers(const lava_layer_desc* desc, int32_t n_layers,

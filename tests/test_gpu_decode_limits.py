@@ -1,5 +1,5 @@
-"""Decode attention at the limits of its arguments: head dimension 64 without a workspace, and heads that
-hold more rows than max_seqlen says."""
+"""Decode attention at the limits of its arguments: head dimension 64 without a workspace and with
+its full precision, and heads that hold more rows than max_seqlen says."""
 import ctypes
 
 import pytest
@@ -60,3 +60,18 @@ def test_heads_longer_than_max_seqlen_stay_inside_the_workspace(d):
     at = 500 + 40000
     _close(out[2 * group:3 * group], q[2 * group:3 * group], k[at:at + 512], v[at:at + 512], [512], group, tol)
     assert bool(torch.isfinite(out).all())
+
+
+@pytest.mark.parametrize("longest", [1024, 1 << 20])   # the one kernel, the listed path
+@pytest.mark.parametrize("n", [40, 100, 300])
+def test_head_dimension_64_rounds_nothing_to_bf16(longest, n):
+    rows, group = [n] * 8, 4
+    desc, q, k, v, hoff, roff, out = _setup(64, rows, group, longest)
+    ws = torch.empty(lava.lava_decode_workspace_bytes(desc, 1), dtype=torch.uint8, device="cuda")
+    lava.lava_decode_attention(desc, q, k, v, hoff, roff, out, ws)
+    kh, vh = k.view(8, n, 64).double(), v.view(8, n, 64).double()
+    p = torch.softmax(torch.einsum("hgd,hnd->hgn", q.view(8, group, 64).double(), kh) / 8, dim=-1)
+    want = torch.einsum("hgn,hnd->hgd", p, vh).view(8 * group, 64)
+    # per block of 16 rows the sums are cut off once (2^-24 on average), and about four roundings of the
+    # logits (of a few units), the exponential, the sum and the quotient; two bf16 terms would give 1.8e-6
+    assert float((out - want).norm() / want.norm()) <= (n / 16 + 5) * 2.0 ** -24
