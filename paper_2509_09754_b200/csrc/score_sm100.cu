@@ -302,7 +302,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
       // cph, in split mode of both halves' (c + 2 cph); each of them belongs to a CTA whose own
       // next pass-2 chunk is c'' >= c, so c' lies at most (cph - 1) / grid ordinals beyond it.
       // With a lead of that many chunks plus one chunk's tiles every such wait ends.  The extra
-      // slots cover the skew between CTAs and the time the statistics take to travel.
+      // slots cover the skew between CTAs and the time the statistics take to travel.  The host
+      // makes the chunks long enough for `need` to stay below the records' limit (chunk_tiles_for).
       int longest = 1;
       for (int b = 0; b < g.batch; ++b) longest = max(longest, m->pref[b + 1] - m->pref[b]);
       longest <<= p.split;
@@ -1113,12 +1114,19 @@ int sm100_first_half(const Geom& g) {
 // 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With fewer than sixteen tiles per CTA in
 // all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
 // 8K (fourteen tiles per CTA) 64 / 66.
+// Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
+// chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
+// serve sequences of up to 0.83 M tokens with split query groups and 1.66 M without.
 int chunk_tiles_for(const Geom& g, int n_layers) {
-  if (options().score_chunk_tiles > 0) return options().score_chunk_tiles;
-  const long long tiles = (long long)n_layers * (g.n_kv_heads << (sm100_first_half(g) ? 1 : 0)) *
-                          ceil_div((int)g.total_tokens, kTile);
   const int sms = sm_count() > 0 ? sm_count() : 148;  // without a device: the part this is tuned for
-  return tiles >= 16LL * sms ? 8 : kMinChunkTiles;
+  const int split = sm100_first_half(g) ? 1 : 0;
+  const int most = (kMaxLeadChunks - 1) * sms >> split;  // chunks of a head
+  const int least = ceil_div(ceil_div(g.max_seqlen, kTile), most);
+  const long long tiles = (long long)n_layers * (g.n_kv_heads << split) * ceil_div((int)g.total_tokens, kTile);
+  const int wanted = options().score_chunk_tiles > 0 ? options().score_chunk_tiles
+                     : tiles >= 16LL * sms           ? 8
+                                                     : kMinChunkTiles;
+  return wanted > least ? wanted : least;
 }
 
 // Slots pass 1 leads pass 2 by beyond what head completion needs.  4 / 8 / 12 / 16 slots with chunks of
