@@ -106,8 +106,9 @@ LAVA_API int32_t lava_version(void);            /* major*10000 + minor*100 + pat
 LAVA_API const char* lava_last_error(void);     /* thread-local text of the last failure, never NULL */
 
 /* Bytes of device scratch that the score and select calls need for `n_layers` layers of this
- * geometry processed in one call.  The first 256 bytes hold the status word; the caller
- * should zero the workspace once after allocating it. */
+ * geometry processed in one call; calls on fewer layers or shorter sequences fit into it as well.
+ * The first 256 bytes hold the status word; the caller should zero the workspace once after
+ * allocating it. */
 LAVA_API size_t lava_workspace_bytes(const lava_layer_desc* desc, int32_t n_layers);
 
 /* Synchronises `stream`, copies the status word to *device_status_out (host) and clears it.
@@ -165,8 +166,10 @@ LAVA_API lava_status lava_score_layers(const lava_layer_desc* desc, int32_t n_la
  *   device_status_out  DEVICE uint32, may be NULL: receives the status word of this call
  *                      (LAVA_DEV_* bits) once `stream` has run past the call
  * Limits and rules:
- *   - A layer whose lava_workspace_bytes(desc, 1) exceeds 8 MiB is rejected with
- *     LAVA_ERR_WORKSPACE before anything is enqueued (about 128K tokens at 32/8 heads, d 128).
+ *   - A layer whose scratch does not fit 8 MiB in any layout is rejected with
+ *     LAVA_ERR_WORKSPACE before anything is enqueued (above 128K tokens at 32/8 heads, d 128).
+ *     Near that size fp32 layers take longer blocks than lava_score_layer gives short sequences,
+ *     and head_dim 64 the CUDA-core path; the results differ by the order of fp32 sums.
  *   - The first call on a device looks up the array's device address (a host-side set-up step,
  *     once per device, with that device current); make that first call before any stream
  *     capture begins.

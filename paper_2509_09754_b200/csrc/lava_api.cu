@@ -5,6 +5,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "lava_internal.cuh"
@@ -135,24 +136,22 @@ lava_status make_geom(const lava_layer_desc* d, Geom* out) {
   return LAVA_OK;
 }
 
-Workspace workspace_layout(const lava_layer_desc* d, int n_layers) {
+// Sizes with the generic path's blocks given; `tensor_path` leaves room for the tensor-core kernels.
+static Workspace layout_with(const lava_layer_desc* d, const Geom* g, int n_layers, int slice_keys,
+                             int score_keys, int v_keys, bool tensor_path) {
   Workspace w;
   const int max_seqlen = d->max_seqlen > 0 ? d->max_seqlen : (int)d->total_tokens;
   const size_t problems = (size_t)n_layers * d->batch;
-  // 64 keys per block up to 2048 tokens, 128 up to 4096, 256 up to 8192, then 512.  Score call in us with
-  // 64 / 128 / 512: one fp32 layer of 1000 tokens with 8 heads 32 / 41 / 122, of 4000 44 / 44 / 123, of 2000
-  // with 32 heads of 128 84 / 66 / 203; 32 layers x 32 heads of 4000 2046 / 1597 / 1397; 16 layers of 8000
-  // - / 2769 / 2722.  The rule looks at the length alone, so a layer gives the same bits alone and among
-  // others.
-  w.slice_keys = 64;
-  while (w.slice_keys < 512 && max_seqlen > 32 * w.slice_keys) w.slice_keys *= 2;
-  w.n_slices = ceil_div(max_seqlen, w.slice_keys);
-  // scores are pooled over up to 8 neighbours on either side: with them a slice is whole tiles of 64 keys
-  w.score_keys = d->pool_kind != LAVA_POOL_NONE && d->pool_kernel / 2 > 8 ? w.slice_keys : w.slice_keys - 16;
-  w.n_score_slices = ceil_div(max_seqlen, w.score_keys);
+  w.tensor_path = tensor_path;
+  w.slice_keys = slice_keys;
+  w.n_slices = ceil_div(max_seqlen, slice_keys);
+  w.score_keys = score_keys;
+  w.n_score_slices = ceil_div(max_seqlen, score_keys);
+  w.v_keys = v_keys;
+  w.n_vslices = ceil_div(max_seqlen, v_keys);
   size_t off = Workspace::kStatusBytes;
   w.off_vpart = off;
-  off = round_up(off + problems * d->n_kv_heads * w.n_slices * sizeof(float), 256);
+  off = round_up(off + problems * d->n_kv_heads * w.n_vslices * sizeof(float), 256);
   w.off_stats = off;
   off = round_up(off + problems * d->n_q_heads * w.n_slices * d->window * sizeof(float2), 256);
   w.off_lse = off;
@@ -162,13 +161,122 @@ Workspace workspace_layout(const lava_layer_desc* d, int n_layers) {
   w.off_ent = off;
   off = round_up(off + problems * d->n_kv_heads * w.n_score_slices * sizeof(double2), 256);
   w.off_sm100 = off;
-  Geom g;
-  const bool tensor_path = make_geom(d, &g) == LAVA_OK && sm100_supported(g);
-  if (tensor_path) off += sm100_layout(g, n_layers).total;
+  if (tensor_path) off += sm100_layout(*g, n_layers).total;
   w.off_tmem = off;
-  if (tensor_path && tmem_supported(g)) off += tmem_layout(g, n_layers).total;
+  if (tensor_path && tmem_supported(*g)) off += tmem_layout(*g, n_layers).total;
   w.total = off;
   return w;
+}
+
+constexpr int kLongSlice = 512;  // keys per block of the generic path in long sequences
+
+Workspace workspace_layout(const lava_layer_desc* d, int n_layers, size_t limit) {
+  const int max_seqlen = d->max_seqlen > 0 ? d->max_seqlen : (int)d->total_tokens;
+  Geom g;
+  // The generic path at its smallest, with the long blocks whatever the length.
+  auto smallest = [&](bool tensor_path) {
+    return layout_with(d, &g, n_layers, kLongSlice, kLongSlice, 2 * kLongSlice, tensor_path);
+  };
+  if (make_geom(d, &g) == LAVA_OK && sm100_supported(g)) {
+    // the generic path serves the "force_generic" option only, and head_dim 64 where there is no room
+    const Workspace w = smallest(true);
+    return w.total <= limit || g.head_dim == 128 ? w : smallest(false);
+  }
+  // 64 keys per block up to 2048 tokens, 128 up to 4096, 256 up to 8192, then 512.  Score call in us with
+  // 64 / 128 / 512: one fp32 layer of 1000 tokens with 8 heads 32 / 41 / 122, of 4000 44 / 44 / 123, of 2000
+  // with 32 heads of 128 84 / 66 / 203; 32 layers x 32 heads of 4000 2046 / 1597 / 1397; 16 layers of 8000
+  // - / 2769 / 2722.  The rule looks at the length alone, so a layer gives the same bits alone and among
+  // others.
+  int slice_keys = 64;
+  while (slice_keys < kLongSlice && max_seqlen > 32 * slice_keys) slice_keys *= 2;
+  for (; slice_keys <= kLongSlice; slice_keys *= 2) {
+    // scores are pooled over up to 8 neighbours on either side: with them a slice is whole tiles of 64 keys
+    const int halo = d->pool_kind != LAVA_POOL_NONE && d->pool_kernel / 2 > 8 ? 0 : 16;
+    const Workspace w = layout_with(d, &g, n_layers, slice_keys, slice_keys - halo, slice_keys, false);
+    if (w.total <= limit) return w;
+  }
+  return smallest(false);
+}
+
+size_t workspace_bytes_for(const lava_layer_desc* d, int n_layers) {
+  // A layout grows with the layers and, between the lengths at which the generic path's blocks double or
+  // the single-pass kernel ends, with the tokens.  So a buffer of this size serves every smaller call.
+  const int max_seqlen = d->max_seqlen > 0 ? d->max_seqlen : (int)d->total_tokens;
+  size_t most = workspace_layout(d, n_layers).total;
+  Geom g;
+  const int single_pass = make_geom(d, &g) == LAVA_OK ? tmem_longest(g) : 0;
+  for (const int length : {2048, 4096, 8192, single_pass})
+    if (length > 0 && length < max_seqlen) {
+      lava_layer_desc shorter = *d;
+      shorter.max_seqlen = length;
+      shorter.total_tokens = std::min<int64_t>(d->total_tokens, (int64_t)d->batch * length);
+      const size_t bytes = workspace_layout(&shorter, n_layers).total;
+      if (bytes > most) most = bytes;
+    }
+  return most;
+}
+
+lava_status score_layers_in(const lava_layer_desc* desc, int n_layers, const void* q_win, const void* k,
+                            const void* v, int64_t q_layer_stride, int64_t k_layer_stride,
+                            int64_t v_layer_stride, const float* vbar_in, float* scores, float* vbar_out,
+                            double* entropy, void* workspace, size_t workspace_bytes, size_t need,
+                            const Workspace& lay, void* stream) {
+  Geom g;
+  lava_status rc = make_geom(desc, &g);
+  if (rc != LAVA_OK) return rc;
+  if (!q_win || !k || !entropy || (!scores && g.total_scores > 0))
+    return fail(LAVA_ERR_INVALID_ARG, "q_win, k, scores and entropy are required");
+  const bool unit_term = (g.flags & (LAVA_FLAG_UNIT_VALUE_NORM | LAVA_FLAG_TOKEN_VALUE_NORM)) != 0;
+  const bool token_term = (g.flags & LAVA_FLAG_TOKEN_VALUE_NORM) != 0;
+  if (!v && !vbar_in && !(unit_term && !token_term))
+    return fail(LAVA_ERR_INVALID_ARG, "v may be NULL only if vbar_in is given");
+  if (unit_term && vbar_in)
+    return fail(LAVA_ERR_INVALID_ARG, "vbar_in must be NULL with a value-term flag");
+  if (token_term && !v) return fail(LAVA_ERR_INVALID_ARG, "the per-token value term needs v");
+  if (!aligned16(q_win) || !aligned16(k) || (v && !aligned16(v)) || !aligned16(scores))
+    return fail(LAVA_ERR_INVALID_ARG, "q_win, k, v and scores must be 16-byte aligned");
+  if (n_layers > 1 && (q_layer_stride % 8 || k_layer_stride % 8 || v_layer_stride % 8 ||
+                       q_layer_stride < 0 || k_layer_stride < 0 || v_layer_stride < 0))
+    return fail(LAVA_ERR_INVALID_ARG, "layer strides must be non-negative multiples of 8");
+  if (!workspace) return fail(LAVA_ERR_WORKSPACE, "workspace is NULL");
+  if (workspace_bytes < need)
+    return fail(LAVA_ERR_WORKSPACE, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
+  if (!aligned16(workspace)) return fail(LAVA_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
+  cudaStream_t st = (cudaStream_t)stream;
+  const void* v_used = v;
+  if (unit_term) {
+    // the score kernels run with a value-norm array of ones and never touch V
+    float* ones = reinterpret_cast<float*>((char*)workspace + lay.off_ones);
+    rc = launch_fill_ones(ones, (long long)n_layers * g.batch * g.n_kv_heads, st);
+    if (rc != LAVA_OK) return rc;
+    vbar_in = ones;
+    v_used = nullptr;
+  }
+  if (lay.tensor_path && !options().force_generic) {
+    // the single-pass kernel (exponentials kept in tensor memory) is opt-in: the exchange of row
+    // statistics between the CTAs outlasts what six exponent buffers can cover, so it is the
+    // slower of the two today
+    if (options().score_kernel == 2 && tmem_supported(g) && tmem_fits(g, tmem_grid(g, n_layers)))
+      rc = launch_score_tmem(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
+                             v_layer_stride, vbar_in, scores, vbar_out, entropy,
+                             (char*)workspace, lay.off_tmem, st);
+    else
+      rc = launch_score_sm100(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
+                              v_layer_stride, vbar_in, scores, vbar_out, entropy,
+                              (char*)workspace, lay.off_sm100,
+                              reinterpret_cast<double2*>((char*)workspace + lay.off_ent), st);
+  } else {
+    rc = launch_score_generic(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
+                              v_layer_stride, vbar_in, scores, vbar_out, entropy,
+                              (char*)workspace, lay, st);
+  }
+  if (rc != LAVA_OK || !token_term) return rc;
+  // VATP: every position's own value-row norm, then the entropy of the final scores
+  rc = launch_token_norm_scale(g, n_layers, v, v_layer_stride, scores, st);
+  if (rc != LAVA_OK) return rc;
+  return launch_entropy_from_scores(g, n_layers, scores, entropy,
+                                    reinterpret_cast<double2*>((char*)workspace + lay.off_ent),
+                                    nullptr, nullptr, nullptr, st);
 }
 
 }  // namespace lava
@@ -227,7 +335,7 @@ int64_t lava_get_option(const char* name) {
 size_t lava_workspace_bytes(const lava_layer_desc* desc, int32_t n_layers) {
   Geom g;
   if (n_layers < 1 || make_geom(desc, &g) != LAVA_OK) return 0;
-  return workspace_layout(desc, n_layers).total;
+  return workspace_bytes_for(desc, n_layers);
 }
 
 lava_status lava_poll_status(void* workspace, void* stream, uint32_t* device_status_out) {
@@ -261,64 +369,12 @@ lava_status lava_score_layers(const lava_layer_desc* desc, int32_t n_layers, con
                               double* entropy, void* workspace, size_t workspace_bytes,
                               void* stream) {
   Geom g;
-  lava_status rc = make_geom(desc, &g);
+  const lava_status rc = make_geom(desc, &g);
   if (rc != LAVA_OK) return rc;
   if (n_layers < 1) return fail(LAVA_ERR_INVALID_ARG, "n_layers must be >= 1");
-  if (!q_win || !k || !entropy || (!scores && g.total_scores > 0))
-    return fail(LAVA_ERR_INVALID_ARG, "q_win, k, scores and entropy are required");
-  const bool unit_term = (g.flags & (LAVA_FLAG_UNIT_VALUE_NORM | LAVA_FLAG_TOKEN_VALUE_NORM)) != 0;
-  const bool token_term = (g.flags & LAVA_FLAG_TOKEN_VALUE_NORM) != 0;
-  if (!v && !vbar_in && !(unit_term && !token_term))
-    return fail(LAVA_ERR_INVALID_ARG, "v may be NULL only if vbar_in is given");
-  if (unit_term && vbar_in)
-    return fail(LAVA_ERR_INVALID_ARG, "vbar_in must be NULL with a value-term flag");
-  if (token_term && !v) return fail(LAVA_ERR_INVALID_ARG, "the per-token value term needs v");
-  if (!aligned16(q_win) || !aligned16(k) || (v && !aligned16(v)) || !aligned16(scores))
-    return fail(LAVA_ERR_INVALID_ARG, "q_win, k, v and scores must be 16-byte aligned");
-  if (n_layers > 1 && (q_layer_stride % 8 || k_layer_stride % 8 || v_layer_stride % 8 ||
-                       q_layer_stride < 0 || k_layer_stride < 0 || v_layer_stride < 0))
-    return fail(LAVA_ERR_INVALID_ARG, "layer strides must be non-negative multiples of 8");
-  const Workspace lay = workspace_layout(desc, n_layers);
-  if (!workspace) return fail(LAVA_ERR_WORKSPACE, "workspace is NULL");
-  if (workspace_bytes < lay.total)
-    return fail(LAVA_ERR_WORKSPACE, "workspace too small: %zu < %zu bytes", workspace_bytes,
-                lay.total);
-  if (!aligned16(workspace)) return fail(LAVA_ERR_INVALID_ARG, "workspace must be 16-byte aligned");
-  cudaStream_t st = (cudaStream_t)stream;
-  const void* v_used = v;
-  if (unit_term) {
-    // the score kernels run with a value-norm array of ones and never touch V
-    float* ones = reinterpret_cast<float*>((char*)workspace + lay.off_ones);
-    rc = launch_fill_ones(ones, (long long)n_layers * g.batch * g.n_kv_heads, st);
-    if (rc != LAVA_OK) return rc;
-    vbar_in = ones;
-    v_used = nullptr;
-  }
-  if (sm100_supported(g) && !options().force_generic) {
-    // the single-pass kernel (exponentials kept in tensor memory) is opt-in: the exchange of row
-    // statistics between the CTAs outlasts what six exponent buffers can cover, so it is the
-    // slower of the two today
-    if (options().score_kernel == 2 && tmem_supported(g) && tmem_fits(g, tmem_grid(g, n_layers)))
-      rc = launch_score_tmem(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
-                             v_layer_stride, vbar_in, scores, vbar_out, entropy,
-                             (char*)workspace, lay.off_tmem, st);
-    else
-      rc = launch_score_sm100(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
-                              v_layer_stride, vbar_in, scores, vbar_out, entropy,
-                              (char*)workspace, lay.off_sm100,
-                              reinterpret_cast<double2*>((char*)workspace + lay.off_ent), st);
-  } else {
-    rc = launch_score_generic(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
-                              v_layer_stride, vbar_in, scores, vbar_out, entropy,
-                              (char*)workspace, lay, st);
-  }
-  if (rc != LAVA_OK || !token_term) return rc;
-  // VATP: every position's own value-row norm, then the entropy of the final scores
-  rc = launch_token_norm_scale(g, n_layers, v, v_layer_stride, scores, st);
-  if (rc != LAVA_OK) return rc;
-  return launch_entropy_from_scores(g, n_layers, scores, entropy,
-                                    reinterpret_cast<double2*>((char*)workspace + lay.off_ent),
-                                    nullptr, nullptr, nullptr, st);
+  return score_layers_in(desc, n_layers, q_win, k, v, q_layer_stride, k_layer_stride, v_layer_stride, vbar_in,
+                         scores, vbar_out, entropy, workspace, workspace_bytes,
+                         workspace_bytes_for(desc, n_layers), workspace_layout(desc, n_layers), stream);
 }
 
 lava_status lava_score_layer(const lava_layer_desc* desc, const void* q_win, const void* k,

@@ -64,11 +64,16 @@ __device__ inline bool batch_has_short_sequence(const Geom& g) {
 // Workspace layout (byte offsets from the workspace base), identical for every caller.
 struct Workspace {
   static constexpr size_t kStatusBytes = 256;
-  // generic score path: keys per block of the statistics (and rows of V), and of the scores
-  int slice_keys, n_slices, score_keys, n_score_slices;
+  bool tensor_path;  // there is room for the tensor-core score kernels where the geometry has them
+  // generic score path: keys per block of the statistics and of the scores, rows of V per block
+  int slice_keys, n_slices, score_keys, n_score_slices, v_keys, n_vslices;
   size_t off_vpart, off_stats, off_lse, off_ones, off_ent, off_sm100, off_tmem, total;
 };
-Workspace workspace_layout(const lava_layer_desc* d, int n_layers);
+// The layout that a call uses.  Given a limit, the first one, from the fastest to the smallest, that fits
+// it; the smallest one where none does.
+Workspace workspace_layout(const lava_layer_desc* d, int n_layers, size_t limit = SIZE_MAX);
+// What is asked of the caller: the most that a call with these or fewer layers and tokens uses.
+size_t workspace_bytes_for(const lava_layer_desc* d, int n_layers);
 
 // Tuning and test knobs of the library (lava_set_option / lava_get_option).  The defaults come from
 // the environment, read once when the first option is looked at; nothing on a call path calls getenv.
@@ -115,6 +120,12 @@ lava_status check_cuda(cudaError_t e, const char* what);
 lava_status make_geom(const lava_layer_desc* d, Geom* out);
 void count_launches(int n);  // bookkeeping for lava_launch_count()
 
+// lava_score_layers with the layout chosen by the caller; `need` is the least workspace that is accepted.
+lava_status score_layers_in(const lava_layer_desc* desc, int n_layers, const void* q_win, const void* k,
+                            const void* v, int64_t q_ls, int64_t k_ls, int64_t v_ls, const float* vbar_in,
+                            float* scores, float* vbar_out, double* entropy, void* workspace,
+                            size_t workspace_bytes, size_t need, const Workspace& lay, void* stream);
+
 // Launchers implemented in the kernel translation units.  Each returns LAVA_OK or the status of
 // a failed launch; all run on `stream`.
 lava_status launch_score_generic(const Geom& g, int n_layers, const void* q, const void* k,
@@ -146,6 +157,7 @@ struct TmemLayout {
   long long kjobs_cap;
   size_t off_sync, sync_bytes, off_part, off_gpart, off_ent, total;
 };
+int tmem_longest(const Geom& g);  // the longest sequence it covers, 0 if the geometry is not one of its
 bool tmem_supported(const Geom& g);
 bool tmem_fits(const Geom& g, int grid);
 int tmem_grid(const Geom& g, int n_layers);

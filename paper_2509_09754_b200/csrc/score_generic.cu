@@ -148,24 +148,26 @@ __device__ void value_norm_slice(const Geom& g, const char* v, int kvh, long lon
 template <int D, bool BF16>
 __global__ void __launch_bounds__(kThreads)
 stats_partial_kernel(Geom g, const char* q, const char* k, const char* v, long long q_ls, long long k_ls,
-                     long long v_ls, float2* stats, float* vpart, int slice_keys, int n_slices, int at_once) {
+                     long long v_ls, float2* stats, float* vpart, int slice_keys, int n_slices, int v_keys,
+                     int n_vslices, int at_once) {
   in_stream_order();
   extern __shared__ __align__(16) float smem[];
   const int prob = blockIdx.z, layer = prob / g.batch, b = prob - layer * g.batch;
   const int slice = blockIdx.x;
   const SeqInfo s = seq_info(g, b);
-  const int key_lo = slice * slice_keys;
-  if (key_lo >= s.n) return;
-  const int key_hi = min(s.n, key_lo + slice_keys);
   const int es = BF16 ? 2 : 4;
   const int batches = (g.group + at_once - 1) / at_once;
   const int unit = blockIdx.y;
   if (unit >= g.n_kv_heads * batches) {
-    const int kvh = unit - g.n_kv_heads * batches;
-    value_norm_slice(g, v + (size_t)layer * v_ls * es, kvh, s.tok0, key_lo, key_hi,
-                     vpart + ((size_t)prob * g.n_kv_heads + kvh) * n_slices + slice);
+    const int kvh = unit - g.n_kv_heads * batches, row_lo = slice * v_keys;
+    if (slice < n_vslices && row_lo < s.n)
+      value_norm_slice(g, v + (size_t)layer * v_ls * es, kvh, s.tok0, row_lo, min(s.n, row_lo + v_keys),
+                       vpart + ((size_t)prob * g.n_kv_heads + kvh) * n_vslices + slice);
     return;
   }
+  const int key_lo = slice * slice_keys;
+  if (key_lo >= s.n) return;
+  const int key_hi = min(s.n, key_lo + slice_keys);
   const int kvh = unit / batches, hb = (unit - kvh * batches) * at_once;
   const int h0 = kvh * g.group + hb, rows = min(at_once, g.group - hb) * g.w_pad;
   float* qs = smem;
@@ -253,9 +255,9 @@ __host__ __device__ inline int a_stride_of(int score_keys) { return score_keys +
 template <int D, bool BF16>
 __global__ void __launch_bounds__(kThreads)
 score_kernel(Geom g, const char* q, const char* k, long long q_ls, long long k_ls, const float2* stats,
-             const float* neg_lse, const float* vpart, const float* vbar_in, float* vbar_out, float* scores, double2* ent_part,
-             unsigned* status, int slice_keys, int n_slices, int score_keys, int n_score_slices,
-             int at_once) {
+             const float* neg_lse, const float* vpart, const float* vbar_in, float* vbar_out, float* scores,
+             double2* ent_part, unsigned* status, int slice_keys, int n_slices, int v_keys, int n_vslices,
+             int score_keys, int n_score_slices, int at_once) {
   in_stream_order();
   extern __shared__ __align__(16) float smem[];
   float* qs = smem;
@@ -279,8 +281,8 @@ score_kernel(Geom g, const char* q, const char* k, long long q_ls, long long k_l
     if (vbar_in) {
       m = vbar_in[(size_t)prob * g.n_kv_heads + kvh];
     } else {
-      const float* p = vpart + ((size_t)prob * g.n_kv_heads + kvh) * n_slices;
-      for (int sl = lane; sl < used; sl += 32) m = fmaxf(m, p[sl]);
+      const float* p = vpart + ((size_t)prob * g.n_kv_heads + kvh) * n_vslices;
+      for (int sl = lane; sl < ceil_div(s.n, v_keys); sl += 32) m = fmaxf(m, p[sl]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
@@ -451,7 +453,7 @@ lava_status launch_generic(const Geom& g, int n_layers, const char* q, const cha
   if (e != cudaSuccess) return check_cuda(e, "cudaFuncSetAttribute(score kernels)");
   launch_in_order(stats_k, dim3(lay.n_slices, g.n_kv_heads * (batches + (vbar_in ? 0 : 1)), problems),
                   kThreads, tile_bytes, stream, g, q, k, v, q_ls, k_ls, v_ls, stats, vpart,
-                  lay.slice_keys, lay.n_slices, at_once);
+                  lay.slice_keys, lay.n_slices, lay.v_keys, lay.n_vslices, at_once);
   // Each score block folds the statistics of its rows itself, unless there are so many blocks that the
   // work weighs more than a launch (the same bits either way): 32 layers of 4000 tokens 2611 us
   // without the launch, 2046 with it; one of 2000 tokens 30.6 without, 32.8 with it.
@@ -464,8 +466,8 @@ lava_status launch_generic(const Geom& g, int n_layers, const char* q, const cha
   }
   launch_in_order(score_k, dim3(lay.n_score_slices, g.n_kv_heads, problems), kThreads, score_bytes, stream,
                   g, q, k, q_ls, k_ls, stats, neg_lse, vpart, vbar_in, vbar_out, scores, ent_part,
-                  reinterpret_cast<unsigned*>(ws), lay.slice_keys, lay.n_slices, lay.score_keys,
-                  lay.n_score_slices, at_once);
+                  reinterpret_cast<unsigned*>(ws), lay.slice_keys, lay.n_slices, lay.v_keys, lay.n_vslices,
+                  lay.score_keys, lay.n_score_slices, at_once);
   launch_in_order(entropy_finalize_kernel, problems, 32, 0, stream, g, ent_part, lay.score_keys,
                   lay.n_score_slices, entropy);
   count_launches(neg_lse ? 4 : 3);

@@ -33,12 +33,12 @@ extern "C" lava_status lava_score_layer_static(const lava_layer_desc* desc, cons
   Geom geom;
   lava_status rc = make_geom(desc, &geom);
   if (rc != LAVA_OK) return rc;
-  const size_t need = workspace_layout(desc, 1).total;
-  if (need > kStaticScratchBytes)
+  const Workspace lay = workspace_layout(desc, 1, kStaticScratchBytes);
+  if (lay.total > kStaticScratchBytes)
     return fail(LAVA_ERR_WORKSPACE,
                 "this layer needs %zu bytes of scratch; the built-in scratch of "
                 "lava_score_layer_static holds %zu bytes: use lava_score_layer with a workspace",
-                need, kStaticScratchBytes);
+                lay.total, kStaticScratchBytes);
   int dev = 0;
   rc = check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
   if (rc != LAVA_OK) return rc;
@@ -59,8 +59,8 @@ extern "C" lava_status lava_score_layer_static(const lava_layer_desc* desc, cons
   // score kernels clear the rest of what they rely on themselves).
   rc = check_cuda(cudaMemsetAsync(scratch, 0, Workspace::kStatusBytes, st), "status clear");
   if (rc != LAVA_OK) return rc;
-  rc = lava_score_layer(desc, q_win, k, v, vbar_in, scores, vbar_out, entropy, scratch,
-                        kStaticScratchBytes, stream);
+  rc = score_layers_in(desc, 1, q_win, k, v, 0, 0, 0, vbar_in, scores, vbar_out, entropy, scratch,
+                       kStaticScratchBytes, lay.total, lay, stream);
   if (rc != LAVA_OK) return rc;
   if (device_status_out)
     rc = check_cuda(cudaMemcpyAsync(device_status_out, scratch, sizeof(uint32_t),

@@ -1052,14 +1052,11 @@ int first_unit_heads(const Geom& g) { return g.group * g.window > 128 ? (g.group
 // Geometry the single-pass kernel covers, whatever the grid: the tensor-core path's geometry,
 // a pooling radius of at most 4, and a head short enough for a part with up to 160 SMs.  Whether
 // a launch really fits is decided against the actual grid in tmem_fits.
-bool tmem_supported(const Geom& g) {
-  if (g.head_dim != 128) return false;
-  if (!sm100_supported(g)) return false;
-  if (g.pool_radius > kMaxRadius) return false;
-  const int nunit = first_unit_heads(g) ? 2 : 1;
-  const int tmax = ceil_div(g.max_seqlen, kTile - 2 * g.pool_radius);
-  return tmax <= (nunit == 1 ? 3 * 160 + 1 : 160 + 1);
+int tmem_longest(const Geom& g) {
+  if (g.head_dim != 128 || !sm100_supported(g) || g.pool_radius > kMaxRadius) return 0;
+  return (first_unit_heads(g) ? 160 + 1 : 3 * 160 + 1) * (kTile - 2 * g.pool_radius);
 }
+bool tmem_supported(const Geom& g) { return g.max_seqlen <= tmem_longest(g); }
 
 TmemLayout tmem_layout(const Geom& g, int n_layers) {
   TmemLayout l;
