@@ -150,6 +150,10 @@ struct Sm100Params {
   unsigned* vbar_bits;      // [heads_total]
   float2* ent_part;         // [heads_total][cph_max][8 consumer warps] (sum s, sum s ln s)
   unsigned* status;
+  // kernel for shared rows: (head, layer) in the maps of K and V and the layer in the queries' are the
+  // indexes times this, 0 where heads or layers share their rows
+  int2 k_at, v_at;
+  int q_at;
 };
 
 // ------------------------------------------------------------------------------------------
@@ -257,7 +261,10 @@ __device__ inline float exp_sum16(const float* c, float scale, float shift) {
 // ------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------
-template <int W, int D>
+// SHARED: some heads or layers of Q, K or V share their rows (stride 0), which a tensor map cannot express.
+// A variant of its own: with the coordinates computed in the one kernel, in the producers or in the chunk
+// records, the ragged batch of 8 (windows of 64) took 1 % longer.
+template <int W, int D, bool SHARED>
 __global__ void __launch_bounds__(kThreads, 1)
 lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
                         const __grid_constant__ CUtensorMap map_k,
@@ -461,7 +468,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
     for (int j = 0; j < nchunks && ok; ++j) {
       if (!kFirst && !chunk_ready(m, j, p.status)) break;
       const Chunk& ck = m->ring[j % kRing];
-      const int nt = kFirst ? ck.n1 : ck.n2, kvh = ck.kvh, layer = ck.layer;
+      const int nt = kFirst ? ck.n1 : ck.n2;
+      const int kvh = SHARED ? ck.kvh * p.k_at.x : ck.kvh, layer = SHARED ? ck.layer * p.k_at.y : ck.layer;
       // a pass-2 tile starts pool_radius keys before the first key it owns (halo for pooling)
       int tok = ck.tok0 + (kFirst ? ck.tile1 * kTile : ck.tile2 * p.out_keys - g.pool_radius);
       for (int t = 0; t < nt && ok; ++t, tok += step) {
@@ -494,8 +502,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
           ok = wait_for(q_empty, (q_loads & 1) ^ 1, m, p.status);
           if (ok) {
             mbar_expect_tx(q_full, S::kTileBytes);
-            tma_load_4d_plain(base + (kFirst ? kOffQ1 : S::kOffQ2), &map_q, 0, ck.q_row0, 0, layer,
-                              q_full);
+            tma_load_4d_plain(base + (kFirst ? kOffQ1 : S::kOffQ2), &map_q, 0, ck.q_row0, 0,
+                              SHARED ? ck.layer * p.q_at : layer, q_full);
             ++q_loads;
           }
         }
@@ -886,8 +894,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
             const Chunk& ck = m->ring[ld.j % kRing];
             const uint32_t bar = smem_u32(&m->v_full[vw][st]);
             mbar_expect_tx(bar, S::kVBytes);
-            tma_load_5d(base + stage0 + st * S::kVBytes, &map_v, 0, ck.tok0 + ld.row, 0, ck.kvh,
-                        ck.layer, bar, drop);
+            tma_load_5d(base + stage0 + st * S::kVBytes, &map_v, 0, ck.tok0 + ld.row, 0,
+                        SHARED ? ck.kvh * p.v_at.x : ck.kvh, SHARED ? ck.layer * p.v_at.y : ck.layer, bar, drop);
           }
           ld.row += parts * kVRows;
           ++nl;
@@ -1204,11 +1212,12 @@ static lava_status encode_rows_map(const Geom& g, int n_layers, const void* x, l
   EncodeTiledFn encode = encode_fn();
   if (!encode) return fail(LAVA_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   const cuuint64_t blocks = (cuuint64_t)g.head_dim / 64;
-  const cuuint64_t dims[5] = {64, (cuuint64_t)g.total_tokens, blocks, (cuuint64_t)g.n_kv_heads,
-                              (cuuint64_t)n_layers};
-  const cuuint64_t hs = (cuuint64_t)sh * 2;
-  const cuuint64_t lb = n_layers > 1 ? (cuuint64_t)ls * 2 : hs * (cuuint64_t)g.n_kv_heads;
-  const cuuint64_t strides[4] = {(cuuint64_t)st * 2, 128, hs > 0 ? hs : 256, lb > 0 ? lb : 256};
+  // heads or layers that share their rows (stride 0) are one to the map
+  const cuuint64_t heads = sh > 0 ? (cuuint64_t)g.n_kv_heads : 1;
+  const cuuint64_t layers = ls > 0 ? (cuuint64_t)n_layers : 1;
+  const cuuint64_t dims[5] = {64, (cuuint64_t)g.total_tokens, blocks, heads, layers};
+  const cuuint64_t strides[4] = {(cuuint64_t)st * 2, 128, sh > 0 ? (cuuint64_t)sh * 2 : 256,
+                                 layers > 1 ? (cuuint64_t)ls * 2 : 256};
   const cuuint32_t box[5] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_blocks, 1, 1};
   const cuuint32_t es[5] = {1, 1, 1, 1, 1};
   if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(x), dims, strides, box, es,
@@ -1224,8 +1233,9 @@ static lava_status encode_query_map(const Geom& g, int n_layers, const void* q, 
   EncodeTiledFn encode = encode_fn();
   if (!encode) return fail(LAVA_ERR_CUDA, "cuTensorMapEncodeTiled is not available");
   const cuuint64_t rows = (cuuint64_t)g.batch * g.n_q_heads * g.window, d = (cuuint64_t)g.head_dim;
-  const cuuint64_t dims[4] = {64, rows, d / 64, (cuuint64_t)n_layers};
-  const cuuint64_t strides[3] = {d * 2, 128, n_layers > 1 ? (cuuint64_t)ls * 2 : rows * d * 2};
+  const cuuint64_t layers = ls > 0 ? (cuuint64_t)n_layers : 1;
+  const cuuint64_t dims[4] = {64, rows, d / 64, layers};
+  const cuuint64_t strides[3] = {d * 2, 128, layers > 1 ? (cuuint64_t)ls * 2 : rows * d * 2};
   const cuuint32_t box[4] = {64, kTile, (cuuint32_t)(d / 64), 1}, es[4] = {1, 1, 1, 1};
   if (encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(q), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -1315,6 +1325,9 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
   p.part = reinterpret_cast<float*>(ws + lay.off_part);
   p.ent_part = reinterpret_cast<float2*>(ws + lay.off_ent);
   p.status = reinterpret_cast<unsigned*>(ws_base);  // the status word opens the workspace
+  p.k_at = make_int2(g.k_sh > 0, k_ls > 0);
+  p.v_at = make_int2(g.v_sh > 0, v_ls > 0);
+  p.q_at = q_ls > 0;
 
   rc = check_cuda(cudaMemsetAsync(ws + lay.off_sync, 0, lay.sync_bytes, stream),
                   "sync scratch clear");
@@ -1325,14 +1338,18 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
     if (rc != LAVA_OK) return rc;
   }
 
-  void (*kern)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const Sm100Params) = nullptr;
   const bool wide = g.head_dim == 128;
-  switch (g.window) {
-    case 16: kern = wide ? lava_score_sm100_kernel<16, 128> : lava_score_sm100_kernel<16, 64>; break;
-    case 32: kern = wide ? lava_score_sm100_kernel<32, 128> : lava_score_sm100_kernel<32, 64>; break;
-    case 64: kern = wide ? lava_score_sm100_kernel<64, 128> : lava_score_sm100_kernel<64, 64>; break;
-    default: kern = wide ? lava_score_sm100_kernel<128, 128> : lava_score_sm100_kernel<128, 64>; break;
-  }
+  const bool shared = (g.n_kv_heads > 1 && (g.k_sh == 0 || (!vbar_in && g.v_sh == 0))) ||
+                      (n_layers > 1 && (q_ls == 0 || k_ls == 0 || (!vbar_in && v_ls == 0)));
+  auto pick = [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    return shared ? (wide ? lava_score_sm100_kernel<W, 128, true> : lava_score_sm100_kernel<W, 64, true>)
+                  : (wide ? lava_score_sm100_kernel<W, 128, false> : lava_score_sm100_kernel<W, 64, false>);
+  };
+  const auto kern = g.window == 16   ? pick(std::integral_constant<int, 16>())
+                    : g.window == 32 ? pick(std::integral_constant<int, 32>())
+                    : g.window == 64 ? pick(std::integral_constant<int, 64>())
+                                     : pick(std::integral_constant<int, 128>());
   const int smem = wide ? (int)Smem<128>::kBytes : (int)Smem<64>::kBytes;
   rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                   "cudaFuncSetAttribute(sm100 score)");
