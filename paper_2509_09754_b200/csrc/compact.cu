@@ -87,17 +87,17 @@ move_head(const Geom& g, int prob, const int* src_pos, const int* hoff_old_all, 
 
 // A step of the cascade: both kinds of rows side by side, 24 us at 8K (one after the other 6 + 23).
 __global__ void __launch_bounds__(256)
-cascade_rows_kernel(Geom g, int n_lists, HeldLists io, const int* hoff_new, const char* k_old,
+cascade_rows_kernel(Geom g, int first, int n_lists, HeldLists io, const int* hoff_new, const char* k_old,
                     const char* v_old, const char* k, const char* v, const int* keep_idx, char* k_new,
                     char* v_new, int blocks_per_head) {
   in_stream_order();
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
-  const int prob = blockIdx.z - g.batch;    // the new layer first: its rows come from further away
+  const int z = first + blockIdx.z, prob = z - g.batch;  // the new layer first: its rows come from further away
   if (prob >= 0)
     move_head(g, prob, io.src_pos, io.hoff_old, hoff_new, io.row_off_old, io.row_off_new, k_old, v_old, k_new,
               v_new, blocks_per_head);
   else
-    compact_head(g, blockIdx.z, k, v, 0, 0, keep_idx, hoff_new + (size_t)n_lists * (g.n_kv_heads + 1),
+    compact_head(g, z, k, v, 0, 0, keep_idx, hoff_new + (size_t)n_lists * (g.n_kv_heads + 1),
                  io.row_off_new + n_lists, k_new, v_new, blocks_per_head);
 }
 
@@ -129,10 +129,14 @@ lava_status launch_cascade_rows(const Geom& g, int n_lists, const HeldLists& io,
                                 const char* k_old, const char* v_old, const void* k, const void* v,
                                 const int* keep_idx, char* k_new, char* v_new, cudaStream_t stream) {
   const int problems = n_lists + g.batch, bph = blocks_per_head(g, problems);
-  const cudaError_t e = launch_in_order(cascade_rows_kernel, dim3(bph, g.n_kv_heads, problems), 256, 0, stream,
-                                        g, n_lists, io, hoff_new, k_old, v_old, (const char*)k,
-                                        (const char*)v, keep_idx, k_new, v_new, bph);
-  count_launches(1);
+  constexpr int kMost = 65535;  // blocks in the third dimension of a grid
+  cudaError_t e = cudaSuccess;
+  for (int first = 0; first < problems && e == cudaSuccess; first += kMost) {
+    const dim3 grid(bph, g.n_kv_heads, std::min(kMost, problems - first));
+    e = launch_in_order(cascade_rows_kernel, grid, 256, 0, stream, g, first, n_lists, io, hoff_new, k_old, v_old,
+                        (const char*)k, (const char*)v, keep_idx, k_new, v_new, bph);
+    count_launches(1);
+  }
   return check_cuda(e, "cascade rows launch");
 }
 

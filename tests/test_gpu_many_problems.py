@@ -1,0 +1,40 @@
+"""Calls of more (layer, sequence) problems than a grid's second and third dimensions can hold."""
+import pytest
+import torch
+
+import paper_2509_09754_b200 as lava
+
+pytestmark = pytest.mark.gpu
+
+
+def test_cascade_of_65536_layers_and_sequences():
+    layers, batch, n, d, w = 64, 1024, 4, 64, 1
+    g = torch.Generator(device="cuda").manual_seed(6)
+    q = torch.randn((layers, batch, 1, w, d), generator=g, device="cuda")
+    k, v = (torch.randn((layers, 1, batch * n, d), generator=g, device="cuda") for _ in range(2))
+    total = torch.full((batch,), 2 * layers, dtype=torch.int64, device="cuda")   # two rows a layer on average
+
+    def run(b0, b1):
+        cu = torch.arange(0, (b1 - b0) * n + 1, n, dtype=torch.int32, device="cuda")
+        qs, ks, vs = q[:, b0:b1].contiguous(), k[:, :, b0 * n:b1 * n].contiguous(), v[:, :, b0 * n:b1 * n].contiguous()
+        desc = lava.LayerDesc.for_tensors(qs[0], ks[0], vs[0], w, cu_seqlens=cu, max_seqlen=n)
+        cas = lava.Cascade(desc, layers, 2 * layers * (b1 - b0), kv_dtype=k.dtype)
+        cas.begin(total[b0:b1].contiguous())
+        for l in range(layers):
+            cas.step(qs[l], ks[l], vs[l])
+        view = {name: t.clone() for name, t in cas.view().items() if torch.is_tensor(t)}
+        cas.close()
+        return view
+
+    whole, halves = run(0, batch), [run(0, batch // 2), run(batch // 2, batch)]
+    for name in ("layer_budget", "head_offsets"):
+        parts = [h[name].view(layers, batch // 2, -1) for h in halves]
+        assert torch.equal(whole[name].view(layers, batch, -1), torch.cat(parts, dim=1))
+    rows = whole["layer_row_offset"].view(-1)[:layers * batch + 1]
+    for i, half in enumerate(halves):
+        part = half["layer_row_offset"].view(-1)[:layers * batch // 2 + 1]
+        for l in range(layers):   # a layer's sequences of one half lie together in both
+            a, b = int(rows[l * batch + i * batch // 2]), int(rows[l * batch + (i + 1) * batch // 2])
+            c, e = int(part[l * batch // 2]), int(part[(l + 1) * batch // 2])
+            for name in ("k_out", "v_out"):
+                assert torch.equal(whole[name][a:b], half[name][c:e])
