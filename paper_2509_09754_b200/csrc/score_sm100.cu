@@ -1020,20 +1020,22 @@ entropy_finalize_sm100_kernel(Geom g, const float2* ent_part, int cph_max, int c
 // order: thread-strided fp32 sums of 32 terms, then fp64.
 constexpr int kEntropySlice = 32768;
 
-// `part` NULL: one block per problem, which finishes it; else the sums of one slice each
+// `part` NULL: one block per problem, which finishes it; else the sums of one slice each.  Slices and
+// problems share the grid's first dimension: the others end at 65535.
 __global__ void __launch_bounds__(1024)
-entropy_from_scores_kernel(Geom g, const float* scores, double2* part, double* entropy,
+entropy_from_scores_kernel(Geom g, const float* scores, int slices, double2* part, double* entropy,
                            const float* vbar_in, const unsigned* vbar_bits, float* vbar_out) {
   in_stream_order();
   if (batch_has_short_sequence(g)) return;
-  const int prob = blockIdx.y, layer = prob / g.batch, b = prob - layer * g.batch;
+  const int prob = blockIdx.x / slices, slice = blockIdx.x - prob * slices;
+  const int layer = prob / g.batch, b = prob - layer * g.batch;
   const SeqInfo s = seq_info(g, b);
-  if (vbar_out && blockIdx.x == 0 && (int)threadIdx.x < g.n_kv_heads) {
+  if (vbar_out && slice == 0 && (int)threadIdx.x < g.n_kv_heads) {
     const size_t head = (size_t)prob * g.n_kv_heads + threadIdx.x;
     vbar_out[head] = vbar_in ? vbar_in[head] : __uint_as_float(vbar_bits[head]);
   }
   const int count = g.n_kv_heads * s.prefix;  // fits: H_kv * total_tokens is below 2^31
-  const int i0 = (int)min((long long)count, (long long)blockIdx.x * kEntropySlice);
+  const int i0 = (int)min((long long)count, (long long)slice * kEntropySlice);
   const int n = min(kEntropySlice, count - i0);
   const float* sc = scores + (size_t)layer * g.total_scores + s.score_off + i0;
   float es = 0.f, et = 0.f;
@@ -1057,7 +1059,7 @@ entropy_from_scores_kernel(Geom g, const float* scores, double2* part, double* e
     a += red[i].x;
     c += red[i].y;
   }
-  if (part) part[(size_t)prob * gridDim.x + blockIdx.x] = make_double2(a, c);
+  if (part) part[blockIdx.x] = make_double2(a, c);
   else entropy[prob] = a > 0.0 ? (log(a) - c / a) / ((double)g.n_kv_heads * (double)s.n) : 0.0;
 }
 
@@ -1155,8 +1157,8 @@ lava_status launch_entropy_from_scores(const Geom& g, int n_layers, const float*
   const long long most = (long long)g.n_kv_heads * (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
   const int slices = most > kEntropySlice ? (int)((most + kEntropySlice - 1) / kEntropySlice) : 1;
   const int problems = n_layers * g.batch;
-  launch_in_order(entropy_from_scores_kernel, dim3(slices, problems), 1024, 0, stream, g, scores, slices
-                  > 1 ? scratch : nullptr, entropy, vbar_in, vbar_bits, vbar_out);
+  launch_in_order(entropy_from_scores_kernel, slices * problems, 1024, 0, stream, g, scores, slices,
+                  slices > 1 ? scratch : nullptr, entropy, vbar_in, vbar_bits, vbar_out);
   if (slices > 1)
     launch_in_order(entropy_from_slices_kernel, problems, 32, 0, stream, g, scratch, slices, entropy);
   count_launches(slices > 1 ? 2 : 1);

@@ -38,3 +38,27 @@ def test_cascade_of_65536_layers_and_sequences():
             c, e = int(part[l * batch // 2]), int(part[(l + 1) * batch // 2])
             for name in ("k_out", "v_out"):
                 assert torch.equal(whole[name][a:b], half[name][c:e])
+
+
+def test_entropies_of_66048_layers_and_sequences():
+    # a split query group (16 x 16 rows), whose entropies are taken from the final scores; one layer's
+    # inputs stand for all
+    layers, batch, n, d, w, group = 129, 512, 40, 64, 16, 16
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q = torch.randn((1, batch, group, w, d), generator=g, device="cuda").bfloat16().expand(layers, -1, -1, -1, -1)
+    k, v = (torch.randn((1, 1, batch * n, d), generator=g, device="cuda").bfloat16().expand(layers, -1, -1, -1)
+            for _ in range(2))
+    cu = torch.arange(0, batch * n + 1, n, dtype=torch.int32, device="cuda")
+    desc = lava.LayerDesc.for_tensors(q[0], k[0], v[0], w, cu_seqlens=cu, max_seqlen=n)
+
+    def score(count):
+        out = (torch.empty((count, desc.total_scores), device="cuda"), torch.empty((count, batch, 1), device="cuda"),
+               torch.empty((count, batch), dtype=torch.float64, device="cuda"))
+        ws = torch.zeros(lava.lava_workspace_bytes(desc, count), dtype=torch.uint8, device="cuda")
+        lava.lava_score_layers(desc, count, q, k, v, q.stride(0), k.stride(0), v.stride(0), None, *out, ws)
+        assert lava.lava_poll_status(ws) == 0
+        return out
+
+    one, many = score(1), score(layers)
+    for a, b in zip(one, many):
+        assert bool((b == a).all())
