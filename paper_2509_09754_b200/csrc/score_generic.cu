@@ -429,6 +429,11 @@ lava_status launch_generic(const Geom& g, int n_layers, const char* q, const cha
                            float* scores, float* vbar_out, double* entropy, char* ws,
                            const Workspace& lay, cudaStream_t stream) {
   const int problems = n_layers * g.batch;
+  // What a group may have does not depend on the length: one query head at a time and blocks of 512 keys, as
+  // if with a whole tile of logits, have to fit 200 KB.
+  if (sizeof(float) * ((size_t)g.w_pad * D + kTK * (D + 4) + (size_t)g.w_pad * (kTK + 1) +
+                       (size_t)g.group * a_stride_of(512)) > 200 * 1024)
+    return fail(LAVA_ERR_UNSUPPORTED, "window/group too large for the generic score kernel");
   float* vpart = reinterpret_cast<float*>(ws + lay.off_vpart);
   float2* stats = reinterpret_cast<float2*>(ws + lay.off_stats);
   double2* ent_part = reinterpret_cast<double2*>(ws + lay.off_ent);
@@ -443,8 +448,6 @@ lava_status launch_generic(const Geom& g, int n_layers, const char* q, const cha
                                                 (size_t)g.group * a_stride_of(lay.score_keys));
   } while (score_bytes > kMaxSmem && at_once > 1);
   const int batches = (g.group + at_once - 1) / at_once;
-  if (score_bytes > kMaxSmem)
-    return fail(LAVA_ERR_UNSUPPORTED, "window/group too large for the generic score kernel");
   auto stats_k = stats_partial_kernel<D, BF16>;
   auto score_k = score_kernel<D, BF16>;
   cudaError_t e = cudaFuncSetAttribute(stats_k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_bytes);
