@@ -26,9 +26,10 @@
 // four warps per pass, each with its own TMEM buffer, so that the loads, reductions, pooling and
 // hand-overs of one group run under the exponentials of the other three.
 //
-// Bound: 2 * G * w exponentials per key at 16 per clock and SM (0.53 ms for 32 layers x 32K tokens at
-// 32/8 heads, w 32) and K + V once from HBM plus K once from L2 (0.66 ms); measured 0.98 ms there
-// (1.17 ms with eight consumer warps that alternated the passes, the predecessor of this kernel).
+// Bound: 2 * G * w exponentials per key at 16 per clock and SM (0.48 ms at 1.9 GHz for 32 layers x 32K
+// tokens at 32/8 heads, w 32) and K + V once from HBM plus K once from L2 (0.66 ms); measured 0.98 ms there
+// in short runs and 1.03 in long ones, under the power cap (1.17 ms with eight consumer warps that
+// alternated the passes, the predecessor of this kernel).
 // What is left is mostly pass 2 waiting for a head's statistics.
 //
 // Every wait (mbarrier, head counters, chunk records, lead) is bounded in time; on expiry the
@@ -659,8 +660,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
   } else if (warp >= kFirstConsumer && warp < kFirstConsumer + 8) {
     // ================= pass-1 consumers: softmax statistics ==================================
     // Group 0 takes the even tiles of a head, group 1 the odd ones (not every other tile of the CTA:
-    // the partial sums, and with them the last bits of the scores, depend on the head alone then).  A
-    // thread's row is summed
+    // the partial sums, and with them the last bits of the scores, depend on the head and on the chunk
+    // length then, not on what else the CTA has).  A thread's row is summed
     // relative to a reference exponent taken from the first block of its chunk, not to a running
     // maximum: fp32 sums keep their relative precision at any scale, the reference is moved by
     // whole powers of two (exactly) when the sum grows, and a tile that would overflow, or that
@@ -1123,7 +1124,8 @@ int sm100_first_half(const Geom& g) {
 // 32K tokens 1079 / 981 / 1151, 32 x 8K 292 / 269 / 286, 28 layers x 128K (7 query heads per KV head)
 // 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With fewer than sixteen tiles per CTA in
 // all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
-// 8K (fourteen tiles per CTA) 64 / 66.
+// 8K (fourteen tiles per CTA) 64 / 66.  So a layer's scores alone and in a call of many layers can differ
+// in their last bits (partial sums of 4 or of 8 tiles).
 // Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
 // chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
 // serve sequences of up to 0.83 M tokens with split query groups and 1.66 M without.
@@ -1141,7 +1143,7 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
 
 // Slots pass 1 leads pass 2 by beyond what head completion needs.  4 / 8 / 12 / 16 slots with chunks of
 // eight tiles: 1300 / 1002 / 981 / 1134 us at 32 layers x 32K; shorter leads let pass 2 wait for the
-// statistics, longer ones lose its K tiles from L2 (0 % more DRAM reads than K and V at 8, 15 % at 16).
+// statistics, longer ones lose its K tiles from L2 (0 % more DRAM reads than K and V at 8, 3 % at 12, 15 % at 16).
 int lead_extra_for() {
   const int forced = options().score_lead_tiles;
   return forced >= 0 ? forced : 12;

@@ -1,13 +1,16 @@
-"""Liveness of the two-pass score kernel's static schedule, checked on the CPU.
+"""Liveness of an interleaved static schedule, checked on the CPU: a model of its own.
 
-The persistent kernel deals chunks of tiles round-robin to its CTAs; inside a CTA two consumer
-groups take the tiles of both passes in a fixed interleaved order, and a pass-2 chunk may only
-start once every pass-1 chunk of its head (owned by other CTAs) has been published.  Whether that
-order can always run to the end depends on how far pass 1 leads pass 2 (`lead_tiles`).  This file
-restates the schedule (chunk enumeration, balanced chunk lengths, the lead formula, the order
-rule) and runs it as a set of sequential actors with monotone dependencies; because conditions
-only ever become true, "some actor can always move until all are done" does not depend on timing.
-A schedule that stalls here would end in the kernel as an expired bounded wait.
+It restates the schedule that the two-pass score kernel had before its consumers were split by pass;
+no code of the repository runs it any more.  The present one is modelled in test_score_lead.py and, with
+the limits taken from the source, in test_score_lead_long.py.
+
+Chunks of tiles are dealt round-robin to CTAs; inside a CTA two consumer groups take the tiles of both
+passes in a fixed interleaved order, and a pass-2 chunk may only start once every pass-1 chunk of its
+head (owned by other CTAs) has been published.  Whether that order can always run to the end depends
+on how far pass 1 leads pass 2 (`lead_tiles`).  The schedule (chunk enumeration, balanced chunk lengths,
+the lead formula, the order rule) runs as a set of sequential actors with monotone dependencies; because
+conditions only ever become true, "some actor can always move until all are done" does not depend on
+timing.
 """
 import math
 import random
