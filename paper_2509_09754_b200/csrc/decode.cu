@@ -817,15 +817,17 @@ decode_generic_kernel(const DecodeParams p) {
 inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
 // Which path (the results are the same): the one kernel saves two launches and spreads a chunk over four
 // warps; the listed one streams with less imbalance and folds all heads at once.  Only the longest length
-// is known here, so the line lies at the most rows that the call may hold, and at more heads than a block
-// takes in three rounds.  One / listed, us (heads x average rows, longest): 128 x 128, 1K: 10 / 15;
-// 512 x 128, 2K: 12 / 17; 256 x 512, 8K: 22 / 26; 112 x 1024, 32K: 22 / 26; 300 x 1000, 6K: 44 / 37;
-// 512 x 700, 6K: 47 / 41; 256 x 2048, 32K: 65 / 54; 1024 x 128, 2K: 21 / 19; 1024 x 500, 3K: 69 / 66;
+// is known here, so the line lies at the most rows that the call may hold, lower where the heads alone are
+// more than the blocks that run at once, and at more heads than a block takes in three rounds.  One /
+// listed, us (heads x average rows, longest): 128 x 128, 1K: 10 / 15; 512 x 128, 2K: 12 / 17; 256 x 512,
+// 8K: 22 / 26; 112 x 1024, 32K: 21 / 26; 384 x 300, 6K: 21 / 26; 300 x 1000, 6K: 44 / 37; 512 x 700, 6K:
+// 47 / 41, at d = 64 37 / 30; 256 x 2048, 32K: 64 / 54; 1024 x 128, 2K: 21 / 19; 1024 x 500, 3K: 69 / 65;
 // 2000 x 31, 300: 20 / 17; 2048 x 128, 16K: 43 / 38.
 int chunks_per_head(const Geom& g) { return (g.max_seqlen + kChunkRows - 1) / kChunkRows; }
 bool listed(const Geom& g, int n_layers) {
   const long long heads = (long long)n_layers * g.batch * g.n_kv_heads;
-  return heads * g.max_seqlen >= (3ll << 20) || heads > 6ll * (sm_count() > 0 ? sm_count() : 148) ||
+  const int blocks = 2 * (sm_count() > 0 ? sm_count() : 148);
+  return heads * g.max_seqlen >= (heads > blocks ? 5ll << 19 : 3ll << 20) || heads > 3ll * blocks ||
          chunks_per_head(g) > kMaxChunks;
 }
 // partial results of all heads at most
@@ -857,10 +859,11 @@ lava_status launch_decode(const DecodeParams& p, int n_layers, cudaStream_t stre
   const lava_status rc = check_cuda(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem),
                                     "decode attention attribute");
   if (rc != LAVA_OK) return rc;
-  // two blocks fit an SM (shared memory); fewer when there cannot be a chunk for every warp
+  // two blocks fit an SM (shared memory); fewer when there cannot be a chunk for every block, or for every
+  // warp of the listed path
   const long long slots = (long long)(sm_count() > 0 ? sm_count() : 1) * 2;
-  const long long most = (long long)part_slots(p.g, n_layers);
-  const int grid = (int)std::max<long long>(1, std::min<long long>(slots, (most + kWarps - 1) / kWarps));
+  const long long most = (long long)part_slots(p.g, n_layers), per_block = list ? kWarps : 1;
+  const int grid = (int)std::max<long long>(1, std::min<long long>(slots, (most + per_block - 1) / per_block));
   if (list) {
     launch_in_order(list_chunks_kernel, 1, 1024, 0, stream, p);
     launch_in_order(decode_listed_kernel<D>, grid, kWarps * 32, smem, stream, p);

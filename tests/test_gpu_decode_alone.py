@@ -51,6 +51,7 @@ def test_a_layer_gives_the_same_bits_alone_and_among_others(d, group):
 @pytest.mark.parametrize("layers,kv,rows,here,there", [
     (1, 4, [131072, 700, 0, 4], 131072, 131073),   # as many chunks as the one kernel's fold looks at
     (8, 4, [1500, 3, 129, 640], 90000, 100000),    # rows at most: 2.9 and 3.2 M
+    (75, 4, [600, 3, 129, 1030], 8700, 8800),      # more heads than blocks at once: 2.61 and 2.64 M
 ])
 def test_both_paths_give_the_same_bits(d, layers, kv, rows, here, there):
     group = 4
