@@ -255,8 +255,10 @@ lava_status score_layers_in(const lava_layer_desc* desc, int n_layers, const voi
   if (lay.tensor_path && !options().force_generic) {
     // the single-pass kernel (exponentials kept in tensor memory) is opt-in: the exchange of row
     // statistics between the CTAs outlasts what six exponent buffers can cover, so it is the
-    // slower of the two today
-    if (options().score_kernel == 2 && tmem_supported(g) && tmem_fits(g, tmem_grid(g, n_layers)))
+    // slower of the two today.  Its maps of Q and K have no form for heads or layers that share rows.
+    const bool shared = (g.n_kv_heads > 1 && g.k_sh == 0) ||
+                        (n_layers > 1 && (q_layer_stride == 0 || k_layer_stride == 0));
+    if (options().score_kernel == 2 && !shared && tmem_supported(g) && tmem_fits(g, tmem_grid(g, n_layers)))
       rc = launch_score_tmem(g, n_layers, q_win, k, v_used, q_layer_stride, k_layer_stride,
                              v_layer_stride, vbar_in, scores, vbar_out, entropy,
                              (char*)workspace, lay.off_tmem, st);
