@@ -1094,13 +1094,17 @@ int sm100_first_half(const Geom& g) {
 // can only start once a whole head is through pass 1, and what lies between the passes has to stay in
 // L2 (chunk + lead tiles of 32 KB in 148 CTAs).  Score call in us for 4 / 8 / 16 tiles: 32 layers x
 // 32K tokens 1079 / 981 / 1151, 32 x 8K 292 / 269 / 286, 28 layers x 128K (7 query heads per KV head)
-// 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With fewer than sixteen tiles per CTA in
+// 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With split query groups the two halves share
+// their K rows, so twice the tiles fit in L2 and a boundary is dearer than its wait, unless heads are short:
+// 8 / 12 / 16 tiles, 28 layers x 128K 2850 / 2735 / 2765, x 32K 705 / 684 / 686, x 8K 207 / 212 / 213, x 3K
+// 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455 / 4400, one layer of it 199 / 192 / 203.
+// With fewer than sixteen tiles per CTA in
 // all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
 // 8K (fourteen tiles per CTA) 64 / 66.  So a layer's scores alone and in a call of many layers can differ
-// in their last bits (partial sums of 4 or of 8 tiles).
+// in their last bits (partial sums of 4, of 8 or of 12 tiles).
 // Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
 // chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
-// serve sequences of up to 0.83 M tokens with split query groups and 1.66 M without.
+// serve sequences of up to 1.66 M tokens, 12 with split query groups 1.25 M.
 int chunk_tiles_for(const Geom& g, int n_layers) {
   const int sms = sm_count() > 0 ? sm_count() : 148;  // without a device: the part this is tuned for
   const int split = sm100_first_half(g) ? 1 : 0;
@@ -1108,8 +1112,9 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
   const int least = ceil_div(ceil_div(g.max_seqlen, kTile), most);
   const long long tiles = (long long)n_layers * (g.n_kv_heads << split) * ceil_div((int)g.total_tokens, kTile);
   const int wanted = options().score_chunk_tiles > 0 ? options().score_chunk_tiles
-                     : tiles >= 16LL * sms           ? 8
-                                                     : kMinChunkTiles;
+                     : tiles < 16LL * sms            ? kMinChunkTiles
+                     : split && g.max_seqlen > 8192  ? 12
+                                                     : 8;
   return wanted > least ? wanted : least;
 }
 
