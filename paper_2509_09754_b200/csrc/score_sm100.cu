@@ -27,10 +27,11 @@
 // hand-overs of one group run under the exponentials of the other three.
 //
 // Bound: 2 * G * w exponentials per key at 16 per clock and SM (0.48 ms at 1.9 GHz for 32 layers x 32K
-// tokens at 32/8 heads, w 32) and K + V once from HBM plus K once from L2 (0.66 ms); measured 0.98 ms there
-// in short runs and 1.03 in long ones, under the power cap (1.17 ms with eight consumer warps that
-// alternated the passes, the predecessor of this kernel).
-// What is left is mostly pass 2 waiting for a head's statistics.
+// tokens at 32/8 heads, w 32) and K + V once from HBM plus K once from L2 (0.66 ms); measured 0.90 to 0.92 ms
+// there in short runs (0.99 to 1.01 before the value rows had a producer of their own).  What is left is mostly
+// latency: pass 2 waits for a head's statistics while pass 1 is held back by the lead.  The consumers are
+// bound by issue and dependent latencies rather than by the exponential unit: with half of the pass-2
+// exponentials as polynomials on the FMA pipe the call took 9 % longer.
 //
 // Every wait (mbarrier, head counters, chunk records, lead) is bounded in time; on expiry the
 // kernel sets LAVA_DEV_WAIT_EXPIRED, every role leaves at its next chunk, copies are drained, TMEM
@@ -48,7 +49,8 @@ constexpr int kTile = 128;           // keys per tile
 constexpr int kVWarps = 2;
 constexpr int kFirstConsumer = 4;    // warps 4..11 pass 1, 12..19 pass 2
 constexpr int kPubWarp = 20, kFirstPrep = 21, kPrepWarps = 4, kFirstV = kFirstPrep + kPrepWarps;
-constexpr int kThreads = 32 * (kFirstV + kVWarps);
+constexpr int kVProdWarp = kFirstV + kVWarps;
+constexpr int kThreads = 32 * (kVProdWarp + 1);
 constexpr int kVRows = 32;           // V rows per stage
 constexpr int kRing = 16;            // chunk records a CTA keeps
 constexpr int kMaxLeadChunks = 12;   // pass 1 is never further ahead than this (see Chunk)
@@ -68,18 +70,18 @@ constexpr uint32_t kOffQ1 = 12288;
 constexpr uint32_t kMiscBytes = 19456;
 // K is loaded in blocks of 64 columns (16 KB), each a stage of its own: a block is free again after
 // its own four MMAs, and the shared memory that the query tiles leave divides more evenly between
-// the passes.  V has kV pieces of 32 rows per warp.
+// the passes.  V has kV pieces of 32 rows.
 template <int D>
 struct Smem {
   static constexpr int kBlocks = D / 64;                          // blocks per tile
-  static constexpr int kK1 = D == 128 ? 3 : 4, kK2 = D == 128 ? 3 : 4, kV = D == 128 ? 2 : 4;
+  static constexpr int kK1 = D == 128 ? 3 : 4, kK2 = D == 128 ? 3 : 4, kV = D == 128 ? 4 : 8;
   static constexpr uint32_t kTileBytes = kBlockBytes * kBlocks;   // [128 x D] bf16
   static constexpr uint32_t kVBytes = kVRows * 128 * kBlocks;     // [32 x D] bf16
   static constexpr uint32_t kOffQ2 = kOffQ1 + kTileBytes;
   static constexpr uint32_t kOffK1 = kOffQ2 + kTileBytes;
   static constexpr uint32_t kOffK2 = kOffK1 + kK1 * kBlockBytes;
   static constexpr uint32_t kOffV = kOffK2 + kK2 * kBlockBytes;
-  static constexpr uint32_t kOffMisc = kOffV + kVWarps * kV * kVBytes;
+  static constexpr uint32_t kOffMisc = kOffV + kV * kVBytes;
   static constexpr uint32_t kBytes = kOffMisc + kMiscBytes + 1024;  // + alignment slack
 };
 
@@ -105,10 +107,10 @@ struct Chunk {
   long long score_base;      // first score of the KV head
 };
 
-constexpr int kMaxStages = 4;
+constexpr int kMaxStages = 4, kMaxVStages = 8;
 struct Misc {
   unsigned long long k1_full[kMaxStages], k1_empty[kMaxStages], k2_full[kMaxStages],
-      k2_empty[kMaxStages], v_full[kVWarps][kMaxStages];
+      k2_empty[kMaxStages], v_full[kMaxVStages], v_empty[kMaxVStages];
   unsigned long long q1_full, q1_empty, q2_full, q2_empty;
   unsigned long long s1_full[2], s1_empty[2], s2_full[2], s2_empty[2];
   unsigned long long pub_full[2], pub_empty[2], prep_full[2], prep_empty[2];
@@ -216,7 +218,7 @@ __device__ __noinline__ bool chunk_wait(Misc* m, int ord, unsigned* status) {
   const long long t0 = clock64();
   while (ld_acquire_cta(&m->ck_count) <= ord) {
     if (m->abort_flag) return false;
-    __nanosleep(32);
+    __nanosleep(128);
     if (clock64() - t0 > m->wait_cycles) give_up(m, status);
   }
   return true;
@@ -325,7 +327,10 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
       mbar_init(smem_u32(&m->k1_empty[s]), 1);
       mbar_init(smem_u32(&m->k2_full[s]), 1);
       mbar_init(smem_u32(&m->k2_empty[s]), 1);
-      for (int w = 0; w < kVWarps; ++w) mbar_init(smem_u32(&m->v_full[w][s]), 1);
+    }
+    for (int s = 0; s < kMaxVStages; ++s) {
+      mbar_init(smem_u32(&m->v_full[s]), 1);
+      mbar_init(smem_u32(&m->v_empty[s]), kVWarps);
     }
     mbar_init(smem_u32(&m->q1_full), 1);
     mbar_init(smem_u32(&m->q1_empty), 1);
@@ -477,7 +482,7 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
           if (slot > m->p2_slot + m->lead_slots) {
             const long long t0 = clock64();
             while (slot > m->p2_slot + m->lead_slots && !m->abort_flag) {
-              __nanosleep(32);
+              __nanosleep(128);
               if (clock64() - t0 > m->wait_cycles) give_up(m, p.status);
             }
           }
@@ -574,7 +579,7 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
         while (ld_acquire(&p.counters[ck.head]) < cph ||
                (pw == 0 && want_v && ld_acquire(&p.vcount[ck.rhead]) < want_v)) {
           if (m->abort_flag) break;
-          __nanosleep(32);
+          __nanosleep(128);
           if (clock64() - t0 > m->wait_cycles) give_up(m, p.status);
         }
         ok = !m->abort_flag && wait_for(smem_u32(&m->prep_empty[slot]), phase ^ 1, m, p.status);
@@ -826,103 +831,106 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
         mbar_arrive(smem_u32(&m->prep_empty[j & 1]));
       }
     }
-  } else if (warp >= kFirstV) {
-    // ================= value-norm warps: the V rows of the CTA's pass-1 chunks ===============
+  } else if (warp == kVProdWarp) {
+    // ================= value-norm producer: the V rows of the CTA's pass-1 chunks =============
+    // Pieces of 32 rows; in split mode the two halves of a query group share the head's pieces.  With the
+    // loads issued by the warps that use them (950 cycles a piece beside the 930 of its sums, two pieces
+    // per warp and tile), pass 2 waited half of its time for the value norms.  Score calls in us with
+    // that, and with this warp: 32 layers x 32K 1007 / 920, x 8K 276 / 247, 16 layers x 8K of head
+    // dimension 64 126 / 115.  Four warps for the sums: 914, 244, 117, but 1 to 2 % slower with split groups.
+    if (!p.vbar_in && lane == 0) {
+      const uint64_t drop = policy_evict_first();
+      int st = 0, n = 0;  // n: pieces issued
+      uint32_t st_phase = 0;
+      bool ok = true;
+      for (int j = 0; j < nchunks && ok; ++j) {
+        if (!chunk_ready(m, j, p.status)) break;
+        const Chunk& ck = m->ring[j % kRing];
+        if (ck.ord != j) give_up(m, p.status);  // (cannot happen, see Chunk)
+        const int kvh = SHARED ? ck.kvh * p.v_at.x : ck.kvh, layer = SHARED ? ck.layer * p.v_at.y : ck.layer;
+        const int end = min(ck.n, (ck.tile1 + ck.n1) * kTile), tok0 = ck.tok0;
+        for (int row = ck.tile1 * kTile + ck.half * kVRows; row < end; row += kVRows << p.split) {
+          ok = wait_for(smem_u32(&m->v_empty[st]), st_phase ^ 1, m, p.status);
+          if (!ok) break;
+          const uint32_t bar = smem_u32(&m->v_full[st]);
+          mbar_expect_tx(bar, S::kVBytes);
+          tma_load_5d(base + S::kOffV + st * S::kVBytes, &map_v, 0, tok0 + row, 0, kvh, layer, bar, drop);
+          ++n;
+          if (++st == S::kV) {
+            st = 0;
+            st_phase ^= 1;
+          }
+        }
+      }
+      // copies still in flight land before this CTA gives up its shared memory
+      for (int i = max(0, n - S::kV); i < n; ++i)
+        wait_for(smem_u32(&m->v_full[i % S::kV]), (uint32_t)((i / S::kV) & 1), m, p.status, false);
+    }
+  } else {
+    // ================= value-norm warps ======================================================
     // Row L1 norms through the register-operand tensor path: the sign bits of the packed bf16
     // values are cleared and the rows multiplied by a matrix of ones (mma.sync m16n8k16, fp32
     // accumulate, exact products).  Which of a row's values lands in which k slot does not matter
     // for a sum, so the swizzled piece is read straight through, 16 bytes per lane: lanes 8r..8r+7
     // hold 64 values of row r, which are rows 2r and 2r + 1 of the operand; four rows go in as the
-    // operand's rows 0..7 and four more as its rows 8..15.  Each warp loads its own pieces of 32
-    // rows, kV of them ahead; in split mode the two halves of a query group share the head's rows.
+    // operand's rows 0..7 and four more as its rows 8..15.  A warp takes kReps groups of
+    // eight rows of every piece.
     if (!p.vbar_in) {
-      const int vw = warp - kFirstV, parts = kVWarps << p.split;
+      const int vw = warp - kFirstV;
       const uint32_t ones = 0x3f803f80u;  // bf16 (1, 1)
-      const uint64_t drop = policy_evict_first();
-      const uint32_t stage0 = S::kOffV + vw * S::kV * S::kVBytes;
-      struct Cursor {
-        int j, row, end;  // chunk ordinal, next row of this warp, end of the chunk's rows
-      };
-      auto open = [&](Cursor& cur) {
-        const Chunk& ck = m->ring[cur.j % kRing];
-        if (ck.ord != cur.j) give_up(m, p.status);  // (cannot happen, see Chunk)
-        cur.row = ck.tile1 * kTile + (vw + kVWarps * ck.half) * kVRows;
-        cur.end = min(ck.n, (ck.tile1 + ck.n1) * kTile);
-      };
-      Cursor ld = {-1, 0, 0}, us = {-1, 0, 0};  // loads issued, pieces used
-      int nl = 0, nu = 0;
-      float best = 0.f;
-      while (!__any_sync(0xffffffffu, m->abort_flag)) {
-        // ---- issue loads as far as stages and chunk records allow ------------------------------
-        while (nl - nu < S::kV) {
-          if (ld.row >= ld.end) {
-            const bool more = ld.j + 1 < nchunks && ld_acquire_cta(&m->ck_count) > ld.j + 1;
-            if (!__all_sync(0xffffffffu, more)) break;
-            ++ld.j;
-            open(ld);
-            continue;
-          }
-          const int st = nl % S::kV;
-          if (lane == 0) {
-            const Chunk& ck = m->ring[ld.j % kRing];
-            const uint32_t bar = smem_u32(&m->v_full[vw][st]);
-            mbar_expect_tx(bar, S::kVBytes);
-            tma_load_5d(base + stage0 + st * S::kVBytes, &map_v, 0, ck.tok0 + ld.row, 0,
-                        SHARED ? ck.kvh * p.v_at.x : ck.kvh, SHARED ? ck.layer * p.v_at.y : ck.layer, bar, drop);
-          }
-          ld.row += parts * kVRows;
-          ++nl;
-        }
-        // ---- close the chunks whose pieces have all been used ----------------------------------
-        while (us.row >= us.end) {
-          if (us.j >= 0) {
+      constexpr int kReps = kVRows / 8 / kVWarps;  // groups of eight rows of a piece that a warp takes
+      const uint8_t* mine = gen + S::kOffV + vw * kReps * 1024 + lane * 16;
+      const int row0 = vw * kReps * 8 + (lane >> 3);
+      int st = 0;
+      uint32_t st_phase = 0;
+      bool ok = true;
+      for (int j = 0; j < nchunks; ++j) {
+        if (!__all_sync(0xffffffffu, ok && chunk_ready(m, j, p.status))) break;
+        const Chunk& ck = m->ring[j % kRing];
+        const int rhead = ck.rhead, end = min(ck.n, (ck.tile1 + ck.n1) * kTile);
+        float best = 0.f;
+        for (int row = ck.tile1 * kTile + ck.half * kVRows; row < end; row += kVRows << p.split) {
+          ok = __all_sync(0xffffffffu, wait_for(smem_u32(&m->v_full[st]), st_phase, m, p.status));
+          if (!ok) break;
+          float e0[kReps], e2[kReps];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-            if (lane == 0) {
-              const int head = m->ring[us.j % kRing].rhead;
-              atomicMax(&p.vbar_bits[head], __float_as_uint(best));
-              red_add_release(&p.vcount[head], 1);
+          for (int u = 0; u < kReps; ++u) {
+            float d0[2] = {0.f, 0.f}, d2[2] = {0.f, 0.f};
+#pragma unroll
+            for (int x = 0; x < S::kBlocks; ++x) {
+              const uint8_t* src = mine + st * S::kVBytes + x * (kVRows * 128) + u * 1024;
+              const uint4 lo = *reinterpret_cast<const uint4*>(src);
+              const uint4 hi = *reinterpret_cast<const uint4*>(src + 512);
+              float d1 = 0.f, d3 = 0.f;
+              mma_bf16_16816(d0[x], d1, d2[x], d3, lo.x & 0x7fff7fffu, hi.x & 0x7fff7fffu,
+                             lo.y & 0x7fff7fffu, hi.y & 0x7fff7fffu, ones, ones);
+              mma_bf16_16816(d0[x], d1, d2[x], d3, lo.z & 0x7fff7fffu, hi.z & 0x7fff7fffu,
+                             lo.w & 0x7fff7fffu, hi.w & 0x7fff7fffu, ones, ones);
             }
-            best = 0.f;
+            e0[u] = d0[0] + d0[1];
+            e2[u] = d2[0] + d2[1];
           }
-          if (us.j + 1 >= nchunks || !__all_sync(0xffffffffu, chunk_ready(m, us.j + 1, p.status))) {
-            us.j = nchunks;
-            break;
-          }
-          ++us.j;
-          open(us);
-        }
-        if (us.j >= nchunks) break;
-        if (nl == nu) continue;  // (the record has only just arrived)
-        const int st = nu % S::kV;
-        wait_for(smem_u32(&m->v_full[vw][st]), (uint32_t)((nu / S::kV) & 1), m, p.status);
-        const uint8_t* piece = gen + stage0 + st * S::kVBytes + lane * 16;
-#pragma unroll 2
-        for (int r8 = 0; r8 < kVRows / 8; ++r8) {
-          float d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+          __syncwarp();  // every lane has read the piece
+          if (lane == 0) mbar_arrive(smem_u32(&m->v_empty[st]));
 #pragma unroll
-          for (int x = 0; x < S::kBlocks; ++x) {
-            const uint8_t* src = piece + x * (kVRows * 128) + r8 * 1024;
-            const uint4 lo = *reinterpret_cast<const uint4*>(src);
-            const uint4 hi = *reinterpret_cast<const uint4*>(src + 512);
-            mma_bf16_16816(d0, d1, d2, d3, lo.x & 0x7fff7fffu, hi.x & 0x7fff7fffu,
-                           lo.y & 0x7fff7fffu, hi.y & 0x7fff7fffu, ones, ones);
-            mma_bf16_16816(d0, d1, d2, d3, lo.z & 0x7fff7fffu, hi.z & 0x7fff7fffu,
-                           lo.w & 0x7fff7fffu, hi.w & 0x7fff7fffu, ones, ones);
+          for (int u = 0; u < kReps; ++u) {
+            const float a0 = e0[u] + __shfl_xor_sync(0xffffffffu, e0[u], 4);
+            const float a2 = e2[u] + __shfl_xor_sync(0xffffffffu, e2[u], 4);
+            if (row + row0 + u * 8 < end) best = fmaxf(best, a0);
+            if (row + row0 + u * 8 + 4 < end) best = fmaxf(best, a2);
           }
-          d0 += __shfl_xor_sync(0xffffffffu, d0, 4);
-          d2 += __shfl_xor_sync(0xffffffffu, d2, 4);
-          const int row = us.row + r8 * 8 + (lane >> 3);
-          if (row < us.end) best = fmaxf(best, d0);
-          if (row + 4 < us.end) best = fmaxf(best, d2);
+          if (++st == S::kV) {
+            st = 0;
+            st_phase ^= 1;
+          }
         }
-        __syncwarp();  // every lane has read the stage before it is loaded again
-        us.row += parts * kVRows;
-        ++nu;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        if (lane == 0) {
+          atomicMax(&p.vbar_bits[rhead], __float_as_uint(best));
+          red_add_release(&p.vcount[rhead], 1);
+        }
       }
-      // copies still in flight land before this CTA gives up its shared memory
-      for (; nu < nl; ++nu)
-        wait_for(smem_u32(&m->v_full[vw][nu % S::kV]), (uint32_t)((nu / S::kV) & 1), m, p.status, false);
     }
   }
 
