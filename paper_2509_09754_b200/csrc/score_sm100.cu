@@ -1105,14 +1105,15 @@ int sm100_first_half(const Geom& g) {
 // 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With split query groups the two halves share
 // their K rows, so twice the tiles fit in L2 and a boundary is dearer than its wait, unless heads are short:
 // 8 / 12 / 16 tiles, 28 layers x 128K 2850 / 2735 / 2765, x 32K 705 / 684 / 686, x 8K 207 / 212 / 213, x 3K
-// 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455 / 4400, one layer of it 199 / 192 / 203.
+// 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455 / 4400, one layer of it 199 / 192 / 203; with the
+// value rows' producer 12 / 16 / 20 tiles, 28 layers x 64K 1404 / 1374 / 1394, x 100001 2196 / 2121 / 2164.
 // With fewer than sixteen tiles per CTA in
 // all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
 // 8K (fourteen tiles per CTA) 64 / 66.  So a layer's scores alone and in a call of many layers can differ
-// in their last bits (partial sums of 4, of 8 or of 12 tiles).
+// in their last bits (partial sums of 4, 8, 12 or 16 tiles).
 // Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
 // chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
-// serve sequences of up to 1.66 M tokens, 12 with split query groups 1.25 M.
+// serve sequences of up to 1.66 M tokens, 16 with split query groups the same.
 int chunk_tiles_for(const Geom& g, int n_layers) {
   const int sms = sm_count() > 0 ? sm_count() : 148;  // without a device: the part this is tuned for
   const int split = sm100_first_half(g) ? 1 : 0;
@@ -1121,6 +1122,7 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
   const long long tiles = (long long)n_layers * (g.n_kv_heads << split) * ceil_div((int)g.total_tokens, kTile);
   const int wanted = options().score_chunk_tiles > 0 ? options().score_chunk_tiles
                      : tiles < 16LL * sms            ? kMinChunkTiles
+                     : split && g.max_seqlen > 32768 ? 16
                      : split && g.max_seqlen > 8192  ? 12
                                                      : 8;
   return wanted > least ? wanted : least;

@@ -1,6 +1,6 @@
-"""Chunk length of split query groups on both sides of the length where it changes, against the
-CUDA-core path.  Both sum in fp32 over keys in another order: 32 window queries and at most 9001 keys
-leave a few times 2^-24 * sqrt(9001), 1e-5, in the 2-norm."""
+"""Chunk length of split query groups on both sides of the lengths where it changes, against the
+CUDA-core path.  Both sum in fp32 over keys in another order, in partial sums of at most 2048 keys: a few
+times 2^-24 * sqrt(2048), below 1e-5, in the 2-norm."""
 import pytest
 import torch
 
@@ -9,7 +9,7 @@ import paper_2509_09754_b200 as lava
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("lens", [(8192,), (8193,), (9001, 33, 4099)])
+@pytest.mark.parametrize("lens", [(8192,), (8193,), (9001, 33, 4099), (32768,), (32771,)])
 def test_chunks_of_split_groups(lens):
     layers, hq, hkv, w, d, n = 5, 28, 4, 32, 128, sum(lens)   # more than sixteen tiles for each of 148 CTAs
     g = torch.Generator(device="cuda").manual_seed(3)
