@@ -11,6 +11,8 @@
 // barriers (no spin waits, no global atomics).
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "lava_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -25,6 +27,12 @@ constexpr int kCoarse = kBins / 32;
 constexpr int kCopies = 4;           // interleaved copies of the histogram: one 16-byte cell per bin
 constexpr int kCacheVec = 3584;      // vectors of four keys kept in shared memory: two CTAs fit an SM
 constexpr int kMaskVec = kBins * kCopies * 4;  // mask bytes that fit where the copies were
+// Candidates: keys whose digits so far are those of the threshold.  Their list takes the second half of
+// that space, the masks then the first, and the candidates of all CTAs the space of the histograms.
+constexpr int kListVec = kMaskVec / 2;           // mask bytes beside a list
+constexpr int kMaxMine = kMaskVec / 2 / 8;       // candidates of one CTA
+constexpr int kMaxCandidates = 2 * kBins;        // candidates of all
+constexpr int kCandBits = 7;                     // digit of a pass over candidates
 constexpr int kMaxCluster = 16;
 constexpr int kSoloKeys = 8192;      // keys that one CTA takes before another is worth its barriers
 constexpr int kFullKeys = 65536;     // keys per CTA up to which CTAs are saved to fit one wave
@@ -40,6 +48,10 @@ struct SelectShared {
   uint2 peer_coarse[kMaxCluster][32];
   unsigned peer_fine[kMaxCluster][32];
   uint2 warp_cnt[kWarps];       // (above tau, equal to tau) per warp
+  // cleared when the kernel starts
+  unsigned n_mine;              // candidates of this CTA in its list
+  unsigned lower[2];            // candidates of the CTAs before this one above / equal to tau
+  alignas(16) unsigned cand_bins[3][1 << kCandBits];
 };
 
 // The two halves of a cluster barrier: what a CTA does between them overlaps the wait for its peers.
@@ -88,11 +100,14 @@ __device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 // narrows the digit down in two steps (64 sums, then the 32 bins below one of them) instead of adding
 // up all 2048 bins; the counts of lower-ranked CTAs fall out of the same reads.  Keys are read as
 // 16-byte vectors, the first 14336 of a CTA stay in shared memory and the rest are read again from L2,
-// so two CTAs share an SM whatever the length.  Kept entries are found once per vector as a mask and
-// a warp emits its contiguous part of the keys with votes.  Against two kernels (keys in registers; all
-// passes from memory) with a fixed cluster of 8 or 16, all 2048 bins added up and two barriers per pass:
-// 32 layers of 1K / 8K / 32K: 20.5 / 27 / 99 us before, 11.4 / 19.4 / 39 now; 28 layers of 128K with 4
-// heads: 164 -> 49; 128 ragged problems of up to 32K with 8 heads: 259 -> 87.
+// so two CTAs share an SM whatever the length.  Kept entries are found once per vector as a mask, and a
+// warp emits its contiguous part of the keys, sixteen to a lane.  Once at most 4096 keys share the
+// threshold's digits (some 1.5 % of pooled scores do after the first pass) they are listed in the read that
+// makes the masks, CTAs exchange the lists behind one barrier, and short passes of seven bits over the
+// lists find the rest of the threshold, instead of further passes over all keys with their exchange.
+// Selections in us with three passes over all keys and votes per 32 vectors, and now: 32 layers of 1K / 8K
+// / 32K 11.4 / 18.3 / 42 -> 10.9 / 15.1 / 29, 28 layers of 128K with 4 heads 53 -> 45, 8 ragged sequences x
+// 32 layers 84 -> 67.
 template <bool LIST, bool ADOPT>
 __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* dyn, const Geom& g, int cl,
                                                const float* scores, const long long* layer_budget,
@@ -139,7 +154,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   int* hoff = head_offsets + (size_t)prob * (g.n_kv_heads + 1);
 
   // this CTA's range [c0, c0 + n) and the aligned vectors that hold it; key e is element e + mis
-  const long long per = (m_total + active - 1) / active;
+  const long long per = (unsigned)(m_total + active - 1) / (unsigned)active;
   const long long c0 = min(m_total, per * rank);
   const int n = (int)(min(m_total, c0 + per) - c0);
   const unsigned* keys = reinterpret_cast<const unsigned*>(
@@ -149,66 +164,76 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   const uint4* vecs = reinterpret_cast<const uint4*>(keys - mis);
   const int n_vec = n > 0 ? (mis + n + 3) / 4 : 0;
   auto inside = [&](int e) { return (unsigned)e < (unsigned)n; };
-  auto fetch = [&](int v) {  // only the vectors at the two ends hold anything but this CTA's keys
-    const int e = 4 * v - mis;
-    if (e >= 0 && e + 4 <= n) return vecs[v];
-    uint4 q;
-    q.x = inside(e) ? keys[e] : 0u;
-    q.y = inside(e + 1) ? keys[e + 1] : 0u;
-    q.z = inside(e + 2) ? keys[e + 2] : 0u;
-    q.w = inside(e + 3) ? keys[e + 3] : 0u;
+  // Keys of a vector.  The vectors at the two ends also hold neighbours' keys (in the same 16 bytes as one of
+  // this CTA's): these become 0, the smallest key, and are left out where it counts.
+  auto fetch = [&](int v) {
+    uint4 q = vecs[v];
+    if (v == 0 || v == n_vec - 1) {
+      const int e = 4 * v - mis;
+      q.x = inside(e) ? q.x : 0u;
+      q.y = inside(e + 1) ? q.y : 0u;
+      q.z = inside(e + 2) ? q.z : 0u;
+      q.w = inside(e + 3) ? q.w : 0u;
+    }
     return q;
   };
-  auto again = [&](int v) { return v < kCacheVec ? cache[v] : fetch(v); };
-  // vectors va..vb (and those between) hold nothing but this CTA's keys
-  auto whole = [&](int va, int vb) { return 4 * va - mis >= 0 && 4 * vb + 4 - mis <= n; };
+
+  // Loops over the keys come four vectors wide for large parts, one ahead of its use for small ones: these
+  // run once after kernels that leave nothing of this one in the instruction caches, and the fetches of
+  // wide loops then cost more than their loads save (32 layers of 1K, first run after a flush: 15.1 us
+  // wide, 13.6 narrow; 28 layers of 128K 35 wide, 44 narrow).
+  const bool wide = n_vec > 8 * kThreads;
 
   // ---- radix passes: find tau and the number of ties to take -------------------------------
   unsigned digits = 0, mask = 0;  // key bits found so far, and which these are
   unsigned k_rem = k_sel;         // entries with those bits that are wanted
   unsigned gt_lower = 0, eq_lower = 0;  // entries above / equal to tau in the CTAs before this one
+  int low = 0, bin = 0;                 // key bits left to find; lane that holds the threshold's bin
+  bool listed = false;                  // few enough keys share the digits: they are listed
   if (k_sel > 0) {
     unsigned* my_copy = copies + (lane & (kCopies - 1));
-#pragma unroll
+#pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
       const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
       const unsigned dmask = pass == 2 ? 1023u : 2047u;
       auto tally = [&](unsigned key) {
-        if (pass == 0 || ((key ^ digits) & mask) == 0u)
-          atomicAdd(&my_copy[((key >> shift) & dmask) * kCopies], 1u);
+        if (((key ^ digits) & mask) == 0u) atomicAdd(&my_copy[((key >> shift) & dmask) * kCopies], 1u);
       };
-      for (int v0 = threadIdx.x; v0 < n_vec; v0 += 4 * kThreads) {
-        uint4 q[4];
-        if (whole(v0, v0 + 3 * kThreads)) {
+      auto pick = [&](int v) { return pass > 0 && v < kCacheVec ? cache[v] : fetch(v); };
+      int v = threadIdx.x;
+      if (wide) {
+        auto sweep = [&](auto first) {  // every key counts in the first pass
+          constexpr bool kFirst = decltype(first)::value;
+          const unsigned want = kFirst ? 0u : mask, by = kFirst ? 21 : shift;
+#pragma unroll 1
+          for (; v + 3 * kThreads < n_vec; v += 4 * kThreads) {
+            uint4 q[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int v = v0 + u * kThreads;
-            q[u] = pass > 0 && v < kCacheVec ? cache[v] : vecs[v];
-          }
+            for (int u = 0; u < 4; ++u) q[u] = kFirst ? fetch(v + u * kThreads) : pick(v + u * kThreads);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (pass == 0 && v0 + u * kThreads < kCacheVec) cache[v0 + u * kThreads] = q[u];
-            tally(q[u].x);
-            tally(q[u].y);
-            tally(q[u].z);
-            tally(q[u].w);
-          }
-        } else {
+            for (int u = 0; u < 4; ++u) {
+              if (kFirst && v + u * kThreads < kCacheVec) cache[v + u * kThreads] = q[u];
+              const unsigned key[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int v = v0 + u * kThreads;
-            if (v < n_vec) q[u] = pass == 0 ? fetch(v) : again(v);
+              for (int j = 0; j < 4; ++j)
+                if (kFirst || ((key[j] ^ digits) & want) == 0u)
+                  atomicAdd(&my_copy[(kFirst ? key[j] >> 21 : (key[j] >> by) & dmask) * kCopies], 1u);
+            }
           }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int v = v0 + u * kThreads, e = 4 * v - mis;
-            if (pass == 0 && v < min(n_vec, kCacheVec)) cache[v] = q[u];
-            if (inside(e)) tally(q[u].x);
-            if (inside(e + 1)) tally(q[u].y);
-            if (inside(e + 2)) tally(q[u].z);
-            if (inside(e + 3)) tally(q[u].w);
-          }
-        }
+        };
+        if (pass == 0) sweep(std::true_type{});
+        else sweep(std::false_type{});
+      }
+      uint4 next = v < n_vec ? pick(v) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+      for (; v < n_vec; v += kThreads) {
+        const uint4 q = next;
+        if (v + kThreads < n_vec) next = pick(v + kThreads);
+        if (pass == 0 && v < kCacheVec) cache[v] = q;
+        tally(q.x);
+        tally(q.y);
+        tally(q.z);
+        tally(q.w);
       }
       __syncthreads();
       unsigned* hist = sh.hist[pass & 1];
@@ -218,7 +243,8 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
         const int bin = i * kThreads + threadIdx.x;
         const uint4 q = cells[bin];
         cells[bin] = make_uint4(0u, 0u, 0u, 0u);
-        const unsigned sum = q.x + q.y + q.z + q.w;
+        unsigned sum = q.x + q.y + q.z + q.w;
+        if (bin == 0 && (digits & mask) == 0u) sum -= 4u * n_vec - n;  // the keys that are not this CTA's
         hist[bin] = sum;
         const unsigned all = __reduce_add_sync(0xffffffffu, sum);
         if (lane == 0) coarse[bin >> 5] = all;
@@ -276,70 +302,190 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       }
       digits |= (unsigned)(group * 32 + 31 - src) << shift;
       mask |= dmask << shift;
+      if (pass < 2) {  // the same in every CTA
+        const unsigned most = active == 1 ? f : __reduce_max_sync(0xffffffffu, lane < active ? sh.peer_fine[lane][src] : 0u);
+        if (__shfl_sync(0xffffffffu, f, src) <= kMaxCandidates &&
+            __shfl_sync(0xffffffffu, most, src) <= kMaxMine && per + 3 <= 4 * kListVec) {
+          listed = true;
+          low = shift;
+          bin = src;
+          break;
+        }
+      }
     }
   }
-  if (active > 1) cluster_arrive();  // this CTA reads no peer's shared memory any more
-  const unsigned tau = k_sel > 0 ? digits : 0xffffffffu;
-  const unsigned ties_wanted = k_sel > 0 ? k_rem : 0u;  // >= 1 when k_sel > 0
+  if (active > 1 && !listed) cluster_arrive();  // this CTA reads no peer's shared memory any more
+  unsigned tau = k_sel > 0 ? digits : 0xffffffffu;
 
   // ---- what is kept: every warp takes consecutive vectors; a mask byte per vector (above tau in
   // the low half, equal to it in the high half), and counts that place the warp's first entry ----
-  const int per_warp = (n_vec + kThreads - 1) / kThreads * 32;
+  const int per_warp = ((n_vec + kWarps - 1) / kWarps + 3) & ~3;
   const int v_first = min(n_vec, warp * per_warp), v_last = min(n_vec, v_first + per_warp);
-  auto compare = [&](const uint4& q) {
-    if (max(max(q.x, q.y), max(q.z, q.w)) < tau) return 0u;
-    const unsigned gt = (q.x > tau ? 1u : 0u) | (q.y > tau ? 2u : 0u) | (q.z > tau ? 4u : 0u) |
-                        (q.w > tau ? 8u : 0u);
-    const unsigned eq = (q.x == tau ? 16u : 0u) | (q.y == tau ? 32u : 0u) | (q.z == tau ? 64u : 0u) |
-                        (q.w == tau ? 128u : 0u);
+  const int v_pad = (v_last + 3) & ~3;  // masks are read four at a time
+  // a mask byte: keys whose digits so far are above the threshold's (low half) and equal to them (high half)
+  const unsigned top = k_sel > 0 ? digits >> low : tau;
+  auto compare = [&](const uint4& q, int v) {
+    const unsigned x = q.x >> low, y = q.y >> low, z = q.z >> low, w = q.w >> low;
+    if (max(max(x, y), max(z, w)) < top) return 0u;
+    const unsigned gt = (x > top ? 1u : 0u) | (y > top ? 2u : 0u) | (z > top ? 4u : 0u) | (w > top ? 8u : 0u);
+    unsigned eq = (x == top ? 16u : 0u) | (y == top ? 32u : 0u) | (z == top ? 64u : 0u) | (w == top ? 128u : 0u);
+    if (top == 0u) {
+      const int e = 4 * v - mis;
+      eq &= (inside(e) ? 16u : 0u) | (inside(e + 1) ? 32u : 0u) | (inside(e + 2) ? 64u : 0u) | (inside(e + 3) ? 128u : 0u);
+    }
     return gt | eq;
-  };
-  auto ends = [&](int v) {  // mask bits of the keys of this CTA
-    const int e = 4 * v - mis;
-    return (inside(e) ? 17u : 0u) | (inside(e + 1) ? 34u : 0u) | (inside(e + 2) ? 68u : 0u) |
-           (inside(e + 3) ? 136u : 0u);
   };
   // without a pass nothing has been put into shared memory (and nothing is kept)
   const int n_cached = k_sel > 0 ? kCacheVec : 0;
   auto key_of = [&](int v) { return v < n_cached ? cache[v] : fetch(v); };
+  unsigned* my_key = reinterpret_cast<unsigned*>(dyn + kListVec);  // candidates, and which element each is
+  unsigned* my_at = my_key + kMaxMine;
   unsigned n_gt = 0, n_eq = 0;
-  for (int v0 = v_first + lane; v0 < v_last; v0 += 128) {
-    uint4 q[4];
-    unsigned m[4];
-    if (v0 + 96 < v_last && whole(v0, v0 + 96)) {
+  auto sift = [&](const uint4& q, int v) {
+    unsigned m = v < v_last ? compare(q, v) : 0u;
+    if (listed && m > 15u) {
+      unsigned at = atomicAdd(&sh.n_mine, (unsigned)__popc(m >> 4));
+#pragma unroll 1
+      for (unsigned rest = m >> 4; rest; rest &= rest - 1u, ++at) {
+        const int j = __ffs(rest) - 1;
+        my_key[at] = j == 0 ? q.x : j == 1 ? q.y : j == 2 ? q.z : q.w;
+        my_at[at] = 4u * v + j;
+      }
+      m &= 15u;
+    }
+    if (v < kMaskVec) masks[v] = (unsigned char)m;
+    n_gt += __popc(m & 15u);
+    n_eq += __popc(m >> 4);
+  };
+  {
+    int v = v_first + lane;
+    if (wide) {
+#pragma unroll 1
+      for (; v + 96 < v_last; v += 128) {
+        uint4 q[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) q[u] = v0 + 32 * u < n_cached ? cache[v0 + 32 * u] : vecs[v0 + 32 * u];
+        for (int u = 0; u < 4; ++u) q[u] = key_of(v + 32 * u);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) m[u] = compare(q[u]);
-    } else {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int v = v0 + 32 * u;
-        m[u] = v < v_last ? compare(key_of(v)) & ends(v) : 0u;
+        for (int u = 0; u < 4; ++u) sift(q[u], v + 32 * u);
       }
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (v0 + 32 * u < min(v_last, kMaskVec)) masks[v0 + 32 * u] = (unsigned char)m[u];
-      n_gt += __popc(m[u] & 15u);
-      n_eq += __popc(m[u] >> 4);
+    uint4 next = v < v_last ? key_of(v) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll 1
+    for (; v < v_pad; v += 32) {
+      const uint4 q = next;
+      if (v + 32 < v_last) next = key_of(v + 32);
+      sift(q, v);
     }
   }
   n_gt = __reduce_add_sync(0xffffffffu, n_gt);
   n_eq = __reduce_add_sync(0xffffffffu, n_eq);
   if (lane == 0) sh.warp_cnt[warp] = make_uint2(n_gt, n_eq);
-  __syncthreads();
+  if (!listed) {
+    __syncthreads();
+  } else {
+    // the candidates of all CTAs, in the order of the CTAs
+    const unsigned* all = my_key;
+    unsigned n_all, n_before = 0;
+    if (active > 1) {
+      cluster.sync();  // the lists are complete, and no peer reads the histograms any more
+      unsigned* gathered = &sh.hist[0][0];
+      const unsigned count = lane < active ? sh.peer_fine[lane][bin] : 0u;
+      const unsigned upto = warp_inclusive(count, lane);
+      n_all = __shfl_sync(0xffffffffu, upto, 31);
+      n_before = __shfl_sync(0xffffffffu, upto - count, rank);
+      const unsigned first = __shfl_sync(0xffffffffu, upto - count, warp);
+      const unsigned many = __shfl_sync(0xffffffffu, count, warp);
+      for (unsigned i0 = lane; i0 < many; i0 += 128) {
+        unsigned x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i0 + 32 * u < many) x[u] = peer_load(my_key + i0 + 32 * u, warp);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i0 + 32 * u < many) gathered[first + i0 + 32 * u] = x[u];
+      }
+      all = gathered;
+      cluster_arrive();  // this CTA reads no peer's shared memory any more
+      __syncthreads();
+    } else {
+      __syncthreads();
+      n_all = sh.n_mine;
+    }
+    // the rest of the threshold's bits
+#pragma unroll 1
+    for (int pass = 0, left = low; left > 0; ++pass) {
+      const int shift = max(0, left - kCandBits);
+      const unsigned dmask = (1u << (left - shift)) - 1u;
+      unsigned* bins = sh.cand_bins[pass];
+      for (unsigned i = threadIdx.x; i < n_all; i += kThreads) {
+        const unsigned key = all[i];
+        if (((key ^ tau) & mask) == 0u) atomicAdd(&bins[(key >> shift) & dmask], 1u);
+      }
+      __syncthreads();
+      // lane l has bins 127 - 4l (w) down to 124 - 4l (x): the highest digits first
+      const uint4 c = *reinterpret_cast<const uint4*>(bins + (1 << kCandBits) - 4 - 4 * lane);
+      const unsigned four = c.x + c.y + c.z + c.w;
+      const unsigned before = warp_inclusive(four, lane) - four;
+      const int src = __ffs(__ballot_sync(0xffffffffu, before < k_rem && k_rem <= before + four)) - 1;
+      unsigned digit = (1u << kCandBits) - 1u - 4u * lane, skip = before;
+      if (k_rem > skip + c.w) {
+        skip += c.w;
+        --digit;
+        if (k_rem > skip + c.z) {
+          skip += c.z;
+          --digit;
+          if (k_rem > skip + c.y) {
+            skip += c.y;
+            --digit;
+          }
+        }
+      }
+      k_rem -= __shfl_sync(0xffffffffu, skip, src);
+      tau |= __shfl_sync(0xffffffffu, digit, src) << shift;
+      mask |= dmask << shift;
+      left = shift;
+    }
+    if (active > 1) {
+      if (low > 10) {  // as many barriers as with two passes over all keys
+        cluster_wait();
+        cluster_arrive();
+      }
+      unsigned above = 0, equal = 0;
+      for (unsigned i = threadIdx.x; i < n_before; i += kThreads) {
+        above += all[i] > tau;
+        equal += all[i] == tau;
+      }
+      above = __reduce_add_sync(0xffffffffu, above);
+      equal = __reduce_add_sync(0xffffffffu, equal);
+      if (lane == 0 && above) atomicAdd(&sh.lower[0], above);
+      if (lane == 0 && equal) atomicAdd(&sh.lower[1], equal);
+    }
+    for (unsigned i = threadIdx.x; i < sh.n_mine; i += kThreads) {
+      const unsigned key = my_key[i], at = my_at[i], v = at >> 2;
+      if (key < tau) continue;
+      const bool eq = key == tau;
+      atomicOr(reinterpret_cast<unsigned*>(masks) + (v >> 2), (eq ? 16u : 1u) << (8 * (v & 3u) + (at & 3u)));
+      atomicAdd(eq ? &sh.warp_cnt[v / per_warp].y : &sh.warp_cnt[v / per_warp].x, 1u);
+    }
+    __syncthreads();
+    gt_lower += sh.lower[0];
+    eq_lower = sh.lower[1];
+  }
+  const unsigned ties_wanted = k_sel > 0 ? k_rem : 0u;  // >= 1 when k_sel > 0
   const uint2 wc = lane < warp ? sh.warp_cnt[lane & (kWarps - 1)] : make_uint2(0u, 0u);
   gt_lower += __reduce_add_sync(0xffffffffu, wc.x);
   unsigned tie_run = eq_lower + __reduce_add_sync(0xffffffffu, wc.y);
   unsigned kept_run = gt_lower + min(tie_run, ties_wanted);  // kept entries before this row
 
-  // ---- ordered emit: 32 vectors at a time ----------------------------------------------------
+  // ---- ordered emit: a row of 128 vectors at a time, four to a lane ---------------------------
   int* out = LIST ? io.pos_new + new0
                   : keep_idx + (size_t)layer * g.total_scores + s.score_off + out_base;
-  // first key of head h, counted from this CTA's first (held inside what the arithmetic can take)
+  // first key of head h, counted from this CTA's first (held inside what the arithmetic can take); the first
+  // 32 heads of a list are read at once, a lane each
+  const int list_start = LIST && lane < n_heads ? hoff_old[lane] - lane * win : 0;
   auto head_start = [&](int h) {
-    const long long at = (LIST ? (long long)(hoff_old[h] - h * win) : (long long)h * s.prefix) - c0;
+    const long long at = (LIST ? (long long)(h < 32 ? __shfl_sync(0xffffffffu, list_start, h) : hoff_old[h] - h * win)
+                               : (long long)h * s.prefix) - c0;
     return (int)min((long long)n, at);
   };
   int next_head = n_heads;  // first head that starts at or after this warp's first key
@@ -349,85 +495,91 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
     const int first = max(0, 4 * v_first - mis);
     if (LIST) {
       next_head = 0;
-      for (int h0 = 0; h0 < n_heads; h0 += 32)
-        next_head += __popc(__ballot_sync(0xffffffffu, h0 + lane < n_heads && head_start(h0 + lane) < first));
+      for (int h0 = 0; h0 < n_heads; h0 += 32) {
+        const int at = h0 == 0 ? list_start : (h0 + lane < n_heads ? hoff_old[h0 + lane] - (h0 + lane) * win : 0);
+        next_head += __popc(__ballot_sync(0xffffffffu, h0 + lane < n_heads && at - c0 < first));
+      }
     } else {
-      next_head = (int)((c0 + first + s.prefix - 1) / s.prefix);
+      next_head = (int)((unsigned)(c0 + first + s.prefix - 1) / (unsigned)s.prefix);
       head_begin = (int)((long long)(next_head - 1) * s.prefix - c0);
     }
     if (next_head < n_heads) next_start = head_start(next_head);
   }
-  for (int v0 = v_first; v0 < v_last; v0 += 32) {
-    const int v = v0 + lane, e = 4 * v - mis;
-    unsigned m = 0;
-    if (v < v_last) m = v < kMaskVec ? masks[v] : compare(key_of(v)) & ends(v);
-    const int row0 = 4 * v0 - mis, row1 = min(n, row0 + 128);
+  for (int v0 = v_first; v0 < v_last; v0 += 128) {
+    const int v = v0 + 4 * lane, e0 = 4 * v - mis;
+    unsigned m = 0;  // a byte per vector
+    if (v < v_last) {
+      if (v < kMaskVec) {
+        m = reinterpret_cast<const unsigned*>(masks)[v >> 2];
+      } else {
+        for (int j = 0; j < 4; ++j)
+          if (v + j < v_last) m |= compare(key_of(v + j), v + j) << (8 * j);
+      }
+    }
+    const int row0 = 4 * v0 - mis, row1 = min(min(n, row0 + 512), 4 * v_last - mis);  // this warp's keys
     const bool starts = next_start < row1;  // a head starts in this row
     if (!__any_sync(0xffffffffu, m != 0u) && !starts) continue;
-    unsigned keep = m & 15u;
-    const unsigned eq = m >> 4;
+    unsigned keep = m & 0x0f0f0f0fu, eq = (m >> 4) & 0x0f0f0f0fu;
     if (__any_sync(0xffffffffu, eq != 0u)) {  // ties are taken in order: the first ties_wanted
-      const unsigned c = __popc(eq);
-      const unsigned upto = warp_inclusive(c, lane);
-      unsigned tie = tie_run + upto - c;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if ((eq >> j) & 1u) {
-          if (tie < ties_wanted) keep |= 1u << j;
-          ++tie;
-        }
+      const unsigned c = __popc(eq), upto = warp_inclusive(c, lane);
+      for (unsigned tie = tie_run + upto - c; eq && tie < ties_wanted; ++tie, eq &= eq - 1u) keep |= eq & (0u - eq);
       tie_run += __shfl_sync(0xffffffffu, upto, 31);
     }
-    unsigned vote[4], row_kept = 0, slot = kept_run;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      vote[j] = __ballot_sync(0xffffffffu, (keep >> j) & 1u);
-      row_kept += __popc(vote[j]);
-      slot += __popc(vote[j] & ((1u << lane) - 1u));
-    }
-    if (keep) {
-      if (LIST) {
-        const uint4 q = key_of(v);
-        const unsigned key[4] = {q.x, q.y, q.z, q.w};
+    const unsigned c = __popc(keep), upto = warp_inclusive(c, lane);
+    const unsigned slot0 = kept_run + upto - c, row_kept = __shfl_sync(0xffffffffu, upto, 31);
+    auto value = [&](int e) {
+      return __uint_as_float(e + mis < 4 * n_cached ? reinterpret_cast<const unsigned*>(cache)[e + mis] : keys[e]);
+    };
+    auto position = [&](int e) {
+      int at = e - head_begin;
+      if (starts)
+        while (at >= s.prefix) at -= s.prefix;
+      return at;
+    };
+    // A lane writes what it keeps of its sixteen keys (bit 8 v + j is element 4 v + j of them); where a row
+    // keeps more than a quarter, lanes take the vectors in turn, so that neighbours write side by side.
+    if (!LIST && row_kept <= 128) {
+      unsigned slot = slot0;
+      for (unsigned rest = keep; rest; rest &= rest - 1u, ++slot) {
+        const int bit = __ffs(rest) - 1, e = e0 + (bit >> 3) * 4 + (bit & 7), at = position(e);
+        out[slot] = at;
+        if (ADOPT) {  // the list of what the layer holds from now on
+          io.pos_new[new0 + slot] = at;
+          io.score_new[new0 + slot] = value(e);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int r = 0; r < 4; ++r) {
+        const int from = 8 * r + (lane >> 2), by = 8 * (lane & 3);
+        const unsigned word = __shfl_sync(0xffffffffu, keep, from);
+        unsigned slot = __shfl_sync(0xffffffffu, slot0, from) + __popc(word & ((1u << by) - 1u));
+        const unsigned four = (word >> by) & 15u;
+        const int e = 4 * (v0 + 32 * r + lane) - mis;
+        int at[4];
+        float x[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if ((keep >> j) & 1u) {
-            out[slot] = io.pos_old[old0 + c0 + e + j];
-            io.score_new[new0 + slot] = __uint_as_float(key[j]);
-            io.src_pos[new0 + slot] = (int)c0 + e + j;
+          if ((four >> j) & 1u) {
+            at[j] = LIST ? io.pos_old[old0 + c0 + e + j] : position(e + j);
+            if (LIST || ADOPT) x[j] = value(e + j);
+          }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((four >> j) & 1u) {
+            out[slot] = at[j];
+            if (ADOPT) io.pos_new[new0 + slot] = at[j];
+            if (LIST || ADOPT) io.score_new[new0 + slot] = x[j];
+            if (LIST) io.src_pos[new0 + slot] = (int)c0 + e + j;
             ++slot;
           }
-      } else {
-        const int pos = e - head_begin;
-        unsigned to = slot;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((keep >> j) & 1u) {
-            int at = pos + j;
-            if (starts)
-              while (at >= s.prefix) at -= s.prefix;
-            out[to] = at;
-            if (ADOPT) io.pos_new[new0 + to] = at;
-            ++to;
-          }
-        if (ADOPT) {  // the list of what the layer holds from now on
-          const uint4 q = key_of(v);
-          const unsigned key[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if ((keep >> j) & 1u) io.score_new[new0 + slot++] = __uint_as_float(key[j]);
-        }
       }
     }
     // heads that start in this row record how many kept entries precede them
     while (next_start < row1) {
-      const int at = next_start - row0, l = at >> 2;
-      unsigned before = kept_run;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        before += __popc(vote[j] & ((1u << l) - 1u));
-        if (j < (at & 3)) before += (vote[j] >> l) & 1u;
-      }
+      const int at = next_start - row0, o = at & 15;
+      const unsigned below = (1u << ((o >> 2) * 8 + (o & 3))) - 1u;
+      const unsigned before = __shfl_sync(0xffffffffu, slot0 + __popc(keep & below), at >> 4);
       const int h = head0 + next_head;
       if (lane == 0) hoff[h] = out_base + (int)before + h * win;
       head_begin = next_start;
@@ -462,6 +614,8 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
   __shared__ SelectShared sh;
   for (int i = threadIdx.x; i < kBins; i += kThreads)
     reinterpret_cast<uint4*>(dyn)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (threadIdx.x < 3 << kCandBits) sh.cand_bins[0][threadIdx.x] = 0u;
+  if (threadIdx.x == 0) sh.n_mine = sh.lower[0] = sh.lower[1] = 0u;
   in_stream_order();
   if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
   select_problem<LIST, ADOPT>(sh, dyn, g, blockIdx.x / cg::this_cluster().num_blocks(), scores, layer_budget,
