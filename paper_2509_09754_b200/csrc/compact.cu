@@ -11,6 +11,10 @@
 namespace lava {
 namespace {
 
+// kAhead: rows a thread has on their way.  1 / 2 / 4 (30, 48, 79 registers): 32 layers x 8K 23.8 / 22.2 /
+// 25.4 us, 28 layers x 128K 20.3 / 20.4 / 23.2, ragged batch of 8 49.6 / 47.3 / 46.7 with eight blocks per
+// SM; where there is little to move one is better (see blocks_for).
+template <int kAhead>
 __device__ __forceinline__ void
 compact_head(const Geom& g, int prob, const char* k, const char* v, long long k_ls, long long v_ls,
              const int* keep_idx, const int* head_offsets, const long long* row_off, char* k_out,
@@ -34,29 +38,45 @@ compact_head(const Geom& g, int prob, const char* k, const char* v, long long k_
 
   const int rows_per_iter = blockDim.x / lanes;
   const int sub = threadIdx.x / lanes, c = threadIdx.x - sub * lanes;
-  for (int r = blockIdx.x * rows_per_iter + sub; r < rows; r += blocks_per_head * rows_per_iter) {
-    const int pos = r < kept ? keep[r] : s.prefix + (r - kept);
-    const long long tok = s.tok0 + pos;
-    const uint4 kk = *reinterpret_cast<const uint4*>(kl + tok * g.k_st * es + c * 16);
-    const uint4 vv = *reinterpret_cast<const uint4*>(vl + tok * g.v_st * es + c * 16);
-    const long long dst = (out_row0 + r) * row_bytes + c * 16;
-    *reinterpret_cast<uint4*>(k_out + dst) = kk;
-    *reinterpret_cast<uint4*>(v_out + dst) = vv;
+  const int step = blocks_per_head * rows_per_iter;
+  for (int r0 = blockIdx.x * rows_per_iter + sub; r0 < rows; r0 += kAhead * step) {
+    long long tok[kAhead];
+    uint4 kk[kAhead], vv[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int r = r0 + u * step;
+      if (r < rows) tok[u] = s.tok0 + (r < kept ? keep[r] : s.prefix + (r - kept));
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (r0 + u * step < rows) {
+        kk[u] = *reinterpret_cast<const uint4*>(kl + tok[u] * g.k_st * es + c * 16);
+        vv[u] = *reinterpret_cast<const uint4*>(vl + tok[u] * g.v_st * es + c * 16);
+      }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (r0 + u * step < rows) {
+        const long long dst = (out_row0 + r0 + u * step) * row_bytes + c * 16;
+        *reinterpret_cast<uint4*>(k_out + dst) = kk[u];
+        *reinterpret_cast<uint4*>(v_out + dst) = vv[u];
+      }
   }
 }
 
+template <int kAhead>
 __global__ void __launch_bounds__(256)
 compact_kernel(Geom g, const char* k, const char* v, long long k_ls, long long v_ls,
                const int* keep_idx, const int* head_offsets, const long long* row_off,
                char* k_out, char* v_out, int blocks_per_head) {
   in_stream_order();
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
-  compact_head(g, blockIdx.z, k, v, k_ls, v_ls, keep_idx, head_offsets, row_off, k_out, v_out,
-               blocks_per_head);
+  compact_head<kAhead>(g, blockIdx.z, k, v, k_ls, v_ls, keep_idx, head_offsets, row_off, k_out, v_out,
+                       blocks_per_head);
 }
 
 // Rows of the lower layers move from the old arena to their place in the new one: for
 // (layer, sequence, head) the kept rows named by the source map, then the w window rows.
+template <int kAhead>
 __device__ __forceinline__ void
 move_head(const Geom& g, int prob, const int* src_pos, const int* hoff_old_all, const int* hoff_new_all,
           const long long* roff_old, const long long* roff_new, const char* k_old, const char* v_old,
@@ -74,18 +94,34 @@ move_head(const Geom& g, int prob, const int* src_pos, const int* hoff_old_all, 
   const long long old_window0 = old0 + ho[kvh + 1] - win;
   const int rows_per_iter = blockDim.x / lanes;
   const int sub = threadIdx.x / lanes, c = threadIdx.x - sub * lanes;
-  for (int r = blockIdx.x * rows_per_iter + sub; r < rows; r += blocks_per_head * rows_per_iter) {
-    // entry p of the old list sits in old row p + kvh*win of the sequence's segment
-    const long long from = r < kept ? old0 + src[r] + (long long)kvh * win : old_window0 + (r - kept);
-    const uint4 kk = *reinterpret_cast<const uint4*>(k_old + from * row_bytes + c * 16);
-    const uint4 vv = *reinterpret_cast<const uint4*>(v_old + from * row_bytes + c * 16);
-    const long long dst = (new0 + h0 + r) * row_bytes + c * 16;
-    *reinterpret_cast<uint4*>(k_new + dst) = kk;
-    *reinterpret_cast<uint4*>(v_new + dst) = vv;
+  const int step = blocks_per_head * rows_per_iter;
+  for (int r0 = blockIdx.x * rows_per_iter + sub; r0 < rows; r0 += kAhead * step) {
+    long long from[kAhead];
+    uint4 kk[kAhead], vv[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int r = r0 + u * step;
+      // entry p of the old list sits in old row p + kvh*win of the sequence's segment
+      if (r < rows) from[u] = r < kept ? old0 + src[r] + (long long)kvh * win : old_window0 + (r - kept);
+    }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (r0 + u * step < rows) {
+        kk[u] = *reinterpret_cast<const uint4*>(k_old + from[u] * row_bytes + c * 16);
+        vv[u] = *reinterpret_cast<const uint4*>(v_old + from[u] * row_bytes + c * 16);
+      }
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (r0 + u * step < rows) {
+        const long long dst = (new0 + h0 + r0 + u * step) * row_bytes + c * 16;
+        *reinterpret_cast<uint4*>(k_new + dst) = kk[u];
+        *reinterpret_cast<uint4*>(v_new + dst) = vv[u];
+      }
   }
 }
 
 // A step of the cascade: both kinds of rows side by side, 24 us at 8K (one after the other 6 + 23).
+template <int kAhead>
 __global__ void __launch_bounds__(256)
 cascade_rows_kernel(Geom g, int first, int n_lists, HeldLists io, const int* hoff_new, const char* k_old,
                     const char* v_old, const char* k, const char* v, const int* keep_idx, char* k_new,
@@ -94,20 +130,33 @@ cascade_rows_kernel(Geom g, int first, int n_lists, HeldLists io, const int* hof
   if (batch_has_short_sequence(g)) return;  // the score layout has no room for such a batch
   const int z = first + blockIdx.z, prob = z - g.batch;  // the new layer first: its rows come from further away
   if (prob >= 0)
-    move_head(g, prob, io.src_pos, io.hoff_old, hoff_new, io.row_off_old, io.row_off_new, k_old, v_old, k_new,
-              v_new, blocks_per_head);
+    move_head<kAhead>(g, prob, io.src_pos, io.hoff_old, hoff_new, io.row_off_old, io.row_off_new, k_old, v_old,
+                      k_new, v_new, blocks_per_head);
   else
-    compact_head(g, z, k, v, 0, 0, keep_idx, hoff_new + (size_t)n_lists * (g.n_kv_heads + 1),
-                 io.row_off_new + n_lists, k_new, v_new, blocks_per_head);
+    compact_head<kAhead>(g, z, k, v, 0, 0, keep_idx, hoff_new + (size_t)n_lists * (g.n_kv_heads + 1),
+                         io.row_off_new + n_lists, k_new, v_new, blocks_per_head);
 }
 
 // Row counts live on the device, so the grid is sized for the bandwidth, not the data: enough
-// blocks per (layer, sequence, head) to fill the GPU, each striding over the head's rows.
-int blocks_per_head(const Geom& g, int problems) {
+// blocks per (layer, sequence, head) to fill the GPU, each striding over the head's rows.  Heads keep
+// uneven numbers of rows: more and shorter blocks even that out where there is much to move, and only
+// cost their launches where there is little, so their number goes with the bytes of K that the rows are
+// taken from.  8 / 16 / 32 blocks per SM, in us: 32 layers x 1K (67 MB) 6.4 / 7.9 / 11.6, 16 layers x 8K of
+// head dimension 64 (134 MB) 5.9 / 7.5 / 11.5, 32 x 8K (537 MB) 22.2 / 21.7 / 22.3, 32 x 32K (2.1 GB) 103 /
+// 91 / 88, ragged batch of 8 (8.6 GB) 47 / 46 / 45; half of 32 x 8K kept 125 with eight blocks of one row
+// ahead, 94 now.  At eight blocks per SM one row ahead is the better: the first two 6.2 and 5.4, four layers
+// of 8K 4.0 (two 4.5).
+struct Blocks {
+  int per_head;
+  bool two_ahead;
+};
+Blocks blocks_for(const Geom& g, int problems) {
   const int heads_total = problems * g.n_kv_heads;
   const int sms = sm_count() > 0 ? sm_count() : 1;
-  const int blocks = std::max(1, (sms * 8 + heads_total - 1) / heads_total);
-  return std::min(blocks, std::max(1, (g.max_seqlen + 15) / 16));
+  const long long bytes = (long long)heads_total * g.max_seqlen * g.head_dim * (g.dtype == LAVA_BF16 ? 2 : 4);
+  const int per_sm = (int)std::min(32ll, std::max(8ll, bytes >> 25));
+  const int blocks = std::max(1, (sms * per_sm + heads_total - 1) / heads_total);
+  return {std::min(blocks, std::max(1, (g.max_seqlen + 15) / 16)), per_sm > 8};
 }
 
 }  // namespace
@@ -116,9 +165,10 @@ lava_status launch_compact(const Geom& g, int n_layers, const void* k, const voi
                            long long k_ls, long long v_ls, const int* keep_idx,
                            const int* head_offsets, const long long* row_off, void* k_out,
                            void* v_out, cudaStream_t stream) {
-  const int bph = blocks_per_head(g, n_layers * g.batch);
+  const Blocks blocks = blocks_for(g, n_layers * g.batch);
+  const int bph = blocks.per_head;
   dim3 grid(bph, g.n_kv_heads, n_layers * g.batch);
-  const cudaError_t e = launch_in_order(compact_kernel, grid, 256, 0, stream, g, (const char*)k,
+  const cudaError_t e = launch_in_order(blocks.two_ahead ? compact_kernel<2> : compact_kernel<1>, grid, 256, 0, stream, g, (const char*)k,
                                         (const char*)v, k_ls, v_ls, keep_idx, head_offsets, row_off,
                                         (char*)k_out, (char*)v_out, bph);
   count_launches(1);
@@ -128,12 +178,14 @@ lava_status launch_compact(const Geom& g, int n_layers, const void* k, const voi
 lava_status launch_cascade_rows(const Geom& g, int n_lists, const HeldLists& io, const int* hoff_new,
                                 const char* k_old, const char* v_old, const void* k, const void* v,
                                 const int* keep_idx, char* k_new, char* v_new, cudaStream_t stream) {
-  const int problems = n_lists + g.batch, bph = blocks_per_head(g, problems);
+  const int problems = n_lists + g.batch;
+  const Blocks blocks = blocks_for(g, problems);
+  const int bph = blocks.per_head;
   constexpr int kMost = 65535;  // blocks in the third dimension of a grid
   cudaError_t e = cudaSuccess;
   for (int first = 0; first < problems && e == cudaSuccess; first += kMost) {
     const dim3 grid(bph, g.n_kv_heads, std::min(kMost, problems - first));
-    e = launch_in_order(cascade_rows_kernel, grid, 256, 0, stream, g, first, n_lists, io, hoff_new, k_old, v_old,
+    e = launch_in_order(blocks.two_ahead ? cascade_rows_kernel<2> : cascade_rows_kernel<1>, grid, 256, 0, stream, g, first, n_lists, io, hoff_new, k_old, v_old,
                         (const char*)k, (const char*)v, keep_idx, k_new, v_new, bph);
     count_launches(1);
   }
