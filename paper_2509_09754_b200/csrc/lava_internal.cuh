@@ -96,7 +96,9 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // any memory of the call.  A chain of short kernels otherwise pays about 1 us at each boundary: eviction
 // of 32 layers of 1K 112 -> 102 us, layer-by-layer cascade at 8K (290 launches) 3650 -> 3300.  No kernel
 // asks for its successor earlier than by ending: blocks that wait on a device still half full are not
-// spread evenly (re-budgeting 32K: 91 us; 104 and 110 with the request after and before the wait).
+// spread evenly (re-budgeting 32K: 91 us; 104 and 110 with the request after and before the wait).  The one
+// exception is the selection among the cascade's lists, whose successor has eight blocks and is independent of
+// it (see select_topk_kernel).
 __device__ inline void in_stream_order() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... P, typename... A>
 cudaError_t launch_in_order(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

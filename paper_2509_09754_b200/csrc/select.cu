@@ -609,17 +609,24 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
 template <bool LIST, bool ADOPT>
 __global__ void __launch_bounds__(kThreads, 2)
 select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, int* keep_idx,
-                   int* head_offsets, HeldLists io) {
+                   int* head_offsets, HeldLists io, bool beside) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ SelectShared sh;
   for (int i = threadIdx.x; i < kBins; i += kThreads)
     reinterpret_cast<uint4*>(dyn)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (threadIdx.x < 3 << kCandBits) sh.cand_bins[0][threadIdx.x] = 0u;
   if (threadIdx.x == 0) sh.n_mine = sh.lower[0] = sh.lower[1] = 0u;
-  in_stream_order();
-  if (batch_has_short_sequence(g)) return;  // every CTA of the cluster sees the same lengths
-  select_problem<LIST, ADOPT>(sh, dyn, g, blockIdx.x / cg::this_cluster().num_blocks(), scores, layer_budget,
-                              keep_idx, head_offsets, io);
+  // A step of the cascade selects among the lists of the lower layers and from the new layer; neither needs
+  // the other, and each is bound by latency.  The kernel of the lists lets its successor start once all its
+  // CTAs know that everything before them has ended; the successor (`beside`) need not wait for more, and
+  // ends after the lists, so that what follows it finds both done.  Cascade of 32 layers x 8K: 3182 us with
+  // one after the other, 2867.
+  if (!ADOPT || !beside) in_stream_order();
+  if (LIST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!batch_has_short_sequence(g))  // every CTA of the cluster sees the same lengths
+    select_problem<LIST, ADOPT>(sh, dyn, g, blockIdx.x / cg::this_cluster().num_blocks(), scores, layer_budget,
+                                keep_idx, head_offsets, io);
+  if (ADOPT && beside) in_stream_order();
 }
 
 // CTAs per problem.  A CTA takes 8192 keys before another pays for the barriers (32 problems of 7936
@@ -676,7 +683,7 @@ lava_status launch_select(const Geom& g, int n_layers, const float* scores,
   if (per_head && m_max > kMaxPerHead)
     return fail(LAVA_ERR_UNSUPPORTED, "per-head selection covers up to %d positions per head", kMaxPerHead);
   return launch(select_topk_kernel<false, false>, problems, m_max, "select_topk launch", stream, g, scores,
-                layer_budget, keep_idx, head_offsets, HeldLists());
+                layer_budget, keep_idx, head_offsets, HeldLists(), false);
 }
 
 lava_status launch_select_cascade(const Geom& g, int n_lists, long long max_held, const float* scores,
@@ -686,14 +693,14 @@ lava_status launch_select_cascade(const Geom& g, int n_lists, long long max_held
     return fail(LAVA_ERR_UNSUPPORTED, "a layer may hold at most %d entries per sequence here", kMaxHeld);
   if (n_lists > 0) {
     const lava_status rc = launch(select_topk_kernel<true, false>, n_lists, max_held, "reselect launch", stream,
-                                  g, nullptr, layer_budget, nullptr, head_offsets, io);
+                                  g, nullptr, layer_budget, nullptr, head_offsets, io, false);
     if (rc != LAVA_OK) return rc;
   }
   const long long m_max = (long long)g.n_kv_heads * (g.max_seqlen > g.window ? g.max_seqlen - g.window : 0);
   HeldLists adopt = io;
   adopt.row_off_new += n_lists;
   return launch(select_topk_kernel<false, true>, g.batch, m_max, "cascade selection launch", stream, g, scores,
-                layer_budget + n_lists, keep_idx, head_offsets + (size_t)n_lists * (g.n_kv_heads + 1), adopt);
+                layer_budget + n_lists, keep_idx, head_offsets + (size_t)n_lists * (g.n_kv_heads + 1), adopt, n_lists > 0);
 }
 
 }  // namespace lava
