@@ -214,6 +214,24 @@ class LayerDesc:
                       self.total_tokens, self.k_stride_head, self.k_stride_tok,
                       self.v_stride_head, self.v_stride_tok, self.sm_scale, self.c_hat)
 
+    # The structure of a call is kept until a field is set (1.4 us to fill, of the 8 to 12 that a call
+    # costs on the host; decode layer by layer is one call a layer).  The lengths' address is looked up
+    # every time: a tensor may move its storage.
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        self.__dict__.pop("_call", None)
+
+    def __getstate__(self):  # copies and pickles leave the structure behind
+        return {k: v for k, v in self.__dict__.items() if k != "_call"}
+
+    def _for_call(self) -> _CDesc:
+        c = self.__dict__.get("_call")
+        if c is None:
+            c = self.__dict__["_call"] = self.to_c()
+        elif self.cu_seqlens is not None:
+            c.cu_seqlens = self.cu_seqlens.data_ptr()
+        return c
+
 
 # ----------------------------------------------------------------------------- plumbing
 def lava_version() -> int:
@@ -225,7 +243,7 @@ def lava_last_error() -> str:
 
 
 def lava_workspace_bytes(desc: LayerDesc, n_layers: int = 1) -> int:
-    c = desc.to_c()
+    c = desc._for_call()
     n = int(load_library().lava_workspace_bytes(ctypes.byref(c), n_layers))
     if n == 0:
         raise LavaError(1, lava_last_error())
@@ -247,7 +265,7 @@ def lava_wo_norm(w_o: torch.Tensor, c_hat_out: torch.Tensor, stream=None) -> Non
 # ----------------------------------------------------------------------------- the four steps
 def lava_score_layer(desc: LayerDesc, q_win, k, v, vbar_in, scores, vbar_out, entropy, workspace,
                      stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_score_layer(
         ctypes.byref(c), _ptr(q_win), _ptr(k), _ptr(v), _ptr(vbar_in), _ptr(scores),
         _ptr(vbar_out), _ptr(entropy), _ptr(workspace), workspace.numel() * workspace.element_size(),
@@ -259,7 +277,7 @@ def lava_score_layer_static(desc: LayerDesc, q_win, k, v, vbar_in, scores, vbar_
     """lava_score_layer without a workspace argument, for callers that cannot allocate device
     memory (the scratch is an 8 MiB array inside the library; larger layers are rejected).
     Calls on one device must not overlap on the GPU: keep them on one stream."""
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_score_layer_static(
         ctypes.byref(c), _ptr(q_win), _ptr(k), _ptr(v), _ptr(vbar_in), _ptr(scores),
         _ptr(vbar_out), _ptr(entropy), _ptr(device_status_out), _stream(stream)))
@@ -268,7 +286,7 @@ def lava_score_layer_static(desc: LayerDesc, q_win, k, v, vbar_in, scores, vbar_
 def lava_score_layers(desc: LayerDesc, n_layers, q_win, k, v, q_layer_stride, k_layer_stride,
                       v_layer_stride, vbar_in, scores, vbar_out, entropy, workspace,
                       stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_score_layers(
         ctypes.byref(c), n_layers, _ptr(q_win), _ptr(k), _ptr(v), q_layer_stride, k_layer_stride,
         v_layer_stride, _ptr(vbar_in), _ptr(scores), _ptr(vbar_out), _ptr(entropy),
@@ -291,7 +309,7 @@ def _ws_args(workspace):
 
 def lava_select_topk(desc: LayerDesc, scores, layer_budget, keep_idx, head_offsets,
                      workspace=None, stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     wp, wb = _ws_args(workspace)
     _check(load_library().lava_select_topk(ctypes.byref(c), _ptr(scores), _ptr(layer_budget),
                                            _ptr(keep_idx), _ptr(head_offsets), wp, wb,
@@ -300,7 +318,7 @@ def lava_select_topk(desc: LayerDesc, scores, layer_budget, keep_idx, head_offse
 
 def lava_select_topk_layers(desc: LayerDesc, n_layers, scores, layer_budget, keep_idx,
                             head_offsets, workspace=None, stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     wp, wb = _ws_args(workspace)
     _check(load_library().lava_select_topk_layers(
         ctypes.byref(c), n_layers, _ptr(scores), _ptr(layer_budget), _ptr(keep_idx),
@@ -309,7 +327,7 @@ def lava_select_topk_layers(desc: LayerDesc, n_layers, scores, layer_budget, kee
 
 def lava_compact_kv(desc: LayerDesc, k, v, keep_idx, head_offsets, layer_row_offset, k_out, v_out,
                     stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_compact_kv(
         ctypes.byref(c), _ptr(k), _ptr(v), _ptr(keep_idx), _ptr(head_offsets),
         _ptr(layer_row_offset), _ptr(k_out), _ptr(v_out), _stream(stream)))
@@ -318,7 +336,7 @@ def lava_compact_kv(desc: LayerDesc, k, v, keep_idx, head_offsets, layer_row_off
 def lava_compact_kv_layers(desc: LayerDesc, n_layers, k, v, k_layer_stride, v_layer_stride,
                            keep_idx, head_offsets, layer_row_offset, k_out, v_out,
                            stream=None) -> None:
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_compact_kv_layers(
         ctypes.byref(c), n_layers, _ptr(k), _ptr(v), k_layer_stride, v_layer_stride,
         _ptr(keep_idx), _ptr(head_offsets), _ptr(layer_row_offset), _ptr(k_out), _ptr(v_out),
@@ -391,53 +409,53 @@ def evict_model(plan: EvictionPlan, q_win, k, v, mode: int = LAVA_BUDGET_DYNAMIC
 
 # ----------------------------------------------------------------------------- sharded selection
 def lava_select_shard_bytes(desc: LayerDesc, n_layers: int) -> int:
-    return load_library().lava_select_shard_bytes(ctypes.byref(desc.to_c()), n_layers)
+    return load_library().lava_select_shard_bytes(ctypes.byref(desc._for_call()), n_layers)
 
 
 def lava_select_shard_layout(desc: LayerDesc, n_layers: int):
     """(hist_offset, hist_bytes, ties_offset, ties_bytes) inside the shard state block."""
     v = [ctypes.c_size_t() for _ in range(4)]
-    _check(load_library().lava_select_shard_layout(ctypes.byref(desc.to_c()), n_layers,
+    _check(load_library().lava_select_shard_layout(ctypes.byref(desc._for_call()), n_layers,
                                                    *[ctypes.byref(x) for x in v]))
     return tuple(int(x.value) for x in v)
 
 
 def lava_select_shard_begin(desc, n_layers, total_kv_heads, layer_budget, state, stream=None):
-    _check(load_library().lava_select_shard_begin(ctypes.byref(desc.to_c()), n_layers, total_kv_heads,
+    _check(load_library().lava_select_shard_begin(ctypes.byref(desc._for_call()), n_layers, total_kv_heads,
                                                   _ptr(layer_budget), _ptr(state), state.numel(),
                                                   _stream(stream)))
 
 
 def lava_select_shard_hist(desc, n_layers, scores, pass_, state, stream=None):
-    _check(load_library().lava_select_shard_hist(ctypes.byref(desc.to_c()), n_layers, _ptr(scores),
+    _check(load_library().lava_select_shard_hist(ctypes.byref(desc._for_call()), n_layers, _ptr(scores),
                                                  pass_, _ptr(state), state.numel(), _stream(stream)))
 
 
 def lava_select_shard_step(desc, n_layers, pass_, state, stream=None):
-    _check(load_library().lava_select_shard_step(ctypes.byref(desc.to_c()), n_layers, pass_,
+    _check(load_library().lava_select_shard_step(ctypes.byref(desc._for_call()), n_layers, pass_,
                                                  _ptr(state), state.numel(), _stream(stream)))
 
 
 def lava_select_shard_count(desc, n_layers, scores, state, stream=None):
-    _check(load_library().lava_select_shard_count(ctypes.byref(desc.to_c()), n_layers, _ptr(scores),
+    _check(load_library().lava_select_shard_count(ctypes.byref(desc._for_call()), n_layers, _ptr(scores),
                                                   _ptr(state), state.numel(), _stream(stream)))
 
 
 def lava_select_shard_emit(desc, n_layers, scores, ties_before_rank, keep_idx, head_offsets,
                            layer_row_offset, state, stream=None):
     _check(load_library().lava_select_shard_emit(
-        ctypes.byref(desc.to_c()), n_layers, _ptr(scores), _ptr(ties_before_rank), _ptr(keep_idx),
+        ctypes.byref(desc._for_call()), n_layers, _ptr(scores), _ptr(ties_before_rank), _ptr(keep_idx),
         _ptr(head_offsets), _ptr(layer_row_offset), _ptr(state), state.numel(), _stream(stream)))
 
 
 def lava_decode_workspace_bytes(desc: LayerDesc, n_layers: int = 1) -> int:
-    return load_library().lava_decode_workspace_bytes(ctypes.byref(desc.to_c()), n_layers)
+    return load_library().lava_decode_workspace_bytes(ctypes.byref(desc._for_call()), n_layers)
 
 
 def lava_decode_attention_layers(desc: LayerDesc, n_layers, q, k_packed, v_packed, head_offsets,
                                  layer_row_offset, out, workspace, stream=None) -> None:
     _check(load_library().lava_decode_attention_layers(
-        ctypes.byref(desc.to_c()), n_layers, _ptr(q), _ptr(k_packed), _ptr(v_packed),
+        ctypes.byref(desc._for_call()), n_layers, _ptr(q), _ptr(k_packed), _ptr(v_packed),
         _ptr(head_offsets), _ptr(layer_row_offset), _ptr(out), _ptr(workspace),
         0 if workspace is None else workspace.numel(), _stream(stream)))
 
@@ -445,7 +463,7 @@ def lava_decode_attention_layers(desc: LayerDesc, n_layers, q, k_packed, v_packe
 def lava_decode_attention(desc: LayerDesc, q, k_packed, v_packed, head_offsets, layer_row_offset,
                           out, workspace, stream=None) -> None:
     _check(load_library().lava_decode_attention(
-        ctypes.byref(desc.to_c()), _ptr(q), _ptr(k_packed), _ptr(v_packed), _ptr(head_offsets),
+        ctypes.byref(desc._for_call()), _ptr(q), _ptr(k_packed), _ptr(v_packed), _ptr(head_offsets),
         _ptr(layer_row_offset), _ptr(out), _ptr(workspace),
         0 if workspace is None else workspace.numel(), _stream(stream)))
 
@@ -455,11 +473,11 @@ def lava_layer_output_loss(desc: LayerDesc, q_win, k, v, keep_idx, head_offsets,
     """Lemma 1 loss (p = 1, last token) and Theorem 1 bound of one layer's selection."""
     lib = load_library()
     d_model = int(w_o.shape[1])
-    need = lib.lava_loss_workspace_bytes(ctypes.byref(desc.to_c()), d_model)
+    need = lib.lava_loss_workspace_bytes(ctypes.byref(desc._for_call()), d_model)
     if workspace is None:
         workspace = torch.empty(need, dtype=torch.uint8, device=k.device)
     _check(lib.lava_layer_output_loss(
-        ctypes.byref(desc.to_c()), _ptr(q_win), _ptr(k), _ptr(v), _ptr(keep_idx), _ptr(head_offsets),
+        ctypes.byref(desc._for_call()), _ptr(q_win), _ptr(k), _ptr(v), _ptr(keep_idx), _ptr(head_offsets),
         _ptr(vbar), _ptr(w_o), _dtype_code(w_o), d_model, _ptr(loss_out), _ptr(bound_out),
         _ptr(workspace), workspace.numel(), _stream(stream)))
     return workspace
@@ -467,7 +485,7 @@ def lava_layer_output_loss(desc: LayerDesc, q_win, k, v, keep_idx, head_offsets,
 
 # ----------------------------------------------------------------------------- layer by layer
 def lava_cascade_state_bytes(desc: LayerDesc, n_layers: int, total_rows: int) -> int:
-    n = load_library().lava_cascade_state_bytes(ctypes.byref(desc.to_c()), n_layers, int(total_rows))
+    n = load_library().lava_cascade_state_bytes(ctypes.byref(desc._for_call()), n_layers, int(total_rows))
     if n == 0:
         raise LavaError(1, "invalid layer descriptor, layer count or row count")
     return n
@@ -553,7 +571,7 @@ def lava_launch_count() -> int:
 
 def lava_score_path(desc: LayerDesc) -> int:
     """0 = CUDA-core path, 1 = tensor-core path, 2 = tensor-core path with split query groups."""
-    c = desc.to_c()
+    c = desc._for_call()
     r = int(load_library().lava_score_path(ctypes.byref(c)))
     if r < 0:
         raise LavaError(1, load_library().lava_last_error().decode("utf-8", "replace"))
@@ -561,7 +579,7 @@ def lava_score_path(desc: LayerDesc) -> int:
 
 
 def lava_host_arena_bytes(desc: LayerDesc, n_layers: int, total_budget_rows: int) -> int:
-    c = desc.to_c()
+    c = desc._for_call()
     n = int(load_library().lava_host_arena_bytes(ctypes.byref(c), n_layers, total_budget_rows))
     if n == 0:
         raise LavaError(1, lava_last_error())
@@ -573,7 +591,7 @@ def lava_evict_model_host(desc: LayerDesc, n_layers, q_win, k, v, seq_lens, tota
     """All tensor arguments except ``arena`` are HOST tensors (pinned for asynchronous copies);
     seq_lens int32 [batch], total_budget int64 [batch].  Results are complete after the stream
     has been synchronised."""
-    c = desc.to_c()
+    c = desc._for_call()
     _check(load_library().lava_evict_model_host(
         ctypes.byref(c), n_layers, _ptr(q_win), _ptr(k), _ptr(v), _ptr(seq_lens),
         _ptr(total_budget), mode, _ptr(layer_budget), _ptr(head_offsets), _ptr(k_out), _ptr(v_out),
