@@ -1107,9 +1107,10 @@ int sm100_first_half(const Geom& g) {
 // 8 / 12 / 16 tiles, 28 layers x 128K 2850 / 2735 / 2765, x 32K 705 / 684 / 686, x 8K 207 / 212 / 213, x 3K
 // 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455 / 4400, one layer of it 199 / 192 / 203; with the
 // value rows' producer 12 / 16 / 20 tiles, 28 layers x 64K 1404 / 1374 / 1394, x 100001 2196 / 2121 / 2164.
-// With fewer than sixteen tiles per CTA in
-// all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; four layers of
-// 8K (fourteen tiles per CTA) 64 / 66.  So a layer's scores alone and in a call of many layers can differ
+// With fewer than twelve tiles per CTA in
+// all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; 4 against 8 tiles at
+// 10.4 tiles per CTA 51.6 / 56.4 (three layers of 8K) and 57 / 61 (24 of 1K), at 12.1 61.2 / 59.0 (28 of 1K),
+// at 13.8 60.3 / 57.1 (four of 8K) and 63.4 / 59.1 (32 of 1K).  So a layer's scores alone and in a call of many layers can differ
 // in their last bits (partial sums of 4, 8, 12 or 16 tiles).
 // Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
 // chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
@@ -1121,7 +1122,7 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
   const int least = ceil_div(ceil_div(g.max_seqlen, kTile), most);
   const long long tiles = (long long)n_layers * (g.n_kv_heads << split) * ceil_div((int)g.total_tokens, kTile);
   const int wanted = options().score_chunk_tiles > 0 ? options().score_chunk_tiles
-                     : tiles < 16LL * sms            ? kMinChunkTiles
+                     : tiles < 12LL * sms            ? kMinChunkTiles
                      : split && g.max_seqlen > 32768 ? 16
                      : split && g.max_seqlen > 8192  ? 12
                                                      : 8;
