@@ -108,8 +108,8 @@ __device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 // Selections in us with three passes over all keys and votes per 32 vectors, and now: 32 layers of 1K / 8K
 // / 32K 11.4 / 18.3 / 42 -> 10.9 / 15.1 / 29, 28 layers of 128K with 4 heads 53 -> 45, 8 ragged sequences x
 // 32 layers 84 -> 67.
-// Where clusters are small and an eighth or more is kept it is the slower one, by less than a fetch of the
-// wide loops in a whole pass: 28 layers of 4000 / 8000 tokens, 4 heads, 13.4 / 14.6 -> 16.0 / 16.5.
+// Slower where clusters are small and an eighth or more is kept: 28 layers of 4000 / 8000 tokens with 4
+// heads 13.4 / 14.6 -> 16.0 / 16.5 (rows emitted by either rule, narrow or unrolled: the same).
 template <bool LIST, bool ADOPT>
 __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* dyn, const Geom& g, int cl,
                                                const float* scores, const long long* layer_budget,
