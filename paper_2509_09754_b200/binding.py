@@ -214,22 +214,36 @@ class LayerDesc:
                       self.total_tokens, self.k_stride_head, self.k_stride_tok,
                       self.v_stride_head, self.v_stride_tok, self.sm_scale, self.c_hat)
 
-    # The structure of a call is kept until a field is set (1.4 us to fill, of the 8 to 12 that a call
-    # costs on the host; decode layer by layer is one call a layer).  The lengths' address is looked up
-    # every time: a tensor may move its storage.
+    # The structure of a call is kept until a field is set (1.4 us to fill, 0.2 to look up, of the 8 to 12
+    # that a call costs on the host; decode layer by layer is one call a layer).  Other threads may set fields
+    # or be inside a call meanwhile: every set leaves a new mark, a structure is stored with the mark that was
+    # read before its fields were, and one that has been handed out is never written again.  The lengths'
+    # address is looked up every time: a tensor may move its storage.
+    __slots__ = ("_mark", "_kept", "__dict__", "__weakref__")  # beside the fields, so not in vars(desc)
+
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
-        self.__dict__.pop("_call", None)
+        object.__setattr__(self, "_mark", object())
 
-    def __getstate__(self):  # copies and pickles leave the structure behind
-        return {k: v for k, v in self.__dict__.items() if k != "_call"}
+    def __delattr__(self, name):
+        object.__delattr__(self, name)
+        object.__setattr__(self, "_mark", object())
+
+    def __getstate__(self):  # copies and pickles hold the fields
+        return dict(self.__dict__)
+
+    def __setstate__(self, state):
+        self.__dict__.update(state)
+        object.__setattr__(self, "_mark", object())
 
     def _for_call(self) -> _CDesc:
-        c = self.__dict__.get("_call")
-        if c is None:
-            c = self.__dict__["_call"] = self.to_c()
-        elif self.cu_seqlens is not None:
-            c.cu_seqlens = self.cu_seqlens.data_ptr()
+        mark, kept = self._mark, getattr(self, "_kept", None)
+        lens = self.cu_seqlens
+        at = None if lens is None else lens.data_ptr()
+        if kept is not None and kept[0] is mark and kept[1] == at:
+            return kept[2]
+        c = self.to_c()
+        object.__setattr__(self, "_kept", (mark, c.cu_seqlens, c))
         return c
 
 
