@@ -166,17 +166,17 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   const uint4* vecs = reinterpret_cast<const uint4*>(keys - mis);
   const int n_vec = n > 0 ? (mis + n + 3) / 4 : 0;
   auto inside = [&](int e) { return (unsigned)e < (unsigned)n; };
-  // Keys of a vector.  The vectors at the two ends also hold neighbours' keys (in the same 16 bytes as one of
-  // this CTA's): these become 0, the smallest key, and are left out where it counts.
+  // Keys of a vector.  The vectors at the two ends may be partly outside this CTA's part, and outside the
+  // array: these go key by key, and what is not this CTA's becomes 0, the smallest key, left out where it counts.
+  const int ragged0 = mis ? 0 : -1, ragged1 = (mis + n) & 3 ? n_vec - 1 : -1;
   auto fetch = [&](int v) {
-    uint4 q = vecs[v];
-    if (v == 0 || v == n_vec - 1) {
-      const int e = 4 * v - mis;
-      q.x = inside(e) ? q.x : 0u;
-      q.y = inside(e + 1) ? q.y : 0u;
-      q.z = inside(e + 2) ? q.z : 0u;
-      q.w = inside(e + 3) ? q.w : 0u;
-    }
+    if (v != ragged0 && v != ragged1) return vecs[v];
+    const int e = 4 * v - mis;
+    uint4 q;
+    q.x = inside(e) ? keys[e] : 0u;
+    q.y = inside(e + 1) ? keys[e + 1] : 0u;
+    q.z = inside(e + 2) ? keys[e + 2] : 0u;
+    q.w = inside(e + 3) ? keys[e + 3] : 0u;
     return q;
   };
 
