@@ -924,6 +924,7 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
             st_phase ^= 1;
           }
         }
+        if (!ok) break;  // without all of its rows the chunk does not count as done
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
         if (lane == 0) {
