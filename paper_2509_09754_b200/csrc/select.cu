@@ -58,6 +58,8 @@ struct SelectShared {
 __device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 
+__device__ inline void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // Address of the same shared-memory location in CTA `rank` of the cluster, and loads through it.
 __device__ inline uint32_t peer_addr(const unsigned* p, int rank) {
   uint32_t a;
@@ -623,8 +625,15 @@ select_topk_kernel(Geom g, const float* scores, const long long* layer_budget, i
   // CTAs know that everything before them has ended; the successor (`beside`) need not wait for more, and
   // ends after the lists, so that what follows it finds both done.  Cascade of 32 layers x 8K: 3182 us with
   // one after the other, 2867.
+  // The successor has no wait of its own in front of what earlier kernels wrote (scores, budgets, offsets,
+  // lengths): that is performed when the wait here has ended, and a fence on either side of the launch orders
+  // it before the successor's reads, which then find no older copies in a cache of their multiprocessor.
   if (!ADOPT || !beside) in_stream_order();
-  if (LIST) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (LIST) {
+    fence_gpu();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
+  if (ADOPT && beside) fence_gpu();
   if (!batch_has_short_sequence(g))  // every CTA of the cluster sees the same lengths
     select_problem<LIST, ADOPT>(sh, dyn, g, blockIdx.x / cg::this_cluster().num_blocks(), scores, layer_budget,
                                 keep_idx, head_offsets, io);
