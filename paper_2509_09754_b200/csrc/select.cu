@@ -1,8 +1,9 @@
 // Layer-wide top-k over the flat score array of one (layer, sequence) (Algorithm 1, Evict).
 //
 // Exact radix select on the fp32 bit patterns (scores are >= 0, so the unsigned patterns order
-// like the values): three digit passes (11, 11, 10 bits) find the k-th largest pattern tau and
-// the number of entries equal to tau that still fit; an ordered compaction then emits, head
+// like the values): digit passes (11, 11, 10 bits), of which a list of the few keys that share the
+// digits so far replaces the last ones, find the k-th largest pattern tau and the number of
+// entries equal to tau that still fit; an ordered compaction then emits, head
 // after head and in ascending position, every entry above tau plus the first ties in flat
 // index order.  Equal scores therefore resolve to the lower flat index, deterministically.
 //
@@ -30,8 +31,9 @@ constexpr int kMaskVec = kBins * kCopies * 4;  // mask bytes that fit where the 
 // Candidates: keys whose digits so far are those of the threshold.  Their list takes the second half of
 // that space, the masks then the first, and the candidates of all CTAs the space of the histograms.
 constexpr int kListVec = kMaskVec / 2;           // mask bytes beside a list
-constexpr int kMaxMine = kMaskVec / 2 / 8;       // candidates of one CTA
-constexpr int kMaxCandidates = 2 * kBins;        // candidates of all
+constexpr int kMaxCandidates = kMaskVec / 2 / 8; // candidates of all CTAs, which one of them may have
+constexpr int kFewCandidates = 256;              // listed whatever their share of the keys
+constexpr int kKeysPerCandidate = 32;            // more than that: up to one key in 32
 constexpr int kCandBits = 7;                     // digit of a pass over candidates
 constexpr int kMaxCluster = 16;
 constexpr int kSoloKeys = 8192;      // keys that one CTA takes before another is worth its barriers
@@ -57,6 +59,13 @@ struct SelectShared {
 // The two halves of a cluster barrier: what a CTA does between them overlaps the wait for its peers.
 __device__ inline void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ inline void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// Sixteen bytes from global to shared memory, and the wait for all of this thread's.
+__device__ inline void copy_async(uint4* dst, const uint4* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ inline void copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 __device__ inline void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
@@ -103,15 +112,18 @@ __device__ inline unsigned warp_inclusive(unsigned x, int lane) {
 // up all 2048 bins; the counts of lower-ranked CTAs fall out of the same reads.  Keys are read as
 // 16-byte vectors, the first 14336 of a CTA stay in shared memory and the rest are read again from L2,
 // so two CTAs share an SM whatever the length.  Kept entries are found once per vector as a mask, and a
-// warp emits its contiguous part of the keys, sixteen to a lane.  Once at most 4096 keys share the
-// threshold's digits (some 1.5 % of pooled scores do after the first pass) they are listed in the read that
-// makes the masks, CTAs exchange the lists behind one barrier, and short passes of seven bits over the
-// lists find the rest of the threshold, instead of further passes over all keys with their exchange.
-// Selections in us with three passes over all keys and votes per 32 vectors, and now: 32 layers of 1K / 8K
-// / 32K 11.4 / 18.3 / 42 -> 10.9 / 15.1 / 29, 28 layers of 128K with 4 heads 53 -> 45, 8 ragged sequences x
-// 32 layers 84 -> 67.
-// Slower where clusters are small and an eighth or more is kept: 28 layers of 4000 / 8000 tokens with 4
-// heads 13.4 / 14.6 -> 16.0 / 16.5 (rows emitted by either rule, narrow or unrolled: the same).
+// warp emits its contiguous part of the keys, sixteen to a lane.  Once few keys share the threshold's digits
+// (some 1.5 % of pooled scores do after the first pass) they are listed in the read that makes the masks, CTAs
+// exchange the lists behind one barrier, and short passes of seven bits over the lists find the rest of the
+// threshold, instead of further passes over all keys with their exchange.
+// A list costs by its length, a digit pass by the keys, so the list is taken up to one key in 32 (256 in any
+// case, 2048 at most): with lists of up to 4096, 4000 tokens x 8 heads cost 16.6 us where half is kept and 15.4
+// at a quarter, now 14.3 and 14.4 (14.2 with three digit passes throughout); 8 ragged sequences x 32 layers at
+// 2 % 71 with lists, 75 up to 512 only.  One in 24 and one in 48 measured the same.
+// Selections in us with three passes over all keys and votes per 32 vectors, and now: 28 layers of 1K x 16
+// heads 14.2 to 15 -> 12.8 to 14.3, 8K x 8 heads 18.3 to 20 -> 16 to 18.3, 32K x 8 36.5 to 43.6 -> 32 to
+// 38, 128K x 4 58 to 73 -> 50 to 61.5 (3 % to half of the entries kept).  4000 tokens x 4 or 8 heads where an
+// eighth or more is kept: 13.7 to 14.2 -> 13.8 to 14.4 in a run of selections, the same after other kernels.
 template <bool LIST, bool ADOPT>
 __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* dyn, const Geom& g, int cl,
                                                const float* scores, const long long* layer_budget,
@@ -185,7 +197,9 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   // Loops over the keys come four vectors wide for large parts, one ahead of its use for small ones: these
   // run once after kernels that leave nothing of this one in the instruction caches, and the fetches of
   // wide loops then cost more than their loads save (32 layers of 1K, first run after a flush: 15.1 us
-  // wide, 13.6 narrow; 28 layers of 128K 35 wide, 44 narrow).
+  // wide, 13.6 narrow; 28 layers of 128K 35 wide, 44 narrow).  The keys of a small part are all on their way
+  // to shared memory at once: one ahead, each of a thread's four or more fetches waited for the one before it
+  // (28 layers of 4000 tokens after a flush 16.2, now 14.3).
   const bool wide = n_vec > 8 * kThreads;
 
   // ---- radix passes: find tau and the number of ties to take -------------------------------
@@ -194,8 +208,18 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   unsigned gt_lower = 0, eq_lower = 0;  // entries above / equal to tau in the CTAs before this one
   int low = 0, bin = 0;                 // key bits left to find; lane that holds the threshold's bin
   bool listed = false;                  // few enough keys share the digits: they are listed
+  const unsigned share = max((unsigned)kFewCandidates, (unsigned)m_total / kKeysPerCandidate);
+  const unsigned list_up_to = per + 3 > 4 * kListVec ? 0u : min((unsigned)kMaxCandidates, share);
   if (k_sel > 0) {
     unsigned* my_copy = copies + (lane & (kCopies - 1));
+    if (!wide) {
+#pragma unroll 1
+      for (int v = threadIdx.x; v < min(n_vec, kCacheVec); v += kThreads) {
+        if (v == ragged0 || v == ragged1) cache[v] = fetch(v);
+        else copy_async(cache + v, vecs + v);
+      }
+      copies_landed();  // until the next barrier a thread reads its own
+    }
 #pragma unroll 1
     for (int pass = 0; pass < 3; ++pass) {
       const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
@@ -203,7 +227,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       auto tally = [&](unsigned key) {
         if (((key ^ digits) & mask) == 0u) atomicAdd(&my_copy[((key >> shift) & dmask) * kCopies], 1u);
       };
-      auto pick = [&](int v) { return pass > 0 && v < kCacheVec ? cache[v] : fetch(v); };
+      auto pick = [&](int v) { return (pass > 0 || !wide) && v < kCacheVec ? cache[v] : fetch(v); };
       int v = threadIdx.x;
       if (wide) {
         auto sweep = [&](auto first) {  // every key counts in the first pass
@@ -307,9 +331,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       digits |= (unsigned)(group * 32 + 31 - src) << shift;
       mask |= dmask << shift;
       if (pass < 2) {  // the same in every CTA
-        const unsigned most = active == 1 ? f : __reduce_max_sync(0xffffffffu, lane < active ? sh.peer_fine[lane][src] : 0u);
-        if (__shfl_sync(0xffffffffu, f, src) <= kMaxCandidates &&
-            __shfl_sync(0xffffffffu, most, src) <= kMaxMine && per + 3 <= 4 * kListVec) {
+        if (__shfl_sync(0xffffffffu, f, src) <= list_up_to) {
           listed = true;
           low = shift;
           bin = src;
@@ -335,7 +357,8 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
     unsigned eq = (x == top ? 16u : 0u) | (y == top ? 32u : 0u) | (z == top ? 64u : 0u) | (w == top ? 128u : 0u);
     if (top == 0u) {
       const int e = 4 * v - mis;
-      eq &= (inside(e) ? 16u : 0u) | (inside(e + 1) ? 32u : 0u) | (inside(e + 2) ? 64u : 0u) | (inside(e + 3) ? 128u : 0u);
+      eq &= (inside(e) ? 16u : 0u) | (inside(e + 1) ? 32u : 0u) | (inside(e + 2) ? 64u : 0u) |
+            (inside(e + 3) ? 128u : 0u);
     }
     return gt | eq;
   };
@@ -343,11 +366,11 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   const int n_cached = k_sel > 0 ? kCacheVec : 0;
   auto key_of = [&](int v) { return v < n_cached ? cache[v] : fetch(v); };
   unsigned* my_key = reinterpret_cast<unsigned*>(dyn + kListVec);  // candidates, and which element each is
-  unsigned* my_at = my_key + kMaxMine;
+  unsigned* my_at = my_key + kMaxCandidates;
   unsigned n_gt = 0, n_eq = 0;
-  auto sift = [&](const uint4& q, int v) {
+  auto sift = [&](const uint4& q, int v, auto may_list) {
     unsigned m = v < v_last ? compare(q, v) : 0u;
-    if (listed && m > 15u) {
+    if (decltype(may_list)::value && listed && m > 15u) {
       unsigned at = atomicAdd(&sh.n_mine, (unsigned)__popc(m >> 4));
 #pragma unroll 1
       for (unsigned rest = m >> 4; rest; rest &= rest - 1u, ++at) {
@@ -364,21 +387,25 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   {
     int v = v_first + lane;
     if (wide) {
+      auto sweep = [&](auto may_list) {
 #pragma unroll 1
-      for (; v + 96 < v_last; v += 128) {
-        uint4 q[4];
+        for (; v + 96 < v_last; v += 128) {
+          uint4 q[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = key_of(v + 32 * u);
+          for (int u = 0; u < 4; ++u) q[u] = key_of(v + 32 * u);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) sift(q[u], v + 32 * u);
-      }
+          for (int u = 0; u < 4; ++u) sift(q[u], v + 32 * u, may_list);
+        }
+      };
+      if (listed) sweep(std::true_type{});
+      else sweep(std::false_type{});
     }
     uint4 next = v < v_last ? key_of(v) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll 1
     for (; v < v_pad; v += 32) {
       const uint4 q = next;
       if (v + 32 < v_last) next = key_of(v + 32);
-      sift(q, v);
+      sift(q, v, std::true_type{});
     }
   }
   n_gt = __reduce_add_sync(0xffffffffu, n_gt);
@@ -450,7 +477,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       left = shift;
     }
     if (active > 1) {
-      if (low > 10) {  // as many barriers as with two passes over all keys
+      if (low > 10 && active < csize) {  // as many barriers as the CTAs without keys take part in
         cluster_wait();
         cluster_arrive();
       }
@@ -540,9 +567,9 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
         while (at >= s.prefix) at -= s.prefix;
       return at;
     };
-    // A lane writes what it keeps of its sixteen keys (bit 8 v + j is element 4 v + j of them); where a row
-    // keeps more than a quarter, lanes take the vectors in turn, so that neighbours write side by side.
-    if (!LIST && row_kept <= 128) {
+    // A lane writes what it keeps of its sixteen keys (bit 8 v + j is element 4 v + j of them); where more than
+    // a quarter of a row is kept, lanes take the vectors in turn, so that neighbours write side by side.
+    if (!LIST && 4 * (int)row_kept <= row1 - row0) {
       unsigned slot = slot0;
       for (unsigned rest = keep; rest; rest &= rest - 1u, ++slot) {
         const int bit = __ffs(rest) - 1, e = e0 + (bit >> 3) * 4 + (bit & 7), at = position(e);
@@ -554,7 +581,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       }
     } else {
 #pragma unroll 1
-      for (int r = 0; r < 4; ++r) {
+      for (int r = 0; r < 4 && v0 + 32 * r < v_last; ++r) {
         const int from = 8 * r + (lane >> 2), by = 8 * (lane & 3);
         const unsigned word = __shfl_sync(0xffffffffu, keep, from);
         unsigned slot = __shfl_sync(0xffffffffu, slot0, from) + __popc(word & ((1u << by) - 1u));
@@ -711,7 +738,8 @@ lava_status launch_select_cascade(const Geom& g, int n_lists, long long max_held
   HeldLists adopt = io;
   adopt.row_off_new += n_lists;
   return launch(select_topk_kernel<false, true>, g.batch, m_max, "cascade selection launch", stream, g, scores,
-                layer_budget + n_lists, keep_idx, head_offsets + (size_t)n_lists * (g.n_kv_heads + 1), adopt, n_lists > 0);
+                layer_budget + n_lists, keep_idx, head_offsets + (size_t)n_lists * (g.n_kv_heads + 1), adopt,
+                n_lists > 0);
 }
 
 }  // namespace lava
