@@ -11,7 +11,8 @@
 namespace lava {
 namespace {
 
-// kAhead: rows a thread has on their way.  1 / 2 / 4 (30, 48, 79 registers): 32 layers x 8K 23.8 / 22.2 /
+// kAhead: rows a thread has on their way.  1 / 2 / 4 (20 and 32 registers for 1 and 2, in the cascade's kernel
+// 30 and 48): 32 layers x 8K 23.8 / 22.2 /
 // 25.4 us, 28 layers x 128K 20.3 / 20.4 / 23.2, ragged batch of 8 49.6 / 47.3 / 46.7 with eight blocks per
 // SM; where there is little to move one is better (see blocks_for).
 template <int kAhead>
@@ -146,6 +147,10 @@ cascade_rows_kernel(Geom g, int first, int n_lists, HeldLists io, const int* hof
 // 91 / 88, ragged batch of 8 (8.6 GB) 47 / 46 / 45; half of 32 x 8K kept 125 with eight blocks of one row
 // ahead, 94 now.  At eight blocks per SM one row ahead is the better: the first two 6.2 and 5.4, four layers
 // of 8K 4.0 (two 4.5).
+// Steps of a cascade follow the same rule although the lists' rows come from the packed copy: cascades of 32
+// layers x 8K at 8 blocks and one row ahead throughout / 16 and two / the rule, in us, 128 rows per head 1717 /
+// 1760 / 1724, 512 2672 / 2678 / 2668, 2048 4727 / 4518 / 4625; 28 x 32K at 1024 3362 / 3395 / 3374; 16 heads x
+// 8K at 512 3798 / 3675 / 3694 (runs of one side differ by up to 1 %).
 struct Blocks {
   int per_head;
   bool two_ahead;
@@ -168,9 +173,9 @@ lava_status launch_compact(const Geom& g, int n_layers, const void* k, const voi
   const Blocks blocks = blocks_for(g, n_layers * g.batch);
   const int bph = blocks.per_head;
   dim3 grid(bph, g.n_kv_heads, n_layers * g.batch);
-  const cudaError_t e = launch_in_order(blocks.two_ahead ? compact_kernel<2> : compact_kernel<1>, grid, 256, 0, stream, g, (const char*)k,
-                                        (const char*)v, k_ls, v_ls, keep_idx, head_offsets, row_off,
-                                        (char*)k_out, (char*)v_out, bph);
+  const auto kernel = blocks.two_ahead ? compact_kernel<2> : compact_kernel<1>;
+  const cudaError_t e = launch_in_order(kernel, grid, 256, 0, stream, g, (const char*)k, (const char*)v, k_ls,
+                                        v_ls, keep_idx, head_offsets, row_off, (char*)k_out, (char*)v_out, bph);
   count_launches(1);
   return check_cuda(e, "compact_kv launch");
 }
@@ -185,7 +190,8 @@ lava_status launch_cascade_rows(const Geom& g, int n_lists, const HeldLists& io,
   cudaError_t e = cudaSuccess;
   for (int first = 0; first < problems && e == cudaSuccess; first += kMost) {
     const dim3 grid(bph, g.n_kv_heads, std::min(kMost, problems - first));
-    e = launch_in_order(blocks.two_ahead ? cascade_rows_kernel<2> : cascade_rows_kernel<1>, grid, 256, 0, stream, g, first, n_lists, io, hoff_new, k_old, v_old,
+    const auto kernel = blocks.two_ahead ? cascade_rows_kernel<2> : cascade_rows_kernel<1>;
+    e = launch_in_order(kernel, grid, 256, 0, stream, g, first, n_lists, io, hoff_new, k_old, v_old,
                         (const char*)k, (const char*)v, keep_idx, k_new, v_new, bph);
     count_launches(1);
   }

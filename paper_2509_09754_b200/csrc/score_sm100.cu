@@ -9,8 +9,8 @@
 //       one thread per row reads its TMEM lane and sums exp2 over the keys the query may see
 //       (Sec. 2: softmax over i <= j).  Work is dealt to CTAs in chunks of consecutive tiles of
 //       one head; a chunk's statistics leave the CTA once, through a publisher warp that also
-//       counts the head's published chunks.  Two more warps stream the chunk's V rows for the
-//       value norm (Theorem 1: max_k ||V[k]||_1).
+//       counts the head's published chunks.  A warp of its own loads the chunk's V rows and two
+//       more sum them for the value norm (Theorem 1: max_k ||V[k]||_1).
 //   pass 2 (scores)      S^T = K Q_g^T (rows = keys, columns = window queries)
 //       one thread per key: a_h[i] = (1/w) sum_t exp2(z - lse_t) per query head in registers,
 //       pooled over the token axis through shared memory, scaled by Vbar * c_hat, reduced with
@@ -32,6 +32,9 @@
 // latency: pass 2 waits for a head's statistics while pass 1 is held back by the lead.  The consumers are
 // bound by issue and dependent latencies rather than by the exponential unit: with half of the pass-2
 // exponentials as polynomials on the FMA pipe the call took 9 % longer.
+//
+// Polls are 128 ns apart; with 32 ns score calls take the same time (32 layers x 1K 51.5 us both, x 8K 263 and
+// 266, one layer of 8K 31.1 and 31.4).
 //
 // Every wait (mbarrier, head counters, chunk records, lead) is bounded in time; on expiry the
 // kernel sets LAVA_DEV_WAIT_EXPIRED, every role leaves at its next chunk, copies are drained, TMEM
@@ -838,6 +841,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
     // per warp and tile), pass 2 waited half of its time for the value norms.  Score calls in us with
     // that, and with this warp: 32 layers x 32K 1007 / 920, x 8K 276 / 247, 16 layers x 8K of head
     // dimension 64 126 / 115.  Four warps for the sums: 914, 244, 117, but 1 to 2 % slower with split groups.
+    // Split groups sum half of the pieces per unit and were not held up by them: 28 layers of 8K 204 / 204,
+    // of 32K 744 / 797, of 128K 3174 / 3320, ragged batch of 8 4507 / 4475.
     if (!p.vbar_in && lane == 0) {
       const uint64_t drop = policy_evict_first();
       int st = 0, n = 0;  // n: pieces issued
@@ -1101,18 +1106,21 @@ int sm100_first_half(const Geom& g) {
 
 // Tiles per chunk.  A boundary costs a reload of the query tile, a publication and a fold, but pass 2
 // can only start once a whole head is through pass 1, and what lies between the passes has to stay in
-// L2 (chunk + lead tiles of 32 KB in 148 CTAs).  Score call in us for 4 / 8 / 16 tiles: 32 layers x
-// 32K tokens 1079 / 981 / 1151, 32 x 8K 292 / 269 / 286, 28 layers x 128K (7 query heads per KV head)
-// 3527 / 3124 / 3290, ragged batch of 8 5434 / 5205 / 5405.  With split query groups the two halves share
-// their K rows, so twice the tiles fit in L2 and a boundary is dearer than its wait, unless heads are short:
-// 8 / 12 / 16 tiles, 28 layers x 128K 2850 / 2735 / 2765, x 32K 705 / 684 / 686, x 8K 207 / 212 / 213, x 3K
-// 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455 / 4400, one layer of it 199 / 192 / 203; with the
-// value rows' producer 12 / 16 / 20 tiles, 28 layers x 64K 1404 / 1374 / 1394, x 100001 2196 / 2121 / 2164.
-// With fewer than twelve tiles per CTA in
-// all, short chunks occupy more CTAs: one layer of 2K 31 / 41 / 41, of 8K 33 / 41 / 62; 4 against 8 tiles at
-// 10.4 tiles per CTA 51.6 / 56.4 (three layers of 8K) and 57 / 61 (24 of 1K), at 12.1 61.2 / 59.0 (28 of 1K),
-// at 13.8 60.3 / 57.1 (four of 8K) and 63.4 / 59.1 (32 of 1K).  So a layer's scores alone and in a call of many layers can differ
-// in their last bits (partial sums of 4, 8, 12 or 16 tiles).
+// L2 (chunk + lead tiles of 32 KB in 148 CTAs).  With split query groups the two halves share their K rows,
+// so twice the tiles fit in L2 and a boundary is dearer than its wait, unless heads are short.  With fewer
+// than twelve tiles per CTA in all, short chunks occupy more CTAs.  Score calls in us, while the value-norm
+// warps still loaded their own rows:
+//   4 / 8 / 16 tiles     32 layers x 32K tokens 1079 / 981 / 1151, 32 x 8K 292 / 269 / 286, one layer of 2K
+//                        31 / 41 / 41, of 8K 33 / 41 / 62
+//   split, 8 / 12 / 16   28 layers x 128K (7 query heads per KV head) 2850 / 2735 / 2765, x 32K 705 / 684 / 686,
+//                        x 8K 207 / 212 / 213, x 3K 111 / 120 / 120, ragged batch of 8 (4K to 16K) 4535 / 4455
+//                        / 4400, one layer of it 199 / 192 / 203
+// and since they have a producer:
+//   split, 12 / 16 / 20  28 layers x 64K 1404 / 1374 / 1394, x 100001 2196 / 2121 / 2164
+//   4 / 8 tiles          at 10.4 tiles per CTA 51.6 / 56.4 (three layers of 8K) and 57 / 61 (24 of 1K), at 12.1
+//                        61.2 / 59.0 (28 of 1K), at 13.8 60.3 / 57.1 (four of 8K) and 63.4 / 59.1 (32 of 1K)
+// So a layer's scores alone and in a call of many layers can differ in their last bits (partial sums of 4, 8,
+// 12 or 16 tiles).
 // Longer sequences take longer chunks, whatever is asked for: the lead that completing a head needs, one
 // chunk per round of CTAs that the head spans (see lead_slots), has to fit the chunk records.  8 tiles
 // serve sequences of up to 1.66 M tokens, 16 with split query groups the same.
