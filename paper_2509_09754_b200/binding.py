@@ -215,7 +215,7 @@ class LayerDesc:
                       self.v_stride_head, self.v_stride_tok, self.sm_scale, self.c_hat)
 
     # The structure of a call is kept until a field is set (1.4 us to fill, 0.2 to look up, of the 8 to 12
-    # that a call costs on the host; decode layer by layer is one call a layer).  Other threads may set fields
+    # that a call costs on the host; decode layer by layer is one call a layer).  Other threads may set attributes
     # or be inside a call meanwhile: every set leaves a new mark, a structure is stored with the mark that was
     # read before its fields were, and one that has been handed out is never written again.  The lengths'
     # address is looked up every time: a tensor may move its storage.
