@@ -841,8 +841,8 @@ lava_score_sm100_kernel(const __grid_constant__ CUtensorMap map_q,
     // per warp and tile), pass 2 waited half of its time for the value norms.  Score calls in us with
     // that, and with this warp: 32 layers x 32K 1007 / 920, x 8K 276 / 247, 16 layers x 8K of head
     // dimension 64 126 / 115.  Four warps for the sums: 914, 244, 117, but 1 to 2 % slower with split groups.
-    // Split groups sum half of the pieces per unit and were not held up by them: 28 layers of 8K 204 / 204,
-    // of 32K 744 / 797, of 128K 3174 / 3320, ragged batch of 8 4507 / 4475.
+    // Split groups sum half of the pieces per unit and gain little: 28 layers of 12K 289 / 287, of 32K 773 /
+    // 765, of 64K 1627 / 1584, of 128K 3174 / 3179, ragged batch of 8 4423 / 4358.
     if (!p.vbar_in && lane == 0) {
       const uint64_t drop = policy_evict_first();
       int st = 0, n = 0;  // n: pieces issued
@@ -1141,9 +1141,13 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
 // Slots pass 1 leads pass 2 by beyond what head completion needs.  4 / 8 / 12 / 16 slots with chunks of
 // eight tiles: 1300 / 1002 / 981 / 1134 us at 32 layers x 32K; shorter leads let pass 2 wait for the
 // statistics, longer ones lose its K tiles from L2 (0 % more DRAM reads than K and V at 8, 3 % at 12, 15 % at 16).
-int lead_extra_for() {
+// Chunks of sixteen (split query groups) take longer to complete and, while a head spans less than a round of
+// CTAs, get nothing for its completion: 12 / 20 / 28 slots, 28 layers x 128K 3555 / 3197 / 3201 (chunks of twelve
+// 3510), x 110000 2746 / 2681 / 2673, x 64K 1628 / 1620 / 1545, x 40000 973 / 977 / 974, 16 layers x 180000 2668 /
+// 2671 / 2695, one layer of 128K 153 / 154 / 159.
+int lead_extra_for(int chunk_tiles) {
   const int forced = options().score_lead_tiles;
-  return forced >= 0 ? forced : 12;
+  return forced >= 0 ? forced : chunk_tiles >= 16 ? 20 : 12;
 }
 
 }  // namespace
@@ -1313,7 +1317,7 @@ lava_status launch_score_sm100(const Geom& g, int n_layers, const void* q, const
   // a head of cph chunks has at most 128 R cph keys, hence at most 128 R cph / out_keys + 1 tiles
   // in pass 2, spread evenly over the chunks
   p.chunk_slots = ceil_div(lay.chunk_tiles * kTile, lay.out_keys) + 2;
-  p.lead_extra = lead_extra_for();
+  p.lead_extra = lead_extra_for(lay.chunk_tiles);
   p.g0 = sm100_first_half(g);
   p.split = p.g0 ? 1 : 0;
   p.wait_cycles = options().wait_limit_cycles;

@@ -43,11 +43,11 @@ def test_chunks_as_short_as_wanted_stall_there():
     assert run([1200000], 1, 1, 1, 32, 3, _chunk_tiles(1200000, 1, 8), SMS, 12)
 
 
-@pytest.mark.parametrize("wanted", [12, 16])
+@pytest.mark.parametrize("wanted,extra", [(12, 12), (16, 12), (16, 20)])
 @pytest.mark.parametrize("factor", [0.5, 1.0, 1.01, 1.6])
-def test_every_wait_ends_with_the_chunks_of_split_groups(wanted, factor):
+def test_every_wait_ends_with_the_chunks_of_split_groups(wanted, extra, factor):
     n = int(factor * ((MAX_LEAD_CHUNKS - 1) * SMS >> 1) * wanted * TILE)
     for heads, radius in ((1, 3), (2, 31)):
-        assert run([n], 1, heads, 1, 32, radius, _chunk_tiles(n, 1, wanted), SMS, extra=12)
-    for lens in ([8193], [32768, 100], [32769, 9000], [131072]):
-        assert run(lens, 2, 4, 1, 32, 3, _chunk_tiles(max(lens), 1, wanted), SMS, extra=12)
+        assert run([n], 1, heads, 1, 32, radius, _chunk_tiles(n, 1, wanted), SMS, extra)
+    for lens in ([8193], [32768, 100], [32769, 9000], [131072], [151552], [151553]):
+        assert run(lens, 2, 4, 1, 32, 3, _chunk_tiles(max(lens), 1, wanted), SMS, extra)
