@@ -199,7 +199,8 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   // wide loops then cost more than their loads save (32 layers of 1K, first run after a flush: 15.1 us
   // wide, 13.6 narrow; 28 layers of 128K 35 wide, 44 narrow).  The keys of a small part are all on their way
   // to shared memory at once: one ahead, each of a thread's four or more fetches waited for the one before it
-  // (28 layers of 4000 tokens after a flush 16.2, now 14.3).
+  // (28 layers of 4000 tokens after a flush 16.2, now 14.3).  A thread that has one fetch only keeps it in
+  // registers on its way (16 layers x 8 sequences of 200 to 800 tokens after a flush 8.5, by way of a copy 9.4).
   const bool wide = n_vec > 8 * kThreads;
 
   // ---- radix passes: find tau and the number of ties to take -------------------------------
@@ -212,7 +213,8 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
   const unsigned list_up_to = per + 3 > 4 * kListVec ? 0u : min((unsigned)kMaxCandidates, share);
   if (k_sel > 0) {
     unsigned* my_copy = copies + (lane & (kCopies - 1));
-    if (!wide) {
+    const bool staged = n_vec > kThreads && !wide;
+    if (staged) {
 #pragma unroll 1
       for (int v = threadIdx.x; v < min(n_vec, kCacheVec); v += kThreads) {
         if (v == ragged0 || v == ragged1) cache[v] = fetch(v);
@@ -227,7 +229,7 @@ __device__ __forceinline__ void select_problem(SelectShared& sh, unsigned char* 
       auto tally = [&](unsigned key) {
         if (((key ^ digits) & mask) == 0u) atomicAdd(&my_copy[((key >> shift) & dmask) * kCopies], 1u);
       };
-      auto pick = [&](int v) { return (pass > 0 || !wide) && v < kCacheVec ? cache[v] : fetch(v); };
+      auto pick = [&](int v) { return (pass > 0 || staged) && v < kCacheVec ? cache[v] : fetch(v); };
       int v = threadIdx.x;
       if (wide) {
         auto sweep = [&](auto first) {  // every key counts in the first pass
