@@ -1144,7 +1144,8 @@ int chunk_tiles_for(const Geom& g, int n_layers) {
 // Chunks of sixteen (split query groups) take longer to complete and, while a head spans less than a round of
 // CTAs, get nothing for its completion: 12 / 20 / 28 slots, 28 layers x 128K 3555 / 3197 / 3201 (chunks of twelve
 // 3510), x 110000 2746 / 2681 / 2673, x 64K 1628 / 1620 / 1545, x 40000 973 / 977 / 974, 16 layers x 180000 2668 /
-// 2671 / 2695, one layer of 128K 153 / 154 / 159.
+// 2671 / 2695, one layer of 128K 153 / 154 / 159.  The longer lead reads 1.47 GB from DRAM where 12 slots read 1.20
+// (four layers of 128K, K + V 1.07).
 int lead_extra_for(int chunk_tiles) {
   const int forced = options().score_lead_tiles;
   return forced >= 0 ? forced : chunk_tiles >= 16 ? 20 : 12;
